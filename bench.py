@@ -63,34 +63,35 @@ CONFIG_ORDER = ["random-undirected-n8-m16", "grid-3x6", "random-directed-n20-m34
 # launches) the bench pins per workload and kernel, from shape sweeps on
 # GB300, so that the timed launches are the ones the instruction counts below
 # were taken from (--autotune lets the autotuner choose instead).  prune 2 =
-# prune-aware prefix arcs; launches 2 = the first launch resolves what the
-# prune can and defers the items left to walk to the second.
+# prune-aware prefix arcs; launches 2 = merged: items whose prefixes leave
+# the same network are walked once.
 SHAPES = {
-    "random-undirected-n24-m40": {"fused": (9, 256, 2, 2, 2), "r_only": (9, 128, 2, 0, 1)},
-    "random-directed-n20-m34": {"fused": (7, 192, 2, 0, 2), "r_only": (7, 128, 2, 0, 2)},
-    "grid-3x6": {"fused": (5, 128, 1, 0, 1), "r_only": (5, 64, 1, 0, 1)},
+    "random-undirected-n24-m40": {"fused": (8, 128, 2, 2, 2), "r_only": (8, 160, 2, 2, 2)},
+    "random-directed-n20-m34": {"fused": (7, 256, 2, 0, 2), "r_only": (7, 256, 2, 0, 2)},
+    "grid-3x6": {"fused": (1, 128, 2, 2, 2), "r_only": (1, 192, 2, 2, 2)},
 }
 
 # Per generated kernel source (first 16 hex digits of its SHA-256, as
 # pbat_kernel_source returns it): warp instructions executed per state
-# (smsp__inst_executed.sum of one launch / 2^m) -- the per-unit figure of the
+# (smsp__inst_executed.sum of the enumeration's launches / 2^m) -- the per-unit figure of the
 # issue-rate roofline -- and DRAM bytes per launch (dram__bytes_read.sum +
 # dram__bytes_write.sum), from one ncu capture of that launch (bench.py
 # --probe with the same workload and shape; summaries in profiles/).  A
 # kernel whose source has changed since has no entry, and its roofline
 # fraction is reported as null.
 COUNTS = {
-    # 24 nodes, 40 arcs: fused (L 9, 256 threads, prune 2, occupancy 2, its two launches
-    # summed) and R-only (L 9, 128, 2, 0, one launch; four walk arcs unrolled)
-    "b080d3e5392bd6e0": (12414443516 / 2**40, 1675264, "profiles/bs_kernel_grad_undirected24x40.md"),
-    "0871ac197eac0d1d": (5902219352 / 2**40, 77568, "profiles/bs_kernel_undirected24x40.md"),
-    # directed, 20 nodes, 34 arcs: fused (7, 192, 2, 0, two launches) and R-only
-    # (7, 128, 2, 0, two launches)
-    "8dff10689adf9178": (22081741 / 2**34, 98304, "profiles/bs_kernel_grad_directed20x34.md"),
-    "fc32829a911d714a": (16006400 / 2**34, 74752, "profiles/bs_kernel_directed20x34.md"),
-    # 3x6 grid: fused (5, 128, 1, 0, 1) and R-only (5, 64, 1, 0, 1)
-    "23c0191c742fbc75": (15952825 / 2**27, 91904, "profiles/bs_kernel_grad_grid3x6.md"),
-    "96d74f15c7df157a": (8078163 / 2**27, 51456, "profiles/bs_kernel_grid3x6.md"),
+    # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
+    "12d89125041c92dd": (52494086 / 2**40, 5643776, "profiles/bs_kernel_grad_undirected24x40.md"),
+    # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
+    "f73d4ef71d415742": (20249019 / 2**40, 559360, "profiles/bs_kernel_undirected24x40.md"),
+    # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
+    "8dccfa2a141e159a": (1023216 / 2**34, 249344, "profiles/bs_kernel_grad_directed20x34.md"),
+    # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
+    "753137a3382ba2aa": (786202 / 2**34, 99840, "profiles/bs_kernel_directed20x34.md"),
+    # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
+    "64f7b6748b6b3400": (1631106 / 2**27, 469248, "profiles/bs_kernel_grad_grid3x6.md"),
+    # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
+    "2d85f5eebf446005": (1037543 / 2**27, 148224, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

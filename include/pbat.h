@@ -90,11 +90,14 @@ typedef struct pbat_options {
                            module takes it as its launch bounds (128 threads, k blocks;
                            0 and -1 = 4 blocks).  Results do not depend on it. */
   int launches;         /* bit-sliced single-network kernels with the prune on: 1 = one
-                           launch; 2 = two launches, the first resolving what the prune can
-                           and deferring the work items left to walk, the second walking
-                           them (at most 2^24 items, else one launch); 0 (default) = two
-                           for the fused kernel with 2^18 to 2^24 items, else one, or the
-                           autotuner's choice when it runs.  Results do not depend on it. */
+                           launch, every work item that the prune leaves walked by itself;
+                           2 = merged: a launch that resolves what the prune can and puts the
+                           items left into classes whose prefixes leave the same network, one
+                           that walks each class once, and for the gradient one that adds the
+                           prefix arcs' (at most 2^24 items and 2^18 classes, else one
+                           launch); 0 (default) = merged from 2^12 items on, else one launch,
+                           or the autotuner's choice when it runs.  Results do not depend on
+                           it. */
   int range_bits;       /* 0 (default) = whole space.  Otherwise only the states whose
                            first range_bits coordinates, read as an integer, lie in
                            [range_lo, range_hi) -- the divisions range_lo..range_hi-1 of
@@ -105,13 +108,15 @@ typedef struct pbat_options {
   double time_budget_s; /* > 0: the device stops after this many seconds and the call
                            returns PBAT_ETIMEOUT; 0 = no limit */
   uint64_t stats[8];    /* out, filled by the last call that took these options:
-                           [0] states enumerated by walking, [1] states resolved by the
-                           prune, [2] bytes copied host -> device, [3] bytes copied
+                           [0] states enumerated by walking (of a class of merged items: one
+                           item's), [1] the other states, resolved by the prune or with
+                           their class, [2] bytes copied host -> device, [3] bytes copied
                            device -> host, [4] summed device time in ns of the
-                           enumeration kernel over the launches since the last read (CUDA
-                           events on the launch stream), [5] kernels launched (one per
-                           bit-sliced launch; the frontier kernel adds a reduce), [6] work
-                           items per launch, [7] launches timed in [4] */
+                           enumeration kernels over the launches since the last read (CUDA
+                           events on the launch stream), [5] kernels launched (bit-sliced:
+                           one per enumeration, merged two or with the gradient three; the
+                           frontier kernel adds a reduce), [6] work items per enumeration,
+                           [7] enumerations timed in [4] */
 } pbat_options;
 
 /* Fill *opt with the defaults above. */

@@ -29,7 +29,9 @@ namespace pbat {
 // Host mirror of BsParams in the kernel source (same field order and types).
 struct BsParamsHost {
   unsigned long long task_lo, n_tasks, budget_ns;
-  int prune, nlev, ex_shift, pad;
+  int prune, nlev, ex_shift;
+  int nlev_hi, mass_exp, slots_log2;
+  int hi_bits[10], hi_off[10];
   int lev_bits[10];
   int lev_off[10];
   unsigned long long thw[32];
@@ -42,8 +44,8 @@ struct BsParamsHost {
 struct JitEntry {
   cudaLibrary_t lib = nullptr;
   cudaKernel_t kernel = nullptr;
-  // the two launches of a two-launch run (single-network kernels only)
-  cudaKernel_t kernel_p1 = nullptr, kernel_p2 = nullptr;
+  // the launches of a merged run (single-network kernels only; p3: fused)
+  cudaKernel_t kernel_p1 = nullptr, kernel_p2 = nullptr, kernel_p3 = nullptr;
   int regs = 0;
 };
 static std::mutex g_jit_mu;
@@ -159,6 +161,10 @@ static int jit_compile(const std::string& src, const DeviceInfo& dev, const char
     cudaGetLastError();
     e.kernel_p1 = e.kernel_p2 = nullptr;
   }
+  if (cudaLibraryGetKernel(&e.kernel_p3, e.lib, (std::string(kname) + "_p3").c_str()) != cudaSuccess) {
+    cudaGetLastError();
+    e.kernel_p3 = nullptr;
+  }
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, (const void*)e.kernel) == cudaSuccess) e.regs = fa.numRegs;
   else cudaGetLastError();
@@ -176,6 +182,14 @@ struct BsGradParamsHost {
   dd inv_p[64], inv_q[64];
 };
 
+// Host mirror of BsFoldParams in the kernel source.
+struct BsFoldParamsHost {
+  unsigned long long p[10];
+  unsigned long long wlow[31];
+  unsigned long long wmid[31];
+  unsigned long long mid[32];
+};
+
 struct BsLaunch {
   BsPlan plan;
   BsParamsHost P;
@@ -190,9 +204,16 @@ struct BsLaunch {
   int nthr = 128;
   size_t smem = 0;
   int per_sm = 1;                     // resident blocks per SM: one-launch kernel
-  int per_sm1 = 1, per_sm2 = 1;       // the two launches of a two-launch run
-  size_t smem1 = 0;                   // shared memory of the first of two fused launches
+  // merged runs
+  int per_sm1 = 1, per_sm2 = 1, per_sm3 = 1;
+  bool unmergeable = false;           // its classes did not fit the table before
+  std::string key;                    // of the plan cache
+  BsFoldParamsHost F;
+  std::vector<unsigned long long> mtab;  // [128] subset sums, [32] mid pattern masses, 128 bits each
 };
+
+constexpr int kMergeThreads = 128;    // BS_MERGE_NTHR
+constexpr int kMaxSlotsLog2 = 18;     // class table of a merged run
 
 // out[v] = product over x < n of (bit x of v ? p : 1 - p) of arc arcs[x], for
 // every v < 2^n, built by doubling: two double-double products per entry.
@@ -235,18 +256,19 @@ static int walk_unroll_bits(const BsPlan& bp) {
 }
 
 static std::string bs_source(const GraphIn& g, const BsPlan& bp, int nthr) {
-  char defs[700];
+  char defs[800];
   const unsigned lane_mask = bp.ell >= 5 ? 0xffffffffu : ((1u << (1 << bp.ell)) - 1u);
   snprintf(defs, sizeof defs,
            "#define BS_M %d\n#define BS_ELL %d\n#define BS_TB %d\n#define BS_L %d\n#define BS_D %d\n"
            "#define BS_NTHR %d\n#define BS_WALK0 %d\n#define BS_TOP %d\n#define BS_NCORE %d\n"
            "#define BS_LANE_MASK 0x%08xu\n#define BS_FULL_COUNTS 0x%016llxull\n#define BS_GRAD %d\n"
            "#define BS_ACC_REG %d\n#define BS_IN_BITS %d\n#define BS_THR_MASK 0x%08xu\n"
-           "#define BS_MINB %d\n#define BS_PEX_MASK 0x%016llxull\n",
+           "#define BS_MINB %d\n#define BS_PEX_MASK 0x%016llxull\n#define BS_MERGE %d\n"
+           "#define BS_NSIG %d\n#define BS_LOW %d\n#define BS_MID %d\n",
            g.m, bp.ell, bp.tb, bp.L, bp.d, nthr, bp.ell + bp.tb, bp.ell + bp.tb + bp.L, bp.ncore,
            lane_mask, full_counts(bp.ell), bp.grad ? 1 : 0, acc_in_registers(bp) ? 1 : 0,
            walk_unroll_bits(bp), bp.tb >= 5 ? 0xffffffffu : ((1u << (1 << bp.tb)) - 1u), bp.minb,
-           bp.pex);
+           bp.pex, bp.nsig >= 0 ? 1 : 0, bp.nsig, bp.low, bp.mid);
   const std::string tmpl = kBsTemplate;
   const size_t cut = tmpl.find("//@@GENERATED@@");
   // only this plan's kernel: the other kernel's section is left out, so that
@@ -258,7 +280,7 @@ static std::string bs_source(const GraphIn& g, const BsPlan& bp, int nthr) {
     if (bp.grad) tail.erase(r0, f0 - r0);
     else tail.erase(f0, f1 + 6 - f0);
   }
-  return std::string(defs) + tmpl.substr(0, cut) + bp.gen + tail;
+  return std::string(defs) + tmpl.substr(0, cut) + bp.gen + bp.gen_sig + tail;
 }
 
 // Generated source for a network (no device needed); see pbat_kernel_source.
@@ -287,7 +309,8 @@ struct BsCached {
   JitEntry jit;
   size_t smem = 0;   // shared memory the kernel attribute was set for
   int per_sm = 0;    // resident blocks per SM at that size (one-launch kernel)
-  int per_sm1 = 0, per_sm2 = 0;   // the two launches of a two-launch run
+  int per_sm1 = 0, per_sm2 = 0, per_sm3 = 0;   // the launches of a merged run
+  bool unmergeable = false;   // more classes than the table holds: one launch from then on
 };
 static std::mutex g_bsplan_mu;
 static std::map<std::string, BsCached> g_bsplan;
@@ -297,13 +320,77 @@ static std::string bs_plan_key(const GraphIn& g, const double* p, bool grad, con
   std::string k;
   auto put = [&](long long v) { k.append((const char*)&v, sizeof v); };
   put(device); put(g.n); put(g.m); put(g.directed); put(g.source); put(g.sink); put(grad);
-  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(nthr); put(o.prune == 2);
+  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(nthr); put(o.prune);
   put(std::max(0, o.occupancy));
   k.append((const char*)g.tail, sizeof(int32_t) * g.m);
   k.append((const char*)g.head, sizeof(int32_t) * g.m);
   if (grad)
     for (int a = 0; a < g.m; ++a) k.push_back(bs_walk_ok(p, a) ? '1' : '0');
   return k;
+}
+
+// Tables of a merged run: masses of the prefix arcs above a block by level,
+// subset sums and masses of the block's low and mid patterns, and for the
+// fold each arc's p and the masses of the arcs folded after it.
+static void merge_tables(const double* p, const pbat_options& o, int m, BsLaunch& bl) {
+  const BsPlan& bp = bl.plan;
+  BsParamsHost& P = bl.P;
+  const int top = bp.ell + bp.tb + bp.L, blk = bp.low + bp.mid, nhi = bp.d - blk;
+  const int* low = bp.perm.data() + top;
+  const int* mid = low + bp.low;
+  const int max_bits = 6;
+  P.nlev_hi = (nhi + max_bits - 1) / max_bits;
+  for (int l = 0, sh = 0; l < P.nlev_hi; ++l) {
+    const int bits = nhi / P.nlev_hi + (l < nhi % P.nlev_hi ? 1 : 0);
+    P.hi_bits[l] = bits;
+    P.hi_off[l] = (int)bl.ptab.size();
+    dd tab[1 << max_bits];
+    product_table(p, bp.perm.data() + top + blk + sh, bits, tab);
+    for (int v = 0; v < (1 << bits); ++v) bl.ptab.push_back(to_mx(tab[v]));
+    sh += bits;
+  }
+  // the enumerated mass is at most 2^-mass_exp
+  const double mass = range_mass(m, p, o);
+  P.mass_exp = mass > 0.0 && mass < 1.0 ? std::max(0, -(ilogb(mass) + 1)) : 0;
+  bl.mtab.assign(2 * (128 + 32), 0ull);
+  dd w[32];
+  product_table(p, low, bp.low, w);
+  uint128_host f[32];
+  for (int j = 0; j < 32; ++j) {
+    u128 v{0, 0};
+    if (j < (1 << bp.low)) v = to_fixed127(w[j]);
+    f[j] = ((uint128_host)v.hi << 64) | v.lo;
+  }
+  for (int b = 0; b < 8; ++b) {
+    uint128_host sum[16];
+    sum[0] = 0;
+    for (int v = 0; v < 16; ++v) {
+      if (v) sum[v] = sum[v & (v - 1)] + f[4 * b + __builtin_ctz((unsigned)v)];
+      bl.mtab[2 * (16 * b + v)] = (unsigned long long)sum[v];
+      bl.mtab[2 * (16 * b + v) + 1] = (unsigned long long)(sum[v] >> 64);
+    }
+  }
+  product_table(p, mid, bp.mid, w);
+  memset(&bl.F, 0, sizeof bl.F);
+  for (int j = 0; j < (1 << bp.mid); ++j) {
+    const u128 v = to_fixed127(w[j]);
+    bl.mtab[2 * (128 + j)] = v.lo;
+    bl.mtab[2 * (128 + j) + 1] = v.hi;
+    bl.F.mid[j] = fixed_u64(w[j], 63);
+  }
+  if (!bp.grad) return;
+  // absent low arcs (blocks of fewer than 32 bits) have p = 0
+  for (int part = 0; part < 2; ++part) {
+    const int* arcs = part ? mid : low;
+    const int n = part ? bp.mid : bp.low;
+    unsigned long long* out = part ? bl.F.wmid : bl.F.wlow;
+    for (int b = 0, at = 0; b < 5; at += 16 >> b, ++b) {
+      if (b < n) bl.F.p[5 * part + b] = fixed_u64(dd_make(p[arcs[b]]), 63);
+      const int above = std::max(0, n - b - 1);
+      product_table(p, arcs + b + 1, above, w);
+      for (int v = 0; v < (1 << above); ++v) out[at + v] = fixed_u64(w[v], 63);
+    }
+  }
 }
 
 // Compile the kernels of several option sets ahead of bs_prepare, on host
@@ -333,7 +420,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
                const DeviceInfo& dev, BsLaunch& bl) {
   bl.nthr = o.block_threads > 0 ? o.block_threads : 128;
   int rc;
-  const std::string key = bs_plan_key(g, p, grad, o, bl.nthr, dev.device);
+  const std::string key = bl.key = bs_plan_key(g, p, grad, o, bl.nthr, dev.device);
   bool cached = false;
   {
     std::lock_guard<std::mutex> lk(g_bsplan_mu);
@@ -341,6 +428,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     if (it != g_bsplan.end()) {
       bl.plan = it->second.plan;
       bl.jit = it->second.jit;
+      bl.unmergeable = it->second.unmergeable;
       cached = true;
     }
   }
@@ -375,6 +463,10 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
   }
   P.task_lo = lo;
   P.n_tasks = hi - lo;
+  // merged runs: a table of twice the items, or one slot per signature
+  while (P.slots_log2 < kMaxSlotsLog2 && P.slots_log2 < bp.nsig &&
+         (1ull << P.slots_log2) < 2 * P.n_tasks)
+    ++P.slots_log2;
   // prefix masses: the d prefix arcs in levels of at most 6 bits (fused
   // kernel: the per-arc excluded tables stay small) or 8 bits (R only); each
   // entry is the double-double product over the level's arcs, rounded to
@@ -408,6 +500,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     sh += bits;
   }
   if (bl.ptab.empty()) bl.ptab.push_back(to_mx(dd_make(1.0)));
+  if (bp.nsig >= 0) merge_tables(p, o, m, bl);
   // lane tables: byte position b, value v -> lane mass (scale 2^62) and the
   // counts of its set lanes by lane popcount class, packed in fields of
   // 8, 11, 12, 12, 11, 8 bits
@@ -427,13 +520,15 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     }
   }
   const int L_in = std::min(bp.L, walk_unroll_bits(bp)), L_out = bp.L - L_in;
+  // the walking launch of a merged run: each warp's counts below the prefix
+  const size_t rel_bytes = bp.nsig >= 0 ? (size_t)(bl.nthr / 32) * (top + 1) * 8 : 0;
   if (!grad) {
     bl.wmid.resize((size_t)1 << bp.L);
     std::vector<dd> wt((size_t)1 << bp.L);
     product_table(p, bp.perm.data() + bp.ell + bp.tb, bp.L, wt.data());
     for (int gi = 0; gi < (1 << bp.L); ++gi) bl.wmid[gi] = fixed_u64(wt[gi], 63);
     bl.smem = (size_t)(4 * 256 * 2 + (1 << bp.L) + (bp.L + 1) * bl.nthr) * 8 +
-              (size_t)(bl.nthr / 32) * 24 + (size_t)(m + 1) * 8;
+              (size_t)(bl.nthr / 32) * 24 + (size_t)(m + 1) * 8 + rel_bytes;
   } else {
     // fused kernel: thread-pattern masses, 128-bit walk masses, fixed-point
     // excluded-arc masses, reciprocals of the walk arcs' p and 1 - p
@@ -472,7 +567,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
       bl.Q.inv_q[k] = dd_recip_dd(dd_one_minus(pk));
     }
     bl.smem = (size_t)(4 * 256 * 2 + 2 * (1 << bp.L) + 4 * 256 + (bp.L + 1) * bl.nthr) * 8 +
-              (size_t)std::max(L_out, 1) * bl.nthr * 16 + (size_t)(m + 1) * 8;
+              (size_t)std::max(L_out, 1) * bl.nthr * 16 + (size_t)(m + 1) * 8 + rel_bytes;
   }
   if (bl.smem > (size_t)dev.smem_optin)
     return fail(PBAT_ERANGE, "bit-sliced kernel needs %zu B of shared memory", bl.smem);
@@ -485,29 +580,28 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
       bl.per_sm = it->second.per_sm;
       bl.per_sm1 = it->second.per_sm1;
       bl.per_sm2 = it->second.per_sm2;
-      bl.smem1 = grad ? (size_t)(m + 1) * 8 : bl.smem;
+      bl.per_sm3 = it->second.per_sm3;
       return PBAT_OK;
     }
   }
   // shared-memory attribute and resident blocks per SM of each entry point
-  // (the first of two fused launches needs only the N_k counts)
-  bl.smem1 = grad ? (size_t)(m + 1) * 8 : bl.smem;
-  auto setup = [&](cudaKernel_t k, size_t smem, int* per_sm) -> int {
+  auto setup = [&](cudaKernel_t k, int nthr, size_t smem, int* per_sm) -> int {
     *per_sm = 1;
     if (!k) return PBAT_OK;
     cudaError_t e = cudaFuncSetAttribute((const void*)k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return fail(PBAT_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, (const void*)k, bl.nthr, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, (const void*)k, nthr, smem);
     if (e != cudaSuccess || *per_sm < 1) {
       cudaGetLastError();
       *per_sm = 1;
     }
     return PBAT_OK;
   };
-  if ((rc = setup(bl.jit.kernel, bl.smem, &bl.per_sm)) ||
-      (rc = setup(bl.jit.kernel_p1, bl.smem1, &bl.per_sm1)) ||
-      (rc = setup(bl.jit.kernel_p2, bl.smem, &bl.per_sm2)))
+  if ((rc = setup(bl.jit.kernel, bl.nthr, bl.smem, &bl.per_sm)) ||
+      (rc = setup(bl.jit.kernel_p1, kMergeThreads, 0, &bl.per_sm1)) ||
+      (rc = setup(bl.jit.kernel_p2, bl.nthr, bl.smem, &bl.per_sm2)) ||
+      (rc = setup(bl.jit.kernel_p3, kMergeThreads, 0, &bl.per_sm3)))
     return rc;
   std::lock_guard<std::mutex> lk(g_bsplan_mu);
   auto it = g_bsplan.find(key);
@@ -516,27 +610,66 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     it->second.per_sm = bl.per_sm;
     it->second.per_sm1 = bl.per_sm1;
     it->second.per_sm2 = bl.per_sm2;
+    it->second.per_sm3 = bl.per_sm3;
   }
   return PBAT_OK;
 }
 
 // Launch with the device copies of the tables (see bs_tables for the order).
-// phase 0: the one-launch kernel; 1, 2: the two launches of a two-launch run.
-cudaError_t bs_launch(const BsLaunch& bl, int grid, cudaStream_t st, const unsigned long long* d_lane,
-                      const unsigned long long* d_thr, const unsigned long long* d_wmid,
-                      const void* d_ptab, const void* d_ptab_ex, const DevWork& W, int phase) {
+// phase 0: the one-launch kernel; 1 to 3: the launches of a merged run.
+cudaError_t bs_launch(const BsLaunch& bl, int grid, cudaStream_t st, const BsTables& T, const DevWork& W,
+                      int phase, int split_log2) {
   const BsParamsHost& P = bl.P;
-  const cudaKernel_t k = phase == 1 ? bl.jit.kernel_p1 : phase == 2 ? bl.jit.kernel_p2 : bl.jit.kernel;
+  const cudaKernel_t k = phase == 1 ? bl.jit.kernel_p1 : phase == 2 ? bl.jit.kernel_p2
+                       : phase == 3 ? bl.jit.kernel_p3 : bl.jit.kernel;
   if (!k) return cudaErrorInvalidDeviceFunction;
-  if (bl.plan.grad) {
-    const BsGradParamsHost& Q = bl.Q;
-    void* args[] = {(void*)&P, (void*)&Q, (void*)&d_lane, (void*)&d_thr, (void*)&d_wmid,
-                    (void*)&d_ptab, (void*)&d_ptab_ex, (void*)&W};
-    return cudaLaunchKernel((const void*)k, dim3(grid), dim3(bl.nthr), args,
-                            phase == 1 ? bl.smem1 : bl.smem, st);
+  // the later launches of a merged run may start while the one before drains
+  // (they wait for its results, see bs_wait_previous in the kernel source)
+  cudaLaunchAttribute early{};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(phase == 1 || phase == 3 ? kMergeThreads : bl.nthr);
+  c.dynamicSmemBytes = phase == 1 || phase == 3 ? 0 : bl.smem;
+  c.stream = st;
+  c.attrs = &early;
+  c.numAttrs = phase >= 2 ? 1 : 0;
+  if (phase == 1) {
+    void* args[] = {(void*)&P, (void*)&T.ptab, (void*)&T.merge, (void*)&split_log2, (void*)&W};
+    return cudaLaunchKernelExC(&c, (const void*)k, args);
   }
-  void* args[] = {(void*)&P, (void*)&d_lane, (void*)&d_wmid, (void*)&d_ptab, (void*)&W};
-  return cudaLaunchKernel((const void*)k, dim3(grid), dim3(bl.nthr), args, bl.smem, st);
+  if (phase == 3) {
+    void* args[] = {(void*)&P, (void*)&bl.F, (void*)&T.ptab, (void*)&W};
+    return cudaLaunchKernelExC(&c, (const void*)k, args);
+  }
+  if (bl.plan.grad) {
+    void* args[] = {(void*)&P, (void*)&bl.Q, (void*)&T.lane, (void*)&T.thr, (void*)&T.walk,
+                    (void*)&T.ptab, (void*)&T.ptab_ex, (void*)&W};
+    return cudaLaunchKernelExC(&c, (const void*)k, args);
+  }
+  void* args[] = {(void*)&P, (void*)&T.lane, (void*)&T.walk, (void*)&T.ptab, (void*)&W};
+  return cudaLaunchKernelExC(&c, (const void*)k, args);
+}
+
+// A merged run met more classes than its table holds: this plan runs its
+// items one by one from now on (the network's structure decides it).
+void bs_mark_unmergeable(const BsLaunch& bl) {
+  std::lock_guard<std::mutex> lk(g_bsplan_mu);
+  auto it = g_bsplan.find(bl.key);
+  if (it != g_bsplan.end()) it->second.unmergeable = true;
+}
+// What a merged run of this plan needs; slots 0: it cannot be merged.
+BsMerge bs_merge(const BsLaunch& bl) {
+  BsMerge r{};
+  const int blk = bl.plan.low + bl.plan.mid;
+  r.blocks = bl.P.n_tasks >> blk;
+  if (bl.plan.nsig < 0 || bl.unmergeable || !bl.jit.kernel_p1 || bl.P.n_tasks > (1ull << 24) ||
+      r.blocks > (1ull << 14) || r.blocks == 0)
+    return r;
+  r.slots = 1ull << bl.P.slots_log2;
+  r.hist = (bl.plan.d + 2) & ~1;   // BS_HIST
+  return r;
 }
 
 // accessors used by the engine
@@ -546,7 +679,7 @@ unsigned long long bs_item_states(const BsLaunch& bl) {
   return 1ull << (bl.plan.ell + bl.plan.tb + bl.plan.L);
 }
 int bs_per_sm(const BsLaunch& bl, int phase) {
-  return phase == 1 ? bl.per_sm1 : phase == 2 ? bl.per_sm2 : bl.per_sm;
+  return phase == 1 ? bl.per_sm1 : phase == 2 ? bl.per_sm2 : phase == 3 ? bl.per_sm3 : bl.per_sm;
 }
 int bs_nthr(const BsLaunch& bl) { return bl.nthr; }
 const std::vector<unsigned long long>& bs_lane_tab(const BsLaunch& bl) { return bl.lane_tab; }
@@ -555,6 +688,7 @@ const std::vector<unsigned long long>& bs_wmid(const BsLaunch& bl) {
 }
 const std::vector<unsigned long long>& bs_thr_tab(const BsLaunch& bl) { return bl.thr_tab; }
 const std::vector<MxHost>& bs_ptab(const BsLaunch& bl) { return bl.ptab; }
+const std::vector<unsigned long long>& bs_mtab(const BsLaunch& bl) { return bl.mtab; }
 const std::vector<MxHost>& bs_ptab_ex(const BsLaunch& bl) { return bl.ptab_ex; }
 bool bs_grad(const BsLaunch& bl) { return bl.plan.grad; }
 
@@ -563,13 +697,16 @@ bool bs_grad(const BsLaunch& bl) { return bl.plan.grad; }
 // with p in [2^-20, 1 - 2^-20] (their sums carry the arc's own factor), A - B
 // for the other prefix arcs (masses without the arc, working minus failed),
 // and A for lane and thread arcs (exact pair differences).
-void bs_finish_grad(const BsLaunch& bl, const dd* acc, int m, double* g_internal) {
+// A merged run sums the prefix arcs of a block as pair differences too.
+void bs_finish_grad(const BsLaunch& bl, const dd* acc, int m, bool merged, double* g_internal) {
   const BsPlan& bp = bl.plan;
   const int walk0 = bp.ell + bp.tb, top = walk0 + bp.L;
   for (int k = 0; k < m; ++k) {
     const dd a = acc[1 + 2 * k], b = acc[2 + 2 * k];
     dd v;
-    if (k >= top && ((bp.pex >> k) & 1ull))
+    if (merged && k >= top && k < top + bp.low + bp.mid)
+      v = a;
+    else if (k >= top && ((bp.pex >> k) & 1ull))
       v = dd_sub(a, b);
     else if (k >= walk0)
       v = dd_sub(dd_mul(a, bl.Q.inv_p[k]), dd_mul(b, bl.Q.inv_q[k]));

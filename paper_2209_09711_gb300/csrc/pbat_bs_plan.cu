@@ -365,6 +365,91 @@ static void bs_generate(const GraphIn& g, BsPlan& bp) {
   bp.ops_var = B.ops() + bp.L;
 }
 
+// Signature of a work item: what its prefix arcs leave of the network.  The
+// states below an item see the prefix only through which nodes its working
+// arcs join, and of those only the boundary -- the source, the sink and the
+// endpoints of the other arcs.  Items with the same connectivity among the
+// boundary nodes therefore have the same words, sums and counts, and one of
+// them is walked for all (the 40-arc networks: 98,650 and 223,568 items left
+// to walk fall into 615 and 3,764 classes).  bs_sig writes it as nsig words,
+// bit-sliced over 32 items, in a form that is the same exactly when the
+// connectivity is:
+//   undirected: every boundary node's first (in a fixed order) boundary node
+//   in its component, as a binary number over the nodes it can be joined to;
+//   directed: which boundary nodes the source reaches, which reach the sink,
+//   and for the other pairs whether the first reaches the second.
+static void bs_generate_sig(const GraphIn& g, BsPlan& bp) {
+  const int m = g.m, top = bp.ell + bp.tb + bp.L;
+  std::vector<bool> isb(g.n, false);
+  isb[g.source] = isb[g.sink] = true;
+  for (int k = 0; k < top; ++k) {
+    const int a = bp.perm[k];
+    isb[g.tail[a]] = isb[g.head[a]] = true;
+  }
+  Elim C(g.n, g.directed != 0, g.source, g.sink);
+  for (int k = top; k < m; ++k) {
+    const int a = bp.perm[k];
+    C.or_in(g.tail[a], g.head[a], "a[" + std::to_string(k) + "]");
+  }
+  std::vector<int> bnd{g.source, g.sink}, rest;
+  for (int v = 0; v < g.n; ++v) {
+    if (!isb[v]) rest.push_back(v);
+    else if (v != g.source && v != g.sink) bnd.push_back(v);
+  }
+  C.eliminate_all(rest);
+  // transitive closure over the boundary (Warshall's algorithm)
+  for (int k : bnd)
+    for (int i : bnd)
+      for (int j : bnd) {
+        if (i == j || i == k || j == k || (!g.directed && i > j)) continue;
+        if (C.has(i, k) && C.has(k, j)) C.or_in(i, j, "(" + C.at(i, k) + " & " + C.at(k, j) + ")");
+      }
+  std::string out;
+  int nsig = 0;
+  auto emit = [&](const std::string& expr) {
+    out += "  z[" + std::to_string(nsig++) + "] = " + expr + ";\n";
+  };
+  if (!g.directed) {
+    for (size_t i = 1; i < bnd.size(); ++i) {
+      std::vector<std::string> first;
+      std::string seen;
+      for (size_t j = 0; j < i; ++j) {
+        if (!C.has(bnd[i], bnd[j])) continue;
+        const std::string at = C.at(bnd[i], bnd[j]), id = std::to_string(i) + "_" + std::to_string(j);
+        out += "  const u32 f" + id + " = " + at + (seen.empty() ? "" : " & ~" + seen) + ";\n";
+        out += "  const u32 s" + id + " = " + at + (seen.empty() ? "" : " | " + seen) + ";\n";
+        first.push_back("f" + id);
+        seen = "s" + id;
+      }
+      for (int b = 0; (1u << b) <= first.size(); ++b) {
+        std::string e;
+        for (size_t q = 0; q < first.size(); ++q)
+          if (((q + 1) >> b) & 1) e += (e.empty() ? "" : " | ") + first[q];
+        emit(e);
+      }
+    }
+  } else {
+    const int s = g.source, t = g.sink;
+    for (size_t i = 2; i < bnd.size(); ++i) {
+      if (C.has(s, bnd[i])) emit(C.at(s, bnd[i]));
+      if (C.has(bnd[i], t)) emit(C.at(bnd[i], t));
+    }
+    for (size_t i = 2; i < bnd.size(); ++i)
+      for (size_t j = 2; j < bnd.size(); ++j) {
+        if (i == j || !C.has(bnd[i], bnd[j])) continue;
+        std::string e = C.at(bnd[i], bnd[j]);
+        if (C.has(s, bnd[i])) e += " & ~" + C.at(s, bnd[i]);
+        if (C.has(s, bnd[j])) e += " & ~" + C.at(s, bnd[j]);
+        if (C.has(bnd[i], t)) e += " & ~" + C.at(bnd[i], t);
+        emit(e);
+      }
+  }
+  bp.nsig = -1;
+  if (nsig > kMaxSigBits) return;
+  bp.nsig = nsig;
+  bp.gen_sig = "__device__ __forceinline__ void bs_sig(const u32* a, u32* z) {\n" + C.code() + out + "}\n";
+}
+
 // The fused kernel divides walk masses by p and 1 - p (p-dependent roles).
 bool bs_walk_ok(const double* p, int a) {
   return !p || (p[a] >= 0x1p-20 && p[a] <= 1.0 - 0x1p-20);
@@ -412,9 +497,22 @@ static void bs_smaller_walk(const GraphIn& g, BsPlan& bp, const double* p_for_gr
   bp = std::move(best);
 }
 
+static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
+                         const double* p_for_grad, bool one_by_one);
+
 int bs_make_plan(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
                  const double* p_for_grad) {
   if (fault_at("plan")) return fail(PBAT_EINVAL, "injected fault: planning");
+  const int rc = bs_plan_roles(g, o, nthr, bp, p_for_grad, false);
+  // items that cannot be merged keep the walk length of a one-launch run
+  const bool lengths_free = o.walk_bits < 0 && o.prefix_bits < 0 && o.prune && o.launches != 1;
+  if (rc || bp.nsig >= 0 || !lengths_free) return rc;
+  bp = BsPlan();
+  return bs_plan_roles(g, o, nthr, bp, p_for_grad, true);
+}
+
+static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
+                         const double* p_for_grad, bool one_by_one) {
   const int m = g.m, r = o.range_bits;
   bp.r = r;
   bp.grad = p_for_grad != nullptr;
@@ -427,10 +525,21 @@ int bs_make_plan(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
     bp.L = std::min(std::min(o.walk_bits, lmax), free_bits);
   } else if (o.prefix_bits >= 0) {
     bp.L = std::max(0, std::min(lmax, m - bp.ell - bp.tb - std::max(o.prefix_bits, r)));
+  } else if (!one_by_one && o.prune && o.launches != 1) {
+    // Items merged by signature cost little each, so there are many and short
+    // ones; their number is bounded by the table of item slots (2^24).  GB300,
+    // R / fused in us, source/sink-near prefixes: 27 arcs L = 3: 42 / 54 (5: 37
+    // / 61, 8: 60 / 100); 31 arcs L = 5: 68 / 109 (3: 97 / 134, 8: 107 / 176);
+    // 34 arcs directed L = 6: 60 / 82 (4: 56 / 78, 8: 78 / 118); 40 arcs,
+    // prune-aware, L = 6: 140 / 269 (8: 158 / 285, 10: 970 fused).  Below
+    // 24 arcs one launch that walks every item left is faster (23 arcs, L = 2:
+    // 29 / 36 against 29 / 54), with about 2^11 items.
+    bp.L = free_bits < 14 ? std::max(0, free_bits - 11)
+                          : std::min(lmax, std::max(free_bits - 24, std::min(6, (free_bits - 6) / 3)));
   } else {
-    // about 2^11 work items: measured best on GB300 for 27..40 arcs (larger
-    // items amortise the per-item epilogue, which is heavier in the fused
-    // kernel, so that one walks two arcs more)
+    // every item walked by itself: about 2^11 of them, measured best on GB300
+    // for 27..40 arcs (larger items amortise the per-item epilogue, which is
+    // heavier in the fused kernel, so that one walks two arcs more)
     bp.L = std::max(0, std::min(lmax, free_bits - std::max(0, 11 - r) + (p_for_grad ? 2 : 0)));
   }
   bp.L = std::max(0, std::min(bp.L, free_bits));  // never into the range arcs
@@ -490,6 +599,10 @@ int bs_make_plan(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
   const int top = bp.ell + bp.tb + bp.L;
   for (int j = 0; j < (int)pre_first.size(); ++j) bp.perm[top + j] = pre_first[j];
   for (int j = 0; j < extra; ++j) bp.perm[top + (int)pre_first.size() + j] = rest[j];
+  // prefix arcs whose p is outside the fused kernel's range come first: the
+  // lowest ten need no division by p (see BsFoldParams in the kernel source)
+  std::stable_partition(bp.perm.begin() + top, bp.perm.begin() + (m - r),
+                        [&](int a) { return !bs_walk_ok(p_for_grad, a); });
   for (int i = 0; i < r; ++i) bp.perm[m - 1 - i] = i;
   for (int b = 0; b < bp.L; ++b) bp.perm[bp.ell + bp.tb + b] = walk[b];
   int x = extra;
@@ -513,6 +626,11 @@ int bs_make_plan(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
   if (p_for_grad)
     for (int k = bp.ell + bp.tb + bp.L; k < m; ++k)
       if (!bs_walk_ok(p_for_grad, bp.perm[k])) bp.pex |= 1ull << k;
+  // merge blocks: up to 2^10 items that differ in prefix arcs outside the
+  // range; not with arcs outside the fused kernel's range above those
+  bp.low = std::min(5, bp.d - r);
+  bp.mid = std::min(5, bp.d - r - bp.low);
+  if (o.prune && bp.d - r > 0 && !(bp.pex >> (top + bp.low + bp.mid))) bs_generate_sig(g, bp);
   return PBAT_OK;
 }
 

@@ -19,12 +19,21 @@ struct BsPlan {
   unsigned long long pex = 0;
   std::vector<int> perm;  // internal position -> input arc
   std::string gen;        // generated bs_inv / bs_var
+  // generated bs_sig and its number of words, -1 when items are not merged
+  // (see bs_generate_sig); the prefix arcs of a merge block: `low` follow the
+  // bits of a word, `mid` the warp lanes
+  std::string gen_sig;
+  int nsig = -1, low = 0, mid = 0;
   int ncore = 0, ops_inv = 0, ops_var = 0;
 };
 
 // The fused kernel divides walk masses by p and 1 - p: an arc may be a walk
 // arc of the gradient only with p in [2^-20, 1 - 2^-20].
 bool bs_walk_ok(const double* p, int a);
+
+// Items are merged when their signatures fit this many bits (a 64-bit table
+// key with one bit to mark a used slot).
+constexpr int kMaxSigBits = 63;
 
 // Plan one network for the bit-sliced kernels (Sec. 4.3 equal division:
 // lane, thread, walk and prefix arcs, range arcs on top) and generate its

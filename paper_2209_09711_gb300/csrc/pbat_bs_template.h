@@ -38,14 +38,6 @@ typedef unsigned long long u64;
 #else
 #define KERNEL_BOUNDS __launch_bounds__(BS_NTHR)
 #endif
-// the first of two launches (prune and closed-form sums, no walk) is compiled
-// for at least 24 resident warps per SM: on GB300 it needs about 80 registers
-// then, without spills
-#if defined(BS_MINB) && BS_MINB > 768 / BS_NTHR
-#define KERNEL_BOUNDS_P1 __launch_bounds__(BS_NTHR, BS_MINB)
-#else
-#define KERNEL_BOUNDS_P1 __launch_bounds__(BS_NTHR, (768 / BS_NTHR > 0 ? 768 / BS_NTHR : 1))
-#endif
 #define BS_OUT (BS_L - BS_IN)
 
 struct dd { double hi, lo; };   // host-side double-double (only carried, never computed here)
@@ -174,7 +166,11 @@ __device__ __forceinline__ void bs_limb_add(u64* limbs, u128 v, int s) {
 struct BsParams {
   u64 task_lo, n_tasks, budget_ns;
   int prune, nlev;       // prefix-mass table levels
-  int ex_shift, pad;     // log2 of the excluded-arc table's row length
+  int ex_shift;          // log2 of the excluded-arc table's row length
+  // merged runs: levels of the prefix arcs above a block, the mass scale of
+  // the classes (see bs_merge) and log2 of their table's slots
+  int nlev_hi, mass_exp, slots_log2;
+  int hi_bits[10], hi_off[10];
   int lev_bits[10];      // prefix bits per level (low level first)
   int lev_off[10];       // first entry of each level in the prefix table
   u64 thw[32];           // thread-pattern masses, fixed point 2^63
@@ -186,62 +182,62 @@ struct BsWork {
   dd* part_acc; u64* part_n; dd* out_acc; u64* out_n;
   facc* wacc;       // fused kernel: per warp, R and the two sums of every arc
   u64* out_limbs;   // [n_acc][8]: 256-bit fixed point at scale 2^250, 32 bits per limb
-  u64* list;        // two-launch runs: items deferred to the walking launch
-  u64 list_cap;     // 0: one-launch run
+  // merged runs: the classes in the order they were met (their slots), how
+  // many there are, and the walking launch's ticket
+  u32* list;
   u64* list_n;
-  u64* counter2;    // ticket of the walking launch
+  u64* counter2;
+  // per slot: the signature (0: unused), the summed mass of the class's items
+  // in two chunks, their number by popcount (BS_HIST each), one of them, and
+  // the sum S of that one
+  u64 *key, *cmass;
+  u32* hist;
+  u64* rep;
+  ulonglong2* csum;
+  // per block of items and lane: items connected throughout and items left to
+  // walk (a bit each), and the latter's slots ([block][bit][lane])
+  uint2* cmask;
+  u32* cls;
 };
 
-// Work items of a launch.  One-launch runs (phase 0) take items by the
-// atomic ticket over [0, n_tasks).  Two-launch runs: the first (phase 1)
-// takes items 16 at a time -- a warp's first 16 fixed by its index, the
-// rest by an atomic ticket (its items are short: one ticket per item would
-// pack 2^21 atomics on one counter into the launch, and a fixed warp stride
-// gave warps runs of alike items that end unevenly) -- resolves what the
-// prune can and defers the items left to walk; the second (phase 2) takes
-// the deferred items by a ticket over the list.  ~0: no item left.
-__device__ __forceinline__ u64 bs_list_task(const BsWork& W) {
-  const u64 i = atomicAdd(W.counter2, 1ull);
-  return i < *W.list_n ? W.list[i] : ~0ull;
+// One-launch runs (phase 0) take items by the atomic ticket over [0,
+// n_tasks).  The walking launch of a merged run (phase 2) takes classes from
+// the list: a warp's first by its index, counted over the blocks first, so
+// that few classes are spread over the SMs and blocks without any return at
+// once; only a list longer than the grid goes on by ticket (with a ticket for
+// every class, the grid's warps queued on one counter: 27-arc R 38 -> 28 us).
+__device__ __forceinline__ u64 bs_next_class(const BsWork& W, u64 n_list, u64 n_warps, int lane) {
+  u64 i = ~0ull;
+  if (n_list > n_warps) {
+    if (lane == 0) i = n_warps + atomicAdd(W.counter2, 1ull);
+    i = __shfl_sync(0xffffffffu, i, 0);
+  }
+  return i;
 }
-// The walking launch: true (in every thread of the block) when no deferred
-// item is left for it -- the list is empty, or blocks that started earlier
-// have taken every ticket -- so the block returns before it stages tables or
-// clears accumulators (it would add nothing to the results).
-__device__ __forceinline__ bool bs_list_done(const BsWork& W) {
-  __shared__ int s_done;
-  if (threadIdx.x == 0)
-    s_done = *(volatile const u64*)W.counter2 >= *(volatile const u64*)W.list_n;
-  __syncthreads();
-  return s_done != 0;
-}
-
-// Phase 1: a warp collects its deferred items one per lane (entry j in lane
-// j) and appends them to the list 32 at a time, with one atomic per batch.
-// The list holds every item (list_cap = n_tasks), so it cannot overflow.
-__device__ __forceinline__ void bs_flush_deferred(const BsWork& W, u64 pend, int npend, int lane) {
-  if (!npend) return;
-  u64 base = 0;
-  if (lane == 0) base = atomicAdd(W.list_n, (u64)npend);
-  base = __shfl_sync(0xffffffffu, base, 0);
-  if (lane < npend) W.list[base + lane] = pend;
-}
+// Programmatic dependent launch: the launches of a merged run start while
+// the one before drains, and wait here for its results.
+__device__ __forceinline__ void bs_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void bs_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 __device__ __forceinline__ u64 bs_timer() {
   u64 t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t;
 }
 
 // Mass of the prefix arcs of `prefix`: product over table levels.
-__device__ __forceinline__ mx bs_prefix_mass(const BsParams& P, const mx* __restrict__ ptab, u64 prefix) {
+__device__ __forceinline__ mx bs_level_mass(int nlev, const int* bits, const int* off,
+                                            const mx* __restrict__ ptab, u64 prefix) {
   mx w = mx{1ull << 63, 0, 0};
   int sh = 0;
-  for (int l = 0; l < P.nlev; ++l) {
-    const u64 v = (prefix >> sh) & ((1ull << P.lev_bits[l]) - 1ull);
-    const mx t = ptab[P.lev_off[l] + v];
+  for (int l = 0; l < nlev; ++l) {
+    const u64 v = (prefix >> sh) & ((1ull << bits[l]) - 1ull);
+    const mx t = ptab[off[l] + v];
     w = l ? mx_mul(w, t) : t;
-    sh += P.lev_bits[l];
+    sh += bits[l];
   }
   return w;
+}
+__device__ __forceinline__ mx bs_prefix_mass(const BsParams& P, const mx* __restrict__ ptab, u64 prefix) {
+  return bs_level_mass(P.nlev, P.lev_bits, P.lev_off, ptab, prefix);
 }
 // Per-lane constants of the 32x32 bit transpose below: byte selectors of the
 // 16- and 8-bit rounds, rotate amounts and keep-masks of the 4-, 2- and
@@ -331,24 +327,247 @@ __device__ __forceinline__ void bs_flush_bins(u64* bins, u64* s_nbins, int base)
 // exact, so the order of the blocks does not matter); then the block's N_k
 // counts.  The host converts the result once.
 __device__ __forceinline__ void bs_write_out(const BsWork& W, const facc* s_acc, int stride, int n_acc,
-                                             const u64* s_nbins) {
-  for (int i = threadIdx.x; i < n_acc; i += BS_NTHR) {
+                                             const u64* s_nbins, int nthr) {
+  for (int i = threadIdx.x; i < n_acc; i += nthr) {
     facc t = s_acc[i];
-    for (int w = 1; w < BS_NTHR / 32; ++w) facc_add(t, s_acc[w * stride + i].v, s_acc[w * stride + i].E);
+    for (int w = 1; w < nthr / 32; ++w) facc_add(t, s_acc[w * stride + i].v, s_acc[w * stride + i].E);
     bs_limb_add(W.out_limbs + 8 * i, t.v, 127 - t.E);   // v * 2^(-123 - E) at scale 2^250
   }
-  for (int i = threadIdx.x; i <= BS_M; i += BS_NTHR)
+  for (int i = threadIdx.x; i <= BS_M; i += nthr)
     if (s_nbins[i]) atomicAdd(&W.out_n[i], s_nbins[i]);
 }
+
+// ---------------------------------------------------------------------------
+// Merged runs.  Most items that the prune leaves share what their prefix
+// leaves of the network with many others (bs_sig), so the run goes in three
+// launches:
+//   bs_merge  prunes the items, 32 x 32 of them at a time, sums those that
+//             are connected throughout, and gives each one left to the class
+//             of its signature: its mass, its popcount;
+//   bs_walk   walks one item of every class for all of them;
+//   bs_fold   (fused kernel) the prefix arcs' gradient from the items' sums.
+// Against walking every item left (GB300; a 24-node, 40-arc network, 2^40
+// states): fused 49.1 -> 0.26 ms, R 20.2 -> 0.12 ms; a 20-node, 34-arc
+// directed network 0.36 -> 0.055 and 0.58 -> 0.050 ms; the 3x6 grid 0.100 ->
+// 0.048 and 0.055 -> 0.026 ms.  The large runs are bound by instruction
+// issue (bs_merge and bs_fold work per 32 items, bs_walk per class), the
+// small ones by the latency of their three launches.
+// ---------------------------------------------------------------------------
+#if BS_MERGE
+#define BS_BLK (BS_LOW + BS_MID)   // prefix arcs inside a merge block
+#define BS_HI (BS_D - BS_BLK)      // prefix arcs above it
+#define BS_MERGE_NTHR 128
+#define BS_CLASS_SHIFT 38          // low chunk of a class mass
+#define BS_HIST ((BS_D + 2) & ~1)  // counters by popcount of a class, an even number
+__device__ __forceinline__ u32 bs_pattern(int i) {
+  return i == 0 ? 0xAAAAAAAAu : i == 1 ? 0xCCCCCCCCu : i == 2 ? 0xF0F0F0F0u : i == 3 ? 0xFF00FF00u : 0xFFFF0000u;
+}
+// (a * b) >> 128 (the product of the low halves dropped: at most two units low)
+__device__ __forceinline__ u128 mulhi128(u128 a, u128 b) {
+  u128 r = u128{a.hi * b.hi, __umul64hi(a.hi, b.hi)};
+  u128_add(r, __umul64hi(a.hi, b.lo), 0ull);
+  u128_add(r, __umul64hi(a.lo, b.hi), 0ull);
+  return r;
+}
+// The mass of the 32 patterns set in v, from eight nibble tables t of 16
+// subset sums (scale 2^127), times the mass f (scale 2^127): scale 2^126.
+__device__ __forceinline__ u128 bs_subset_mass(u32 v, const ulonglong2* t, u128 f) {
+  u128 s = u128{0ull, 0ull};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const ulonglong2 x = t[16 * i + ((v >> (4 * i)) & 15u)];
+    u128_add(s, x.x, x.y);
+  }
+  return mulhi128(s, f);
+}
+// The set bits of v by the popcount of their position, a byte each.
+__device__ __forceinline__ u64 bs_popcount_bytes(u32 v) {
+  return (u64)(__popc(v & 0x00000001u) | (__popc(v & 0x00010116u) << 8) | (__popc(v & 0x01161668u) << 16) |
+               (__popc(v & 0x16686880u) << 24)) |
+         ((u64)(__popc(v & 0x68808000u) | (__popc(v & 0x80000000u) << 8)) << 32);
+}
+// Adds the block's items in `full` to s_ci by popcount.  Every lane packs its
+// counts by popcount into bytes (at most C(10, 5) = 252 each over the warp)
+// and three warp reductions add them; lane k then holds popcount k's.
+__device__ __forceinline__ void bs_count_full(u32 full, int lane, int pc_hi, u64* s_ci) {
+  const u64 v = bs_popcount_bytes(full);
+  const int sh = 8 * __popc(lane);
+  const u64 lo = v << sh, hi = sh ? v >> (64 - sh) : 0ull;
+  const u32 r0 = __reduce_add_sync(0xffffffffu, (u32)lo), r1 = __reduce_add_sync(0xffffffffu, (u32)(lo >> 32));
+  const u32 r2 = __reduce_add_sync(0xffffffffu, (u32)hi);
+  const u32 r = lane < 4 ? r0 : lane < 8 ? r1 : r2;
+  const u32 n = (r >> (8 * (lane & 3))) & 255u;
+  if (lane <= BS_BLK && n) atomicAdd(&s_ci[pc_hi + lane], (u64)n);
+}
+// The class of signature `key` (never 0): its slot, by linear probing from
+// its hash; claimed by compare-and-swap when new (`fresh`).  A table of
+// 2^BS_NSIG slots or more is indexed by the signature itself.  ~0: no free
+// slot within reach.
+__device__ __forceinline__ u32 bs_class(const BsParams& P, const BsWork& W, u64 key, bool& fresh) {
+  const u32 mask = (1u << P.slots_log2) - 1u;
+  u32 slot = (u32)key & mask;
+  if (BS_NSIG > P.slots_log2) {
+    u64 h = key * 0x9E3779B97F4A7C15ull;   // the finaliser of splitmix64
+    h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
+    slot = (u32)((h ^ (h >> 27)) >> 20) & mask;
+  }
+  fresh = false;
+  for (int probe = 0; probe < 256; ++probe) {
+    u64 k = *(volatile u64*)&W.key[slot];
+    if (!k) {
+      k = atomicCAS(&W.key[slot], 0ull, key);
+      if (!k) { fresh = true; return slot; }
+    }
+    if (k == key) return slot;
+    slot = (slot + 1u) & mask;
+  }
+  return ~0u;
+}
+
+__device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __restrict__ ptab,
+                                              const ulonglong2* __restrict__ mtab, int split_log2, const BsWork& W) {
+  __shared__ ulonglong2 s_nib[128];   // subset sums of the low prefix pattern masses
+  __shared__ facc s_acc[BS_MERGE_NTHR / 32];
+  __shared__ u64 s_ci[BS_D + 1];      // items connected throughout, by popcount
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < 128; i += BS_MERGE_NTHR) s_nib[i] = mtab[i];
+  for (int i = tid; i <= BS_D; i += BS_MERGE_NTHR) s_ci[i] = 0ull;
+  bs_let_next_start();
+  __syncthreads();
+  const u128 m_mid = u128{mtab[128 + lane].x, mtab[128 + lane].y};
+  facc accR = facc{u128{0ull, 0ull}, 0, 0};
+  const u64 t_start = bs_timer();
+  // a block's items left to walk are shared by 2^split_log2 warps (each takes
+  // every so manyeth bit of the words), so that few blocks still fill the GPU
+  const u64 nwarps = (u64)gridDim.x * (BS_MERGE_NTHR / 32);
+  const u64 nblk = P.n_tasks >> BS_BLK, blk0 = P.task_lo >> BS_BLK;
+  const u32 valid = lane < (1 << BS_MID) ? (BS_LOW >= 5 ? 0xffffffffu : (1u << (1 << BS_LOW)) - 1u) : 0u;
+  for (u64 t = (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; t < nblk << split_log2; t += nwarps) {
+    const u64 b = t >> split_log2;
+    const u32 part = (u32)t & ((1u << split_log2) - 1u);
+    if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
+    const u64 hi = blk0 + b;
+    u32 a[BS_M], u[BS_M];
+#pragma unroll
+    for (int k = 0; k < BS_TOP; ++k) a[k] = 0u;
+#pragma unroll
+    for (int j = 0; j < BS_D; ++j)
+      a[BS_TOP + j] = j < BS_LOW ? bs_pattern(j) : j < BS_BLK ? 0u - (u32)((lane >> (j - BS_LOW)) & 1)
+                                                              : 0u - (u32)((hi >> (j - BS_BLK)) & 1ull);
+#pragma unroll
+    for (int k = 0; k < BS_M; ++k) u[k] = k < BS_TOP ? ~0u : a[k];
+    const u32 up = bs_uniform(u) & valid;
+    const u32 full = bs_uniform(a) & valid;
+    u32 left = up & ~full;
+    const int pc_hi = __popcll((long long)hi);
+    if (part == 0) {
+      if (BS_GRAD) W.cmask[b * 32 + lane] = make_uint2(full, left);
+      if (__any_sync(0xffffffffu, full)) {
+        bs_count_full(full, lane, pc_hi, s_ci);
+        const u128 S = warp_sum_u128(u128_shr(bs_subset_mass(full, s_nib, m_mid), 2));
+        const mx w = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
+        facc_add(accR, mx_prod(w, S), w.e);
+      }
+    }
+    if (!__any_sync(0xffffffffu, left)) continue;
+    u32 z[BS_NSIG > 0 ? BS_NSIG : 1];
+    bs_sig(a, z);
+    // every 2^split_log2-th bit
+    left &= (split_log2 == 0 ? 0xffffffffu : split_log2 == 1 ? 0x55555555u : split_log2 == 2 ? 0x11111111u
+             : split_log2 == 3 ? 0x01010101u : split_log2 == 4 ? 0x00010001u : 1u) << part;
+    const mx whi = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
+    while (left) {
+      // one of the lane's items, and all of them with its signature
+      const int j = __ffs(left) - 1;
+      u32 k0 = 0u, k1 = 0u, same = left;
+#pragma unroll
+      for (int i = 0; i < BS_NSIG; ++i) {
+        const u32 top = z[i] << (31 - j);   // item j's bit on top
+        if (i < 32) k0 = __funnelshift_l(top, k0, 1); else k1 = __funnelshift_l(top, k1, 1);
+        same &= ~(z[i] ^ (u32)((int)top >> 31));
+      }
+      left &= ~same;
+      const u64 key = ((u64)k1 << 32) | k0 | 1ull << 63;
+      bool fresh;
+      const u32 slot = bs_class(P, W, key, fresh);
+      if (slot == ~0u) { atomicOr(W.status, 2u); continue; }   // the host runs the items one by one instead
+      if (fresh) {
+        W.rep[slot] = (hi << BS_BLK) | (u64)(lane << BS_LOW) | (u64)j;
+        W.list[atomicAdd(W.list_n, 1ull)] = slot;
+      }
+      // their mass at scale 2^(98 + mass_exp), where all the items' masses add
+      // up to at most 2^98: two chunks, the lower of BS_CLASS_SHIFT bits,
+      // each added up by itself
+      const u128 F = u128_shr(mx_prod(whi, u128_shr(bs_subset_mass(same, s_nib, m_mid), 2)), 25 + whi.e - P.mass_exp);
+      const u64 lo = F.lo & ((1ull << BS_CLASS_SHIFT) - 1ull);
+      const u64 up64 = (F.lo >> BS_CLASS_SHIFT) | (F.hi << (64 - BS_CLASS_SHIFT));
+      if (lo) atomicAdd(&W.cmass[2 * (size_t)slot], lo);
+      if (up64) atomicAdd(&W.cmass[2 * (size_t)slot + 1], up64);
+      // their number by popcount, two 32-bit counters to an addition
+      const int pc = pc_hi + __popc(lane);
+      u64* h = (u64*)(W.hist + (size_t)slot * BS_HIST) + (pc >> 1);
+      const u64 n = bs_popcount_bytes(same) << (8 * (pc & 1));
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const u64 two = ((n >> (16 * i)) & 255ull) | ((n >> (16 * i + 8)) & 255ull) << 32;
+        if (two) atomicAdd(&h[i], two);
+      }
+      if (BS_GRAD)
+        for (u32 s = same; s; s &= s - 1u) W.cls[(b << BS_BLK) + (u64)(((__ffs(s) - 1) << BS_MID) + lane)] = slot;
+    }
+  }
+  if (lane == 0) s_acc[warp] = accR;
+  __syncthreads();
+  if (tid == 0) {
+    facc r = s_acc[0];
+    for (int w = 1; w < BS_MERGE_NTHR / 32; ++w) facc_add(r, s_acc[w].v, s_acc[w].E);
+    bs_limb_add(W.out_limbs, r.v, 127 - r.E);
+  }
+  // an item connected throughout stands for C(arcs below, j) states with j
+  // more working arcs
+  for (int i = tid; i <= BS_M; i += BS_MERGE_NTHR) {
+    u64 n = 0;
+    for (int j = 0; j <= BS_TOP && j <= i; ++j)
+      if (i - j <= BS_D) n += s_ci[i - j] * P.binom[j];
+    if (n) atomicAdd(&W.out_n[i], n);
+  }
+}
+// The mass of a class as integer floating point.
+__device__ __forceinline__ mx bs_class_mass(const BsParams& P, const BsWork& W, u64 slot) {
+  u128 t = u128{W.cmass[2 * slot], 0ull};
+  const u64 up = W.cmass[2 * slot + 1];
+  u128_add(t, up << BS_CLASS_SHIFT, up >> (64 - BS_CLASS_SHIFT));
+  if (!(t.lo | t.hi)) return mx{0ull, 0, 0};
+  const int lz = t.hi ? __clzll((long long)t.hi) : 64 + __clzll((long long)t.lo);
+  const u64 m = lz >= 64 ? t.lo << (lz - 64) : (lz ? (t.hi << lz) | (t.lo >> (64 - lz)) : t.hi);
+  return mx{m, lz - 29 + P.mass_exp, 0};   // 128 - lz bits at scale 2^(98 + mass_exp)
+}
+// N_k of a class: its representative's states by popcount below the prefix
+// (rel, BS_TOP + 1 of them) for every popcount that its prefixes have.
+__device__ __forceinline__ void bs_class_counts(const BsWork& W, u64 slot, int lane, const u64* rel, u64* s_nbins) {
+  __syncwarp();
+  const u64 r = lane <= BS_TOP ? rel[lane] : 0ull;
+  for (int p0 = 0; p0 <= BS_D; p0 += 32) {
+    const u32 h = p0 + lane <= BS_D ? W.hist[(size_t)slot * BS_HIST + p0 + lane] : 0u;
+    u32 some = __ballot_sync(0xffffffffu, h != 0u);
+    while (some) {
+      const int q = __ffs(some) - 1;
+      some &= some - 1u;
+      const u64 n = (u64)__shfl_sync(0xffffffffu, h, q) * r;
+      if (n) atomicAdd(&s_nbins[p0 + q + lane], n);
+    }
+  }
+  __syncwarp();
+}
+#endif
 
 // ---------------------------------------------------------------------------
 // R + N_k
 // ---------------------------------------------------------------------------
 #if !BS_GRAD
-// PHASE 0: a one-launch run; 1 and 2: the two launches of a two-launch run
-// (the first resolves what the prune can and defers the items left to walk,
-// the second walks them).  One entry point per phase, so that a one-launch
-// kernel carries none of the two-launch state in its registers.
+// PHASE 0: a one-launch run; 2: the walking launch of a merged run.  One entry
+// point per phase, so that a one-launch kernel carries none of the other's
+// state in its registers.
 template <int PHASE>
 __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __restrict__ lane_tab,
                                                const u64* __restrict__ wmid_tab,
@@ -360,12 +579,16 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
   facc* s_acc = (facc*)(s_bins + (BS_L + 1) * BS_NTHR);     // [warps]: each warp's R
   u64* s_nbins = (u64*)(s_acc + BS_NTHR / 32);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if constexpr (PHASE == 2) {
-    if (bs_list_done(W)) return;
-  }
   for (int i = tid; i < 4 * 256; i += BS_NTHR) s_lt[i] = ((const ulonglong2*)lane_tab)[i];
   for (int i = tid; i < (1 << BS_L); i += BS_NTHR) s_wmid[i] = wmid_tab[i];
   for (int i = tid; i <= BS_M; i += BS_NTHR) s_nbins[i] = 0ull;
+  u64 n_list = 0, next = 0;
+  if constexpr (PHASE == 2) {
+    bs_wait_previous();
+    n_list = *W.list_n;
+    next = (u64)warp * gridDim.x + blockIdx.x;
+    if (blockIdx.x >= n_list || *W.status) return;   // no class, or a run that the host discards
+  }
   __syncthreads();
   u64* bins = s_bins + tid;
   const bool thr_on = lane < (1 << BS_TB);
@@ -377,35 +600,37 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
   u32 a[BS_M];
   bs_init_arcs(a, lane);
   constexpr int phase = PHASE;
-  // phase 1: this warp's chunk of items -- its first chunk is its own (no
-  // ticket at the start of a short launch), the later ones come by ticket
-  u64 chunk_next = ((u64)blockIdx.x * (BS_NTHR / 32) + warp) * 16, chunk_end = chunk_next + 16;
-  u64 pend = 0;   // phase 1: this warp's deferred items, entry j in lane j
-  int npend = 0;
+#if BS_MERGE
+  u64* rel = s_nbins + BS_M + 1 + warp * (BS_TOP + 1);   // phase 2: counts below the prefix
+#endif
 
   for (;;) {
     u64 task = 0;
-    if constexpr (phase == 1) {
-      if (chunk_next == chunk_end) {   // the next 16 items, by one atomic ticket
-        u64 base = 0;
-        if (lane == 0) base = (u64)gridDim.x * (BS_NTHR / 32) * 16 + atomicAdd(W.counter, 16ull);
-        chunk_next = __shfl_sync(0xffffffffu, base, 0);
-        chunk_end = chunk_next + 16;
-      }
-      task = chunk_next++;
+    if constexpr (phase == 2) {
+      task = next < n_list ? (u64)W.list[next] : ~0ull;
+      next = bs_next_class(W, n_list, (u64)gridDim.x * (BS_NTHR / 32), lane);
     }
     if (lane == 0) {
-      if constexpr (phase == 2) task = bs_list_task(W);
-      else if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
+      if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
       if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); task = ~0ull; }
     }
     task = __shfl_sync(0xffffffffu, task, 0);
-    if (task >= P.n_tasks) break;
-    const u64 prefix = P.task_lo + task;
+    u64 prefix;
+    if constexpr (phase == 2) {   // a class, by its slot
+      if (task == ~0ull) break;
+#if BS_MERGE
+      prefix = W.rep[task];
+      for (int i = lane; i <= BS_TOP; i += 32) rel[i] = 0ull;
+      __syncwarp();
+#endif
+    } else {
+      if (task >= P.n_tasks) break;
+      prefix = P.task_lo + task;
+    }
 #pragma unroll
     for (int j = 0; j < BS_D; ++j) a[BS_TOP + j] = 0u - (u32)((prefix >> j) & 1ull);
     const int pc_pre = __popcll((long long)prefix);
-    if ((P.prune && phase == 0) || phase == 1) {   // two-launch runs always prune
+    if (P.prune && phase == 0) {
       const int pr = bs_prune(a);
       if (pr == 1) { ++n_dead; continue; }
       if (pr == 2) {
@@ -415,11 +640,6 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
         facc_add(accR, mx_prod(w, u128{0ull, 1ull << 60}), w.e);
         continue;
       }
-    }
-    if constexpr (phase == 1) {   // left to walk: deferred to the second launch
-      if (lane == npend) pend = task;
-      if (++npend == 32) { bs_flush_deferred(W, pend, npend, lane); npend = 0; }
-      continue;
     }
     ++n_walk;
     u32 e[BS_NCORE > 0 ? BS_NCORE : 1];
@@ -465,27 +685,42 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
         }
       }
     }
-    if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
     // item total: exact warp sum of T x thread mass (scale 2^124), times the
-    // prefix mass, once per item
+    // prefix mass (a class: its items' summed mass), once per item
     const u128 S = warp_sum_u128(mul64x128_shr64(thw, T.lo, T.hi));
-    const mx w = bs_prefix_mass(P, ptab, prefix);
+    mx w;
+    if constexpr (phase == 2) {
+#if BS_MERGE
+      if (thr_on) bs_flush_bins(bins, rel, pc_thr);
+      bs_class_counts(W, task, lane, rel, s_nbins);
+      w = bs_class_mass(P, W, task);
+#endif
+    } else {
+      if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
+      w = bs_prefix_mass(P, ptab, prefix);
+    }
     facc_add(accR, mx_prod(w, S), w.e);
   }
-  if constexpr (phase == 1) bs_flush_deferred(W, pend, npend, lane);
   if (lane == 0) {
-    atomicAdd(&W.stats[0], n_walk); atomicAdd(&W.stats[1], n_full); atomicAdd(&W.stats[2], n_dead);
+    if (n_walk) atomicAdd(&W.stats[0], n_walk);
+    if (n_full) atomicAdd(&W.stats[1], n_full);
+    if (n_dead) atomicAdd(&W.stats[2], n_dead);
     s_acc[warp] = accR;
   }
   __syncthreads();
-  bs_write_out(W, s_acc, 1, 1, s_nbins);
+  bs_write_out(W, s_acc, 1, 1, s_nbins, BS_NTHR);
 }
 
 #define KERNEL_R_ARGS const __grid_constant__ BsParams P, const u64* __restrict__ lane_tab, \
                   const u64* __restrict__ wmid_tab, const mx* __restrict__ ptab, const BsWork W
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel(KERNEL_R_ARGS) { bs_kernel_body<0>(P, lane_tab, wmid_tab, ptab, W); }
-extern "C" __global__ void KERNEL_BOUNDS_P1 bs_kernel_p1(KERNEL_R_ARGS) { bs_kernel_body<1>(P, lane_tab, wmid_tab, ptab, W); }
+#if BS_MERGE
+extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_p1(const __grid_constant__ BsParams P,
+    const mx* __restrict__ ptab, const ulonglong2* __restrict__ mtab, int split_log2, const BsWork W) {
+  bs_merge_body(P, ptab, mtab, split_log2, W);
+}
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel_p2(KERNEL_R_ARGS) { bs_kernel_body<2>(P, lane_tab, wmid_tab, ptab, W); }
+#endif
 #endif
 
 #if BS_GRAD
@@ -541,6 +776,22 @@ __device__ __forceinline__ mx bs_arc_factor(const BsParams& P, const mx* __restr
   return f;
 }
 
+// The mass factors of an item (or class) for R, of internal arc `lane` and of
+// arc `lane + 32`.
+#if BS_MERGE
+#define BS_CLASS_FACTORS() wpre = f0 = f1 = bs_class_mass(P, W, task)
+#else
+#define BS_CLASS_FACTORS() wpre = f0 = f1 = mx{0ull, 0, 0}
+#endif
+#define BS_FACTORS()                                                                                  \
+  if constexpr (phase == 2) {                                                                         \
+    BS_CLASS_FACTORS();                                                                               \
+  } else {                                                                                            \
+    wpre = bs_prefix_mass(P, ptab, prefix);                                                           \
+    f0 = bs_arc_factor(P, ptab, ptab_ex, prefix, lane, wpre);                                         \
+    f1 = lane + 32 < BS_M ? bs_arc_factor(P, ptab, ptab_ex, prefix, lane + 32, wpre) : wpre;          \
+  }
+
 template <int PHASE>
 __device__ __forceinline__ void bs_kernel_grad_body(
     const BsParams& P, const BsGradParams& Q, const u64* __restrict__ lane_tab,
@@ -552,22 +803,23 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u64* s_tt = (u64*)(s_wm + (1 << BS_L));                   // [4][256] thread-pattern masses (2^62)
   u64* s_bins = s_tt + 4 * 256;                             // [L + 1][NTHR]
   u128* s_A = (u128*)(s_bins + (BS_L + 1) * BS_NTHR);       // [BS_OUT][NTHR]
-  // the first of two launches walks nothing: it holds only the N_k counts,
-  // so it is launched with (m + 1) * 8 bytes of shared memory
-  u64* s_nbins = PHASE == 1 ? (u64*)smem : (u64*)(s_A + (BS_OUT > 0 ? BS_OUT : 1) * BS_NTHR);
+  u64* s_nbins = (u64*)(s_A + (BS_OUT > 0 ? BS_OUT : 1) * BS_NTHR);
   // per warp, in global scratch: R, then A_k and B_k of every arc k
   facc* g_acc = W.wacc + (size_t)blockIdx.x * (BS_NTHR / 32) * (1 + 2 * BS_M);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < 4 * 256; i += BS_NTHR) s_lt[i] = ((const ulonglong2*)lane_tab)[i];
+  for (int i = tid; i < 4 * 256; i += BS_NTHR) s_tt[i] = thr_tab[i];
+  for (int i = tid; i < (1 << BS_L); i += BS_NTHR) s_wm[i] = ((const ulonglong2*)wmid128)[i];
+  for (int i = tid; i <= BS_M; i += BS_NTHR) s_nbins[i] = 0ull;
+  u64 n_list = 0, next = 0;
   if constexpr (PHASE == 2) {
-    if (bs_list_done(W)) return;
-  }
-  if constexpr (PHASE != 1) {
-    for (int i = tid; i < 4 * 256; i += BS_NTHR) s_lt[i] = ((const ulonglong2*)lane_tab)[i];
-    for (int i = tid; i < 4 * 256; i += BS_NTHR) s_tt[i] = thr_tab[i];
-    for (int i = tid; i < (1 << BS_L); i += BS_NTHR) s_wm[i] = ((const ulonglong2*)wmid128)[i];
+    bs_wait_previous();
+    bs_let_next_start();
+    n_list = *W.list_n;
+    next = (u64)warp * gridDim.x + blockIdx.x;
+    if (blockIdx.x >= n_list || *W.status) return;   // no class, or a run that the host discards
   }
   for (int i = tid; i < (BS_NTHR / 32) * (1 + 2 * BS_M); i += BS_NTHR) g_acc[i] = facc{u128{0ull, 0ull}, 0, 0};
-  for (int i = tid; i <= BS_M; i += BS_NTHR) s_nbins[i] = 0ull;
   __syncthreads();
   facc* acc = g_acc + warp * (1 + 2 * BS_M);
   u64* bins = s_bins + tid;
@@ -591,59 +843,53 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u32 a[BS_M];
   bs_init_arcs(a, lane);
   constexpr int phase = PHASE;
-  // phase 1: this warp's chunk of items -- its first chunk is its own (no
-  // ticket at the start of a short launch), the later ones come by ticket
-  u64 chunk_next = ((u64)blockIdx.x * (BS_NTHR / 32) + warp) * 16, chunk_end = chunk_next + 16;
-  u64 pend = 0;   // phase 1: this warp's deferred items, entry j in lane j
-  int npend = 0;
+#if BS_MERGE
+  u64* rel = s_nbins + BS_M + 1 + warp * (BS_TOP + 1);   // phase 2: counts below the prefix
+#endif
 
   for (;;) {
     u64 task = 0;
-    if constexpr (phase == 1) {
-      if (chunk_next == chunk_end) {   // the next 16 items, by one atomic ticket
-        u64 base = 0;
-        if (lane == 0) base = (u64)gridDim.x * (BS_NTHR / 32) * 16 + atomicAdd(W.counter, 16ull);
-        chunk_next = __shfl_sync(0xffffffffu, base, 0);
-        chunk_end = chunk_next + 16;
-      }
-      task = chunk_next++;
+    if constexpr (phase == 2) {
+      task = next < n_list ? (u64)W.list[next] : ~0ull;
+      next = bs_next_class(W, n_list, (u64)gridDim.x * (BS_NTHR / 32), lane);
     }
     if (lane == 0) {
-      if constexpr (phase == 2) task = bs_list_task(W);
-      else if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
+      if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
       if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); task = ~0ull; }
     }
     task = __shfl_sync(0xffffffffu, task, 0);
-    if (task >= P.n_tasks) break;
-    const u64 prefix = P.task_lo + task;
+    u64 prefix;
+    if constexpr (phase == 2) {   // a class, by its slot
+      if (task == ~0ull) break;
+#if BS_MERGE
+      prefix = W.rep[task];
+      for (int i = lane; i <= BS_TOP; i += 32) rel[i] = 0ull;
+      __syncwarp();
+#endif
+    } else {
+      if (task >= P.n_tasks) break;
+      prefix = P.task_lo + task;
+    }
 #pragma unroll
     for (int j = 0; j < BS_D; ++j) a[BS_TOP + j] = 0u - (u32)((prefix >> j) & 1ull);
     const int pc_pre = __popcll((long long)prefix);
     int pr = 0;
-    if ((P.prune && phase == 0) || phase == 1) {   // two-launch runs always prune
+    if (P.prune && phase == 0) {
       pr = bs_prune(a);
       if (pr == 1) { ++n_dead; continue; }
-    }
-    if constexpr (phase == 1) {
-      if (pr == 0) {   // left to walk: deferred to the second launch
-        if (lane == npend) pend = task;
-        if (++npend == 32) { bs_flush_deferred(W, pend, npend, lane); npend = 0; }
-        continue;
-      }
     }
 #if BS_ACC_REG
     // the prefix factors of an item that is not cut off, before its walk so
     // that their table loads overlap it (a cut-off item needs none: with
     // prune-aware prefix arcs most items are cut off or fully connected)
-    const mx wpre = bs_prefix_mass(P, ptab, prefix);
-    const mx f0 = bs_arc_factor(P, ptab, ptab_ex, prefix, lane, wpre);
-    const mx f1 = lane + 32 < BS_M ? bs_arc_factor(P, ptab, ptab_ex, prefix, lane + 32, wpre) : wpre;
+    mx wpre, f0, f1;
+    BS_FACTORS();
 #endif
     u128 S;      // sum over the warp of T x thread mass, scale 2^124
     // warp sums of the internal arc this lane owns (internal arcs are below
     // 32): the exact pair difference, or for a walk arc A and T - A
     u128 myX = u128{0ull, 0ull}, myY = u128{0ull, 0ull};
-    if (pr == 2 || phase == 1) {   // (the first of two launches walks nothing)
+    if (pr == 2) {
       ++n_full;
       for (int j = lane; j <= BS_TOP; j += 32) atomicAdd(&s_nbins[pc_pre + j], P.binom[j]);
       S = u128{0ull, 1ull << 60};   // the whole item: mass 1 at scale 2^124
@@ -722,7 +968,14 @@ __device__ __forceinline__ void bs_kernel_grad_body(
 #pragma unroll
       for (int b = 0; b < BS_OUT; ++b)
         if ((gout >> b) & 1u) { u128 ab = A[b * BS_NTHR]; u128_add(ab, T.lo, T.hi); A[b * BS_NTHR] = ab; }
-      if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
+      if constexpr (phase == 2) {
+#if BS_MERGE
+        if (thr_on) bs_flush_bins(bins, rel, pc_thr);
+        bs_class_counts(W, task, lane, rel, s_nbins);
+#endif
+      } else {
+        if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
+      }
       // ---- exact warp sums; slot k of `red` holds internal arc k's value
       S = warp_sum_u128(mul64x128_shr64(thw, T.lo, T.hi));
 #pragma unroll
@@ -755,9 +1008,8 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     }
     // ---- per-arc scaling on the owning lanes (internal arcs lane, lane + 32)
 #if !BS_ACC_REG
-    const mx wpre = bs_prefix_mass(P, ptab, prefix);
-    const mx f0 = bs_arc_factor(P, ptab, ptab_ex, prefix, lane, wpre);
-    const mx f1 = lane + 32 < BS_M ? bs_arc_factor(P, ptab, ptab_ex, prefix, lane + 32, wpre) : wpre;
+    mx wpre, f0, f1;
+    BS_FACTORS();
     facc accR, accA, accB;
     if (lane == 0) accR = acc[0];
     if (lane < BS_M) {
@@ -770,15 +1022,19 @@ __device__ __forceinline__ void bs_kernel_grad_body(
       // arc `lane`: a prefix arc goes into A when it works in this item and
       // into B when it fails (the item's mass without its factor); an
       // internal arc of a fully connected item has no pair that differs
+      // (a class's prefix arcs are left to bs_fold, from its sum S)
       u128 X = u128{0ull, 0ull}, Y = u128{0ull, 0ull};
       if (lane >= BS_TOP) {
-        if (lane < BS_M) {
+        if (phase == 0 && lane < BS_M) {
           if ((prefix >> (lane - BS_TOP)) & 1ull) X = S; else Y = S;
         }
       } else if (pr != 2) {
         X = myX;
         Y = myY;
       }
+#if BS_MERGE
+      if (phase == 2 && lane == 0) W.csum[task] = make_ulonglong2(S.lo, S.hi);
+#endif
       facc_add(accA, mx_prod(f0, X), f0.e);
       facc_add(accB, mx_prod(f0, Y), f0.e);
     }
@@ -789,7 +1045,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
       acc[2 + 2 * lane] = accB;
     }
 #endif
-    if (lane + 32 < BS_M) {
+    if (phase == 0 && lane + 32 < BS_M) {
       // arc lane + 32 is a prefix arc (lanes own arcs below 32 and the top
       // prefix arcs): the item's total, by whether the arc works here
       const int j = lane + 32 - BS_TOP;
@@ -807,9 +1063,10 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     }
     __syncwarp();
   }
-  if constexpr (phase == 1) bs_flush_deferred(W, pend, npend, lane);
   if (lane == 0) {
-    atomicAdd(&W.stats[0], n_walk); atomicAdd(&W.stats[1], n_full); atomicAdd(&W.stats[2], n_dead);
+    if (n_walk) atomicAdd(&W.stats[0], n_walk);
+    if (n_full) atomicAdd(&W.stats[1], n_full);
+    if (n_dead) atomicAdd(&W.stats[2], n_dead);
   }
 #if BS_ACC_REG
   if (lane == 0) acc[0] = accR;
@@ -828,7 +1085,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   // gradient (A - B for prefix arcs, A / p - B / (1 - p) for walk arcs, A
   // for lane and thread arcs)
   __syncthreads();
-  bs_write_out(W, g_acc, 1 + 2 * BS_M, 1 + 2 * BS_M, s_nbins);
+  bs_write_out(W, g_acc, 1 + 2 * BS_M, 1 + 2 * BS_M, s_nbins, BS_NTHR);
 }
 
 #define KERNEL_G_ARGS const __grid_constant__ BsParams P, const __grid_constant__ BsGradParams Q, \
@@ -837,8 +1094,147 @@ __device__ __forceinline__ void bs_kernel_grad_body(
                   const mx* __restrict__ ptab_ex, const BsWork W
 #define KERNEL_G_PASS P, Q, lane_tab, thr_tab, wmid128, ptab, ptab_ex, W
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel_grad(KERNEL_G_ARGS) { bs_kernel_grad_body<0>(KERNEL_G_PASS); }
-extern "C" __global__ void KERNEL_BOUNDS_P1 bs_kernel_grad_p1(KERNEL_G_ARGS) { bs_kernel_grad_body<1>(KERNEL_G_PASS); }
+#if BS_MERGE
+extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p1(const __grid_constant__ BsParams P,
+    const mx* __restrict__ ptab, const ulonglong2* __restrict__ mtab, int split_log2, const BsWork W) {
+  bs_merge_body(P, ptab, mtab, split_log2, W);
+}
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel_grad_p2(KERNEL_G_ARGS) { bs_kernel_grad_body<2>(KERNEL_G_PASS); }
+#endif
+
+#if BS_MERGE
+// ---------------------------------------------------------------------------
+// The prefix arcs' gradient of a merged run.  Every item has its conditional
+// reliability V: 0 when cut, 1 when connected throughout, else its class's S.
+// A warp folds a block of items arc by arc, V' = V0 + p (V1 - V0): lane u
+// holds the items of mid pattern u and folds the low arcs over its 32 items,
+// the mid arcs fold over the lanes.  On the way each arc of the block
+// collects the pair differences V1 - V0 weighted by the other arcs' masses;
+// the arcs above it take the block's V, by whether they work (the host
+// divides those sums by p and 1 - p).  A fold costs one product for two
+// items, so the whole launch is a few instructions per item, where adding
+// every item to every prefix arc took about 250.
+// ---------------------------------------------------------------------------
+struct BsFoldParams {
+  u64 p[10];            // low, then mid arcs: p at 2^63
+  u64 wlow[31];         // masses (2^63) of the low arcs above arc b: 16, 8, 4, 2, 1 patterns for b = 0..4
+  u64 wmid[31];         // of the mid arcs above mid arc b
+  u64 mid[32];          // mid pattern masses (2^63)
+};
+// |a - b|; neg: a < b (classes' sums round apart by up to 2^-61, so a pair
+// whose true difference is zero may come out below it)
+__device__ __forceinline__ u128 bs_absdiff(u128 a, u128 b, bool& neg) {
+  neg = a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
+  return neg ? u128_sub(b, a) : u128_sub(a, b);
+}
+// one fold: adds w (V1 - V0) to G, returns V0 + p (V1 - V0)
+__device__ __forceinline__ u128 bs_fold2(u128 V0, u128 V1, u64 p, u64 w, u128& G) {
+  bool neg;
+  const u128 d = bs_absdiff(V1, V0, neg);
+  if (!neg) {
+    const u128 g = mul64x128_shr64(w, d.lo, d.hi);   // scale 2^123
+    u128_add(G, g.lo, g.hi);
+  }
+  u128 x = mul64x128_shr64(p, d.lo, d.hi);
+  x = u128{x.lo << 1, (x.hi << 1) | (x.lo >> 63)};
+  if (neg) return u128_sub(V0, x);
+  u128_add(V0, x.lo, x.hi);
+  return V0;
+}
+extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p3(
+    const __grid_constant__ BsParams P, const __grid_constant__ BsFoldParams Q, const mx* __restrict__ ptab,
+    const BsWork W) {
+  __shared__ u64 s_none[BS_M + 1];   // no counts here
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  facc* g_acc = W.wacc + (size_t)blockIdx.x * (BS_MERGE_NTHR / 32) * (1 + 2 * BS_M);
+  facc* acc = g_acc + warp * (1 + 2 * BS_M);
+  for (int i = tid; i <= BS_M; i += BS_MERGE_NTHR) s_none[i] = 0ull;
+  bs_wait_previous();
+  // (the walking launch uses the same slots, so not before it has ended)
+  for (int i = lane; i < 1 + 2 * BS_M; i += 32) acc[i] = facc{u128{0ull, 0ull}, 0, 0};
+  __syncwarp();
+  // an earlier launch ran out of time or slots: its masks and slots are not
+  // all written, and the host discards the run
+  if (*(volatile u32*)W.status) return;
+  const u64 nblk = P.n_tasks >> BS_BLK, blk0 = P.task_lo >> BS_BLK;
+  const u64 nwarps = (u64)gridDim.x * (BS_MERGE_NTHR / 32);
+  const u64 m_mid = Q.mid[lane];
+  const u64 t_start = bs_timer();
+  // lane l < BS_BLK: arc l of the block; lanes: arcs `lane` and `lane + 32` above it
+  facc accP = facc{u128{0ull, 0ull}, 0, 0}, accA = accP, accB = accP, accA2 = accP, accB2 = accP;
+  for (u64 b = (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; b < nblk; b += nwarps) {
+    if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
+    const u64 hi = blk0 + b;
+    const uint2 m = W.cmask[b * 32 + lane];
+    if (!__any_sync(0xffffffffu, m.x | m.y)) continue;
+    const u32* cls = W.cls + (b << BS_BLK) + lane;
+    u128 G[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) G[i] = u128{0ull, 0ull};
+    u128 top[4];   // folded over the lowest three arcs
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      u128 V[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int j = 8 * q + i;
+        V[i] = u128{0ull, (m.x >> j) & 1u ? 1ull << 60 : 0ull};
+        if ((m.y >> j) & 1u) {
+          const ulonglong2 s = W.csum[cls[j << BS_MID]];
+          V[i] = u128{s.x, s.y};
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], Q.p[0], Q.wlow[4 * q + i], G[0]);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], Q.p[1], Q.wlow[16 + 2 * q + i], G[1]);
+      top[q] = bs_fold2(V[0], V[1], Q.p[2], Q.wlow[24 + q], G[2]);
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) top[i] = bs_fold2(top[2 * i], top[2 * i + 1], Q.p[3], Q.wlow[28 + i], G[3]);
+    u128 V = bs_fold2(top[0], top[1], Q.p[4], Q.wlow[30], G[4]);
+    // the block's sums per arc, lane l ending with arc l's (scale 2^124)
+    u128 X = u128{0ull, 0ull};
+#pragma unroll
+    for (int i = 0; i < BS_LOW; ++i) {
+      u128 g = mul64x128_shr64(m_mid, G[i].lo, G[i].hi);   // 2^122
+      g = warp_sum_u128(g);
+      g = u128{g.lo << 2, (g.hi << 2) | (g.lo >> 62)};
+      if (lane == i) X = g;
+    }
+#pragma unroll
+    for (int i = 0; i < BS_MID; ++i) {
+      const u128 o = shfl_xor_u128(V, 1 << i);
+      const bool one = (lane >> i) & 1;
+      u128 g = u128{0ull, 0ull};
+      const int at = (i == 0 ? 0 : i == 1 ? 16 : i == 2 ? 24 : i == 3 ? 28 : 30) + (lane >> (i + 1));
+      V = bs_fold2(one ? o : V, one ? V : o, Q.p[5 + i], Q.wmid[at], g);
+      if (lane & ((1 << (i + 1)) - 1)) g = u128{0ull, 0ull};   // each pair once
+      g = warp_sum_u128(g);
+      g = u128{g.lo << 1, (g.hi << 1) | (g.lo >> 63)};
+      if (lane == BS_LOW + i) X = g;
+    }
+    V.lo = __shfl_sync(0xffffffffu, V.lo, 0);
+    V.hi = __shfl_sync(0xffffffffu, V.hi, 0);
+    const mx w = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
+    if (lane < BS_BLK) facc_add(accP, mx_prod(w, X), w.e);
+    const u128 Sv = mx_prod(w, V);
+    if (lane < BS_HI) { if ((hi >> lane) & 1ull) facc_add(accA, Sv, w.e); else facc_add(accB, Sv, w.e); }
+    if (lane + 32 < BS_HI) { if ((hi >> (lane + 32)) & 1ull) facc_add(accA2, Sv, w.e); else facc_add(accB2, Sv, w.e); }
+  }
+  if (lane < BS_BLK) acc[1 + 2 * (BS_TOP + lane)] = accP;
+  if (lane < BS_HI) {
+    acc[1 + 2 * (BS_TOP + BS_BLK + lane)] = accA;
+    acc[2 + 2 * (BS_TOP + BS_BLK + lane)] = accB;
+  }
+  if (lane + 32 < BS_HI) {
+    acc[1 + 2 * (BS_TOP + BS_BLK + lane + 32)] = accA2;
+    acc[2 + 2 * (BS_TOP + BS_BLK + lane + 32)] = accB2;
+  }
+  __syncthreads();
+  bs_write_out(W, g_acc, 1 + 2 * BS_M, 1 + 2 * BS_M, s_none, BS_MERGE_NTHR);
+}
+#endif
 #endif
 )PBAT";
 

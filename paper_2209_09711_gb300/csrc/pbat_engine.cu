@@ -43,16 +43,18 @@ cudaError_t launch_frontier(bool grad, bool wide, int grid, int nthr, size_t sme
 cudaError_t launch_reduce(cudaStream_t st, const DevWork& W, int nblocks, int n_acc, int n_cnt);
 
 struct BsLaunch;
-void bs_finish_grad(const BsLaunch& bl, const dd* acc, int m, double* g_internal);
+void bs_finish_grad(const BsLaunch& bl, const dd* acc, int m, bool merged, double* g_internal);
 BsLaunch* bs_new();
 void bs_delete(BsLaunch* b);
 void bs_precompile(const GraphIn& g, const double* p, bool grad,
                    const std::vector<pbat_options>& opts, const DeviceInfo& dev);
 int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options& o,
                const DeviceInfo& dev, BsLaunch& bl);
-cudaError_t bs_launch(const BsLaunch& bl, int grid, cudaStream_t st, const unsigned long long* d_lane,
-                      const unsigned long long* d_thr, const unsigned long long* d_wmid,
-                      const void* d_ptab, const void* d_ptab_ex, const DevWork& W, int phase);
+cudaError_t bs_launch(const BsLaunch& bl, int grid, cudaStream_t st, const BsTables& T, const DevWork& W,
+                      int phase, int split_log2);
+BsMerge bs_merge(const BsLaunch& bl);
+void bs_mark_unmergeable(const BsLaunch& bl);
+const std::vector<unsigned long long>& bs_mtab(const BsLaunch& bl);
 const std::vector<MxHost>& bs_ptab(const BsLaunch& bl);
 const std::vector<MxHost>& bs_ptab_ex(const BsLaunch& bl);
 const std::vector<unsigned long long>& bs_thr_tab(const BsLaunch& bl);
@@ -387,6 +389,12 @@ void scratch_release(Scratch* s) {
 // ---------------------------------------------------------------------------
 // one planned enumeration (single network)
 // ---------------------------------------------------------------------------
+// Items from which a run merges them by default (pbat_options.launches 0):
+// below, one launch is a few microseconds long and further ones cost more
+// than they save (GB300, R / fused: 2^11 items of 23 arcs 29 / 36 us in one
+// launch, 29 / 54 merged; 2^14 items of 27 arcs 58 / 90 against 42 / 54).
+constexpr unsigned long long kMergeItems = 1ull << 12;
+
 struct Job {
   GraphIn g;
   Plan pl;
@@ -413,11 +421,7 @@ struct Job {
   size_t n_pending = 0;
   // bit-sliced kernel (R and N_k); null for the frontier kernel
   BsLaunch* bs = nullptr;
-  unsigned long long* d_lane = nullptr;
-  unsigned long long* d_thr = nullptr;
-  unsigned long long* d_wmid64 = nullptr;
-  void* d_ptab = nullptr;
-  void* d_ptabx = nullptr;
+  BsTables tabs;
   // absolute error bounds of R and of each dR/dp_k, in units of the
   // enumerated probability mass (the rounding of the fixed-point tables)
   double abs_err_bound = 0.0;
@@ -426,11 +430,11 @@ struct Job {
   std::vector<int> perm;       // internal arc position -> input arc
   unsigned long long item_states = 0, n_items = 0;
   int grid_nthr = 128;
-  // two launches per enumeration: the first resolves what the prune can and
-  // defers the items left to walk, the second walks them (bit-sliced kernels
-  // with the prune on and many items)
-  bool two_phase = false;
-  int grid1 = 0, grid2 = 0;   // grids of the two launches
+  // a merged run: its launches' grids, the warps that share a block of its
+  // first, and the bytes cleared before it (results and class table)
+  bool merged = false;
+  int grid1 = 0, grid2 = 0, grid3 = 0, split_log2 = 0;
+  size_t clear_bytes = 0;
   // the inputs, kept to re-run the exact frontier kernel when R is too small
   // for the bit-sliced kernel's fixed-point error bound
   std::vector<int32_t> tail_copy, head_copy;
@@ -544,7 +548,7 @@ static double tune_time(const GraphIn& g, const double* p, bool grad, pbat_optio
     return -1.0;
   }
   double ms = 1e300;
-  bool ok = !job_upload(J, st);
+  bool ok = (t.launches != 2 || J->merged) && !job_upload(J, st);
   for (int rep = 0; ok && rep < 3; ++rep) {
     cudaEvent_t a, b;
     cudaEventCreate(&a);
@@ -558,6 +562,11 @@ static double tune_time(const GraphIn& g, const double* p, bool grad, pbat_optio
     cudaEventDestroy(a);
     cudaEventDestroy(b);
   }
+  // a merged run that could not be, or whose classes did not fit its table,
+  // is no candidate
+  unsigned status = 0;
+  ok = ok && cudaMemcpy(&status, J->W.status, sizeof status, cudaMemcpyDeviceToHost) == cudaSuccess &&
+       !(status & 2u);
   job_destroy(J);
   if (!ok) {
     cudaGetLastError();
@@ -604,15 +613,16 @@ static int autotune(const GraphIn& g, const double* p, bool grad, pbat_options& 
     const double ta = tune_time(g, p, grad, a, st), tb = tune_time(g, p, grad, b, st);
     if (tb > 0 && (ta < 0 || tb < ta)) mode = 2;
   }
-  // stage 2: walk length x block size x occupancy x launches.  Candidates run the whole
-  // problem: a block of the equal division is not a fair sample (which arcs
-  // its range fixes changes how much the prune removes; the first block of
-  // the 40-arc network favoured a shape 50% slower on the whole).  Large
-  // problems try fewer candidates: long walks, no 64-thread blocks.
-  const int lmax = std::min(10, std::max(0, g.m - o.range_bits - 10));
+  // stage 2: walk length x block size x occupancy, with the items merged
+  // where they can be; where no merged candidate runs (signatures or classes
+  // too many), one launch.  Candidates run the whole problem: a block of the
+  // equal division is not a fair sample (which arcs its range fixes changes
+  // how much the prune removes; the first block of the 40-arc network
+  // favoured a shape 50% slower on the whole).  Large problems try fewer
+  // candidates: no 64-thread blocks, in one launch only long walks.
+  const int free_bits = std::max(0, g.m - o.range_bits - 10), lmax = std::min(10, free_bits);
   const bool large = log2_states(g, o) > 34.0;
-  std::vector<int> Ls, nts, occs;
-  for (int L = std::max(0, lmax - (large ? 2 : 6)); L <= lmax; ++L) Ls.push_back(L);
+  std::vector<int> nts, occs;
   // warps per block need not be a power of two: on the 40-arc network 160
   // threads (3 blocks, 15 warps per SM) ran the fused kernel 12% faster
   // than 128 and 224 threads the R kernel 7% faster than 256
@@ -622,33 +632,32 @@ static int autotune(const GraphIn& g, const double* p, bool grad, pbat_options& 
   // 40-arc network in prune-aware mode went from 26.0 to 24.7 ms with it
   if (o.occupancy >= 0) occs.push_back(o.occupancy);
   else occs = {0, 2};
-  // one launch or two (with the prune on): the deferral pays where walked
-  // items are long and few, or where the prune resolves nearly every item
-  std::vector<int> launch_modes;
-  if (o.launches) launch_modes.push_back(o.launches);
-  else if (mode) launch_modes = {1, 2};
-  else launch_modes.push_back(1);
-  std::vector<pbat_options> cands;
-  for (int L : Ls)
-    for (int nt : nts)
-      for (int oc : occs)
-        for (int nl : launch_modes) {
+  double best_ms = 1e300;
+  TuneChoice best{-1, 128, mode, 0, 1};
+  for (const bool merge : {true, false}) {
+    if (merge ? (!mode || o.launches == 1) : best.L >= 0) continue;
+    // merged: around the planner's choice (see bs_plan_roles)
+    const int mid = (free_bits - 6) / 3;
+    const int lo = merge ? std::max({0, free_bits - 24, mid - 3}) : std::max(0, lmax - (large ? 2 : 6));
+    std::vector<pbat_options> cands;
+    for (int L = lo; L <= (merge ? std::min(lmax, mid + 1) : lmax); ++L)
+      for (int nt : nts)
+        for (int oc : occs) {
           if (oc * nt > 2048) continue;
           pbat_options t = o;
           t.prune = mode;
           t.walk_bits = L;
           t.block_threads = nt;
           t.occupancy = oc;
-          t.launches = nl;
+          t.launches = merge ? 2 : 1;
           cands.push_back(t);
         }
-  bs_precompile(g, p, grad, cands, dev);
-  double best_ms = 1e300;
-  TuneChoice best{-1, 128, mode, 0, 1};
-  for (const pbat_options& t : cands) {
-    const double ms = tune_time(g, p, grad, t, st);
-    if (ms > 0 && ms < best_ms)
-      best_ms = ms, best = TuneChoice{t.walk_bits, t.block_threads, t.prune, t.occupancy, t.launches};
+    bs_precompile(g, p, grad, cands, dev);
+    for (const pbat_options& t : cands) {
+      const double ms = tune_time(g, p, grad, t, st);
+      if (ms > 0 && ms < best_ms)
+        best_ms = ms, best = TuneChoice{t.walk_bits, t.block_threads, t.prune, t.occupancy, t.launches};
+    }
   }
   cudaStreamDestroy(st);
   if (best.L < 0) return PBAT_OK;  // keep the planner's defaults
@@ -736,22 +745,11 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   }
   J->n_items = n_items;
   J->grid_nthr = nthr;
-  // Deferring the walked items to a second launch lets the whole grid share
-  // them at the end instead of meeting them in ticket order: with the
-  // prune-aware plan of the 40-arc network 9% of the items are walked, each
-  // about 10^5 instructions per warp, spread over the whole ticket range, so
-  // the last ones otherwise start late (fused kernel on GB300: 22.7 -> 20.8
-  // ms at the best shapes).  The first launch visits the items with a fixed
-  // warp stride and appends deferred items 32 at a time.  The R kernel's
-  // items are shorter and it stays faster in one launch (7.7 against 8.0
-  // ms), so by default only the fused kernel defers; opt.launches (or the
-  // autotuner) chooses otherwise.  Small item counts keep one launch by
-  // default (the second costs a launch latency).
-  const bool can_two = J->bs && o.prune && n_items <= (1ull << 24);
-  J->two_phase = can_two && (o.launches == 2 ||
-                             (o.launches == 0 && grad && n_items >= (1ull << 18)));
-  // the list has a slot for every item (at most 128 MiB), so it never fills
-  const unsigned long long list_cap = J->two_phase ? n_items : 0;
+  // Items merged by signature, or every item by itself in one launch (see
+  // bs_merge_body in the kernel source).  Below kMergeItems items the run is
+  // a few microseconds long and further launches cost more than they save.
+  const BsMerge mg = J->bs && o.prune && o.launches != 1 ? bs_merge(*J->bs) : BsMerge{};
+  J->merged = mg.slots > 0 && (o.launches == 2 || n_items >= kMergeItems);
   const long long warps_per_block = nthr / 32;
   long long grid = (long long)per_sm * J->dev.sms;
   // never more warps than work items
@@ -759,10 +757,16 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
                           warps_per_block - 1) / warps_per_block;
   grid = std::max(1LL, std::min(grid, need));
   J->grid = (int)grid;
-  if (J->bs) {
-    // the two launches of a two-launch run fill the GPU at their own occupancy
-    J->grid1 = (int)std::max(1LL, std::min((long long)bs_per_sm(*J->bs, 1) * J->dev.sms, need));
-    J->grid2 = (int)std::max(1LL, std::min((long long)bs_per_sm(*J->bs, 2) * J->dev.sms, need));
+  if (J->merged) {
+    auto fit = [&](int phase, unsigned long long warps, int per_block) {
+      const long long want = (long long)((warps + per_block - 1) / per_block);
+      return (int)std::max(1LL, std::min((long long)bs_per_sm(*J->bs, phase) * J->dev.sms, want));
+    };
+    // few blocks: up to 32 warps share one (its items' latency is in the way)
+    while (J->split_log2 < 5 && (mg.blocks << (J->split_log2 + 1)) <= 8ull * J->dev.sms) ++J->split_log2;
+    J->grid1 = fit(1, mg.blocks << J->split_log2, 4);
+    J->grid2 = fit(2, std::min(n_items, mg.slots), (int)warps_per_block);
+    J->grid3 = fit(3, mg.blocks, 4);
   }
   const int m = g.m;
   // accumulators per block: the frontier kernel and the bit-sliced R kernel
@@ -777,33 +781,44 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   const size_t o_counter = off; off = up16(off + 8);
   const size_t o_status = off; off = up16(off + 4);
   const size_t o_stats = off; off = up16(off + 3 * 8);
-  const size_t o_list_n = off; off = up16(off + 8);     // deferred-item count and ticket
+  const size_t o_list_n = off; off = up16(off + 8);     // number of classes and their ticket
   const size_t o_counter2 = off; off = up16(off + 8);
   const size_t o_out_n = off; off = up16(off + (size_t)(m + 1) * 8);
   const size_t limbs_bytes = J->bs ? (size_t)n_acc * 8 * 8 : 0;
   const size_t o_out_limbs = off; off = up16(off + limbs_bytes);
   J->reset_bytes = off;
+  // the class table of a merged run, cleared with the results
+  const size_t slots = J->merged ? (size_t)mg.slots : 0;
+  const size_t o_key = off; off = up16(off + slots * 8);
+  const size_t o_cmass = off; off = up16(off + slots * 16);
+  const size_t o_hist = off; off = up16(off + slots * mg.hist * 4);
+  J->clear_bytes = off;
   // the frontier kernel: per-block partials and the fixed-order reduction
   const size_t part_bytes = J->bs ? 0 : (size_t)grid * n_acc * sizeof(dd);
   const size_t o_part_acc = off; off = up16(off + part_bytes);
   const size_t o_part_n = off; off = up16(off + (J->bs ? 0 : (size_t)grid * (m + 1) * 8));
   const size_t o_out_acc = off; off = up16(off + (size_t)n_acc * sizeof(dd));
   // per-warp slots of every block of the largest of the launches' grids
-  const long long grid_max = std::max<long long>(grid, std::max(J->grid1, J->grid2));
-  const size_t wacc_bytes =
-      (J->bs && bs_grad(*J->bs)) ? (size_t)grid_max * (nthr / 32) * (1 + 2 * m) * 24 : 0;
+  const long long warps_max = std::max<long long>(std::max<long long>(grid, J->grid2) * warps_per_block, J->grid3 * 4LL);
+  const size_t wacc_bytes = (J->bs && bs_grad(*J->bs)) ? (size_t)warps_max * (1 + 2 * m) * 24 : 0;
   const size_t o_wacc = off; off = up16(off + wacc_bytes);
   const size_t o_wmid = off; off = up16(off + wmid.size() * sizeof(u128));
-  size_t o_lane = 0, o_thr = 0, o_wmid64 = 0, o_ptab = 0, o_ptabx = 0, o_tab_end = 0;
+  size_t o_lane = 0, o_thr = 0, o_wmid64 = 0, o_ptab = 0, o_ptabx = 0, o_mtab = 0, o_tab_end = 0;
   if (J->bs) {
     o_lane = off; off = up16(off + bs_lane_tab(*J->bs).size() * 8);
     o_thr = off; off = up16(off + bs_thr_tab(*J->bs).size() * 8);
     o_wmid64 = off; off = up16(off + bs_wmid(*J->bs).size() * 8);
     o_ptab = off; off = up16(off + bs_ptab(*J->bs).size() * sizeof(MxHost));
     o_ptabx = off; off = up16(off + bs_ptab_ex(*J->bs).size() * sizeof(MxHost));
+    o_mtab = off; off = up16(off + (J->merged ? bs_mtab(*J->bs).size() * 8 : 0));
     o_tab_end = off;
   }
-  const size_t o_list = off; off = up16(off + (size_t)list_cap * 8);
+  const size_t o_list = off; off = up16(off + slots * 4);
+  const size_t o_rep = off; off = up16(off + slots * 8);
+  const bool fold = J->merged && grad;
+  const size_t o_csum = off; off = up16(off + (fold ? slots * 16 : 0));
+  const size_t o_cmask = off; off = up16(off + (fold ? (size_t)mg.blocks * 32 * 8 : 0));
+  const size_t o_cls = off; off = up16(off + (fold ? (size_t)n_items * 4 : 0));
   const size_t dbytes = off;
   // host (pinned) layout: results + staging of the walk table
   // the first reset_bytes mirror the device's result region (one copy back)
@@ -831,8 +846,14 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   J->W.out_n = (unsigned long long*)(d + o_out_n);
   J->W.out_limbs = limbs_bytes ? (unsigned long long*)(d + o_out_limbs) : nullptr;
   J->W.wacc = wacc_bytes ? (void*)(d + o_wacc) : nullptr;
-  J->W.list = list_cap ? (unsigned long long*)(d + o_list) : nullptr;
-  J->W.list_cap = list_cap;
+  J->W.list = (unsigned int*)(d + o_list);
+  J->W.key = (unsigned long long*)(d + o_key);
+  J->W.cmass = (unsigned long long*)(d + o_cmass);
+  J->W.hist = (unsigned int*)(d + o_hist);
+  J->W.rep = (unsigned long long*)(d + o_rep);
+  J->W.csum = (void*)(d + o_csum);
+  J->W.cmask = (void*)(d + o_cmask);
+  J->W.cls = (unsigned int*)(d + o_cls);
   J->W.list_n = (unsigned long long*)(d + o_list_n);
   J->W.counter2 = (unsigned long long*)(d + o_counter2);
   J->d_wmid = (u128*)(d + o_wmid);
@@ -858,11 +879,13 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
     memcpy(hb + o_wmid64, wm.data(), wm.size() * 8);
     memcpy(hb + o_ptab, pt.data(), pt.size() * sizeof(MxHost));
     if (!px.empty()) memcpy(hb + o_ptabx, px.data(), px.size() * sizeof(MxHost));
-    J->d_lane = (unsigned long long*)(d + o_lane);
-    J->d_thr = (unsigned long long*)(d + o_thr);
-    J->d_wmid64 = (unsigned long long*)(d + o_wmid64);
-    J->d_ptab = (void*)(d + o_ptab);
-    J->d_ptabx = (void*)(d + o_ptabx);
+    if (J->merged) memcpy(hb + o_mtab, bs_mtab(*J->bs).data(), bs_mtab(*J->bs).size() * 8);
+    J->tabs.lane = d + o_lane;
+    J->tabs.thr = d + o_thr;
+    J->tabs.walk = d + o_wmid64;
+    J->tabs.ptab = d + o_ptab;
+    J->tabs.ptab_ex = d + o_ptabx;
+    J->tabs.merge = d + o_mtab;
     J->wmid_host_staging = h + h_lane;
     J->wmid_bytes = o_tab_end - o_lane;
     J->d_wmid = (u128*)(d + o_lane);  // upload destination
@@ -915,7 +938,7 @@ static void event_pairs_release(int device, std::vector<std::pair<cudaEvent_t, c
 int job_launch(Job* J, cudaStream_t st) {
   NvtxRange nv("pbat launch");
   if (fault_at("launch")) return fail(PBAT_ECUDA, "injected fault: kernel launch");
-  PBAT_CUDA(cudaMemsetAsync(J->W.counter, 0, J->reset_bytes, st));  // counter, status, stats, results
+  PBAT_CUDA(cudaMemsetAsync(J->W.counter, 0, J->clear_bytes, st));  // counter, status, stats, results, classes
   const bool timed = J->n_pending < 65536;
   if (timed && J->n_pending == J->evs.size()) {
     std::pair<cudaEvent_t, cudaEvent_t> e;
@@ -924,14 +947,12 @@ int job_launch(Job* J, cudaStream_t st) {
     J->evs.push_back(e);
   }
   if (timed) PBAT_CUDA(cudaEventRecord(J->evs[J->n_pending].first, st));
-  if (J->bs && !J->two_phase) {
-    PBAT_CUDA(bs_launch(*J->bs, J->grid, st, J->d_lane, J->d_thr, J->d_wmid64, J->d_ptab,
-                        J->d_ptabx, J->W, 0));
+  if (J->bs && !J->merged) {
+    PBAT_CUDA(bs_launch(*J->bs, J->grid, st, J->tabs, J->W, 0, 0));
   } else if (J->bs) {
-    PBAT_CUDA(bs_launch(*J->bs, J->grid1, st, J->d_lane, J->d_thr, J->d_wmid64, J->d_ptab,
-                        J->d_ptabx, J->W, 1));
-    PBAT_CUDA(bs_launch(*J->bs, J->grid2, st, J->d_lane, J->d_thr, J->d_wmid64, J->d_ptab,
-                        J->d_ptabx, J->W, 2));
+    PBAT_CUDA(bs_launch(*J->bs, J->grid1, st, J->tabs, J->W, 1, J->split_log2));
+    PBAT_CUDA(bs_launch(*J->bs, J->grid2, st, J->tabs, J->W, 2, 0));
+    if (bs_grad(*J->bs)) PBAT_CUDA(bs_launch(*J->bs, J->grid3, st, J->tabs, J->W, 3, 0));
   }
   else
     PBAT_CUDA(launch_frontier(J->pl.grad, J->pl.wide, J->grid, J->pl.nthr, J->pl.smem, st, J->P,
@@ -945,6 +966,20 @@ int job_launch(Job* J, cudaStream_t st) {
 }
 
 void job_destroy(Job* J);
+
+int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* dRdp_out,
+             pbat_options* opt);
+
+// The same question under other options, in place of J's results.
+static int job_rerun(Job* J, pbat_options o, cudaStream_t st, double* R_out, uint64_t* Nk_out,
+                     double* dRdp_out, pbat_options* opt) {
+  Job* F = nullptr;
+  int rc = job_create(J->g, J->p_copy.data(), J->pl.grad, &o, &F);
+  if (!rc && !(rc = job_upload(F, st)) && !(rc = job_launch(F, st)))
+    rc = job_read(F, st, R_out, Nk_out, J->pl.grad ? dRdp_out : nullptr, opt);
+  job_destroy(F);
+  return rc;
+}
 
 // Copy results to the host and wait; convert to input arc order.
 int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* dRdp_out,
@@ -961,12 +996,23 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
   if (*J->h_status & 1u)
     return fail(PBAT_ETIMEOUT, "time budget of %.3f s ran out on the device",
                 J->opt_copy.time_budget_s);
+  if (*J->h_status & 2u) {
+    // more classes than the table holds (the network's structure decides
+    // that): every item by itself, now and from now on
+    bs_mark_unmergeable(*J->bs);
+    pbat_options o = J->opt_copy;
+    o.launches = 1;
+    J->merged = false;
+    J->n_pending = 0;
+    return job_rerun(J, o, st, R_out, Nk_out, dRdp_out, opt);
+  }
   if (J->bs)
     for (int i = 0; i < J->n_acc; ++i) J->h_acc[i] = limbs256_to_dd(J->h_limbs + 8 * i);
   if (opt) {
     const unsigned long long item = J->item_states;
-    opt->stats[0] = J->h_stats[0] * item;
-    opt->stats[1] = (J->h_stats[1] + J->h_stats[2]) * item;
+    opt->stats[0] = J->h_stats[0] * item;   // a class counts once
+    opt->stats[1] = J->merged ? (J->n_items - J->h_stats[0]) * item
+                              : (J->h_stats[1] + J->h_stats[2]) * item;
     opt->stats[2] = J->wmid_bytes;
     opt->stats[3] = J->reset_bytes + (J->bs ? 0 : J->n_acc * sizeof(dd));
     double ns = 0.0;
@@ -978,8 +1024,8 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
         cudaGetLastError();
     }
     opt->stats[4] = (unsigned long long)ns;
-    // one kernel per launch, two in two-phase runs; the frontier kernel adds its reduce
-    opt->stats[5] = (J->bs ? (J->two_phase ? 2 : 1) : 2) * J->n_pending;
+    // one kernel per launch, two (fused: three) in merged runs; the frontier kernel adds its reduce
+    opt->stats[5] = (J->bs ? (J->merged ? (bs_grad(*J->bs) ? 3 : 2) : 1) : 2) * J->n_pending;
     opt->stats[6] = J->n_items;
     opt->stats[7] = J->n_pending;
   }
@@ -988,7 +1034,7 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
   std::vector<double> gi;
   if (J->bs && dRdp_out) {
     gi.resize(m);
-    bs_finish_grad(*J->bs, J->h_acc, m, gi.data());
+    bs_finish_grad(*J->bs, J->h_acc, m, J->merged, gi.data());
   }
   // The bit-sliced kernels' error bounds against the accuracy promised:
   // R within 1e-12 relative; each dR/dp_k within 1e-12 of max(|g_k|,
@@ -1009,12 +1055,7 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
     // kernel, whose tables are exact to 2^-100
     pbat_options o = J->opt_copy;
     o.algo = PBAT_ALGO_FRONTIER;
-    Job* F = nullptr;
-    int rc = job_create(J->g, J->p_copy.data(), J->pl.grad, &o, &F);
-    if (!rc && !(rc = job_upload(F, st)) && !(rc = job_launch(F, st)))
-      rc = job_read(F, st, R_out, Nk_out, J->pl.grad ? dRdp_out : nullptr, opt);
-    job_destroy(F);
-    return rc;
+    return job_rerun(J, o, st, R_out, Nk_out, dRdp_out, opt);
   }
   *R_out = R;
   if (Nk_out)

@@ -54,6 +54,19 @@ struct Scratch {
 int scratch_acquire(int device, size_t dbytes, size_t hbytes, Scratch** out);
 void scratch_release(Scratch* s);
 
+// Device copies of a bit-sliced plan's tables.
+struct BsTables {
+  const void *lane = nullptr, *thr = nullptr, *walk = nullptr, *ptab = nullptr, *ptab_ex = nullptr;
+  const void* merge = nullptr;
+};
+// Sizes of a merged run (bit-sliced plans): blocks of items, slots of the
+// class table (0: not to be merged), popcounts kept per class.
+struct BsMerge {
+  unsigned long long blocks = 0, slots = 0;
+  int hist = 0;
+};
+
+double range_mass(int m, const double* p, const pbat_options& o);
 int run_single(const GraphIn& g, const double* p, bool grad, pbat_options* opt, void* stream,
                double* R_out, uint64_t* Nk_out, double* dRdp_out);
 

@@ -50,13 +50,19 @@ struct DevWork {
   unsigned long long* out_n;    // [m + 1]
   void* wacc;                   // fused bit-sliced kernel: per-warp accumulators (24 B each)
   unsigned long long* out_limbs;  // bit-sliced kernels: [n_acc][8] 256-bit fixed point, scale 2^250
-  // two-phase bit-sliced launches: the first defers the items its prune
-  // leaves to walk to `list` (capacity list_cap, count list_n), the second
-  // walks them, taking them by the ticket counter2
-  unsigned long long* list;
-  unsigned long long list_cap;
+  // merged runs of the bit-sliced kernels (BsWork in the kernel source): the
+  // classes' slots, their count and ticket, the class table, and per item
+  // what the gradient's last launch reads
+  unsigned int* list;
   unsigned long long* list_n;
   unsigned long long* counter2;
+  unsigned long long* key;
+  unsigned long long* cmass;
+  unsigned int* hist;
+  unsigned long long* rep;
+  void* csum;
+  void* cmask;
+  unsigned int* cls;
 };
 
 }  // namespace pbat

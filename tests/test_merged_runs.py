@@ -1,0 +1,165 @@
+"""Merged runs of the bit-sliced kernels: items whose prefixes leave the same
+network share one walk.  On the CPU, the generated signature program is
+evaluated in Python and compared with the connectivity it stands for; on the
+GPU, merged runs are compared with one-launch runs and the oracle at the
+sizes where blocks of items, words of signatures and tables change shape."""
+import re
+
+import pytest
+
+import oracle
+import synth
+
+FULL = 0xFFFFFFFF
+
+
+@pytest.fixture(scope="module")
+def pb():
+    from paper_2209_09711_gb300 import build
+    build.build()
+    import paper_2209_09711_gb300 as mod
+    return mod
+
+
+def _signature_program(src):
+    perm = [int(x) for x in src.splitlines()[0].split(":")[1].split()]
+    defs = {k: v for k, v in re.findall(r"#define (BS_\w+) (-?\w+)", src)}
+    body = src[src.index("void bs_sig("):]
+    return perm, defs, body[:body.index("\n}\n")]
+
+
+def _evaluate(body, a, n):
+    env, z = {"a": a}, [0] * n
+    for line in body.splitlines()[1:]:
+        m = re.match(r"\s*const u32 (\w+) = (.*);$", line)
+        if m:
+            env[m.group(1)] = eval(m.group(2), {}, env) & FULL
+            continue
+        m = re.match(r"\s*z\[(\d+)\] = (.*);$", line)
+        z[int(m.group(1))] = eval(m.group(2), {}, env) & FULL
+    return z
+
+
+def _residual(net, prefix, on, free):
+    """What the working prefix arcs leave between the boundary nodes: who
+    reaches whom, without what the source reaches and what reaches the sink
+    already say."""
+    s, t = net.source, net.sink
+    bound = sorted({s, t} | {v for k in free for v in (net.tail[k], net.head[k])})
+    reach = {v: {v} for v in range(net.n)}
+    grew = True
+    while grew:
+        grew = False
+        for k, works in zip(prefix, on):
+            if not works:
+                continue
+            u, v = net.tail[k], net.head[k]
+            for x, y in ((u, v),) if net.directed else ((u, v), (v, u)):
+                if net.directed and (y == s or x == t):
+                    continue
+                for r in reach.values():
+                    if x in r and y not in r:
+                        r.add(y)
+                        grew = True
+    pairs = {(x, y) for x in bound for y in bound if x != y and y in reach[x]}
+    if net.directed:
+        pairs = {(x, y) for x, y in pairs
+                 if x == s or y == t or not ((s, x) in pairs or (s, y) in pairs or (x, t) in pairs)}
+    return frozenset(pairs)
+
+
+@pytest.mark.parametrize("directed", [False, True])
+@pytest.mark.parametrize("prune", [1, 2])
+def test_signature_is_the_residual_network(pb, directed, prune):
+    """Over 32 random items at a time, those whose prefix does not join source
+    and sink: equal signatures exactly where the prefix leaves the same
+    connectivity."""
+    for seed in range(10):
+        rng = synth.SplitMix64(8100 + seed)
+        n, m = 3 + rng.below(9), 14 + rng.below(14)
+        net = synth.random_small(8200 + seed, n=n, m=m, directed=directed)
+        src = pb.kernel_source(net, pb.options(walk_bits=seed % 3, prune=prune))
+        perm, D, body = _signature_program(src)
+        top, nsig = int(D["BS_TOP"]), int(D["BS_NSIG"])
+        assert int(D["BS_MERGE"]) == 1 and 0 <= nsig <= 63
+        words = [rng.next_u64() & FULL for _ in range(m)]
+        z = _evaluate(body, [0] * top + words[top:], nsig)
+        items = [[(words[k] >> i) & 1 for k in range(top, m)] for i in range(32)]
+        sig = [tuple((w >> i) & 1 for w in z) for i in range(32)]
+        res = [_residual(net, perm[top:], on, perm[:top]) for on in items]
+        st = (net.source, net.sink)   # items that join these are not classed
+        left = [i for i in range(32) if st not in res[i]]
+        for i in left:
+            for j in left:
+                assert (sig[i] == sig[j]) == (res[i] == res[j]), (seed, i, j)
+
+
+def _same(a, b, tol):
+    return abs(a - b) <= tol
+
+
+def _check(pb, net, p=None, grad=True, ref=None, merged=True, **opt):
+    one = pb.reliability_net(net, p=p, grad=grad, opts=pb.options(launches=1, algo=pb.ALGO_BITSLICE, **opt))
+    two = pb.reliability_net(net, p=p, grad=grad, opts=pb.options(launches=2, algo=pb.ALGO_BITSLICE, **opt))
+    assert one.stats[5] == 1
+    if merged:
+        assert two.stats[5] == (3 if grad else 2)
+    assert two.Nk == one.Nk
+    # the bit-sliced bounds: R within 2^-61 + 2^-59 (+ the R kernel's walk
+    # masses, 2^(L-64) with L <= 10), each gradient entry within 2^-57, either
+    # run, and their rounding to doubles
+    assert _same(two.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+    if grad:
+        for x, y in zip(two.grad, one.grad):
+            assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (x, y)
+    if ref is not None:
+        assert two.Nk == ref.Nk
+        assert _same(two.R, ref.R, 1e-12 * ref.R + 1e-300)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m", [11, 12, 15, 16, 19, 20, 21, 22])
+@pytest.mark.parametrize("directed", [False, True])
+def test_merged_runs_at_block_edges(pb, m, directed):
+    """One to twelve prefix arcs: blocks of two items up to full ones, one
+    block and several, with and without walk arcs."""
+    for seed in range(2):
+        net = synth.random_small(9300 + 10 * m + seed, n=4 + (m + seed) % 7, m=m, directed=directed, p_lo=0.2, p_hi=0.99)
+        for grad in (False, True):
+            ref = oracle.enumerate_states(net) if m < 20 else None
+            for walk in {0, min(3, m - 11)}:
+                _check(pb, net, grad=grad, ref=ref, walk_bits=walk, prune=1 + seed)
+
+
+@pytest.mark.gpu
+def test_merged_runs_of_ranges_and_extreme_reliabilities(pb):
+    """Equal divisions whose blocks are smaller than a word, and arcs that
+    always work or never do among the prefix arcs (with too many of them the
+    fused kernel is not merged)."""
+    net = synth.random_small(611, n=7, m=20, p_lo=0.1, p_hi=0.95)
+    for bits in (1, 6, 9):
+        for lo in (0, 1):
+            for grad in (False, True):
+                ref = oracle.enumerate_states(net, prefix_bits=bits, prefix_lo=lo, prefix_hi=lo + 1)
+                _check(pb, net, grad=grad, ref=ref, walk_bits=0, range_bits=bits, range_lo=lo, range_hi=lo + 1)
+    for bad in (1, 4, 11, 16):
+        p = [(1.0 if k % 3 else 0.0) if k < bad else q for k, q in enumerate(net.p)]
+        ref = oracle.enumerate_states(net, p=p)
+        for grad in (False, True):
+            _check(pb, net, p=p, grad=grad, ref=ref, merged=not grad, walk_bits=0)
+
+
+@pytest.mark.gpu
+def test_more_classes_than_the_table_holds(pb):
+    """A network of 2^24 items in more than 2^18 classes: the merged run is
+    given up and every item walked, with the same counts and reliability, for
+    a kept plan from its first read on."""
+    tail, head, rng = synth.random_connected_undirected(20, 38, 902)
+    net = synth.Network(20, tail, head, synth.uniform_p(rng, 38, 0.7, 0.95), 0, 19)
+    want = pb.reliability_net(net, opts=pb.options(autotune=0, launches=1, walk_bits=4))
+    plan = pb.Plan(net, opts=pb.options(autotune=0, launches=2, walk_bits=4))
+    for _ in range(2):
+        plan.execute()
+        res = plan.read()
+        assert res.stats[5] == 1
+        assert res.Nk == want.Nk and _same(res.R, want.R, 1e-12 * want.R)
