@@ -81,17 +81,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "12d89125041c92dd": (52494086 / 2**40, 5643776, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "37df6b1409896506": (52898657 / 2**40, 5649664, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "f73d4ef71d415742": (20249019 / 2**40, 559360, "profiles/bs_kernel_undirected24x40.md"),
+    "bcf1dfc496e39eac": (20601601 / 2**40, 563712, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "8dccfa2a141e159a": (1023216 / 2**34, 249344, "profiles/bs_kernel_grad_directed20x34.md"),
+    "94e55a18f9749108": (1135726 / 2**34, 263680, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "753137a3382ba2aa": (786202 / 2**34, 99840, "profiles/bs_kernel_directed20x34.md"),
+    "2f33d29f92400dc4": (879618 / 2**34, 108032, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "64f7b6748b6b3400": (1631106 / 2**27, 469248, "profiles/bs_kernel_grad_grid3x6.md"),
+    "a1c4af05cd02c1c0": (1715071 / 2**27, 478208, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "2d85f5eebf446005": (1037543 / 2**27, 148224, "profiles/bs_kernel_grid3x6.md"),
+    "037ffde57a2a4231": (1129100 / 2**27, 156672, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

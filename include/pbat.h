@@ -158,14 +158,14 @@ typedef struct pbat_graph {
 } pbat_graph;
 
 /*
- * Many networks, each with n_pvec arc-reliability vectors, in one
- * persistent launch (captured once in a CUDA graph and replayed).  Each
- * state's connectivity is computed once and weighted by every p-vector.
- * With dRdp_out, one launch of the gradient module gives R, N_k and dR/dp
- * for every (network, p-vector); pairs whose R or gradient the bit-sliced
- * fixed-point bounds cannot certify to 1e-12 (small R) are re-run exactly
- * with the frontier kernel, one enumeration each.  opt->stats[4] holds the
- * device time of the batched launch in ns.
+ * Many networks, each with n_pvec arc-reliability vectors, in one launch of
+ * a CUDA graph (captured once and replayed).  Each state's connectivity is
+ * computed once and weighted by every p-vector.
+ * With dRdp_out, the gradient module gives R, N_k and dR/dp for every
+ * (network, p-vector); pairs whose R or gradient the bit-sliced fixed-point
+ * bounds cannot certify to 1e-12 (small R) are re-run exactly with the
+ * frontier kernel, one enumeration each.  opt->stats[4] holds the device time
+ * of the graph in ns, stats[5] its launches (1).
  *   p         per graph g: n_pvec x m_g doubles (vector-major), concatenated in
  *             graph order
  *   R_out     out, n_graphs x n_pvec doubles (graph-major)

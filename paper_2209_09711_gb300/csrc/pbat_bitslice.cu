@@ -13,6 +13,7 @@
 #include <memory>
 #include <mutex>
 #include <queue>
+#include <set>
 #include <string>
 #include <thread>
 #include <vector>
@@ -64,8 +65,10 @@ static bool nvrtc_cubin(const std::string& src, int cc, std::vector<char>& cubin
     return false;
   }
   const std::string arch = "-arch=sm_" + std::to_string(cc) + "a";
-  const char* opts[] = {arch.c_str(), "-std=c++17", "-lineinfo", "-diag-suppress=177"};
-  const nvrtcResult rc = nvrtcCompileProgram(prog, 4, opts);
+  // a batch's networks are functions of their own: compiled on several threads
+  const bool split = src.find("#define BSB_MERGE 1") != std::string::npos;
+  const char* opts[] = {arch.c_str(), "-std=c++17", "-lineinfo", "-diag-suppress=177", "--split-compile=8"};
+  const nvrtcResult rc = nvrtcCompileProgram(prog, split ? 5 : 4, opts);
   if (rc != NVRTC_SUCCESS) {
     size_t ls = 0;
     nvrtcGetProgramLogSize(prog, &ls);
@@ -153,14 +156,20 @@ static int jit_compile(const std::string& src, const DeviceInfo& dev, const char
   JitEntry e;
   cudaError_t ce = cudaLibraryLoadData(&e.lib, cubin.data(), nullptr, nullptr, 0, nullptr, nullptr, 0);
   if (ce != cudaSuccess) return fail(PBAT_ECUDA, "cudaLibraryLoadData: %s", cudaGetErrorString(ce));
-  ce = cudaLibraryGetKernel(&e.kernel, e.lib, kname);
-  if (ce != cudaSuccess) return fail(PBAT_ECUDA, "cudaLibraryGetKernel: %s", cudaGetErrorString(ce));
-  // optional per-phase entry points: absent from the batched modules
+  // the launches of merged runs; a merged single-network module has only
+  // these, and its walking launch in the one-launch kernel's place
   if (cudaLibraryGetKernel(&e.kernel_p1, e.lib, (std::string(kname) + "_p1").c_str()) != cudaSuccess ||
       cudaLibraryGetKernel(&e.kernel_p2, e.lib, (std::string(kname) + "_p2").c_str()) != cudaSuccess) {
     cudaGetLastError();
     e.kernel_p1 = e.kernel_p2 = nullptr;
   }
+  ce = cudaLibraryGetKernel(&e.kernel, e.lib, kname);
+  if (ce != cudaSuccess && e.kernel_p2) {
+    cudaGetLastError();
+    e.kernel = e.kernel_p2;
+    ce = cudaSuccess;
+  }
+  if (ce != cudaSuccess) return fail(PBAT_ECUDA, "cudaLibraryGetKernel: %s", cudaGetErrorString(ce));
   if (cudaLibraryGetKernel(&e.kernel_p3, e.lib, (std::string(kname) + "_p3").c_str()) != cudaSuccess) {
     cudaGetLastError();
     e.kernel_p3 = nullptr;
@@ -206,7 +215,6 @@ struct BsLaunch {
   int per_sm = 1;                     // resident blocks per SM: one-launch kernel
   // merged runs
   int per_sm1 = 1, per_sm2 = 1, per_sm3 = 1;
-  bool unmergeable = false;           // its classes did not fit the table before
   std::string key;                    // of the plan cache
   BsFoldParamsHost F;
   std::vector<unsigned long long> mtab;  // [128] subset sums, [32] mid pattern masses, 128 bits each
@@ -268,7 +276,7 @@ static std::string bs_source(const GraphIn& g, const BsPlan& bp, int nthr) {
            g.m, bp.ell, bp.tb, bp.L, bp.d, nthr, bp.ell + bp.tb, bp.ell + bp.tb + bp.L, bp.ncore,
            lane_mask, full_counts(bp.ell), bp.grad ? 1 : 0, acc_in_registers(bp) ? 1 : 0,
            walk_unroll_bits(bp), bp.tb >= 5 ? 0xffffffffu : ((1u << (1 << bp.tb)) - 1u), bp.minb,
-           bp.pex, bp.nsig >= 0 ? 1 : 0, bp.nsig, bp.low, bp.mid);
+           bp.pex, bp.merge ? 1 : 0, bp.nsig, bp.low, bp.mid);
   const std::string tmpl = kBsTemplate;
   const size_t cut = tmpl.find("//@@GENERATED@@");
   // only this plan's kernel: the other kernel's section is left out, so that
@@ -280,7 +288,7 @@ static std::string bs_source(const GraphIn& g, const BsPlan& bp, int nthr) {
     if (bp.grad) tail.erase(r0, f0 - r0);
     else tail.erase(f0, f1 + 6 - f0);
   }
-  return std::string(defs) + tmpl.substr(0, cut) + bp.gen + bp.gen_sig + tail;
+  return std::string(defs) + tmpl.substr(0, cut) + bp.gen + (bp.merge ? bp.gen_sig : "") + tail;
 }
 
 // Generated source for a network (no device needed); see pbat_kernel_source.
@@ -320,7 +328,7 @@ static std::string bs_plan_key(const GraphIn& g, const double* p, bool grad, con
   std::string k;
   auto put = [&](long long v) { k.append((const char*)&v, sizeof v); };
   put(device); put(g.n); put(g.m); put(g.directed); put(g.source); put(g.sink); put(grad);
-  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(nthr); put(o.prune);
+  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(nthr); put(o.prune); put(o.launches);
   put(std::max(0, o.occupancy));
   k.append((const char*)g.tail, sizeof(int32_t) * g.m);
   k.append((const char*)g.head, sizeof(int32_t) * g.m);
@@ -329,15 +337,63 @@ static std::string bs_plan_key(const GraphIn& g, const double* p, bool grad, con
   return k;
 }
 
+// A merge block's masses: subset sums by nibble of its low patterns (nib, 128
+// entries) and its mid patterns (mid, 32), 128 bits each at scale 2^127.
+static void block_tables(const double* p, const int* arcs, int low, int mid, unsigned long long* nib,
+                         unsigned long long* out_mid) {
+  dd w[32];
+  product_table(p, arcs, low, w);
+  uint128_host f[32];
+  for (int j = 0; j < 32; ++j) {
+    u128 v{0, 0};
+    if (j < (1 << low)) v = to_fixed127(w[j]);
+    f[j] = ((uint128_host)v.hi << 64) | v.lo;
+  }
+  for (int b = 0; b < 8; ++b) {
+    uint128_host sum[16];
+    sum[0] = 0;
+    for (int v = 0; v < 16; ++v) {
+      if (v) sum[v] = sum[v & (v - 1)] + f[4 * b + __builtin_ctz((unsigned)v)];
+      nib[2 * (16 * b + v)] = (unsigned long long)sum[v];
+      nib[2 * (16 * b + v) + 1] = (unsigned long long)(sum[v] >> 64);
+    }
+  }
+  product_table(p, arcs + low, mid, w);
+  for (int j = 0; j < 32; ++j) {
+    u128 v{0, 0};
+    if (j < (1 << mid)) v = to_fixed127(w[j]);
+    out_mid[2 * j] = v.lo;
+    out_mid[2 * j + 1] = v.hi;
+  }
+}
+
+// What the fold takes per arc of a block: its p and the masses of the arcs
+// folded after it; absent low arcs (blocks of fewer than 32 bits) have p = 0.
+static void fold_tables(const double* p, const int* arcs, int low, int mid, BsFoldParamsHost& F) {
+  memset(&F, 0, sizeof F);
+  dd w[32];
+  product_table(p, arcs + low, mid, w);
+  for (int j = 0; j < (1 << mid); ++j) F.mid[j] = fixed_u64(w[j], 63);
+  for (int part = 0; part < 2; ++part) {
+    const int* a = arcs + (part ? low : 0);
+    const int n = part ? mid : low;
+    unsigned long long* out = part ? F.wmid : F.wlow;
+    for (int b = 0, at = 0; b < 5; at += 16 >> b, ++b) {
+      if (b < n) F.p[5 * part + b] = fixed_u64(dd_make(p[a[b]]), 63);
+      const int above = std::max(0, n - b - 1);
+      product_table(p, a + b + 1, above, w);
+      for (int v = 0; v < (1 << above); ++v) out[at + v] = fixed_u64(w[v], 63);
+    }
+  }
+}
+
 // Tables of a merged run: masses of the prefix arcs above a block by level,
-// subset sums and masses of the block's low and mid patterns, and for the
-// fold each arc's p and the masses of the arcs folded after it.
+// the block's, and the fold's.
 static void merge_tables(const double* p, const pbat_options& o, int m, BsLaunch& bl) {
   const BsPlan& bp = bl.plan;
   BsParamsHost& P = bl.P;
   const int top = bp.ell + bp.tb + bp.L, blk = bp.low + bp.mid, nhi = bp.d - blk;
   const int* low = bp.perm.data() + top;
-  const int* mid = low + bp.low;
   const int max_bits = 6;
   P.nlev_hi = (nhi + max_bits - 1) / max_bits;
   for (int l = 0, sh = 0; l < P.nlev_hi; ++l) {
@@ -353,44 +409,8 @@ static void merge_tables(const double* p, const pbat_options& o, int m, BsLaunch
   const double mass = range_mass(m, p, o);
   P.mass_exp = mass > 0.0 && mass < 1.0 ? std::max(0, -(ilogb(mass) + 1)) : 0;
   bl.mtab.assign(2 * (128 + 32), 0ull);
-  dd w[32];
-  product_table(p, low, bp.low, w);
-  uint128_host f[32];
-  for (int j = 0; j < 32; ++j) {
-    u128 v{0, 0};
-    if (j < (1 << bp.low)) v = to_fixed127(w[j]);
-    f[j] = ((uint128_host)v.hi << 64) | v.lo;
-  }
-  for (int b = 0; b < 8; ++b) {
-    uint128_host sum[16];
-    sum[0] = 0;
-    for (int v = 0; v < 16; ++v) {
-      if (v) sum[v] = sum[v & (v - 1)] + f[4 * b + __builtin_ctz((unsigned)v)];
-      bl.mtab[2 * (16 * b + v)] = (unsigned long long)sum[v];
-      bl.mtab[2 * (16 * b + v) + 1] = (unsigned long long)(sum[v] >> 64);
-    }
-  }
-  product_table(p, mid, bp.mid, w);
-  memset(&bl.F, 0, sizeof bl.F);
-  for (int j = 0; j < (1 << bp.mid); ++j) {
-    const u128 v = to_fixed127(w[j]);
-    bl.mtab[2 * (128 + j)] = v.lo;
-    bl.mtab[2 * (128 + j) + 1] = v.hi;
-    bl.F.mid[j] = fixed_u64(w[j], 63);
-  }
-  if (!bp.grad) return;
-  // absent low arcs (blocks of fewer than 32 bits) have p = 0
-  for (int part = 0; part < 2; ++part) {
-    const int* arcs = part ? mid : low;
-    const int n = part ? bp.mid : bp.low;
-    unsigned long long* out = part ? bl.F.wmid : bl.F.wlow;
-    for (int b = 0, at = 0; b < 5; at += 16 >> b, ++b) {
-      if (b < n) bl.F.p[5 * part + b] = fixed_u64(dd_make(p[arcs[b]]), 63);
-      const int above = std::max(0, n - b - 1);
-      product_table(p, arcs + b + 1, above, w);
-      for (int v = 0; v < (1 << above); ++v) out[at + v] = fixed_u64(w[v], 63);
-    }
-  }
+  block_tables(p, low, bp.low, bp.mid, bl.mtab.data(), bl.mtab.data() + 256);
+  if (bp.grad) fold_tables(p, low, bp.low, bp.mid, bl.F);
 }
 
 // Compile the kernels of several option sets ahead of bs_prepare, on host
@@ -423,13 +443,20 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
   const std::string key = bl.key = bs_plan_key(g, p, grad, o, bl.nthr, dev.device);
   bool cached = false;
   {
-    std::lock_guard<std::mutex> lk(g_bsplan_mu);
+    std::unique_lock<std::mutex> lk(g_bsplan_mu);
     auto it = g_bsplan.find(key);
     if (it != g_bsplan.end()) {
       bl.plan = it->second.plan;
       bl.jit = it->second.jit;
-      bl.unmergeable = it->second.unmergeable;
       cached = true;
+      if (it->second.unmergeable) {
+        // its classes did not fit the table before (the network's structure
+        // decides that): one launch
+        pbat_options one = o;
+        one.launches = 1;
+        lk.unlock();
+        return bs_prepare(g, p, grad, one, dev, bl);
+      }
     }
   }
   if (!cached) {
@@ -464,7 +491,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
   P.task_lo = lo;
   P.n_tasks = hi - lo;
   // merged runs: a table of twice the items, or one slot per signature
-  while (P.slots_log2 < kMaxSlotsLog2 && P.slots_log2 < bp.nsig &&
+  while (bp.merge && P.slots_log2 < kMaxSlotsLog2 && P.slots_log2 < bp.nsig &&
          (1ull << P.slots_log2) < 2 * P.n_tasks)
     ++P.slots_log2;
   // prefix masses: the d prefix arcs in levels of at most 6 bits (fused
@@ -500,7 +527,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     sh += bits;
   }
   if (bl.ptab.empty()) bl.ptab.push_back(to_mx(dd_make(1.0)));
-  if (bp.nsig >= 0) merge_tables(p, o, m, bl);
+  if (bp.merge) merge_tables(p, o, m, bl);
   // lane tables: byte position b, value v -> lane mass (scale 2^62) and the
   // counts of its set lanes by lane popcount class, packed in fields of
   // 8, 11, 12, 12, 11, 8 bits
@@ -521,7 +548,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
   }
   const int L_in = std::min(bp.L, walk_unroll_bits(bp)), L_out = bp.L - L_in;
   // the walking launch of a merged run: each warp's counts below the prefix
-  const size_t rel_bytes = bp.nsig >= 0 ? (size_t)(bl.nthr / 32) * (top + 1) * 8 : 0;
+  const size_t rel_bytes = bp.merge ? (size_t)(bl.nthr / 32) * (top + 1) * 8 : 0;
   if (!grad) {
     bl.wmid.resize((size_t)1 << bp.L);
     std::vector<dd> wt((size_t)1 << bp.L);
@@ -662,11 +689,8 @@ void bs_mark_unmergeable(const BsLaunch& bl) {
 // What a merged run of this plan needs; slots 0: it cannot be merged.
 BsMerge bs_merge(const BsLaunch& bl) {
   BsMerge r{};
-  const int blk = bl.plan.low + bl.plan.mid;
-  r.blocks = bl.P.n_tasks >> blk;
-  if (bl.plan.nsig < 0 || bl.unmergeable || !bl.jit.kernel_p1 || bl.P.n_tasks > (1ull << 24) ||
-      r.blocks > (1ull << 14) || r.blocks == 0)
-    return r;
+  if (!bl.plan.merge) return r;
+  r.blocks = bl.P.n_tasks >> (bl.plan.low + bl.plan.mid);
   r.slots = 1ull << bl.P.slots_log2;
   r.hist = (bl.plan.d + 2) & ~1;   // BS_HIST
   return r;
@@ -743,6 +767,17 @@ struct BGraphHost {
   unsigned long long full_counts;
   unsigned long long pex_mask;
   unsigned long long binom[64];
+  int low, mid, nhi, nsig, slots_log2, pad2;
+  unsigned long long blk_begin, slot_base, item_base;
+};
+// Host mirror of BMerge in the kernel source.
+struct BMergeHost {
+  void *key, *id_of, *net, *rep, *hist, *cmass, *csum, *cmask, *ent, *n_classes, *ticket;
+  unsigned long long n_blocks;
+  int split_log2, parts;
+  unsigned cap;
+  int hist_stride;
+  const void *nib, *mid, *fold;
 };
 
 constexpr int kBsbThreads = 128;
@@ -750,6 +785,9 @@ constexpr int kBsbMinBlocks = 4;  // default launch bounds: 4 blocks of 128 thre
 constexpr int kBsbMaxWalk = 5;  // 2^L connectivity words per thread staged in shared memory
 constexpr int kBsbLimbs = 8;    // 32-bit chunks of a 256-bit value at scale 2^250, in 64-bit atomics
 constexpr int kBsbMaxGraphs = 256;
+constexpr unsigned long long kBsbMaxItems = 1ull << 24;   // merged: of all networks together
+constexpr unsigned kBsbMaxClasses = 1u << 23;   // classes x p-vectors (the gradient: 32 B each)
+constexpr int kBsbFold = 104;   // 64-bit words of BsFoldParams
 
 struct BsBatch {
   std::string key;
@@ -774,10 +812,28 @@ struct BsBatch {
   bool grad = false;
   std::vector<std::string> elig;   // input order, one '0'/'1' per arc
   size_t o_wm2 = 0, o_tt = 0, o_lwex = 0, o_thwex = 0, o_ptex = 0, n_out = 0;
+  // merged modules (BMerge in the kernel source): items with the same
+  // signature walked once.  per_item: every item by itself instead
+  bool per_item = false, merged = false;
+  int nsig_max = 0, grid1 = 0, grid2 = 0, grid3 = 0;
+  size_t smem1 = 0, o_nib = 0, o_mid = 0, o_fold = 0, key_bytes = 0;
+  Scratch* mscr = nullptr;
+  BMergeHost M{};
 };
+
+// Signatures and items within the merged module's limits.
+static bool bsb_mergeable(const std::vector<BsPlan>& plans, const pbat_options& o) {
+  unsigned long long items = 0;
+  for (const BsPlan& bp : plans) {
+    if (!o.prune || bp.nsig < 0 || bp.d > 24) return false;
+    items += 1ull << bp.d;
+  }
+  return items <= kBsbMaxItems;
+}
 
 static std::mutex g_bsb_mu;
 static std::vector<BsBatch*> g_bsb;
+static std::set<std::string> g_bsb_unmergeable;   // batches whose classes did not fit
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -824,6 +880,8 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
     items[i] = 1ull << E.plans[i].d;
     E.lmax = std::max(E.lmax, E.plans[i].L);
   }
+  E.merged = !E.per_item && bsb_mergeable(E.plans, o);
+  for (const BsPlan& bp : E.plans) E.nsig_max = std::max(E.nsig_max, bp.nsig);
   E.order.resize(G);
   for (int i = 0; i < G; ++i) E.order[i] = i;
   std::stable_sort(E.order.begin(), E.order.end(), [&](int a, int b) { return items[a] > items[b]; });
@@ -832,35 +890,39 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   E.minb = o.occupancy > 0 ? o.occupancy : kBsbMinBlocks;
   std::string src = "#define BSB_NTHR " + std::to_string(kBsbThreads) + "\n#define BSB_LMAX " +
                     std::to_string(E.lmax) + "\n#define BSB_MINB " + std::to_string(E.minb) + "\n" +
-                    tmpl.substr(0, tmpl.find("//@@GENERATED@@"));
+                    "#define BSB_GRAD " + std::to_string(E.grad ? 1 : 0) + "\n#define BSB_MERGE " +
+                    std::to_string(E.merged ? 1 : 0) + "\n#define BSB_SCATTER " +
+                    (E.grad ? "bs_batch_grad_p2" : "bs_batch_p2") + "\n" + tmpl.substr(0, tmpl.find("//@@GENERATED@@"));
   for (int r = 0; r < G; ++r) {
     const BsPlan& bp = E.plans[E.order[r]];
-    std::string gen = bp.gen;
+    std::string gen = E.merged ? bp.gen + bp.gen_sig : bp.gen;
     auto rep = [&](const std::string& a, const std::string& b) {
       const size_t at = gen.find(a);
       if (at != std::string::npos) gen.replace(at, a.size(), b);
     };
     rep("__device__ __forceinline__ void bs_inv(", "static __device__ __forceinline__ void inv(");
     rep("__device__ __forceinline__ u32 bs_var(", "static __device__ __forceinline__ u32 var(");
+    rep("__device__ __forceinline__ void bs_sig(", "static __device__ __forceinline__ void sig(");
     const int m = graphs[E.order[r]].n_arcs;
     const unsigned lane_mask = bp.ell >= 5 ? 0xffffffffu : ((1u << (1 << bp.ell)) - 1u);
     char head[400];
     snprintf(head, sizeof head,
              "struct G%d {\n  static constexpr int M = %d, ELL = %d, TB = %d, L = %d, D = %d, NCORE = %d,"
-             " WALK0 = %d, TOP = %d;\n  static constexpr u32 LANE_MASK = 0x%08xu;\n",
-             r, m, bp.ell, bp.tb, bp.L, bp.d, bp.ncore, bp.ell + bp.tb, bp.ell + bp.tb + bp.L, lane_mask);
+             " WALK0 = %d, TOP = %d, LOW = %d, MID = %d, NSIG = %d;\n  static constexpr u32 LANE_MASK = 0x%08xu;\n",
+             r, m, bp.ell, bp.tb, bp.L, bp.d, bp.ncore, bp.ell + bp.tb, bp.ell + bp.tb + bp.L, bp.low, bp.mid,
+             std::max(0, bp.nsig), lane_mask);
     src += head + gen + "};\n";
   }
   // shared memory: per-thread N_k bins, the item's connectivity words (and,
   // in the gradient module, their lane transposes), per-warp N_k counts
-  std::string kern = E.grad ?
+  const char* head_g =
       "extern \"C\" __global__ void __launch_bounds__(BSB_NTHR, BSB_MINB)\n"
       "bs_batch_grad(const BGraph* __restrict__ graphs, int G, int K, int Kp, u64 total,\n"
       "         const u64* __restrict__ lt, const u64* __restrict__ nt, const u64* __restrict__ wm2,\n"
       "         const mx* __restrict__ pt, const u64* __restrict__ thw, const u64* __restrict__ tt,\n"
       "         const u64* __restrict__ lwex, const u64* __restrict__ thwex,\n"
       "         const mx* __restrict__ ptex, u64* limbs, u64* nk,\n"
-      "         u64* counter, u32* status, u64 budget_ns) {\n"
+      "         u64* counter, u32* status, u64 budget_ns, const BMerge A) {\n"
       "  extern __shared__ __align__(16) u64 s_bins[];\n"
       "  const int lane = threadIdx.x & 31;\n"
       "  const BsTr tr = bs_tr_init(lane);\n"
@@ -868,27 +930,45 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  u32* cw = (u32*)(s_bins + (BSB_LMAX + 1) * BSB_NTHR) + threadIdx.x;\n"
       "  u32* ctw = (u32*)(s_bins + (BSB_LMAX + 1) * BSB_NTHR) + ((size_t)1 << BSB_LMAX) * BSB_NTHR +\n"
       "             threadIdx.x;\n"
-      "  u64* nkw = s_bins + (BSB_LMAX + 1) * BSB_NTHR + ((size_t)1 << BSB_LMAX) * BSB_NTHR +\n"
-      "             (threadIdx.x >> 5) * 65;\n"
-      "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n"
-    :
+      "  u64* s_nk = s_bins + (BSB_LMAX + 1) * BSB_NTHR + ((size_t)1 << BSB_LMAX) * BSB_NTHR;\n";
+  const char* head_r =
       "extern \"C\" __global__ void __launch_bounds__(BSB_NTHR, BSB_MINB)\n"
       "bs_batch(const BGraph* __restrict__ graphs, int G, int K, int Kp, u64 total,\n"
       "         const u64* __restrict__ lt, const u64* __restrict__ nt, const u64* __restrict__ wm,\n"
       "         const mx* __restrict__ pt, const u64* __restrict__ thw, u64* limbs, u64* nk,\n"
-      "         u64* counter, u32* status, u64 budget_ns) {\n"
+      "         u64* counter, u32* status, u64 budget_ns, const BMerge A) {\n"
       "  extern __shared__ __align__(16) u64 s_bins[];\n"
       "  const int lane = threadIdx.x & 31;\n"
       "  u64* bins = s_bins + threadIdx.x;\n"
       "  u32* cw = (u32*)(s_bins + (BSB_LMAX + 1) * BSB_NTHR) + threadIdx.x;\n"
-      "  u64* nkw = s_bins + (BSB_LMAX + 1) * BSB_NTHR + (((size_t)1 << BSB_LMAX) * BSB_NTHR) / 2 +\n"
-      "             (threadIdx.x >> 5) * 65;\n"
-      "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n";
+      "  u64* s_nk = s_bins + (BSB_LMAX + 1) * BSB_NTHR + (((size_t)1 << BSB_LMAX) * BSB_NTHR + 1) / 2;\n";
+  std::string kern = E.grad ? head_g : head_r;
   kern +=
+      "  u64* nkw = s_nk + (threadIdx.x >> 5) * 65;\n"
+      "  u64* rel = s_nk + (BSB_NTHR / 32) * 65 + (threadIdx.x >> 5) * 33;   // merged: counts below the prefix\n"
+      "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n"
       "  int cur = -1;   // network whose counts nkw holds\n"
-      "  const u64 t0 = bs_timer();\n"
+      "  const u64 t0 = bs_timer();\n";
+  kern += E.merged ?
+      "  rel[lane] = 0ull;\n"
+      "  if (*(volatile u32*)status) return;\n"
+      "  const u64 n_cls = *A.n_classes, n_warps = (u64)gridDim.x * (BSB_NTHR / 32);\n"
+      "  u64 next = (u64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;\n"
+      "  __syncwarp();\n"
+      "  for (;;) {\n"
+      "    const u64 cls = next;\n"
+      "    if (cls >= n_cls) break;\n"
+      "    if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); break; }\n"
+      "    next = ~0ull;\n"
+      "    if (n_cls > n_warps) {\n"
+      "      if (lane == 0) next = n_warps + atomicAdd(A.ticket, 1ull);\n"
+      "      next = __shfl_sync(0xffffffffu, next, 0);\n"
+      "    }\n"
+      "    const int lo = (int)A.net[cls];\n"
+      "    const u64 prefix = A.rep[cls];\n" :
       "  for (;;) {\n"
       "    u64 task = 0;\n"
+      "    const u64 cls = 0;\n"
       "    if (lane == 0) {\n"
       "      task = atomicAdd(counter, 1ull);\n"
       "      if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); task = ~0ull; }\n"
@@ -897,14 +977,16 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "    if (task >= total) break;\n"
       "    int lo = 0, hi = G - 1;\n"
       "    while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (graphs[mid].task_begin <= task) lo = mid; else hi = mid - 1; }\n"
+      "    const u64 prefix = task - graphs[lo].task_begin;\n";
+  kern +=
       "    const BGraph* __restrict__ Bp = graphs + lo;\n"
       "    if (lo != cur) {\n"
       "      __syncwarp();\n"
       "      if (cur >= 0) bsb_flush_counts(graphs + cur, nkw, nk, lane);\n"
       "      cur = lo;\n"
-      "    }\n"
-      "    const u64 prefix = task - Bp->task_begin;\n"
-      "    const int prune = Bp->prune;\n"
+      "    }\n";
+  kern += E.merged ? "    const int prune = 0;\n" : "    const int prune = Bp->prune;\n";
+  kern +=
       "    int st = 0;\n"
       "    switch (lo) {\n";
   for (int r = 0; r < G; ++r)
@@ -913,12 +995,36 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   kern += "    }\n";
   kern += E.grad ?
           "    if (st) bsb_finish_grad(Bp, st, prefix, lane, K, Kp, lt, nt, wm2, pt, thw, tt, lwex, thwex,\n"
-          "                            ptex, limbs, nkw, bins, cw, ctw, tr);\n" :
-          "    if (st) bsb_finish(Bp, st, prefix, lane, K, Kp, lt, nt, wm, pt, thw, limbs, nkw, bins, cw);\n";
+          "                            ptex, limbs, nkw, bins, cw, ctw, tr, A, cls, rel);\n" :
+          "    if (st) bsb_finish(Bp, st, prefix, lane, K, Kp, lt, nt, wm, pt, thw, limbs, nkw, bins, cw, A, cls, rel);\n";
   kern +=
           "    __syncwarp();\n  }\n"
           "  __syncwarp();\n"
           "  if (cur >= 0) bsb_flush_counts(graphs + cur, nkw, nk, lane);\n}\n";
+  if (E.merged) {
+    kern += std::string("extern \"C\" __global__ void __launch_bounds__(BSB_MNTHR) ") +
+            (E.grad ? "bs_batch_grad_p1" : "bs_batch_p1") +
+            "(const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A,\n"
+            "    u64* limbs, u64* nk, u32* status, u64 budget_ns) {\n"
+            "  extern __shared__ u32 s_sig[];\n"
+            "  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;\n"
+            "  u32* zs = s_sig + warp * " + std::to_string(std::max(1, E.nsig_max) * 32) + ";\n"
+            "  const u64 t0 = bs_timer();\n"
+            "  for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks << A.split_log2;\n"
+            "       v += (u64)gridDim.x * (BSB_MNTHR / 32)) {\n"
+            "    const u64 t = v >> A.split_log2;\n"
+            "    if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); break; }\n"
+            "    const int net = bsb_block_net(graphs, G, t);\n"
+            "    const u64 hi = t - graphs[net].blk_begin;\n"
+            "    u32 full = 0u, left = 0u;\n"
+            "    switch (net) {\n";
+    for (int r = 0; r < G; ++r)
+      kern += "      case " + std::to_string(r) + ": bsb_classify<G" + std::to_string(r) +
+              ">(hi, lane, zs, full, left); break;\n";
+    kern += "    }\n"
+            "    bsb_merge_block(graphs + net, net, t, hi, (int)(v & ((1ull << A.split_log2) - 1ull)), lane, K, zs, full, left, pt, A, limbs, nk, status);\n"
+            "  }\n}\n";
+  }
   std::string bt = kBsBatchTemplate;
   const size_t cut = bt.find("//@@BATCH_KERNEL@@");
   src += bt.substr(0, cut) + kern;
@@ -936,6 +1042,8 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   unsigned long long begin = 0;
   size_t lt = 0, nt = 0, wm = 0, pt = 0, th = 0;
   size_t wm2 = 0, tt = 0, lwex = 0, thwex = 0, ptex = 0, outl = 0;   // gradient module
+  unsigned long long blocks = 0, slots = 0;   // merged modules
+  int d_max = 0;
   int nk_off = 0;
   std::vector<int> nk_offs(G);
   for (int i = 0; i < G; ++i) {
@@ -954,10 +1062,17 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
     b.gidx = i;
     b.m = graphs[i].n_arcs;
     b.prune = o.prune ? 1 : 0;
-    b.nlev = (bp.d + 6) / 7;   // levels of at most 7 bits: small per-p-vector tables
+    b.low = bp.low;
+    b.mid = bp.mid;
+    b.nhi = bp.d - bp.low - bp.mid;
+    b.nsig = std::max(0, bp.nsig);
+    // prefix masses (merged: of the arcs above a block) in levels of at most
+    // 7 bits: small per-p-vector tables
+    const int nl = E.merged ? b.nhi : bp.d;
+    b.nlev = (nl + 6) / 7;
     int off = 0;
     for (int l = 0; l < b.nlev; ++l) {
-      b.lev_bits[l] = bp.d / b.nlev + (l < bp.d % b.nlev ? 1 : 0);
+      b.lev_bits[l] = nl / b.nlev + (l < nl % b.nlev ? 1 : 0);
       b.lev_off[l] = off;
       off += 1 << b.lev_bits[l];
     }
@@ -978,6 +1093,16 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
     b.d = bp.d;
     b.thr_mask = bp.tb >= 5 ? 0xffffffffu : ((1u << (1 << bp.tb)) - 1u);
     b.pex_mask = bp.pex;
+    if (E.merged) {
+      while (b.slots_log2 < b.nsig && (1ull << b.slots_log2) < 2 * items[i]) ++b.slots_log2;
+      b.blk_begin = blocks;
+      b.slot_base = slots;
+      b.item_base = b.task_begin;
+      blocks += 1ull << b.nhi;
+      slots += 1ull << b.slots_log2;
+      d_max = std::max(d_max, bp.d);
+      if (!E.grad) b.out_off = i * K * kBsbLimbs;
+    }
     if (E.grad) {
       b.wm2_off = (int)wm2; wm2 += (size_t)2 * ((size_t)1 << bp.L) * Kp;
       b.tt_off = (int)tt; tt += (size_t)1024 * Kp;
@@ -1002,17 +1127,58 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   E.o_lwex = off; off = a256(off + 8 * lwex);
   E.o_thwex = off; off = a256(off + 8 * thwex);
   E.o_ptex = off; off = a256(off + sizeof(MxHost) * ptex);
+  const size_t gk = E.merged ? (size_t)G * K : 0;
+  E.o_nib = off; off = a256(off + 16 * 128 * gk);
+  E.o_mid = off; off = a256(off + 16 * 32 * gk);
+  E.o_fold = off; off = a256(off + (E.grad ? 8 * kBsbFold * gk : 0));
   E.o_upload_end = off;
   E.o_limbs = off; off = a256(off + 8 * E.n_out);
   E.o_nk = off; off = a256(off + 8 * (size_t)E.nk_total);
-  E.o_counter = off; off = a256(off + 8);
+  E.o_counter = off; off = a256(off + 3 * 8);   // and, merged, the number of classes and their ticket
   E.o_status = off; off = a256(off + 4);
   E.o_end = off;
   if ((rc = scratch_acquire(dev.device, E.o_end, E.o_end, &E.scr))) return rc;
   memcpy((char*)E.scr->hmem + E.o_graphs, E.bg.data(), sizeof(BGraphHost) * G);
   E.smem = (size_t)(E.lmax + 1) * kBsbThreads * 8 +
            ((size_t)1 << E.lmax) * kBsbThreads * 4 * (E.grad ? 2 : 1) +
-           (size_t)(kBsbThreads / 32) * 65 * 8;
+           (size_t)(kBsbThreads / 32) * (65 + 33) * 8 + 8;
+  if (E.merged) {
+    BMergeHost& M = E.M;
+    M.n_blocks = blocks;
+    M.cap = (unsigned)std::min<unsigned long long>(E.total, std::max(kBsbMaxClasses / 64, kBsbMaxClasses / K));
+    M.hist_stride = (d_max + 2) & ~1;
+    size_t mo = 0;
+    auto take = [&](size_t bytes) { const size_t at = mo; mo = a256(mo + bytes); return at; };
+    E.key_bytes = 8 * (size_t)slots;
+    const size_t key = take(E.key_bytes), id_of = take(4 * (size_t)slots), net = take(4ull * M.cap);
+    const size_t rep = take(8ull * M.cap), hist = take(4ull * M.cap * M.hist_stride);
+    const size_t cmass = take(16ull * M.cap * K), csum = take(E.grad ? 16ull * M.cap * K : 0);
+    const size_t cmask = take(8ull * 32 * blocks), ent = take(8ull * E.total);
+    if ((rc = scratch_acquire(dev.device, mo, 0, &E.mscr))) return rc;
+    char* d = (char*)E.mscr->dmem;
+    char* u = (char*)E.scr->dmem;
+    M.key = d + key; M.id_of = d + id_of; M.net = d + net; M.rep = d + rep; M.hist = d + hist;
+    M.cmass = d + cmass; M.csum = d + csum; M.cmask = d + cmask; M.ent = d + ent;
+    M.n_classes = u + E.o_counter + 8; M.ticket = u + E.o_counter + 16;
+    M.nib = u + E.o_nib; M.mid = u + E.o_mid; M.fold = u + E.o_fold;
+    E.smem1 = (size_t)(kMergeThreads / 32) * std::max(1, E.nsig_max) * 32 * 4;
+    auto fit = [&](cudaKernel_t k, size_t smem, unsigned long long warps) {
+      int n = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void*)k, kMergeThreads, smem) != cudaSuccess || n < 1) {
+        cudaGetLastError();
+        n = 1;
+      }
+      return (int)std::max(1ull, std::min((unsigned long long)n * dev.sms, (warps + kMergeThreads / 32 - 1) / (kMergeThreads / 32)));
+    };
+    // a block is a few hundred microseconds of one warp's latency: enough warps
+    // to fill the SMs with 32 each
+    M.parts = 1;
+    while (M.split_log2 < 5 && (blocks << M.split_log2) < 32ull * dev.sms) ++M.split_log2;
+    while (M.parts < std::min(K, 32) && blocks * M.parts < 64ull * dev.sms) M.parts *= 2;
+    E.grid1 = fit(E.jit.kernel_p1, E.smem1, blocks << M.split_log2);
+    E.grid2 = fit(E.jit.kernel_p2, 0, blocks * M.parts);
+    if (E.grad) E.grid3 = fit(E.jit.kernel_p3, 0, blocks * K);
+  }
   cudaError_t e = cudaFuncSetAttribute((const void*)E.jit.kernel,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)E.smem);
   if (e != cudaSuccess) return fail(PBAT_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
@@ -1081,13 +1247,14 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
       product_table(pv, bp.perm.data() + bp.ell, bp.tb, tw);
       for (int t = 0; t < 32; ++t)
         th[b.thw_off + (size_t)t * Kp + k] = t < (1 << bp.tb) ? fixed_u64(tw[t], 63) : 0ull;
+      const int blk = E.merged ? bp.low + bp.mid : 0;
       MxHost* ptk = pt + b.pt_off + (size_t)k * b.pt_size;
       if (b.nlev == 0) ptk[0] = to_mx(dd_make(1.0));
       for (int l = 0, sh = 0; l < b.nlev; ++l) {
         dd tab[1 << 7];
-        product_table(pv, bp.perm.data() + top + sh, b.lev_bits[l], tab);
+        product_table(pv, bp.perm.data() + top + blk + sh, b.lev_bits[l], tab);
         for (int v = 0; v < (1 << b.lev_bits[l]); ++v) ptk[b.lev_off[l] + v] = to_mx(tab[v]);
-        if (E.grad)
+        if (E.grad && !E.merged)
           for (int jj = 0; jj < b.lev_bits[l]; ++jj) {
             if (!((bp.pex >> (top + sh + jj)) & 1ull)) continue;   // divided by p on the host
             // the level's product without prefix arc sh + jj, indexed by the
@@ -1102,6 +1269,13 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
               row[v] = to_mx(ex[(v & ((1 << jj) - 1)) | ((v >> (jj + 1)) << jj)]);
           }
         sh += b.lev_bits[l];
+      }
+      if (E.merged) {
+        const size_t gk = (size_t)r * K + k;
+        block_tables(pv, bp.perm.data() + top, bp.low, bp.mid, (unsigned long long*)(h + E.o_nib) + 256 * gk,
+                     (unsigned long long*)(h + E.o_mid) + 64 * gk);
+        if (E.grad)
+          fold_tables(pv, bp.perm.data() + top, bp.low, bp.mid, *(BsFoldParamsHost*)((unsigned long long*)(h + E.o_fold) + kBsbFold * gk));
       }
       if (E.grad) {
         // 128-bit walk masses, thread-pattern byte tables, and the lane and
@@ -1156,12 +1330,24 @@ static int bsb_enqueue(BsBatch& E, cudaStream_t st, unsigned long long budget_ns
   const void *wm2 = d + E.o_wm2, *tt = d + E.o_tt, *lwex = d + E.o_lwex, *thwex = d + E.o_thwex;
   const void* ptex = d + E.o_ptex;
   void* args[] = {(void*)&graphs, &G, &K, &Kp, &total, (void*)&lt, (void*)&nt, (void*)&wm,
-                  (void*)&pt, (void*)&thw, &limbs, &nk, &counter, &status, &bud};
+                  (void*)&pt, (void*)&thw, &limbs, &nk, &counter, &status, &bud, (void*)&E.M};
   void* gargs[] = {(void*)&graphs, &G, &K, &Kp, &total, (void*)&lt, (void*)&nt, (void*)&wm2,
                    (void*)&pt, (void*)&thw, (void*)&tt, (void*)&lwex, (void*)&thwex, (void*)&ptex,
-                   &limbs, &nk, &counter, &status, &bud};
+                   &limbs, &nk, &counter, &status, &bud, (void*)&E.M};
+  if (E.merged) {
+    void* a1[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &limbs, &nk, &status, &bud};
+    void* a2[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &status};
+    if ((e = cudaMemsetAsync(E.M.key, 0, E.key_bytes, st)) != cudaSuccess ||
+        (e = cudaLaunchKernel((const void*)E.jit.kernel_p1, dim3(E.grid1), dim3(kMergeThreads), a1, E.smem1, st)) != cudaSuccess ||
+        (e = cudaLaunchKernel((const void*)E.jit.kernel_p2, dim3(E.grid2), dim3(kMergeThreads), a2, 0, st)) != cudaSuccess)
+      return fail(PBAT_ECUDA, "batched launch: %s", cudaGetErrorString(e));
+  }
   e = cudaLaunchKernel((const void*)E.jit.kernel, dim3(E.grid), dim3(kBsbThreads),
                        E.grad ? gargs : args, E.smem, st);
+  if (e == cudaSuccess && E.merged && E.grad) {
+    void* a3[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &limbs, &status};
+    e = cudaLaunchKernel((const void*)E.jit.kernel_p3, dim3(E.grid3), dim3(kMergeThreads), a3, 0, st);
+  }
   if (e != cudaSuccess) return fail(PBAT_ECUDA, "batched launch: %s", cudaGetErrorString(e));
   return PBAT_OK;
 }
@@ -1194,7 +1380,7 @@ int bsb_source_for(int G, const pbat_graph* graphs, int K, const pbat_options& o
 // and 5.91 ms).  Returns false when no candidate ran (the planner's
 // defaults are kept).
 static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, const pbat_options& o,
-                     cudaStream_t st, const DeviceInfo& dev, const std::vector<std::string>* elig,
+                     cudaStream_t st, const DeviceInfo& dev, const std::vector<std::string>* elig, bool per_item,
                      int* best_L, int* best_prune, int* best_occ) {
   double best_ms = 1e300;
   bool found = false;
@@ -1205,6 +1391,7 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
     return false;
   }
   auto new_batch = [&](BsBatch& T) {
+    T.per_item = per_item;
     if (elig) {
       T.grad = true;
       T.elig = *elig;
@@ -1227,15 +1414,21 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
     BsBatch T;
     new_batch(T);
     if (bsb_build(T, G, graphs, K, t, dev) != PBAT_OK) {
-      if (T.scr) scratch_release(T.scr);
+      scratch_release(T.scr);
+      scratch_release(T.mscr);
       clear_error();
       return;
     }
     bsb_tables(T, graphs, p);
     bool ok = cudaMemcpyAsync(T.scr->dmem, T.scr->hmem, T.o_upload_end, cudaMemcpyHostToDevice, st) ==
               cudaSuccess;
-    ok = ok && cudaEventRecord(a, st) == cudaSuccess && bsb_enqueue(T, st, 0) == PBAT_OK &&
-         cudaEventRecord(b, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    // (merged runs are short: the second of two counts)
+    for (int rep = 0; ok && rep < (T.merged ? 2 : 1); ++rep)
+      ok = cudaEventRecord(a, st) == cudaSuccess && bsb_enqueue(T, st, 0) == PBAT_OK &&
+           cudaEventRecord(b, st) == cudaSuccess && cudaStreamSynchronize(st) == cudaSuccess;
+    unsigned status = 0;
+    ok = ok && cudaMemcpy(&status, (char*)T.scr->dmem + T.o_status, sizeof status, cudaMemcpyDeviceToHost) == cudaSuccess &&
+         !(status & 2u);
     float ms = 0.f;
     if (ok && cudaEventElapsedTime(&ms, a, b) == cudaSuccess && ms < best_ms) {
       best_ms = ms;
@@ -1249,6 +1442,7 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
       clear_error();
     }
     scratch_release(T.scr);
+    scratch_release(T.mscr);
   };
   std::vector<pbat_options> cands;
   for (int mode : (o.prune == 1 ? std::vector<int>{1, 2} : std::vector<int>{o.prune}))
@@ -1281,31 +1475,40 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
   NvtxRange nv("pbat batched");
   if (G > kBsbMaxGraphs) return PBAT_ENOTSUP;
   BsBatch* E = nullptr;
+  bool per_item = false;
   {
     std::lock_guard<std::mutex> lk(g_bsb_mu);
+    per_item = g_bsb_unmergeable.count(key) != 0;
     for (auto* e : g_bsb)
-      if (!e->busy && e->key == key) { e->busy = true; E = e; break; }
+      if (!e->busy && e->key == key && e->per_item == per_item) { e->busy = true; E = e; break; }
   }
   if (!E) {
     pbat_options ob = o;
     if (o.autotune && o.walk_bits < 0) {
       int L = -1, mode = o.prune, occ = o.occupancy;
-      if (bsb_tune(G, graphs, K, p, o, st, dev, elig, &L, &mode, &occ)) {
+      if (bsb_tune(G, graphs, K, p, o, st, dev, elig, per_item, &L, &mode, &occ)) {
         ob.walk_bits = L;
         ob.prune = mode;
         ob.occupancy = occ;
       }
+    } else if (o.walk_bits < 0 && o.prune && !per_item) {
+      // untuned and merged: shorter walks than one by one (GB300, 20 networks
+      // x 7 p-vectors, L = 5 / 4 / 3: gradient 551 / 358 / 414 us, R 157 / 135 /
+      // 151; 64 x 16, R 3.0 / 2.7 / 3.4 ms)
+      ob.walk_bits = 4;
     }
     std::unique_ptr<BsBatch> ne(new BsBatch());
     ne->key = key;
     ne->busy = true;
+    ne->per_item = per_item;
     if (elig) {
       ne->grad = true;
       ne->elig = *elig;
     }
     int rc = bsb_build(*ne, G, graphs, K, ob, dev);
     if (rc) {
-      if (ne->scr) scratch_release(ne->scr);
+      scratch_release(ne->scr);
+      scratch_release(ne->mscr);
       return rc;
     }
     E = ne.release();
@@ -1368,6 +1571,15 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
   }
+  if (*(unsigned int*)(h + E->o_status) & 2u) {
+    // more classes than fit: every item by itself, now and from now on
+    {
+      std::lock_guard<std::mutex> lk(g_bsb_mu);
+      g_bsb_unmergeable.insert(key);
+      E->busy = false;
+    }
+    return run_batched_bs(G, graphs, K, p, o, st, R_out, Nk_out, key, dev, kernel_ns, elig, dRdp_out, coarse);
+  }
   if (*(unsigned int*)(h + E->o_status) & 1u) return done(fail(PBAT_ETIMEOUT, "time budget ran out on the device"));
   const unsigned long long* limbs = (const unsigned long long*)(h + E->o_limbs);
   const unsigned long long* nk = (const unsigned long long*)(h + E->o_nk);
@@ -1412,7 +1624,9 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
           const dd B = limbs256_to_dd(base + (size_t)(2 + 2 * q) * kBsbLimbs);
           const int a = bp.perm[q];
           dd v;
-          if (q >= top && ((bp.pex >> q) & 1ull))
+          if (E->merged && q >= top && q < top + b.low + b.mid)
+            v = A;   // pair differences (bs_batch_grad_p3)
+          else if (q >= top && ((bp.pex >> q) & 1ull))
             v = dd_sub(A, B);
           else if (q >= walk0)
             v = dd_sub(dd_mul(A, dd_recip(pk[a])), dd_mul(B, dd_recip_dd(dd_one_minus(pk[a]))));

@@ -38,7 +38,8 @@ namespace pbat {
 // ---------------------------------------------------------------------------
 class Elim {
  public:
-  Elim(int n, bool directed, int s, int t) : n_(n), dir_(directed), s_(s), t_(t), E_(n * n) {}
+  Elim(int n, bool directed, int s, int t, const char* name = "v")
+      : n_(n), dir_(directed), s_(s), t_(t), name_(name), E_(n * n) {}
 
   bool has(int i, int j) const { return !at(i, j).empty(); }
   const std::string& at(int i, int j) const {
@@ -50,7 +51,7 @@ class Elim {
     if (i == j) return;
     if (dir_ && (j == s_ || i == t_)) return;  // no s-t path enters s or leaves t
     std::string& e = ref(i, j);
-    const std::string v = "v" + std::to_string(nvar_++);
+    const std::string v = name_ + std::to_string(nvar_++);
     if (e.empty())
       code_ += "  const u32 " + v + " = " + expr + ";\n";
     else
@@ -127,6 +128,7 @@ class Elim {
   int n_;
   bool dir_;
   int s_, t_;
+  std::string name_;   // of the generated variables
   std::vector<std::string> E_;
   std::string code_;
   int nvar_ = 0, ops_ = 0;
@@ -378,6 +380,7 @@ static void bs_generate(const GraphIn& g, BsPlan& bp) {
 //   in its component, as a binary number over the nodes it can be joined to;
 //   directed: which boundary nodes the source reaches, which reach the sink,
 //   and for the other pairs whether the first reaches the second.
+// It also gives the prune's answer for the 32 items (dn, up).
 static void bs_generate_sig(const GraphIn& g, BsPlan& bp) {
   const int m = g.m, top = bp.ell + bp.tb + bp.L;
   std::vector<bool> isb(g.n, false);
@@ -447,7 +450,40 @@ static void bs_generate_sig(const GraphIn& g, BsPlan& bp) {
   bp.nsig = -1;
   if (nsig > kMaxSigBits) return;
   bp.nsig = nsig;
-  bp.gen_sig = "__device__ __forceinline__ void bs_sig(const u32* a, u32* z) {\n" + C.code() + out + "}\n";
+  // The two ends of the prune come from the same closure: an item is connected
+  // throughout when its prefix alone joins source and sink (dn), and not cut
+  // when the prefix does so together with every other arc (up): the boundary
+  // graph with its undirected components of other arcs contracted, or for
+  // directed networks with these arcs added, eliminated down to the pair.
+  std::vector<int> comp(g.n);
+  for (int v = 0; v < g.n; ++v) comp[v] = v;
+  if (!g.directed)
+    for (bool grew = true; grew;) {
+      grew = false;
+      for (int k = 0; k < top; ++k) {
+        const int u = g.tail[bp.perm[k]], v = g.head[bp.perm[k]], c = std::min(comp[u], comp[v]);
+        if (comp[u] != c || comp[v] != c) comp[u] = comp[v] = c, grew = true;
+      }
+    }
+  const int s = comp[g.source], t = comp[g.sink];
+  const std::string dn = C.has(g.source, g.sink) ? C.at(g.source, g.sink) : "0u";
+  std::string up = "0xffffffffu", ucode;
+  if (s != t) {
+    Elim U(g.n, g.directed != 0, s, t, "x");
+    for (int i : bnd)
+      for (int j : bnd)
+        if (i != j && (g.directed || i < j) && C.has(i, j)) U.or_in(comp[i], comp[j], C.at(i, j));
+    if (g.directed)
+      for (int k = 0; k < top; ++k) U.or_in(g.tail[bp.perm[k]], g.head[bp.perm[k]], "0xffffffffu");
+    std::vector<int> inner;
+    for (int v : bnd)
+      if (comp[v] == v && v != s && v != t) inner.push_back(v);
+    U.eliminate_all(inner);
+    ucode = U.code();
+    up = U.has(s, t) ? U.at(s, t) : "0u";
+  }
+  bp.gen_sig = "__device__ __forceinline__ void bs_sig(const u32* a, u32* z, u32& dn, u32& up) {\n" + C.code() + out +
+               ucode + "  dn = " + dn + ";\n  up = " + up + ";\n}\n";
 }
 
 // The fused kernel divides walk masses by p and 1 - p (p-dependent roles).
@@ -630,7 +666,10 @@ static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPl
   // range; not with arcs outside the fused kernel's range above those
   bp.low = std::min(5, bp.d - r);
   bp.mid = std::min(5, bp.d - r - bp.low);
-  if (o.prune && bp.d - r > 0 && !(bp.pex >> (top + bp.low + bp.mid))) bs_generate_sig(g, bp);
+  if (o.prune && !(bp.pex >> (top + bp.low + bp.mid))) bs_generate_sig(g, bp);
+  const unsigned long long items = r > 0 ? (o.range_hi - o.range_lo) << (bp.d - r) : 1ull << bp.d;
+  bp.merge = bp.nsig >= 0 && o.launches != 1 && bp.d - r <= 24 && items > 0 && items <= kMaxMergeItems &&
+             items >> (bp.low + bp.mid) <= kMaxMergeBlocks && (o.launches == 2 || items >= kMergeItems);
   return PBAT_OK;
 }
 

@@ -24,6 +24,7 @@ struct BsPlan {
   // bits of a word, `mid` the warp lanes
   std::string gen_sig;
   int nsig = -1, low = 0, mid = 0;
+  bool merge = false;     // a merged run: its launches' kernels, not the one-launch kernel
   int ncore = 0, ops_inv = 0, ops_var = 0;
 };
 
@@ -34,6 +35,13 @@ bool bs_walk_ok(const double* p, int a);
 // Items are merged when their signatures fit this many bits (a 64-bit table
 // key with one bit to mark a used slot).
 constexpr int kMaxSigBits = 63;
+// Items from which a run merges them by default (pbat_options.launches 0):
+// below, one launch is a few microseconds long and further ones cost more
+// than they save (GB300, R / fused: 2^11 items of 23 arcs 29 / 36 us in one
+// launch, 29 / 54 merged; 2^14 items of 27 arcs 58 / 90 against 42 / 54).
+constexpr unsigned long long kMergeItems = 1ull << 12;
+constexpr unsigned long long kMaxMergeItems = 1ull << 24;   // a slot number for each in the fused kernel
+constexpr unsigned long long kMaxMergeBlocks = 1ull << 14;
 
 // Plan one network for the bit-sliced kernels (Sec. 4.3 equal division:
 // lane, thread, walk and prefix arcs, range arcs on top) and generate its

@@ -274,6 +274,182 @@ __device__ __forceinline__ u32 bs_transpose32(u32 x, const BsTr& t) {
   return x;
 }
 
+__device__ __forceinline__ u32 bs_pattern(int i) {
+  return i == 0 ? 0xAAAAAAAAu : i == 1 ? 0xCCCCCCCCu : i == 2 ? 0xF0F0F0F0u : i == 3 ? 0xFF00FF00u : 0xFFFF0000u;
+}
+// (a * b) >> 128 (the product of the low halves dropped: at most two units low)
+__device__ __forceinline__ u128 mulhi128(u128 a, u128 b) {
+  u128 r = u128{a.hi * b.hi, __umul64hi(a.hi, b.hi)};
+  u128_add(r, __umul64hi(a.hi, b.lo), 0ull);
+  u128_add(r, __umul64hi(a.lo, b.hi), 0ull);
+  return r;
+}
+// The mass of the 32 patterns set in v, from eight nibble tables t of 16
+// subset sums (scale 2^127), times the mass f (scale 2^127): scale 2^126.
+__device__ __forceinline__ u128 bs_subset_mass(u32 v, const ulonglong2* t, u128 f) {
+  u128 s = u128{0ull, 0ull};
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const ulonglong2 x = t[16 * i + ((v >> (4 * i)) & 15u)];
+    u128_add(s, x.x, x.y);
+  }
+  return mulhi128(s, f);
+}
+// Every 2^split_log2-th bit, from bit `part` on: one warp's share of a
+// block's words when 2^split_log2 warps work on it.
+__device__ __forceinline__ u32 bs_part_mask(int split_log2, u32 part) {
+  return (split_log2 == 0 ? 0xffffffffu : split_log2 == 1 ? 0x55555555u : split_log2 == 2 ? 0x11111111u
+          : split_log2 == 3 ? 0x01010101u : split_log2 == 4 ? 0x00010001u : 1u) << part;
+}
+// The set bits of v by the popcount of their position, a byte each.
+__device__ __forceinline__ u64 bs_popcount_bytes(u32 v) {
+  return (u64)(__popc(v & 0x00000001u) | (__popc(v & 0x00010116u) << 8) | (__popc(v & 0x01161668u) << 16) |
+               (__popc(v & 0x16686880u) << 24)) |
+         ((u64)(__popc(v & 0x68808000u) | (__popc(v & 0x80000000u) << 8)) << 32);
+}
+// Counts of a block's items in `full` by popcount inside the block, lane k
+// ending with popcount k's.  Every lane packs its own into bytes (at most
+// C(10, 5) = 252 each over the warp) and three warp reductions add them.
+__device__ __forceinline__ u32 bs_block_counts(u32 full, int lane) {
+  const u64 v = bs_popcount_bytes(full);
+  const int sh = 8 * __popc(lane);
+  const u64 lo = v << sh, hi = sh ? v >> (64 - sh) : 0ull;
+  const u32 r0 = __reduce_add_sync(0xffffffffu, (u32)lo), r1 = __reduce_add_sync(0xffffffffu, (u32)(lo >> 32));
+  const u32 r2 = __reduce_add_sync(0xffffffffu, (u32)hi);
+  const u32 r = lane < 4 ? r0 : lane < 8 ? r1 : r2;
+  return (r >> (8 * (lane & 3))) & 255u;
+}
+// The class of signature `key` (never 0): its slot, by linear probing from
+// its hash; claimed by compare-and-swap when new (`fresh`).  A table of
+// 2^nsig slots or more is indexed by the signature itself.  ~0: no free slot
+// within reach.
+__device__ __forceinline__ u32 bs_class(u64* table, int slots_log2, int nsig, u64 key, bool& fresh) {
+  const u32 mask = (1u << slots_log2) - 1u;
+  u32 slot = (u32)key & mask;
+  if (nsig > slots_log2) {
+    u64 h = key * 0x9E3779B97F4A7C15ull;   // the finaliser of splitmix64
+    h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
+    slot = (u32)((h ^ (h >> 27)) >> 20) & mask;
+  }
+  fresh = false;
+  for (int probe = 0; probe < 256; ++probe) {
+    u64 k = *(volatile u64*)&table[slot];
+    if (!k) {
+      k = atomicCAS(&table[slot], 0ull, key);
+      if (!k) { fresh = true; return slot; }
+    }
+    if (k == key) return slot;
+    slot = (slot + 1u) & mask;
+  }
+  return ~0u;
+}
+
+// A mass m (integer floating point hi times the 128-bit v, scale 2^124) at
+// scale 2^(98 + mass_exp), where all the items' masses add up to at most
+// 2^98, added to a class's two chunks -- the lower of BS_CLASS_SHIFT bits --
+// each by itself; and the mass back from its chunks.
+#define BS_CLASS_SHIFT 38
+__device__ __forceinline__ void bs_add_mass(u64* chunks, mx hi, u128 v, int mass_exp) {
+  const u128 F = u128_shr(mx_prod(hi, v), 25 + hi.e - mass_exp);
+  const u64 lo = F.lo & ((1ull << BS_CLASS_SHIFT) - 1ull);
+  const u64 up = (F.lo >> BS_CLASS_SHIFT) | (F.hi << (64 - BS_CLASS_SHIFT));
+  if (lo) atomicAdd(&chunks[0], lo);
+  if (up) atomicAdd(&chunks[1], up);
+}
+__device__ __forceinline__ mx bs_class_mass(const u64* chunks, int mass_exp) {
+  u128 t = u128{chunks[0], 0ull};
+  const u64 up = chunks[1];
+  u128_add(t, up << BS_CLASS_SHIFT, up >> (64 - BS_CLASS_SHIFT));
+  if (!(t.lo | t.hi)) return mx{0ull, 0, 0};
+  const int lz = t.hi ? __clzll((long long)t.hi) : 64 + __clzll((long long)t.lo);
+  const u64 m = lz >= 64 ? t.lo << (lz - 64) : (lz ? (t.hi << lz) | (t.lo >> (64 - lz)) : t.hi);
+  return mx{m, lz - 29 + mass_exp, 0};   // 128 - lz bits at scale 2^(98 + mass_exp)
+}
+// Adds the popcounts of the items in `same` of a lane to a class's counters
+// (h, by popcount), two 32-bit counters to an addition; pc: the popcount of
+// their common arcs.
+__device__ __forceinline__ void bs_add_counts(u32* h, u32 same, int pc) {
+  u64* p = (u64*)h + (pc >> 1);
+  const u64 n = bs_popcount_bytes(same) << (8 * (pc & 1));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const u64 two = ((n >> (16 * i)) & 255ull) | ((n >> (16 * i + 8)) & 255ull) << 32;
+    if (two) atomicAdd(&p[i], two);
+  }
+}
+// |a - b|; neg: a < b (classes' sums round apart by up to 2^-61, so a pair
+// whose true difference is zero may come out below it)
+__device__ __forceinline__ u128 bs_absdiff(u128 a, u128 b, bool& neg) {
+  neg = a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
+  return neg ? u128_sub(b, a) : u128_sub(a, b);
+}
+// one fold: adds w (V1 - V0) to G, returns V0 + p (V1 - V0)
+__device__ __forceinline__ u128 bs_fold2(u128 V0, u128 V1, u64 p, u64 w, u128& G) {
+  bool neg;
+  const u128 d = bs_absdiff(V1, V0, neg);
+  if (!neg) {
+    const u128 g = mul64x128_shr64(w, d.lo, d.hi);   // scale 2^123
+    u128_add(G, g.lo, g.hi);
+  }
+  u128 x = mul64x128_shr64(p, d.lo, d.hi);
+  x = u128{x.lo << 1, (x.hi << 1) | (x.lo >> 63)};
+  if (neg) return u128_sub(V0, x);
+  u128_add(V0, x.lo, x.hi);
+  return V0;
+}
+// A fold block's 32 items per lane: V over them by the five low arcs (see
+// bs_kernel_grad_p3).  V(j): item j's conditional reliability (scale 2^124);
+// p, w: the low arcs' p and the masses above each, as in BsFoldParams.
+template <class Item>
+__device__ __forceinline__ u128 bs_fold_low(const u64* p, const u64* w, u128 (&G)[5], Item item) {
+  u128 top[4];   // folded over the lowest three arcs
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    u128 V[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) V[i] = item(8 * q + i);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[0], w[4 * q + i], G[0]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[1], w[16 + 2 * q + i], G[1]);
+    top[q] = bs_fold2(V[0], V[1], p[2], w[24 + q], G[2]);
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) top[i] = bs_fold2(top[2 * i], top[2 * i + 1], p[3], w[28 + i], G[3]);
+  return bs_fold2(top[0], top[1], p[4], w[30], G[4]);
+}
+// The mid arcs over the lanes, and the block's sums per arc (scale 2^124):
+// lane l ends with low arc l's, lane `low` + l with mid arc l's, in X; every
+// lane with the block's V.
+__device__ __forceinline__ u128 bs_fold_mid(u128 V, const u128 (&G)[5], int low, int mid, const u64* p, const u64* w,
+                                            u64 m_mid, int lane, u128& X) {
+  X = u128{0ull, 0ull};
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    if (i >= low) break;
+    u128 g = mul64x128_shr64(m_mid, G[i].lo, G[i].hi);   // 2^122
+    g = warp_sum_u128(g);
+    g = u128{g.lo << 2, (g.hi << 2) | (g.lo >> 62)};
+    if (lane == i) X = g;
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    if (i >= mid) break;
+    const u128 o = shfl_xor_u128(V, 1 << i);
+    const bool one = (lane >> i) & 1;
+    u128 g = u128{0ull, 0ull};
+    const int at = (i == 0 ? 0 : i == 1 ? 16 : i == 2 ? 24 : i == 3 ? 28 : 30) + (lane >> (i + 1));
+    V = bs_fold2(one ? o : V, one ? V : o, p[i], w[at], g);
+    if (lane & ((1 << (i + 1)) - 1)) g = u128{0ull, 0ull};   // each pair once
+    g = warp_sum_u128(g);
+    g = u128{g.lo << 1, (g.hi << 1) | (g.lo >> 63)};
+    if (lane == low + i) X = g;
+  }
+  V.lo = __shfl_sync(0xffffffffu, V.lo, 0);
+  V.hi = __shfl_sync(0xffffffffu, V.hi, 0);
+  return V;
+}
+
 //@@GENERATED@@
 // connectivity of one uniform state (every word 0 or ~0): the prune test
 __device__ __forceinline__ u32 bs_uniform(const u32* a) {
@@ -357,73 +533,7 @@ __device__ __forceinline__ void bs_write_out(const BsWork& W, const facc* s_acc,
 #define BS_BLK (BS_LOW + BS_MID)   // prefix arcs inside a merge block
 #define BS_HI (BS_D - BS_BLK)      // prefix arcs above it
 #define BS_MERGE_NTHR 128
-#define BS_CLASS_SHIFT 38          // low chunk of a class mass
 #define BS_HIST ((BS_D + 2) & ~1)  // counters by popcount of a class, an even number
-__device__ __forceinline__ u32 bs_pattern(int i) {
-  return i == 0 ? 0xAAAAAAAAu : i == 1 ? 0xCCCCCCCCu : i == 2 ? 0xF0F0F0F0u : i == 3 ? 0xFF00FF00u : 0xFFFF0000u;
-}
-// (a * b) >> 128 (the product of the low halves dropped: at most two units low)
-__device__ __forceinline__ u128 mulhi128(u128 a, u128 b) {
-  u128 r = u128{a.hi * b.hi, __umul64hi(a.hi, b.hi)};
-  u128_add(r, __umul64hi(a.hi, b.lo), 0ull);
-  u128_add(r, __umul64hi(a.lo, b.hi), 0ull);
-  return r;
-}
-// The mass of the 32 patterns set in v, from eight nibble tables t of 16
-// subset sums (scale 2^127), times the mass f (scale 2^127): scale 2^126.
-__device__ __forceinline__ u128 bs_subset_mass(u32 v, const ulonglong2* t, u128 f) {
-  u128 s = u128{0ull, 0ull};
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    const ulonglong2 x = t[16 * i + ((v >> (4 * i)) & 15u)];
-    u128_add(s, x.x, x.y);
-  }
-  return mulhi128(s, f);
-}
-// The set bits of v by the popcount of their position, a byte each.
-__device__ __forceinline__ u64 bs_popcount_bytes(u32 v) {
-  return (u64)(__popc(v & 0x00000001u) | (__popc(v & 0x00010116u) << 8) | (__popc(v & 0x01161668u) << 16) |
-               (__popc(v & 0x16686880u) << 24)) |
-         ((u64)(__popc(v & 0x68808000u) | (__popc(v & 0x80000000u) << 8)) << 32);
-}
-// Adds the block's items in `full` to s_ci by popcount.  Every lane packs its
-// counts by popcount into bytes (at most C(10, 5) = 252 each over the warp)
-// and three warp reductions add them; lane k then holds popcount k's.
-__device__ __forceinline__ void bs_count_full(u32 full, int lane, int pc_hi, u64* s_ci) {
-  const u64 v = bs_popcount_bytes(full);
-  const int sh = 8 * __popc(lane);
-  const u64 lo = v << sh, hi = sh ? v >> (64 - sh) : 0ull;
-  const u32 r0 = __reduce_add_sync(0xffffffffu, (u32)lo), r1 = __reduce_add_sync(0xffffffffu, (u32)(lo >> 32));
-  const u32 r2 = __reduce_add_sync(0xffffffffu, (u32)hi);
-  const u32 r = lane < 4 ? r0 : lane < 8 ? r1 : r2;
-  const u32 n = (r >> (8 * (lane & 3))) & 255u;
-  if (lane <= BS_BLK && n) atomicAdd(&s_ci[pc_hi + lane], (u64)n);
-}
-// The class of signature `key` (never 0): its slot, by linear probing from
-// its hash; claimed by compare-and-swap when new (`fresh`).  A table of
-// 2^BS_NSIG slots or more is indexed by the signature itself.  ~0: no free
-// slot within reach.
-__device__ __forceinline__ u32 bs_class(const BsParams& P, const BsWork& W, u64 key, bool& fresh) {
-  const u32 mask = (1u << P.slots_log2) - 1u;
-  u32 slot = (u32)key & mask;
-  if (BS_NSIG > P.slots_log2) {
-    u64 h = key * 0x9E3779B97F4A7C15ull;   // the finaliser of splitmix64
-    h = (h ^ (h >> 30)) * 0xBF58476D1CE4E5B9ull;
-    slot = (u32)((h ^ (h >> 27)) >> 20) & mask;
-  }
-  fresh = false;
-  for (int probe = 0; probe < 256; ++probe) {
-    u64 k = *(volatile u64*)&W.key[slot];
-    if (!k) {
-      k = atomicCAS(&W.key[slot], 0ull, key);
-      if (!k) { fresh = true; return slot; }
-    }
-    if (k == key) return slot;
-    slot = (slot + 1u) & mask;
-  }
-  return ~0u;
-}
-
 __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __restrict__ ptab,
                                               const ulonglong2* __restrict__ mtab, int split_log2, const BsWork& W) {
   __shared__ ulonglong2 s_nib[128];   // subset sums of the low prefix pattern masses
@@ -447,34 +557,28 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
     const u32 part = (u32)t & ((1u << split_log2) - 1u);
     if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
     const u64 hi = blk0 + b;
-    u32 a[BS_M], u[BS_M];
-#pragma unroll
-    for (int k = 0; k < BS_TOP; ++k) a[k] = 0u;
+    u32 a[BS_M], z[BS_NSIG > 0 ? BS_NSIG : 1], dn, up;
 #pragma unroll
     for (int j = 0; j < BS_D; ++j)
       a[BS_TOP + j] = j < BS_LOW ? bs_pattern(j) : j < BS_BLK ? 0u - (u32)((lane >> (j - BS_LOW)) & 1)
                                                               : 0u - (u32)((hi >> (j - BS_BLK)) & 1ull);
-#pragma unroll
-    for (int k = 0; k < BS_M; ++k) u[k] = k < BS_TOP ? ~0u : a[k];
-    const u32 up = bs_uniform(u) & valid;
-    const u32 full = bs_uniform(a) & valid;
-    u32 left = up & ~full;
+    bs_sig(a, z, dn, up);
+    const u32 full = dn & valid;
+    u32 left = up & valid & ~full;
     const int pc_hi = __popcll((long long)hi);
     if (part == 0) {
       if (BS_GRAD) W.cmask[b * 32 + lane] = make_uint2(full, left);
       if (__any_sync(0xffffffffu, full)) {
-        bs_count_full(full, lane, pc_hi, s_ci);
+        const u32 n = bs_block_counts(full, lane);
+        if (lane <= BS_BLK && n) atomicAdd(&s_ci[pc_hi + lane], (u64)n);
         const u128 S = warp_sum_u128(u128_shr(bs_subset_mass(full, s_nib, m_mid), 2));
         const mx w = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
         facc_add(accR, mx_prod(w, S), w.e);
       }
     }
     if (!__any_sync(0xffffffffu, left)) continue;
-    u32 z[BS_NSIG > 0 ? BS_NSIG : 1];
-    bs_sig(a, z);
     // every 2^split_log2-th bit
-    left &= (split_log2 == 0 ? 0xffffffffu : split_log2 == 1 ? 0x55555555u : split_log2 == 2 ? 0x11111111u
-             : split_log2 == 3 ? 0x01010101u : split_log2 == 4 ? 0x00010001u : 1u) << part;
+    left &= bs_part_mask(split_log2, part);
     const mx whi = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
     while (left) {
       // one of the lane's items, and all of them with its signature
@@ -489,29 +593,14 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
       left &= ~same;
       const u64 key = ((u64)k1 << 32) | k0 | 1ull << 63;
       bool fresh;
-      const u32 slot = bs_class(P, W, key, fresh);
+      const u32 slot = bs_class(W.key, P.slots_log2, BS_NSIG, key, fresh);
       if (slot == ~0u) { atomicOr(W.status, 2u); continue; }   // the host runs the items one by one instead
       if (fresh) {
         W.rep[slot] = (hi << BS_BLK) | (u64)(lane << BS_LOW) | (u64)j;
         W.list[atomicAdd(W.list_n, 1ull)] = slot;
       }
-      // their mass at scale 2^(98 + mass_exp), where all the items' masses add
-      // up to at most 2^98: two chunks, the lower of BS_CLASS_SHIFT bits,
-      // each added up by itself
-      const u128 F = u128_shr(mx_prod(whi, u128_shr(bs_subset_mass(same, s_nib, m_mid), 2)), 25 + whi.e - P.mass_exp);
-      const u64 lo = F.lo & ((1ull << BS_CLASS_SHIFT) - 1ull);
-      const u64 up64 = (F.lo >> BS_CLASS_SHIFT) | (F.hi << (64 - BS_CLASS_SHIFT));
-      if (lo) atomicAdd(&W.cmass[2 * (size_t)slot], lo);
-      if (up64) atomicAdd(&W.cmass[2 * (size_t)slot + 1], up64);
-      // their number by popcount, two 32-bit counters to an addition
-      const int pc = pc_hi + __popc(lane);
-      u64* h = (u64*)(W.hist + (size_t)slot * BS_HIST) + (pc >> 1);
-      const u64 n = bs_popcount_bytes(same) << (8 * (pc & 1));
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const u64 two = ((n >> (16 * i)) & 255ull) | ((n >> (16 * i + 8)) & 255ull) << 32;
-        if (two) atomicAdd(&h[i], two);
-      }
+      bs_add_mass(W.cmass + 2 * (size_t)slot, whi, u128_shr(bs_subset_mass(same, s_nib, m_mid), 2), P.mass_exp);
+      bs_add_counts(W.hist + (size_t)slot * BS_HIST, same, pc_hi + __popc(lane));
       if (BS_GRAD)
         for (u32 s = same; s; s &= s - 1u) W.cls[(b << BS_BLK) + (u64)(((__ffs(s) - 1) << BS_MID) + lane)] = slot;
     }
@@ -531,16 +620,6 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
       if (i - j <= BS_D) n += s_ci[i - j] * P.binom[j];
     if (n) atomicAdd(&W.out_n[i], n);
   }
-}
-// The mass of a class as integer floating point.
-__device__ __forceinline__ mx bs_class_mass(const BsParams& P, const BsWork& W, u64 slot) {
-  u128 t = u128{W.cmass[2 * slot], 0ull};
-  const u64 up = W.cmass[2 * slot + 1];
-  u128_add(t, up << BS_CLASS_SHIFT, up >> (64 - BS_CLASS_SHIFT));
-  if (!(t.lo | t.hi)) return mx{0ull, 0, 0};
-  const int lz = t.hi ? __clzll((long long)t.hi) : 64 + __clzll((long long)t.lo);
-  const u64 m = lz >= 64 ? t.lo << (lz - 64) : (lz ? (t.hi << lz) | (t.lo >> (64 - lz)) : t.hi);
-  return mx{m, lz - 29 + P.mass_exp, 0};   // 128 - lz bits at scale 2^(98 + mass_exp)
 }
 // N_k of a class: its representative's states by popcount below the prefix
 // (rel, BS_TOP + 1 of them) for every popcount that its prefixes have.
@@ -693,7 +772,7 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
 #if BS_MERGE
       if (thr_on) bs_flush_bins(bins, rel, pc_thr);
       bs_class_counts(W, task, lane, rel, s_nbins);
-      w = bs_class_mass(P, W, task);
+      w = bs_class_mass(W.cmass + 2 * task, P.mass_exp);
 #endif
     } else {
       if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
@@ -713,8 +792,9 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
 
 #define KERNEL_R_ARGS const __grid_constant__ BsParams P, const u64* __restrict__ lane_tab, \
                   const u64* __restrict__ wmid_tab, const mx* __restrict__ ptab, const BsWork W
+#if !BS_MERGE
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel(KERNEL_R_ARGS) { bs_kernel_body<0>(P, lane_tab, wmid_tab, ptab, W); }
-#if BS_MERGE
+#else
 extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_p1(const __grid_constant__ BsParams P,
     const mx* __restrict__ ptab, const ulonglong2* __restrict__ mtab, int split_log2, const BsWork W) {
   bs_merge_body(P, ptab, mtab, split_log2, W);
@@ -779,7 +859,7 @@ __device__ __forceinline__ mx bs_arc_factor(const BsParams& P, const mx* __restr
 // The mass factors of an item (or class) for R, of internal arc `lane` and of
 // arc `lane + 32`.
 #if BS_MERGE
-#define BS_CLASS_FACTORS() wpre = f0 = f1 = bs_class_mass(P, W, task)
+#define BS_CLASS_FACTORS() wpre = f0 = f1 = bs_class_mass(W.cmass + 2 * task, P.mass_exp)
 #else
 #define BS_CLASS_FACTORS() wpre = f0 = f1 = mx{0ull, 0, 0}
 #endif
@@ -1093,8 +1173,9 @@ __device__ __forceinline__ void bs_kernel_grad_body(
                   const u64* __restrict__ wmid128, const mx* __restrict__ ptab, \
                   const mx* __restrict__ ptab_ex, const BsWork W
 #define KERNEL_G_PASS P, Q, lane_tab, thr_tab, wmid128, ptab, ptab_ex, W
+#if !BS_MERGE
 extern "C" __global__ void KERNEL_BOUNDS bs_kernel_grad(KERNEL_G_ARGS) { bs_kernel_grad_body<0>(KERNEL_G_PASS); }
-#if BS_MERGE
+#else
 extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p1(const __grid_constant__ BsParams P,
     const mx* __restrict__ ptab, const ulonglong2* __restrict__ mtab, int split_log2, const BsWork W) {
   bs_merge_body(P, ptab, mtab, split_log2, W);
@@ -1121,26 +1202,6 @@ struct BsFoldParams {
   u64 wmid[31];         // of the mid arcs above mid arc b
   u64 mid[32];          // mid pattern masses (2^63)
 };
-// |a - b|; neg: a < b (classes' sums round apart by up to 2^-61, so a pair
-// whose true difference is zero may come out below it)
-__device__ __forceinline__ u128 bs_absdiff(u128 a, u128 b, bool& neg) {
-  neg = a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo);
-  return neg ? u128_sub(b, a) : u128_sub(a, b);
-}
-// one fold: adds w (V1 - V0) to G, returns V0 + p (V1 - V0)
-__device__ __forceinline__ u128 bs_fold2(u128 V0, u128 V1, u64 p, u64 w, u128& G) {
-  bool neg;
-  const u128 d = bs_absdiff(V1, V0, neg);
-  if (!neg) {
-    const u128 g = mul64x128_shr64(w, d.lo, d.hi);   // scale 2^123
-    u128_add(G, g.lo, g.hi);
-  }
-  u128 x = mul64x128_shr64(p, d.lo, d.hi);
-  x = u128{x.lo << 1, (x.hi << 1) | (x.lo >> 63)};
-  if (neg) return u128_sub(V0, x);
-  u128_add(V0, x.lo, x.hi);
-  return V0;
-}
 extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p3(
     const __grid_constant__ BsParams P, const __grid_constant__ BsFoldParams Q, const mx* __restrict__ ptab,
     const BsWork W) {
@@ -1171,51 +1232,16 @@ extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p3(
     u128 G[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) G[i] = u128{0ull, 0ull};
-    u128 top[4];   // folded over the lowest three arcs
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      u128 V[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = 8 * q + i;
-        V[i] = u128{0ull, (m.x >> j) & 1u ? 1ull << 60 : 0ull};
-        if ((m.y >> j) & 1u) {
-          const ulonglong2 s = W.csum[cls[j << BS_MID]];
-          V[i] = u128{s.x, s.y};
-        }
+    u128 V = bs_fold_low(Q.p, Q.wlow, G, [&](int j) {
+      u128 v = u128{0ull, (m.x >> j) & 1u ? 1ull << 60 : 0ull};
+      if ((m.y >> j) & 1u) {
+        const ulonglong2 s = W.csum[cls[j << BS_MID]];
+        v = u128{s.x, s.y};
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], Q.p[0], Q.wlow[4 * q + i], G[0]);
-#pragma unroll
-      for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], Q.p[1], Q.wlow[16 + 2 * q + i], G[1]);
-      top[q] = bs_fold2(V[0], V[1], Q.p[2], Q.wlow[24 + q], G[2]);
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i) top[i] = bs_fold2(top[2 * i], top[2 * i + 1], Q.p[3], Q.wlow[28 + i], G[3]);
-    u128 V = bs_fold2(top[0], top[1], Q.p[4], Q.wlow[30], G[4]);
-    // the block's sums per arc, lane l ending with arc l's (scale 2^124)
-    u128 X = u128{0ull, 0ull};
-#pragma unroll
-    for (int i = 0; i < BS_LOW; ++i) {
-      u128 g = mul64x128_shr64(m_mid, G[i].lo, G[i].hi);   // 2^122
-      g = warp_sum_u128(g);
-      g = u128{g.lo << 2, (g.hi << 2) | (g.lo >> 62)};
-      if (lane == i) X = g;
-    }
-#pragma unroll
-    for (int i = 0; i < BS_MID; ++i) {
-      const u128 o = shfl_xor_u128(V, 1 << i);
-      const bool one = (lane >> i) & 1;
-      u128 g = u128{0ull, 0ull};
-      const int at = (i == 0 ? 0 : i == 1 ? 16 : i == 2 ? 24 : i == 3 ? 28 : 30) + (lane >> (i + 1));
-      V = bs_fold2(one ? o : V, one ? V : o, Q.p[5 + i], Q.wmid[at], g);
-      if (lane & ((1 << (i + 1)) - 1)) g = u128{0ull, 0ull};   // each pair once
-      g = warp_sum_u128(g);
-      g = u128{g.lo << 1, (g.hi << 1) | (g.lo >> 63)};
-      if (lane == BS_LOW + i) X = g;
-    }
-    V.lo = __shfl_sync(0xffffffffu, V.lo, 0);
-    V.hi = __shfl_sync(0xffffffffu, V.hi, 0);
+      return v;
+    });
+    u128 X;   // the block's sums, lane l: arc l's
+    V = bs_fold_mid(V, G, BS_LOW, BS_MID, Q.p + 5, Q.wmid, m_mid, lane, X);
     const mx w = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
     if (lane < BS_BLK) facc_add(accP, mx_prod(w, X), w.e);
     const u128 Sv = mx_prod(w, V);
@@ -1271,7 +1297,32 @@ struct BGraph {
   u64 full_counts;
   u64 pex_mask;   // gradient module: prefix arcs using the excluded-arc tables
   u64 binom[64];
+  // merged modules: the arcs of a block and above it, the signature, and
+  // where this network's blocks, slots and items begin (see BMerge)
+  int low, mid, nhi, nsig, slots_log2, pad2;
+  u64 blk_begin, slot_base, item_base;
 };
+// Work arrays of a merged batch.  Slots hold signatures and the class that
+// each stands for; a class its network, one of its items, its number of items
+// by popcount, and per p-vector its mass (two chunks) and its sum S.  Blocks:
+// per lane the items connected throughout and left to walk (a bit each);
+// items: the slot, and for the first of a lane with that slot the lane's items
+// with it.
+struct BMerge {
+  u64* key; u32* id_of;
+  u32* net; u64* rep; u32* hist; u64* cmass; ulonglong2* csum;
+  uint2* cmask; uint2* ent;
+  u64* n_classes; u64* ticket;
+  u64 n_blocks;
+  // few blocks: 2^split_log2 warps share one in the first (its words and its
+  // p-vectors), `parts` in the second launch (its p-vectors)
+  int split_log2, parts;
+  u32 cap; int hist_stride;
+  const ulonglong2* nib; const ulonglong2* mid; const u64* fold;
+};
+#ifndef BSB_MERGE
+#define BSB_MERGE 0
+#endif
 
 // add P * 2^(-123 - e) (P < 2^124, e >= 0) to the 256-bit limbs (scale 2^250)
 __device__ __forceinline__ void bsb_limb_add(u64* limbs, u128 P, int e) { bs_limb_add(limbs, P, 127 - e); }
@@ -1303,12 +1354,19 @@ __device__ __forceinline__ u32 bsb_uniform(const u32* a) {
   return G::var(e, w);
 }
 
+// A merged module walks few items and holds two functions per network: these
+// are calls, compiled apart (64 networks: NVRTC 11.7 s inlined, 5.4 s so).
+#if BSB_MERGE
+#define BSB_NETWORK __noinline__
+#else
+#define BSB_NETWORK __forceinline__
+#endif
 // The per-network part of one item: its state words, the monotone prune,
 // and the connectivity word of every walk state into cw (stride BSB_NTHR).
 // Returns 0 when every state of the item is cut, 1 when every state is
 // connected, 2 when cw holds the item's words.
 template <class G>
-__device__ __forceinline__ int bsb_conn(u64 prefix, int lane, int prune, u32* cw) {
+__device__ BSB_NETWORK int bsb_conn(u64 prefix, int lane, int prune, u32* cw) {
   u32 a[G::M];
 #pragma unroll
   for (int i = 0; i < G::ELL; ++i)
@@ -1359,6 +1417,37 @@ __device__ __forceinline__ void bsb_flush_counts(const BGraph* __restrict__ B, u
   __syncwarp();
 }
 
+// N_k of a class: its item's counts below the prefix (rel) for every popcount
+// that its prefixes have, into the warp's counts nkw.
+__device__ __forceinline__ void bsb_class_counts(const BMerge& A, u64 cls, int d, int top, int lane, u64* rel, u64* nkw) {
+  __syncwarp();
+  const u64 r = lane <= top ? rel[lane] : 0ull;
+  const u32* h = A.hist + cls * A.hist_stride;
+  for (int q = 0; q <= d; ++q) {
+    const u32 n = h[q];
+    if (n && r) nkw[q + lane] += n * r;
+    __syncwarp();
+  }
+  if (lane <= top) rel[lane] = 0ull;
+  __syncwarp();
+}
+// this thread's counts c11 by walk popcount + lane class: an item's to nkw, a
+// class's below the prefix, then for all its items
+#if BSB_MERGE
+#define BSB_COUNTS()                                                          \
+  if (thr_on) {                                                               \
+    _Pragma("unroll") for (int i = 0; i < 11; ++i)                            \
+      if (c11[i]) atomicAdd(&rel[__popc(lane) + i], c11[i]);                  \
+  }                                                                           \
+  bsb_class_counts(A, cls, Bp->d, top, lane, rel, nkw)
+#else
+#define BSB_COUNTS()                                                          \
+  if (thr_on) {                                                               \
+    _Pragma("unroll") for (int i = 0; i < 11; ++i)                            \
+      if (c11[i]) atomicAdd(&nkw[pc_pre + __popc(lane) + i], c11[i]);         \
+  }
+#endif
+
 // N_k counts go to the warp's own array nkw (indexed by k within the
 // network), which the kernel flushes to global memory when the warp moves
 // to another network and at the end.
@@ -1366,7 +1455,7 @@ __device__ __forceinline__ void bsb_finish(const BGraph* __restrict__ Bp, int st
                                            int Kp, const u64* __restrict__ lt, const u64* __restrict__ nt,
                                            const u64* __restrict__ wm, const mx* __restrict__ pt,
                                            const u64* __restrict__ thw, u64* limbs, u64* nkw, u64* bins,
-                                           const u32* cw) {
+                                           const u32* cw, const BMerge& A, u64 cls, u64* rel) {
   constexpr int nsh[6] = BS_NK_SHIFTS, nwd[6] = BS_NK_WIDTHS;
   const int gidx = Bp->gidx, L = Bp->L, tb = Bp->tb, nlev = Bp->nlev, top = Bp->top;
   const int lt_off = Bp->lt_off, nt_off = Bp->nt_off, wm_off = Bp->wm_off, pt_off = Bp->pt_off;
@@ -1415,12 +1504,7 @@ __device__ __forceinline__ void bsb_finish(const BGraph* __restrict__ Bp, int st
 #pragma unroll
       for (int cl = 0; cl < 6; ++cl) c11[r + cl] += (n >> nsh[cl]) & ((1ull << nwd[cl]) - 1ull);
     }
-    if (thr_on) {
-      const int base = pc_pre + __popc(lane);
-#pragma unroll
-      for (int i = 0; i < 11; ++i)
-        if (c11[i]) atomicAdd(&nkw[base + i], c11[i]);
-    }
+    BSB_COUNTS();
   }
   const u64* ltg = lt + lt_off;
   const u64* wmg = wm + wm_off;
@@ -1486,7 +1570,8 @@ __device__ __forceinline__ void bsb_finish(const BGraph* __restrict__ Bp, int st
       u128_add(T[0], got.lo, got.hi);
     }
     if (!(lane & 1) && idx < kc) {
-      const mx w = bsb_prefix_mass(gpt + (size_t)(k0 + idx) * pt_size, nlev, lev_bits, lev_off, prefix);
+      const mx w = BSB_MERGE ? bs_class_mass(A.cmass + 2 * (cls * K + k0 + idx), 0)
+          : bsb_prefix_mass(gpt + (size_t)(k0 + idx) * pt_size, nlev, lev_bits, lev_off, prefix);
       bsb_limb_add(glimbs + (size_t)(k0 + idx) * BSB_LIMBS, mx_prod(w, T[0]), w.e);
     }
   }
@@ -1529,7 +1614,7 @@ __device__ __forceinline__ void bsb_finish_grad(
     const u64* __restrict__ lt, const u64* __restrict__ nt, const u64* __restrict__ wm2,
     const mx* __restrict__ pt, const u64* __restrict__ thw, const u64* __restrict__ tt,
     const u64* __restrict__ lwex, const u64* __restrict__ thwex, const mx* __restrict__ ptex,
-    u64* limbs, u64* nkw, u64* bins, const u32* cw, u32* ctw, const BsTr& tr) {
+    u64* limbs, u64* nkw, u64* bins, const u32* cw, u32* ctw, const BsTr& tr, const BMerge& A, u64 cls, u64* rel) {
   constexpr int nsh[6] = BS_NK_SHIFTS, nwd[6] = BS_NK_WIDTHS;
   const int L = Bp->L, tb = Bp->tb, ell = Bp->ell, top = Bp->top, m = Bp->m, nlev = Bp->nlev;
   const int pt_size = Bp->pt_size, d = Bp->d;
@@ -1566,12 +1651,7 @@ __device__ __forceinline__ void bsb_finish_grad(
 #pragma unroll
       for (int cl = 0; cl < 6; ++cl) c11[r + cl] += (n >> nsh[cl]) & ((1ull << nwd[cl]) - 1ull);
     }
-    if (thr_on) {
-      const int base = pc_pre + __popc(lane);
-#pragma unroll
-      for (int i = 0; i < 11; ++i)
-        if (c11[i]) atomicAdd(&nkw[base + i], c11[i]);
-    }
+    BSB_COUNTS();
     // ---- the lane transposes, once per word: lane j then holds the
     // threads' bits of lane pattern j (lanes past the thread patterns hold
     // no thread's states); zero when no lane's word is partly connected
@@ -1656,9 +1736,19 @@ __device__ __forceinline__ void bsb_finish_grad(
     // ---- prefix factors of p-vector k and the additions to its results
     const mx* tk = pt + Bp->pt_off + (size_t)k * pt_size;
     const mx* exk = ptex + Bp->ptex_off + ((size_t)k * d << 7);
-    const mx wpre = bsb_prefix_mass(tk, nlev, lev_bits, lev_off, prefix);
+    const mx wpre = BSB_MERGE ? bs_class_mass(A.cmass + 2 * (cls * K + k), 0)
+                              : bsb_prefix_mass(tk, nlev, lev_bits, lev_off, prefix);
     u64* out = gl + (size_t)k * stride * BSB_LIMBS;
     if (lane == 0) bsb_limb_add(out, mx_prod(wpre, S), wpre.e);
+#if BSB_MERGE
+    // a class's prefix arcs are left to bs_batch_grad_p3, from its sum S
+    if (lane == 0) A.csum[cls * K + k] = make_ulonglong2(S.lo, S.hi);
+    if (lane < top) {
+      bsb_limb_add(out + (1 + 2 * lane) * BSB_LIMBS, mx_prod(wpre, myX), wpre.e);
+      bsb_limb_add(out + (2 + 2 * lane) * BSB_LIMBS, mx_prod(wpre, myY), wpre.e);
+    }
+    continue;
+#endif
     if (lane < m) {
       u128 X = u128{0ull, 0ull}, Y = u128{0ull, 0ull};
       mx f = wpre;
@@ -1686,6 +1776,183 @@ __device__ __forceinline__ void bsb_finish_grad(
     }
   }
 }
+#if BSB_MERGE
+// ---------------------------------------------------------------------------
+// Merged batches: as the single networks' merged runs (bs_merge_body), for
+// every network and p-vector at once.
+//   bs_batch*_p1  prunes every network's items, 32 x 32 at a time, sums those
+//                 connected throughout, and interns the signatures of the others
+//   bs_batch*_p2  adds each item's masses and popcount to its class
+//   bs_batch*     walks one item of every class (bsb_conn, bsb_finish)
+//   bs_batch*_p3  (gradient) folds the prefix arcs, per block and p-vector
+// GB300, against a walk for every item left: 64 networks x 16 p-vectors, R
+// 9.6 -> 0.62 ms; 20 x 7 with the gradient 0.91 -> 0.36 ms (prune 1), 0.16
+// (prune 2).  The walking launch is bound by instruction issue and the table
+// rows it reads through L1, the others by the latency of the table and the
+// class memory, hence the several warps per block of items.
+// ---------------------------------------------------------------------------
+#define BSB_MNTHR 128
+// The per-network part of a block: which of its items are connected
+// throughout and which are left to walk, and the latter's signatures, one
+// word per bit and lane, in zs.
+template <class G>
+__device__ __noinline__ void bsb_classify(u64 hi, int lane, u32* zs, u32& full, u32& left) {
+  constexpr int BLK = G::LOW + G::MID;
+  u32 a[G::M], z[G::NSIG > 0 ? G::NSIG : 1], dn, up;
+#pragma unroll
+  for (int j = 0; j < G::D; ++j)
+    a[G::TOP + j] = j < G::LOW ? bs_pattern(j) : j < BLK ? 0u - (u32)((lane >> (j - G::LOW)) & 1)
+                                                          : 0u - (u32)((hi >> (j - BLK)) & 1ull);
+  G::sig(a, z, dn, up);
+  const u32 valid = lane < (1 << G::MID) ? (G::LOW >= 5 ? 0xffffffffu : (1u << (1 << G::LOW)) - 1u) : 0u;
+  full = dn & valid;
+  left = up & valid & ~full;
+#pragma unroll
+  for (int i = 0; i < G::NSIG; ++i) zs[i * 32 + lane] = z[i];
+}
+__device__ __forceinline__ int bsb_block_net(const BGraph* __restrict__ graphs, int G, u64 t) {
+  int lo = 0, hi = G - 1;
+  while (lo < hi) { const int mid = (lo + hi + 1) >> 1; if (graphs[mid].blk_begin <= t) lo = mid; else hi = mid - 1; }
+  return lo;
+}
+// mass of the arcs above a block (the levels of a merged batch's table)
+__device__ __forceinline__ mx bsb_hi_mass(const BGraph* __restrict__ B, const mx* __restrict__ pt, int k, u64 hi) {
+  return bs_level_mass(B->nlev, B->lev_bits, B->lev_off, pt + B->pt_off + (size_t)k * B->pt_size, hi);
+}
+// What bsb_merge does with a block once its network's part is done.
+__device__ __forceinline__ void bsb_merge_block(const BGraph* __restrict__ B, int net, u64 t, u64 hi, int part, int lane, int K,
+                                                const u32* zs, u32 full, u32 left, const mx* __restrict__ pt,
+                                                const BMerge& A, u64* limbs, u64* nk, u32* status) {
+  const int low = B->low, mid = B->mid, blk = low + mid, top = B->top, nsig = B->nsig;
+  const int pc_hi = __popcll((long long)hi);
+  if (part == 0) A.cmask[t * 32 + lane] = make_uint2(full, left);
+  if (__any_sync(0xffffffffu, full)) {
+    if (part == 0) {
+      // lane q: states with pc_hi + q working arcs, over the items' popcounts
+      const u32 n = bs_block_counts(full, lane);
+      u64 s = 0;
+      for (int i = 0; i <= blk; ++i) {
+        const u64 c = __shfl_sync(0xffffffffu, n, i);
+        if (lane >= i && lane - i <= top) s += c * __ldg(&B->binom[lane - i]);
+      }
+      if (s) atomicAdd(&nk[B->nk_off + pc_hi + lane], s);
+    }
+    for (int k = part; k < K; k += 1 << A.split_log2) {
+      const size_t gk = (size_t)net * K + k;
+      const ulonglong2 mm = __ldg(&A.mid[gk * 32 + lane]);
+      const u128 S = warp_sum_u128(u128_shr(bs_subset_mass(full, A.nib + gk * 128, u128{mm.x, mm.y}), 2));
+      if (lane == 0) {
+        const mx w = bsb_hi_mass(B, pt, k, hi);
+        bsb_limb_add(limbs + B->out_off + (size_t)k * (BSB_GRAD ? 1 + 2 * B->m : 1) * BSB_LIMBS, mx_prod(w, S), w.e);
+      }
+    }
+  }
+  left &= bs_part_mask(A.split_log2, part);
+  while (left) {
+    const int j = __ffs(left) - 1;
+    u32 k0 = 0u, k1 = 0u, same = left;
+    for (int i = 0; i < nsig; ++i) {
+      const u32 z = zs[i * 32 + lane], b = z << (31 - j);   // item j's bit on top
+      if (i < 32) k0 = __funnelshift_l(b, k0, 1); else k1 = __funnelshift_l(b, k1, 1);
+      same &= ~(z ^ (u32)((int)b >> 31));
+    }
+    left &= ~same;
+    bool fresh;
+    const u32 at = bs_class(A.key + B->slot_base, B->slots_log2, nsig, ((u64)k1 << 32) | k0 | 1ull << 63, fresh);
+    if (at == ~0u) { atomicOr(status, 2u); continue; }   // the host walks the items one by one instead
+    const u32 slot = (u32)B->slot_base + at;
+    if (fresh) {
+      const u64 id = atomicAdd(A.n_classes, 1ull);
+      if (id < A.cap) {
+        A.id_of[slot] = (u32)id;
+        A.net[id] = (u32)net;
+        A.rep[id] = (hi << blk) | (u64)(lane << low) | (u64)j;
+        for (int i = 0; i < A.hist_stride; ++i) A.hist[id * A.hist_stride + i] = 0u;
+        for (int i = 0; i < 2 * K; ++i) A.cmass[2 * id * K + i] = 0ull;
+      } else {
+        atomicOr(status, 2u);
+      }
+    }
+    uint2* e = A.ent + B->item_base + (hi << blk) + lane;
+    for (u32 s = same; s; s &= s - 1u) {
+      const int i = __ffs(s) - 1;
+      e[i << mid] = make_uint2(slot, i == j ? same : 0u);
+    }
+  }
+}
+extern "C" __global__ void __launch_bounds__(BSB_MNTHR) BSB_SCATTER(
+    const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u32* status) {
+  __shared__ mx s_hi[BSB_MNTHR / 32][64];
+  if (*(volatile u32*)status) return;   // out of time or slots: the host discards the run
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks * A.parts; v += (u64)gridDim.x * (BSB_MNTHR / 32)) {
+    const u64 t = v / A.parts;
+    const int part = (int)(v - t * A.parts);
+    u32 left = A.cmask[t * 32 + lane].y;
+    if (!__any_sync(0xffffffffu, left)) continue;
+    const int net = bsb_block_net(graphs, G, t);
+    const BGraph* __restrict__ B = graphs + net;
+    const u64 hi = t - B->blk_begin;
+    const int mid = B->mid, blk = B->low + mid, pc = __popcll((long long)hi) + __popc(lane);
+    __syncwarp();
+    for (int k = part + lane * A.parts; k < K; k += 32 * A.parts) s_hi[warp][k] = bsb_hi_mass(B, pt, k, hi);
+    __syncwarp();
+    uint2* e = A.ent + B->item_base + (hi << blk) + lane;
+    while (left) {
+      const int j = __ffs(left) - 1;
+      const uint2 x = e[j << mid];
+      left &= ~x.y;   // the first item of its class in the lane has them all
+      const u32 id = A.id_of[x.x];
+      if (part == 0) bs_add_counts(A.hist + (size_t)id * A.hist_stride, x.y, pc);
+      for (int k = part; k < K; k += A.parts) {
+        const size_t gk = (size_t)net * K + k;
+        const ulonglong2 mm = __ldg(&A.mid[gk * 32 + lane]);
+        bs_add_mass(A.cmass + 2 * ((size_t)id * K + k), s_hi[warp][k],
+                    u128_shr(bs_subset_mass(x.y, A.nib + gk * 128, u128{mm.x, mm.y}), 2), 0);
+      }
+    }
+  }
+}
+#if BSB_GRAD
+extern "C" __global__ void __launch_bounds__(BSB_MNTHR) bs_batch_grad_p3(
+    const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u64* limbs,
+    const u32* status) {
+  if (*(volatile const u32*)status) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (u64 t = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; t < A.n_blocks * K; t += (u64)gridDim.x * (BSB_MNTHR / 32)) {
+    const u64 b = t / K;
+    const int k = (int)(t - b * K);
+    const uint2 m = A.cmask[b * 32 + lane];
+    if (!__any_sync(0xffffffffu, m.x | m.y)) continue;
+    const int net = bsb_block_net(graphs, G, b);
+    const BGraph* __restrict__ B = graphs + net;
+    const u64 hi = b - B->blk_begin;
+    const int low = B->low, mid = B->mid, blk = low + mid, nhi = B->nhi, top = B->top;
+    const u64* __restrict__ f = A.fold + ((size_t)net * K + k) * 104;   // laid out as BsFoldParams
+    const uint2* e = A.ent + B->item_base + (hi << blk) + lane;
+    u128 Gs[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) Gs[i] = u128{0ull, 0ull};
+    u128 V = bs_fold_low(f, f + 10, Gs, [&](int j) {
+      u128 v = u128{0ull, (m.x >> j) & 1u ? 1ull << 60 : 0ull};
+      if ((m.y >> j) & 1u) {
+        const ulonglong2 s = A.csum[(size_t)A.id_of[e[j << mid].x] * K + k];
+        v = u128{s.x, s.y};
+      }
+      return v;
+    });
+    u128 X;
+    V = bs_fold_mid(V, Gs, low, mid, f + 5, f + 41, f[72 + lane], lane, X);
+    const mx w = bsb_hi_mass(B, pt, k, hi);
+    u64* out = limbs + B->out_off + (size_t)k * (1 + 2 * B->m) * BSB_LIMBS;
+    if (lane < blk) bsb_limb_add(out + (1 + 2 * (top + lane)) * BSB_LIMBS, mx_prod(w, X), w.e);
+    const u128 Sv = mx_prod(w, V);
+    for (int q = lane; q < nhi; q += 32)
+      bsb_limb_add(out + (((hi >> q) & 1ull ? 1 : 2) + 2 * (top + blk + q)) * BSB_LIMBS, Sv, w.e);
+  }
+}
+#endif
+#endif
 //@@BATCH_KERNEL@@
 )PBAT";
 }  // namespace pbat

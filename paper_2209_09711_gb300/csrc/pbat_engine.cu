@@ -389,12 +389,6 @@ void scratch_release(Scratch* s) {
 // ---------------------------------------------------------------------------
 // one planned enumeration (single network)
 // ---------------------------------------------------------------------------
-// Items from which a run merges them by default (pbat_options.launches 0):
-// below, one launch is a few microseconds long and further ones cost more
-// than they save (GB300, R / fused: 2^11 items of 23 arcs 29 / 36 us in one
-// launch, 29 / 54 merged; 2^14 items of 27 arcs 58 / 90 against 42 / 54).
-constexpr unsigned long long kMergeItems = 1ull << 12;
-
 struct Job {
   GraphIn g;
   Plan pl;
@@ -745,11 +739,10 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   }
   J->n_items = n_items;
   J->grid_nthr = nthr;
-  // Items merged by signature, or every item by itself in one launch (see
-  // bs_merge_body in the kernel source).  Below kMergeItems items the run is
-  // a few microseconds long and further launches cost more than they save.
-  const BsMerge mg = J->bs && o.prune && o.launches != 1 ? bs_merge(*J->bs) : BsMerge{};
-  J->merged = mg.slots > 0 && (o.launches == 2 || n_items >= kMergeItems);
+  // items merged by signature, or every item by itself in one launch (see
+  // bs_merge_body in the kernel source)
+  const BsMerge mg = J->bs ? bs_merge(*J->bs) : BsMerge{};
+  J->merged = mg.slots > 0;
   const long long warps_per_block = nthr / 32;
   long long grid = (long long)per_sm * J->dev.sms;
   // never more warps than work items
@@ -970,13 +963,15 @@ void job_destroy(Job* J);
 int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* dRdp_out,
              pbat_options* opt);
 
-// The same question under other options, in place of J's results.
-static int job_rerun(Job* J, pbat_options o, cudaStream_t st, double* R_out, uint64_t* Nk_out,
+// The same question under other options, in place of J's results; keep: J
+// becomes that job, so that a plan's next enumeration runs it at once.
+static int job_rerun(Job* J, pbat_options o, bool keep, cudaStream_t st, double* R_out, uint64_t* Nk_out,
                      double* dRdp_out, pbat_options* opt) {
   Job* F = nullptr;
   int rc = job_create(J->g, J->p_copy.data(), J->pl.grad, &o, &F);
   if (!rc && !(rc = job_upload(F, st)) && !(rc = job_launch(F, st)))
     rc = job_read(F, st, R_out, Nk_out, J->pl.grad ? dRdp_out : nullptr, opt);
+  if (keep && !rc) std::swap(*J, *F);
   job_destroy(F);
   return rc;
 }
@@ -1002,9 +997,8 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
     bs_mark_unmergeable(*J->bs);
     pbat_options o = J->opt_copy;
     o.launches = 1;
-    J->merged = false;
     J->n_pending = 0;
-    return job_rerun(J, o, st, R_out, Nk_out, dRdp_out, opt);
+    return job_rerun(J, o, true, st, R_out, Nk_out, dRdp_out, opt);
   }
   if (J->bs)
     for (int i = 0; i < J->n_acc; ++i) J->h_acc[i] = limbs256_to_dd(J->h_limbs + 8 * i);
@@ -1055,7 +1049,7 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
     // kernel, whose tables are exact to 2^-100
     pbat_options o = J->opt_copy;
     o.algo = PBAT_ALGO_FRONTIER;
-    return job_rerun(J, o, st, R_out, Nk_out, dRdp_out, opt);
+    return job_rerun(J, o, false, st, R_out, Nk_out, dRdp_out, opt);
   }
   *R_out = R;
   if (Nk_out)

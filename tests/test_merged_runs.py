@@ -31,13 +31,18 @@ def _signature_program(src):
 def _evaluate(body, a, n):
     env, z = {"a": a}, [0] * n
     for line in body.splitlines()[1:]:
+        line = re.sub(r"\b(0x[0-9a-f]+|0)u\b", r"\1", line)
         m = re.match(r"\s*const u32 (\w+) = (.*);$", line)
         if m:
             env[m.group(1)] = eval(m.group(2), {}, env) & FULL
             continue
-        m = re.match(r"\s*z\[(\d+)\] = (.*);$", line)
-        z[int(m.group(1))] = eval(m.group(2), {}, env) & FULL
-    return z
+        m = re.match(r"\s*(z\[(\d+)\]|dn|up) = (.*);$", line)
+        value = eval(m.group(3), {}, env) & FULL
+        if m.group(2):
+            z[int(m.group(2))] = value
+        else:
+            env[m.group(1)] = value
+    return z, env["dn"], env["up"]
 
 
 def _residual(net, prefix, on, free):
@@ -73,21 +78,26 @@ def _residual(net, prefix, on, free):
 def test_signature_is_the_residual_network(pb, directed, prune):
     """Over 32 random items at a time, those whose prefix does not join source
     and sink: equal signatures exactly where the prefix leaves the same
-    connectivity."""
+    connectivity.  And both ends of the prune, for every item."""
     for seed in range(10):
         rng = synth.SplitMix64(8100 + seed)
         n, m = 3 + rng.below(9), 14 + rng.below(14)
         net = synth.random_small(8200 + seed, n=n, m=m, directed=directed)
-        src = pb.kernel_source(net, pb.options(walk_bits=seed % 3, prune=prune))
+        src = pb.kernel_source(net, pb.options(walk_bits=seed % 3, prune=prune, launches=2))
         perm, D, body = _signature_program(src)
         top, nsig = int(D["BS_TOP"]), int(D["BS_NSIG"])
         assert int(D["BS_MERGE"]) == 1 and 0 <= nsig <= 63
         words = [rng.next_u64() & FULL for _ in range(m)]
-        z = _evaluate(body, [0] * top + words[top:], nsig)
+        z, dn, up = _evaluate(body, [0] * top + words[top:], nsig)
         items = [[(words[k] >> i) & 1 for k in range(top, m)] for i in range(32)]
         sig = [tuple((w >> i) & 1 for w in z) for i in range(32)]
         res = [_residual(net, perm[top:], on, perm[:top]) for on in items]
         st = (net.source, net.sink)   # items that join these are not classed
+        for i, on in enumerate(items):
+            rest = sum(1 << (m - 1 - a) for a in perm[:top])
+            x = sum(1 << (m - 1 - a) for a, works in zip(perm[top:], on) if works)
+            assert bool((dn >> i) & 1) == oracle.connected(net, x)
+            assert bool((up >> i) & 1) == oracle.connected(net, x | rest)
         left = [i for i in range(32) if st not in res[i]]
         for i in left:
             for j in left:
@@ -163,3 +173,30 @@ def test_more_classes_than_the_table_holds(pb):
         res = plan.read()
         assert res.stats[5] == 1
         assert res.Nk == want.Nk and _same(res.R, want.R, 1e-12 * want.R)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("vectors", [1, 7, 17, 40])
+@pytest.mark.parametrize("grad", [False, True])
+def test_merged_batches(pb, vectors, grad):
+    """Networks from ones without prefix arcs to several blocks of items, in
+    one batch, against batches that walk every item (the prune off) and the
+    oracle."""
+    nets = [synth.random_small(4400 + m, n=4 + m % 6, m=m, directed=bool(m & 1), p_lo=0.3, p_hi=0.99)
+            for m in (6, 10, 11, 13, 16, 17, 19, 22)]
+    rng = synth.SplitMix64(90 + vectors)
+    pvecs = [[synth.uniform_p(rng, net.m, 0.3, 0.99) for _ in range(vectors)] for net in nets]
+    for prune, walk in ((1, -1), (1, 0), (2, 1)):
+        opts = dict(autotune=0, algo=pb.ALGO_BITSLICE, walk_bits=walk)
+        R, Nk, g = pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(prune=prune, **opts))
+        R0, Nk0, g0 = pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(prune=0, **opts))
+        assert Nk == Nk0
+        for i, net in enumerate(nets):
+            if net.m < 17 and prune == 1:
+                ref = oracle.enumerate_states(net, p=pvecs[i][0])
+                assert Nk[i] == ref.Nk and _same(R[i][0], ref.R, 1e-12 * ref.R)
+            for k in range(vectors):   # the bounds of _check; walk masses 2^(5-64) at most
+                assert _same(R[i][k], R0[i][k], 2 * 2.0**-53 * R0[i][k] + 2.0**-57)
+                if grad:
+                    for x, y in zip(g[i][k], g0[i][k]):
+                        assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (net.name, k)
