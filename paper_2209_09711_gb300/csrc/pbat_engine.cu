@@ -191,16 +191,21 @@ int make_plan(const GraphIn& g, const double* p, bool grad, const pbat_options& 
   pl.ell = std::min(kMaxLaneBits, m - r);
   const int free_bits = m - r - pl.ell;
   const int lmax = grad ? kMaxWalkBitsGrad : kMaxWalkBitsR;
-  // enough work items to keep every warp of the persistent grid busy
-  int want_items_log2 = 14;
   if (o.walk_bits >= 0) {
     pl.L = std::min(o.walk_bits, std::min(lmax, free_bits));
   } else if (o.prefix_bits >= 0) {
     const int d = std::max(o.prefix_bits, r);
     pl.L = std::max(0, std::min(lmax, m - pl.ell - d));
   } else {
-    const int extra_prefix = std::max(0, want_items_log2 - r);
-    pl.L = std::max(0, std::min(lmax, free_bits - extra_prefix));
+    // Between items enough to fill the SMs and walks long enough to carry an
+    // item's prune and sums.  GB300, R / gradient in us: 19 arcs L = 4 38 / 59
+    // (0: 105 / 204, 8: 124 / 138); 23 arcs L = 6 90 / 159 (4: 124 / 298, 9: 335
+    // / 341); 25 arcs L = 7 231 / 386 (5: 284 / 715, 10: 704 / 710); 30 arcs
+    // L = 9 3.7 / 8.3 ms (6: 5.4 / 12.7, 11: 6.0 ms).
+    int space = free_bits;   // log2 of the lane patterns enumerated
+    if (r > 0)
+      for (uint64_t x = o.range_hi - o.range_lo; x > 1; x >>= 1) ++space;
+    pl.L = std::max(0, std::min(std::min(lmax, free_bits), (space - 6) / 2));
   }
   pl.d = m - pl.ell - pl.L;
   // Internal arc order: internal position k holds input arc m-1-k, so the
@@ -294,18 +299,16 @@ void build_params(const GraphIn& g, const double* p, const Plan& pl, const pbat_
   const int nl = 1 << pl.ell;
   for (int j = 0; j < 32; ++j) {
     if (j >= nl) {
-      P.lane_w[j] = dd{0.0, 0.0};
-      for (int i = 0; i < kMaxLaneBits; ++i) P.lane_w_ex[i][j] = dd{0.0, 0.0};
       continue;
     }
     dd w = dd_make(1.0);
     for (int i = 0; i < pl.ell; ++i) w = dd_mul(w, arc_w(p, pl.perm[i], (j >> i) & 1));
-    P.lane_w[j] = w;
+    P.lane_w[j] = to_lane_mass(w);
     for (int x = 0; x < pl.ell; ++x) {
       dd we = dd_make(1.0);
       for (int i = 0; i < pl.ell; ++i)
         if (i != x) we = dd_mul(we, arc_w(p, pl.perm[i], (j >> i) & 1));
-      P.lane_w_ex[x][j] = we;
+      P.lane_w_ex[x][j] = to_lane_mass(we);
     }
   }
   for (int j = 0; j < 64; ++j) P.binom[j] = binom_u64(pl.ell + pl.L, j);

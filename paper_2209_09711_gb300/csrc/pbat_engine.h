@@ -9,6 +9,7 @@
 #include <math.h>
 
 #include "pbat.h"
+#include "pbat_internal.h"
 #include "pbat_num.cuh"
 
 namespace pbat {
@@ -117,6 +118,22 @@ inline u128 to_fixed127(dd v) {
   else if (v.lo < 0)
     r -= scaled_round_u(-v.lo, 127);
   return u128{(uint64_t)r, (uint64_t)(r >> 64)};
+}
+
+// v in [0, 1] as the frontier kernel's lane masses hold it
+inline LaneMass to_lane_mass(dd v) {
+  LaneMass out{{0, 0}, 0, 0};
+  if (!(v.hi > 0.0)) return out;
+  int k;
+  frexp(v.hi, &k);   // v.hi in [2^(k-1), 2^k)
+  uint128_host r = scaled_round_u(v.hi, 127 - k);
+  if (v.lo > 0)
+    r += scaled_round_u(v.lo, 127 - k);
+  else if (v.lo < 0)
+    r -= scaled_round_u(-v.lo, 127 - k);
+  out.m = u128{(uint64_t)r, (uint64_t)(r >> 64)};
+  out.e = -k;
+  return out;
 }
 
 // Products of arc reliabilities in the kernels' integer floating point:

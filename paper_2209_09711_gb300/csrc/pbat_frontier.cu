@@ -89,28 +89,101 @@ __device__ __noinline__ bool state_connected(const FrontierParams& P, unsigned l
   return (reach & tb) != 0;
 }
 
-__device__ __forceinline__ dd warp_sum(dd v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    dd w;
-    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    v = dd_add(v, w);
-  }
-  return v;
+// Exact sum over the warp (every lane gets it) of values below 2^127: five
+// chunks of at most 26 bits, whose 32-lane sums fit 31 bits, one hardware
+// warp reduction each (the top chunk holds 23 bits).
+__device__ __forceinline__ u128 warp_sum_u128(u128 v) {
+  const uint32_t c0 = (uint32_t)(v.lo & 0x3ffffffull), c1 = (uint32_t)((v.lo >> 26) & 0x3ffffffull);
+  const uint32_t c2 = (uint32_t)(((v.lo >> 52) | (v.hi << 12)) & 0x3ffffffull);
+  const uint32_t c3 = (uint32_t)((v.hi >> 14) & 0x3ffffffull), c4 = (uint32_t)(v.hi >> 40);
+  const unsigned long long s0 = __reduce_add_sync(0xffffffffu, c0), s1 = __reduce_add_sync(0xffffffffu, c1);
+  const unsigned long long s2 = __reduce_add_sync(0xffffffffu, c2), s3 = __reduce_add_sync(0xffffffffu, c3);
+  const unsigned long long s4 = __reduce_add_sync(0xffffffffu, c4);
+  u128 r = u128{s0, 0ull};
+  u128_add_to(r, u128{s1 << 26, 0ull});
+  u128_add_to(r, u128{s2 << 52, s2 >> 12});
+  u128_add_to(r, u128{0ull, s3 << 14});
+  u128_add_to(r, u128{0ull, s4 << 40});
+  return r;
+}
+// (a * b) >> 128, at most two units low (the product of the low halves dropped)
+__device__ __forceinline__ u128 mulhi128(u128 a, u128 b) {
+  u128 r = u128{a.hi * b.hi, __umul64hi(a.hi, b.hi)};
+  u128_add_to(r, u128{__umul64hi(a.hi, b.lo), 0ull});
+  u128_add_to(r, u128{__umul64hi(a.lo, b.hi), 0ull});
+  return r;
+}
+// Sum over the warp of T (scale 2^127) times a lane's mass: the sum is
+// returned times 2^*e.  Each product keeps 126 significant bits and is shifted
+// to the largest one's exponent, so the sum is good to 2^-115 of itself
+// however small the masses are.
+__device__ __forceinline__ u128 warp_sum_scaled(u128 T, const LaneMass& w, int* e) {
+  const int lz = T.hi ? __clzll((long long)T.hi) : 64 + __clzll((long long)T.lo);
+  const bool some = (T.lo | T.hi) && (w.m.lo | w.m.hi);
+  u128 n = T;   // T << lz
+  if (lz >= 64) n = u128{0ull, n.lo};
+  const int r = lz & 63;
+  if (r) n = u128{n.lo << r, (n.hi << r) | (n.lo >> (64 - r))};
+  const u128 p = mulhi128(n, w.m);   // below 2^127: the product is p 2^(-126 - E)
+  const int E = some ? lz + w.e : 1 << 20;
+  const int lo = (int)__reduce_min_sync(0xffffffffu, (unsigned)(E + (1 << 16))) - (1 << 16);
+  const int sh = some ? E - lo + 5 : 128;
+  u128 q = u128_zero();
+  if (sh < 64) q = u128{(p.lo >> sh) | (p.hi << (64 - sh)), p.hi >> sh};
+  else if (sh < 128) q = u128{p.hi >> (sh - 64), 0ull};
+  *e = lo >= (1 << 19) ? 0 : 5 - 126 - lo;
+  return warp_sum_u128(q);
 }
 
-// Mass of the prefix arcs of `prefix`, optionally without prefix arc `skip`.
-__device__ __forceinline__ dd prefix_mass(const FrontierParams& P, unsigned long long prefix,
-                                          int skip) {
-  const int base = P.lane_bits + P.walk_bits;
-  dd w = dd{1.0, 0.0};
-  for (int j = 0; j < P.prefix_bits; ++j) {
-    if (j == skip) continue;
-    const int k = base + j;
-    w = ((prefix >> j) & 1ull) ? dd_mul_d(w, P.p[k]) : dd_mul(w, P.q[k]);
+__device__ __forceinline__ dd shfl_dd(dd v, int src) {
+  return dd{__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src)};
+}
+// Mass of the prefix arcs of `prefix` (every lane), and with EX for lane j's
+// prefix arc (j < 32, and j + 32) the mass without it: products over the
+// lanes, one factor each, by shuffles -- FP64 runs at 1/64 of the FP32 rate
+// here, and a product over the arcs in turn, in every lane, was half of an
+// item's FP64 work.
+template <bool EX>
+__device__ __forceinline__ dd prefix_mass(const FrontierParams& P, unsigned long long prefix, int lane, dd* ex) {
+  const int base = P.lane_bits + P.walk_bits, d = P.prefix_bits;
+  dd whole = dd{1.0, 0.0}, ex0 = whole, ex1 = whole;
+  for (int j0 = 0; j0 < d; j0 += 32) {
+    const int j = j0 + lane;
+    dd f = dd{1.0, 0.0};
+    if (j < d) f = ((prefix >> j) & 1ull) ? dd{P.p[base + j], 0.0} : P.q[base + j];
+    // up: the product of this lane's factor and those below it (with EX);
+    // all: of every lane's factor
+    dd all = f;
+    if (EX) {
+      dd up = f, dn = f;
+      for (int o = 1; o < 32 && o < d - j0; o <<= 1) {
+        const dd a = dd{__shfl_up_sync(0xffffffffu, up.hi, o), __shfl_up_sync(0xffffffffu, up.lo, o)};
+        const dd b = dd{__shfl_down_sync(0xffffffffu, dn.hi, o), __shfl_down_sync(0xffffffffu, dn.lo, o)};
+        if (lane >= o) up = dd_mul(up, a);
+        if (lane + o < 32) dn = dd_mul(dn, b);
+      }
+      all = shfl_dd(dn, 0);
+      dd below = dd{__shfl_up_sync(0xffffffffu, up.hi, 1), __shfl_up_sync(0xffffffffu, up.lo, 1)};
+      dd above = dd{__shfl_down_sync(0xffffffffu, dn.hi, 1), __shfl_down_sync(0xffffffffu, dn.lo, 1)};
+      if (lane == 0) below = dd{1.0, 0.0};
+      if (lane == 31) above = dd{1.0, 0.0};
+      const dd x = dd_mul(below, above);
+      if (j0 == 0) ex0 = x; else ex1 = dd_mul(x, whole);
+    } else {
+      for (int o = 16; o > 0; o >>= 1) {
+        if (o >= d - j0 && o > 1) continue;   // only ones up there
+        all = dd_mul(all, dd{__shfl_xor_sync(0xffffffffu, all.hi, o), __shfl_xor_sync(0xffffffffu, all.lo, o)});
+      }
+      all = shfl_dd(all, 0);
+    }
+    if (j0 > 0 && EX) ex0 = dd_mul(ex0, all);
+    whole = dd_mul(whole, all);
   }
-  return w;
+  if (EX) {
+    ex[0] = ex0;
+    ex[1] = ex1;
+  }
+  return whole;
 }
 
 __device__ __forceinline__ void acc_signed(dd& slot, dd v, bool plus) {
@@ -141,7 +214,11 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
   dd* s_wacc = reinterpret_cast<dd*>(smem + off);
   off = align16(off + (size_t)nwarps * (1 + m) * sizeof(dd));
   unsigned long long* s_nbins = reinterpret_cast<unsigned long long*>(smem + off);
+  if (GRAD) off = align16(off + (size_t)(m + 1) * sizeof(unsigned long long));
+  LaneMass* s_lwx = reinterpret_cast<LaneMass*>(smem + off);   // lane masses without each lane arc
 
+  if (GRAD)
+    for (int i = tid; i < ell * 32; i += nthr) s_lwx[i] = P.lane_w_ex[i >> 5][i & 31];
   for (int i = tid; i < nW; i += nthr) s_wmid[i] = wmid_g[i];
   for (int i = tid; i < nwarps * (1 + m); i += nthr) s_wacc[i] = dd{0.0, 0.0};
   for (int i = tid; i <= m; i += nthr) s_nbins[i] = 0ull;
@@ -154,6 +231,7 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
   dd* wacc = s_wacc + (size_t)warp * (1 + m);
   const M sbit = (M)1 << P.source, tbit = (M)1 << P.sink;
   const bool lane_on = lane < (1 << ell);
+  const LaneMass lw = P.lane_w[lane];   // zero past the lane patterns
   const int top = ell + L;  // first prefix arc
   const unsigned long long t_start = globaltimer_ns();
   unsigned long long n_walk = 0, n_full = 0, n_dead = 0;
@@ -171,7 +249,6 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
     if (task >= P.n_tasks) break;
     const unsigned long long prefix = P.task_lo + task;
     const unsigned long long xpre = top < 64 ? (prefix << top) : 0ull;
-    const dd wpre = prefix_mass(P, prefix, -1);
     const int pc_pre = __popcll((long long)prefix);
 
     if (P.prune) {
@@ -182,10 +259,12 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
       if (state_connected(P, xpre)) {
         ++n_full;
         for (int j = lane; j <= top; j += 32) atomicAdd(&s_nbins[pc_pre + j], P.binom[j]);
+        dd ex[2];
+        const dd wpre = prefix_mass<GRAD>(P, prefix, lane, ex);
         if (lane == 0) wacc[0] = dd_add(wacc[0], wpre);
         if (GRAD) {
           for (int j = lane; j < P.prefix_bits; j += 32)
-            acc_signed(wacc[1 + top + j], prefix_mass(P, prefix, j), (prefix >> j) & 1ull);
+            acc_signed(wacc[1 + top + j], j < 32 ? ex[0] : ex[1], (prefix >> j) & 1ull);
         }
         continue;
       }
@@ -255,28 +334,53 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
         if (cnt) atomicAdd(&s_nbins[base + c], (unsigned long long)cnt);
       }
     }
-    const dd t = dd_ldexp(u128_to_dd(T), -127);
-    const dd lw = lane_on ? P.lane_w[lane] : dd{0.0, 0.0};
-    const dd wsum = warp_sum(dd_mul(lw, t));
+    // Sums over the lanes are integers to a common exponent (warp_sum_scaled);
+    // every arc's ends on the lane that owns it, which scales all of them at
+    // once in double-double.  (In double-double throughout, 14 warp sums of
+    // five rounds were 1,300 FP64 instructions per item, and FP64 issues at
+    // 1/64 of the FP32 rate: 23 arcs, 16,384 items, 1.30 ms; 0.29 so.)
+    int eS;
+    const u128 S = warp_sum_scaled(T, lw, &eS);
+    dd ex[2];
+    const dd wpre = prefix_mass<GRAD>(P, prefix, lane, ex);
+    const dd wsum = dd_ldexp(u128_to_dd(S), eS);
     if (lane == 0) wacc[0] = dd_add(wacc[0], dd_mul(wpre, wsum));
     if (GRAD) {
+      // of internal arc `lane`: a walk arc's masses with it working (X) and
+      // failed (Y), a lane arc's pair differences (X)
+      u128 X = u128_zero(), Y = u128_zero();
+      int eX = 0, eY = 0;
       for (int b = 0; b < L; ++b) {
-        const int k = ell + b;
         const u128 A = seg_acc[b * nthr];
-        const dd a = dd_ldexp(u128_to_dd(A), -127);
-        const dd z = dd_ldexp(u128_to_dd(u128_sub(T, A)), -127);
-        dd y = dd_sub(dd_mul(a, P.inv_p[k]), dd_mul(z, P.inv_q[k]));
-        y = warp_sum(dd_mul(lw, y));
-        if (lane == (k & 31)) wacc[1 + k] = dd_add(wacc[1 + k], dd_mul(wpre, y));
+        int ea, ez;
+        const u128 sa = warp_sum_scaled(A, lw, &ea), sz = warp_sum_scaled(u128_sub(T, A), lw, &ez);
+        if (lane == ell + b) {
+          X = sa;
+          Y = sz;
+          eX = ea;
+          eY = ez;
+        }
       }
       for (int i = 0; i < ell; ++i) {
-        dd y = lane_on ? dd_mul(P.lane_w_ex[i][lane], t) : dd{0.0, 0.0};
-        if (!((lane >> i) & 1)) y = dd_neg(y);
-        y = warp_sum(y);
-        if (lane == i) wacc[1 + i] = dd_add(wacc[1 + i], dd_mul(wpre, y));
+        // the pair's lane with the arc working holds the larger T (exactly)
+        const u128 o = u128{__shfl_xor_sync(0xffffffffu, T.lo, 1 << i), __shfl_xor_sync(0xffffffffu, T.hi, 1 << i)};
+        const u128 df = (lane >> i) & 1 ? u128_sub(T, o) : u128_zero();
+        int eg;
+        const u128 sg = warp_sum_scaled(df, s_lwx[i * 32 + lane], &eg);
+        if (lane == i) {
+          X = sg;
+          eX = eg;
+        }
+      }
+      if (lane < top) {
+        dd y = dd_ldexp(u128_to_dd(X), eX);
+        if (lane >= ell)
+          y = dd_sub(dd_mul(y, P.inv_p[lane]), dd_mul(dd_ldexp(u128_to_dd(Y), eY), P.inv_q[lane]));
+        wacc[1 + lane] = dd_add(wacc[1 + lane], dd_mul(wpre, y));
       }
       for (int j = lane; j < P.prefix_bits; j += 32)
-        acc_signed(wacc[1 + top + j], dd_mul(prefix_mass(P, prefix, j), wsum), (prefix >> j) & 1ull);
+        acc_signed(wacc[1 + top + j], dd_mul(j < 32 ? ex[0] : ex[1], wsum), (prefix >> j) & 1ull);
+      __syncwarp();
     }
   }
 
@@ -335,7 +439,8 @@ size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide) 
   off = align16(off + (size_t)(L + 1) * nthr * sizeof(uint32_t));
   if (grad) off = align16(off + (size_t)2 * L * nthr * sizeof(u128));
   off = align16(off + (size_t)(nthr / 32) * (1 + m) * sizeof(dd));
-  off += (size_t)(m + 1) * sizeof(unsigned long long);
+  off = align16(off + (size_t)(m + 1) * sizeof(unsigned long long));
+  if (grad) off += (size_t)kMaxLaneBits * 32 * sizeof(LaneMass);
   return off;
 }
 

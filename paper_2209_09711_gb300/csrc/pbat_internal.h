@@ -14,6 +14,12 @@ constexpr int kMaxLaneBits = 5;       // one warp lane per low-arc pattern
 constexpr int kMaxWalkBitsR = 12;     // Gray-walk arcs per thread, R only
 constexpr int kMaxWalkBitsGrad = 10;  // with the gradient segment sums
 
+// A lane pattern's mass as m * 2^(-127 - e), m in [2^126, 2^127] or zero.
+struct LaneMass {
+  u128 m;
+  int e, pad;
+};
+
 // Everything a frontier-kernel launch needs that is not a table, passed by
 // value (it lives in the kernel parameter bank, read with uniform indices).
 // Arc index k below is the INTERNAL arc position: bit k of a state word.
@@ -33,8 +39,8 @@ struct FrontierParams {
   double p[64];                 // p_k
   dd q[64];                     // 1 - p_k, exact
   dd inv_p[64], inv_q[64];      // 1/p_k, 1/(1-p_k) for walk arcs (gradient)
-  dd lane_w[32];                // mass of each lane pattern: prod over lane arcs
-  dd lane_w_ex[kMaxLaneBits][32];  // the same without lane arc i's factor
+  LaneMass lane_w[32];          // mass of each lane pattern: prod over lane arcs
+  LaneMass lane_w_ex[kMaxLaneBits][32];  // the same without lane arc i's factor
   unsigned long long binom[64];    // C(lane_bits + walk_bits, j)
 };
 

@@ -117,7 +117,10 @@ static int run_noalloc(const GraphIn& g, const double* p, const pbat_options* op
   } else if (o.prefix_bits >= 0) {
     L = std::max(0, std::min(kNoAllocMaxWalkBits, m - ell - std::max(o.prefix_bits, r)));
   } else {
-    L = std::max(0, std::min(kNoAllocMaxWalkBits, free_bits - std::max(0, 14 - r)));
+    int space = free_bits;   // the split of make_plan
+    if (r > 0)
+      for (uint64_t x = o.range_hi - o.range_lo; x > 1; x >>= 1) ++space;
+    L = std::max(0, std::min(std::min(kNoAllocMaxWalkBits, free_bits), (space - 6) / 2));
   }
   const int d = m - ell - L;
   if (d >= 64) return fail(PBAT_ERANGE, "prefix of %d bits is too deep", d);
@@ -191,12 +194,11 @@ static int run_noalloc(const GraphIn& g, const double* p, const pbat_options* op
   }
   for (int j = 0; j < 32; ++j) {
     if (j >= (1 << ell)) {
-      P.lane_w[j] = dd{0.0, 0.0};
       continue;
     }
     dd w = dd_make(1.0);
     for (int i = 0; i < ell; ++i) w = dd_mul(w, arc_w(p, m - 1 - i, (j >> i) & 1));
-    P.lane_w[j] = w;
+    P.lane_w[j] = to_lane_mass(w);
   }
   for (int j = 0; j < 64; ++j) P.binom[j] = binom_u64(ell + L, j);
   u128* wmid = g_na_wmid;
