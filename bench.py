@@ -81,17 +81,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "37df6b1409896506": (52898657 / 2**40, 5649664, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "144a0eff24a2e04d": (51080047 / 2**40, 5656576, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "bcf1dfc496e39eac": (20601601 / 2**40, 563712, "profiles/bs_kernel_undirected24x40.md"),
+    "d6bbbd149d626633": (18785233 / 2**40, 563968, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "94e55a18f9749108": (1135726 / 2**34, 263680, "profiles/bs_kernel_grad_directed20x34.md"),
+    "a1a59d928cebfbe7": (1143022 / 2**34, 258560, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "2f33d29f92400dc4": (879618 / 2**34, 108032, "profiles/bs_kernel_directed20x34.md"),
+    "2070c50cd69727f3": (879618 / 2**34, 107520, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "a1c4af05cd02c1c0": (1715071 / 2**27, 478208, "profiles/bs_kernel_grad_grid3x6.md"),
+    "2f12e7d3edd30eb2": (1648898 / 2**27, 475904, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "037ffde57a2a4231": (1129100 / 2**27, 156672, "profiles/bs_kernel_grid3x6.md"),
+    "e9d8951d579e3800": (1067596 / 2**27, 156672, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

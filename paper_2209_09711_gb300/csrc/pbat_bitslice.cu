@@ -547,8 +547,7 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     }
   }
   const int L_in = std::min(bp.L, walk_unroll_bits(bp)), L_out = bp.L - L_in;
-  // the walking launch of a merged run: each warp's counts below the prefix
-  const size_t rel_bytes = bp.merge ? (size_t)(bl.nthr / 32) * (top + 1) * 8 : 0;
+  const size_t rel_bytes = (size_t)(bl.nthr / 32) * (top + 1) * 4;   // each warp's item counts
   if (!grad) {
     bl.wmid.resize((size_t)1 << bp.L);
     std::vector<dd> wt((size_t)1 << bp.L);
@@ -945,12 +944,12 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   std::string kern = E.grad ? head_g : head_r;
   kern +=
       "  u64* nkw = s_nk + (threadIdx.x >> 5) * 65;\n"
-      "  u64* rel = s_nk + (BSB_NTHR / 32) * 65 + (threadIdx.x >> 5) * 33;   // merged: counts below the prefix\n"
+      "  u32* rel = (u32*)(s_nk + (BSB_NTHR / 32) * 65) + (threadIdx.x >> 5) * 33;   // merged: counts below the prefix\n"
       "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n"
       "  int cur = -1;   // network whose counts nkw holds\n"
       "  const u64 t0 = bs_timer();\n";
   kern += E.merged ?
-      "  rel[lane] = 0ull;\n"
+      "  rel[lane] = 0u;\n"
       "  if (*(volatile u32*)status) return;\n"
       "  const u64 n_cls = *A.n_classes, n_warps = (u64)gridDim.x * (BSB_NTHR / 32);\n"
       "  u64 next = (u64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;\n"

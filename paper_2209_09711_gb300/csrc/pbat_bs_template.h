@@ -484,17 +484,32 @@ __device__ __forceinline__ int bs_prune(const u32* a) {
   return (ext & 2u) ? 2 : 0;
 }
 
-__device__ __forceinline__ void bs_flush_bins(u64* bins, u64* s_nbins, int base) {
+// An item's counts by popcount below the prefix, into the warp's own rel
+// (BS_TOP + 1, cleared here): 32-bit additions in shared memory, which are
+// one instruction, where 64-bit ones are a compare-and-swap loop that the
+// threads of one popcount run in turn (an item has at most C(20, 10) =
+// 184,756 states of one popcount).  Then the warp adds them to the block's
+// (bs_item_counts) or a class's (bs_class_counts), a lane per popcount.
+__device__ __forceinline__ void bs_flush_bins(u64* bins, u32* rel, int lane) {
   constexpr int sh[6] = BS_NK_SHIFTS, wd[6] = BS_NK_WIDTHS;
+  if (lane <= BS_TOP) rel[lane] = 0u;
+  __syncwarp();
+  if (lane < (1 << BS_TB)) {
+    u32* mine = rel + __popc(lane);
 #pragma unroll 1
-  for (int r = 0; r <= BS_L; ++r) {
-    const u64 n = bins[r * BS_NTHR];
+    for (int r = 0; r <= BS_L; ++r) {
+      const u64 n = bins[r * BS_NTHR];
 #pragma unroll
-    for (int cl = 0; cl < 6; ++cl) {
-      const u64 c = (n >> sh[cl]) & ((1ull << wd[cl]) - 1ull);
-      if (c) atomicAdd(&s_nbins[base + r + cl], c);
+      for (int cl = 0; cl < 6; ++cl) {
+        const u32 c = (u32)(n >> sh[cl]) & ((1u << wd[cl]) - 1u);
+        if (c) atomicAdd(&mine[r + cl], c);
+      }
     }
   }
+  __syncwarp();
+}
+__device__ __forceinline__ void bs_item_counts(const u32* rel, u64* s_nbins, int pc_pre, int lane) {
+  if (lane <= BS_TOP && rel[lane]) atomicAdd(&s_nbins[pc_pre + lane], (u64)rel[lane]);
 }
 
 // End of a block: entry i combines the warps' floating accumulators
@@ -623,9 +638,8 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
 }
 // N_k of a class: its representative's states by popcount below the prefix
 // (rel, BS_TOP + 1 of them) for every popcount that its prefixes have.
-__device__ __forceinline__ void bs_class_counts(const BsWork& W, u64 slot, int lane, const u64* rel, u64* s_nbins) {
-  __syncwarp();
-  const u64 r = lane <= BS_TOP ? rel[lane] : 0ull;
+__device__ __forceinline__ void bs_class_counts(const BsWork& W, u64 slot, int lane, const u32* rel, u64* s_nbins) {
+  const u64 r = lane <= BS_TOP ? rel[lane] : 0u;
   for (int p0 = 0; p0 <= BS_D; p0 += 32) {
     const u32 h = p0 + lane <= BS_D ? W.hist[(size_t)slot * BS_HIST + p0 + lane] : 0u;
     u32 some = __ballot_sync(0xffffffffu, h != 0u);
@@ -671,7 +685,6 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
   __syncthreads();
   u64* bins = s_bins + tid;
   const bool thr_on = lane < (1 << BS_TB);
-  const int pc_thr = __popc(lane & ((1 << BS_TB) - 1));
   const u64 thw = thr_on ? P.thw[lane] : 0ull;
   const u64 t_start = bs_timer();
   u64 n_walk = 0, n_full = 0, n_dead = 0;
@@ -679,9 +692,7 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
   u32 a[BS_M];
   bs_init_arcs(a, lane);
   constexpr int phase = PHASE;
-#if BS_MERGE
-  u64* rel = s_nbins + BS_M + 1 + warp * (BS_TOP + 1);   // phase 2: counts below the prefix
-#endif
+  u32* rel = (u32*)(s_nbins + BS_M + 1) + warp * (BS_TOP + 1);   // an item's counts below the prefix
 
   for (;;) {
     u64 task = 0;
@@ -699,8 +710,6 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
       if (task == ~0ull) break;
 #if BS_MERGE
       prefix = W.rep[task];
-      for (int i = lane; i <= BS_TOP; i += 32) rel[i] = 0ull;
-      __syncwarp();
 #endif
     } else {
       if (task >= P.n_tasks) break;
@@ -768,14 +777,14 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
     // prefix mass (a class: its items' summed mass), once per item
     const u128 S = warp_sum_u128(mul64x128_shr64(thw, T.lo, T.hi));
     mx w;
+    bs_flush_bins(bins, rel, lane);
     if constexpr (phase == 2) {
 #if BS_MERGE
-      if (thr_on) bs_flush_bins(bins, rel, pc_thr);
       bs_class_counts(W, task, lane, rel, s_nbins);
       w = bs_class_mass(W.cmass + 2 * task, P.mass_exp);
 #endif
     } else {
-      if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
+      bs_item_counts(rel, s_nbins, pc_pre, lane);
       w = bs_prefix_mass(P, ptab, prefix);
     }
     facc_add(accR, mx_prod(w, S), w.e);
@@ -906,7 +915,6 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u128* A = s_A + tid;
   const BsTr tr = bs_tr_init(lane);
   const bool thr_on = lane < (1 << BS_TB);
-  const int pc_thr = __popc(lane & ((1 << BS_TB) - 1));
   const u64 thw = thr_on ? P.thw[lane] : 0ull;
   const u64 t_start = bs_timer();
   u64 n_walk = 0, n_full = 0, n_dead = 0;
@@ -923,9 +931,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u32 a[BS_M];
   bs_init_arcs(a, lane);
   constexpr int phase = PHASE;
-#if BS_MERGE
-  u64* rel = s_nbins + BS_M + 1 + warp * (BS_TOP + 1);   // phase 2: counts below the prefix
-#endif
+  u32* rel = (u32*)(s_nbins + BS_M + 1) + warp * (BS_TOP + 1);   // an item's counts below the prefix
 
   for (;;) {
     u64 task = 0;
@@ -943,8 +949,6 @@ __device__ __forceinline__ void bs_kernel_grad_body(
       if (task == ~0ull) break;
 #if BS_MERGE
       prefix = W.rep[task];
-      for (int i = lane; i <= BS_TOP; i += 32) rel[i] = 0ull;
-      __syncwarp();
 #endif
     } else {
       if (task >= P.n_tasks) break;
@@ -1048,13 +1052,13 @@ __device__ __forceinline__ void bs_kernel_grad_body(
 #pragma unroll
       for (int b = 0; b < BS_OUT; ++b)
         if ((gout >> b) & 1u) { u128 ab = A[b * BS_NTHR]; u128_add(ab, T.lo, T.hi); A[b * BS_NTHR] = ab; }
+      bs_flush_bins(bins, rel, lane);
       if constexpr (phase == 2) {
 #if BS_MERGE
-        if (thr_on) bs_flush_bins(bins, rel, pc_thr);
         bs_class_counts(W, task, lane, rel, s_nbins);
 #endif
       } else {
-        if (thr_on) bs_flush_bins(bins, s_nbins, pc_pre + pc_thr);
+        bs_item_counts(rel, s_nbins, pc_pre, lane);
       }
       // ---- exact warp sums; slot k of `red` holds internal arc k's value
       S = warp_sum_u128(mul64x128_shr64(thw, T.lo, T.hi));
@@ -1419,16 +1423,16 @@ __device__ __forceinline__ void bsb_flush_counts(const BGraph* __restrict__ B, u
 
 // N_k of a class: its item's counts below the prefix (rel) for every popcount
 // that its prefixes have, into the warp's counts nkw.
-__device__ __forceinline__ void bsb_class_counts(const BMerge& A, u64 cls, int d, int top, int lane, u64* rel, u64* nkw) {
+__device__ __forceinline__ void bsb_class_counts(const BMerge& A, u64 cls, int d, int top, int lane, u32* rel, u64* nkw) {
   __syncwarp();
-  const u64 r = lane <= top ? rel[lane] : 0ull;
+  const u64 r = lane <= top ? rel[lane] : 0u;
   const u32* h = A.hist + cls * A.hist_stride;
   for (int q = 0; q <= d; ++q) {
     const u32 n = h[q];
     if (n && r) nkw[q + lane] += n * r;
     __syncwarp();
   }
-  if (lane <= top) rel[lane] = 0ull;
+  if (lane <= top) rel[lane] = 0u;
   __syncwarp();
 }
 // this thread's counts c11 by walk popcount + lane class: an item's to nkw, a
@@ -1437,7 +1441,7 @@ __device__ __forceinline__ void bsb_class_counts(const BMerge& A, u64 cls, int d
 #define BSB_COUNTS()                                                          \
   if (thr_on) {                                                               \
     _Pragma("unroll") for (int i = 0; i < 11; ++i)                            \
-      if (c11[i]) atomicAdd(&rel[__popc(lane) + i], c11[i]);                  \
+      if (c11[i]) atomicAdd(&rel[__popc(lane) + i], (u32)c11[i]);             \
   }                                                                           \
   bsb_class_counts(A, cls, Bp->d, top, lane, rel, nkw)
 #else
@@ -1455,7 +1459,7 @@ __device__ __forceinline__ void bsb_finish(const BGraph* __restrict__ Bp, int st
                                            int Kp, const u64* __restrict__ lt, const u64* __restrict__ nt,
                                            const u64* __restrict__ wm, const mx* __restrict__ pt,
                                            const u64* __restrict__ thw, u64* limbs, u64* nkw, u64* bins,
-                                           const u32* cw, const BMerge& A, u64 cls, u64* rel) {
+                                           const u32* cw, const BMerge& A, u64 cls, u32* rel) {
   constexpr int nsh[6] = BS_NK_SHIFTS, nwd[6] = BS_NK_WIDTHS;
   const int gidx = Bp->gidx, L = Bp->L, tb = Bp->tb, nlev = Bp->nlev, top = Bp->top;
   const int lt_off = Bp->lt_off, nt_off = Bp->nt_off, wm_off = Bp->wm_off, pt_off = Bp->pt_off;
@@ -1614,7 +1618,7 @@ __device__ __forceinline__ void bsb_finish_grad(
     const u64* __restrict__ lt, const u64* __restrict__ nt, const u64* __restrict__ wm2,
     const mx* __restrict__ pt, const u64* __restrict__ thw, const u64* __restrict__ tt,
     const u64* __restrict__ lwex, const u64* __restrict__ thwex, const mx* __restrict__ ptex,
-    u64* limbs, u64* nkw, u64* bins, const u32* cw, u32* ctw, const BsTr& tr, const BMerge& A, u64 cls, u64* rel) {
+    u64* limbs, u64* nkw, u64* bins, const u32* cw, u32* ctw, const BsTr& tr, const BMerge& A, u64 cls, u32* rel) {
   constexpr int nsh[6] = BS_NK_SHIFTS, nwd[6] = BS_NK_WIDTHS;
   const int L = Bp->L, tb = Bp->tb, ell = Bp->ell, top = Bp->top, m = Bp->m, nlev = Bp->nlev;
   const int pt_size = Bp->pt_size, d = Bp->d;
