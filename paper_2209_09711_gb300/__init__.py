@@ -11,6 +11,7 @@ import ctypes
 import os
 import threading
 from dataclasses import dataclass
+from itertools import chain
 from typing import List, Optional, Sequence
 
 import numpy as np
@@ -210,6 +211,40 @@ def reliability_net(net, p=None, grad: bool = False, opts: Optional[Options] = N
                        net.directed, grad, opts, stream)
 
 
+# numpy layout of Graph: a batch's descriptors are filled column by column
+_GRAPH_DTYPE = np.dtype({"names": [f[0] for f in Graph._fields_],
+                         "formats": [np.intp if f[0] in ("tail", "head") else np.int32 for f in Graph._fields_],
+                         "offsets": [getattr(Graph, f[0]).offset for f in Graph._fields_],
+                         "itemsize": ctypes.sizeof(Graph)})
+
+
+def _graphs(nets):
+    """The networks as an array of Graph, what it points into, and their sizes."""
+    lists = [x if isinstance(x, (list, tuple)) else np.asarray(x, dtype=np.int32)
+             for net in nets for x in (net.tail, net.head)]
+    sizes = [len(x) for x in lists]
+    ends = np.fromiter(chain.from_iterable(lists), np.int32, sum(sizes))
+    table = np.zeros(len(nets), dtype=_GRAPH_DTYPE)
+    at = ends.ctypes.data + 4 * np.cumsum([0] + sizes[:-1])
+    table["tail"], table["head"] = at[0::2], at[1::2]
+    ms = sizes[0::2]
+    table["n_arcs"] = ms
+    table["n_nodes"] = [net.n for net in nets]
+    table["directed"] = [int(net.directed) for net in nets]
+    table["source"] = [net.source for net in nets]
+    table["sink"] = [net.sink for net in nets]
+    return table.ctypes.data_as(ctypes.POINTER(Graph)), (table, ends), ms
+
+
+def _rows(pv, K):
+    """The K reliability vectors of one network, end to end."""
+    if (isinstance(pv, (list, tuple)) and len(pv) == K and all(isinstance(row, (list, tuple)) for row in pv)
+            and len({len(row) for row in pv}) == 1):
+        # lists of floats: half the time of np.asarray
+        return np.fromiter(chain.from_iterable(pv), np.float64, K * len(pv[0]))
+    return np.asarray(pv, dtype=np.float64).reshape(K, -1).ravel()
+
+
 def reliability_batched(nets, pvecs, grad: bool = False, want_nk: bool = True,
                         opts: Optional[Options] = None, stream: int = 0):
     """Batched call: nets is a list of networks, pvecs[g] a list of n_pvec
@@ -217,17 +252,10 @@ def reliability_batched(nets, pvecs, grad: bool = False, want_nk: bool = True,
     lib = load()
     G = len(nets)
     K = len(pvecs[0])
-    keep = []
-    graphs = (Graph * G)()
-    for i, net in enumerate(nets):
-        t, tp = _i32(net.tail)
-        h, hp = _i32(net.head)
-        keep += [t, h]
-        graphs[i] = Graph(net.n, len(t), tp, hp, int(net.directed), net.source, net.sink)
-    flat = np.concatenate([np.asarray(pv, dtype=np.float64).reshape(K, -1).ravel() for pv in pvecs])
+    graphs, keep, ms = _graphs(nets)
+    flat = np.concatenate([_rows(pv, K) for pv in pvecs])
     pv, pp = _f64(flat)
     R = np.zeros(G * K, dtype=np.float64)
-    ms = [len(net.tail) for net in nets]
     Nk = np.zeros(sum(m + 1 for m in ms), dtype=np.uint64) if want_nk else None
     gr = np.zeros(flat.shape[0], dtype=np.float64) if grad else None
     o = opts if opts is not None else options()
@@ -243,7 +271,7 @@ def reliability_batched(nets, pvecs, grad: bool = False, want_nk: bool = True,
     goff = 0
     for m in ms:
         if want_nk:
-            Nks.append([int(v) for v in Nk[off:off + m + 1]])
+            Nks.append(Nk[off:off + m + 1].tolist())
         off += m + 1
         if grad:
             grads.append(gr[goff:goff + K * m].reshape(K, m))

@@ -463,6 +463,8 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
     if ((rc = bs_make_plan(g, o, bl.nthr, bl.plan, grad ? p : nullptr))) return rc;
     const std::string src = bs_source(g, bl.plan, bl.nthr);
     if ((rc = jit_compile(src, dev, grad ? "bs_kernel_grad" : "bs_kernel", &bl.jit))) return rc;
+    bl.plan.gen.clear();   // compiled: a cached plan is copied on every call
+    bl.plan.gen_sig.clear();
     std::lock_guard<std::mutex> lk(g_bsplan_mu);
     g_bsplan[key] = BsCached{bl.plan, bl.jit, 0, 0};
   }
@@ -503,15 +505,18 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
   P.nlev = (bp.d + max_bits - 1) / max_bits;
   P.ex_shift = max_bits;
   bl.ptab.clear();
-  bl.ptab_ex.assign(grad ? (size_t)bp.d << max_bits : 0, MxHost{0, 0, 0});
-  for (int l = 0, sh = 0; l < P.nlev; ++l) {
+  // (a merged run takes the levels above its blocks, merge_tables; excluded
+  // masses are read only for arcs of pex)
+  const bool excluded_tab = grad && bp.pex && !bp.merge;
+  bl.ptab_ex.assign(excluded_tab ? (size_t)bp.d << max_bits : 0, MxHost{0, 0, 0});
+  for (int l = 0, sh = 0; l < P.nlev && !bp.merge; ++l) {
     const int bits = bp.d / P.nlev + (l < bp.d % P.nlev ? 1 : 0);
     P.lev_bits[l] = bits;
     P.lev_off[l] = (int)bl.ptab.size();
     std::vector<dd> tab((size_t)1 << bits);
     product_table(p, bp.perm.data() + top + sh, bits, tab.data());
     for (int v = 0; v < (1 << bits); ++v) bl.ptab.push_back(to_mx(tab[v]));
-    if (grad)
+    if (excluded_tab)
       for (int jj = 0; jj < bits; ++jj) {
         // the level's product without arc jj: a table over the other arcs,
         // indexed by v with bit jj removed
@@ -815,6 +820,8 @@ struct BsBatch {
   // signature walked once.  per_item: every item by itself instead
   bool per_item = false, merged = false;
   int nsig_max = 0, grid1 = 0, grid2 = 0, grid3 = 0;
+  bool static_ready = false;
+  size_t o_perm = 0, o_poff = 0, o_p = 0, n_p = 0;
   size_t smem1 = 0, o_nib = 0, o_mid = 0, o_fold = 0, key_bytes = 0;
   Scratch* mscr = nullptr;
   BMergeHost M{};
@@ -1130,6 +1137,10 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   E.o_nib = off; off = a256(off + 16 * 128 * gk);
   E.o_mid = off; off = a256(off + 16 * 32 * gk);
   E.o_fold = off; off = a256(off + (E.grad ? 8 * kBsbFold * gk : 0));
+  for (int i = 0; i < G; ++i) E.n_p += (size_t)K * graphs[i].n_arcs;
+  E.o_perm = off; off = a256(off + (E.merged ? 64 * (size_t)G : 0));
+  E.o_poff = off; off = a256(off + (E.merged ? 8 * (size_t)G : 0));
+  E.o_p = off; off = a256(off + (E.merged ? 8 * E.n_p : 0));
   E.o_upload_end = off;
   E.o_limbs = off; off = a256(off + 8 * E.n_out);
   E.o_nk = off; off = a256(off + 8 * (size_t)E.nk_total);
@@ -1192,6 +1203,21 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   return PBAT_OK;
 }
 
+// Packed N counts by lane class of every byte of a word (the same for every
+// p-vector).
+static void bsb_count_table(int ell, unsigned long long* nt) {
+  for (int v = 0; v < 1024; ++v) {
+    const int by = v >> 8, val = v & 255;
+    unsigned long long n = 0;
+    for (int k = 0; k < 8; ++k) {
+      const int j = 8 * by + k;
+      if (!((val >> k) & 1) || j >= (1 << ell)) continue;
+      n += 1ull << kNkShift[__builtin_popcount((unsigned)j)];
+    }
+    nt[v] = n;
+  }
+}
+
 static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
   char* h = (char*)E.scr->hmem;
   unsigned long long* lt = (unsigned long long*)(h + E.o_lt);
@@ -1219,16 +1245,7 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
     const int i = b.gidx, m = b.m;
     const BsPlan& bp = E.plans[i];
     const int top = bp.ell + bp.tb + bp.L;
-    for (int v = 0; v < 1024; ++v) {  // packed N counts by lane class (same for every p-vector)
-      const int by = v >> 8, val = v & 255;
-      unsigned long long n = 0;
-      for (int k = 0; k < 8; ++k) {
-        const int j = 8 * by + k;
-        if (!((val >> k) & 1) || j >= (1 << bp.ell)) continue;
-        n += 1ull << kNkShift[__builtin_popcount((unsigned)j)];
-      }
-      nt[b.nt_off + v] = n;
-    }
+    bsb_count_table(bp.ell, nt + b.nt_off);
     for (int k = K; k < Kp; ++k) {  // padding p-vector: zero mass
       for (int v = 0; v < 1024; ++v) lt[b.lt_off + (size_t)v * Kp + k] = 0;
       for (int gi = 0; gi < (1 << bp.L); ++gi) wm[b.wm_off + (size_t)gi * Kp + k] = 0;
@@ -1246,14 +1263,13 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
       product_table(pv, bp.perm.data() + bp.ell, bp.tb, tw);
       for (int t = 0; t < 32; ++t)
         th[b.thw_off + (size_t)t * Kp + k] = t < (1 << bp.tb) ? fixed_u64(tw[t], 63) : 0ull;
-      const int blk = E.merged ? bp.low + bp.mid : 0;
       MxHost* ptk = pt + b.pt_off + (size_t)k * b.pt_size;
       if (b.nlev == 0) ptk[0] = to_mx(dd_make(1.0));
       for (int l = 0, sh = 0; l < b.nlev; ++l) {
         dd tab[1 << 7];
-        product_table(pv, bp.perm.data() + top + blk + sh, b.lev_bits[l], tab);
+        product_table(pv, bp.perm.data() + top + sh, b.lev_bits[l], tab);
         for (int v = 0; v < (1 << b.lev_bits[l]); ++v) ptk[b.lev_off[l] + v] = to_mx(tab[v]);
-        if (E.grad && !E.merged)
+        if (E.grad)
           for (int jj = 0; jj < b.lev_bits[l]; ++jj) {
             if (!((bp.pex >> (top + sh + jj)) & 1ull)) continue;   // divided by p on the host
             // the level's product without prefix arc sh + jj, indexed by the
@@ -1268,13 +1284,6 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
               row[v] = to_mx(ex[(v & ((1 << jj) - 1)) | ((v >> (jj + 1)) << jj)]);
           }
         sh += b.lev_bits[l];
-      }
-      if (E.merged) {
-        const size_t gk = (size_t)r * K + k;
-        block_tables(pv, bp.perm.data() + top, bp.low, bp.mid, (unsigned long long*)(h + E.o_nib) + 256 * gk,
-                     (unsigned long long*)(h + E.o_mid) + 64 * gk);
-        if (E.grad)
-          fold_tables(pv, bp.perm.data() + top, bp.low, bp.mid, *(BsFoldParamsHost*)((unsigned long long*)(h + E.o_fold) + kBsbFold * gk));
       }
       if (E.grad) {
         // 128-bit walk masses, thread-pattern byte tables, and the lane and
@@ -1315,6 +1324,173 @@ static void bsb_tables(BsBatch& E, const pbat_graph* graphs, const double* p) {
   for (int t = 0; t < nthreads; ++t)
     pool.emplace_back(build_range, E.G * t / nthreads, E.G * (t + 1) / nthreads);
   for (auto& th_ : pool) th_.join();
+}
+
+// The tables of a merged batch, built on the device: one block per (network,
+// p-vector) reads the network's reliabilities and writes every table that
+// bsb_tables builds on the host for the other modules, from pattern masses in
+// double-double and exact subset sums.  (Built on 16 host threads and copied,
+// they were 1.5 of the 3.0 ms of a 64 x 16 call, GB300.)  A few thousand FP64
+// operations a block; the writes are one 8-byte word per row of p-vectors.
+struct BsbBuild {
+  const BGraphHost* graphs;
+  const unsigned char* perm;         // [launch order][64]: internal position -> input arc
+  const unsigned long long* p_off;   // launch order: first reliability of the network
+  const double* p;
+  unsigned long long *lt, *wm, *thw, *wm2, *tt, *lwex, *thwex, *nib, *mid, *fold;
+  MxHost* pt;
+  int K, Kp, grad;
+};
+__device__ inline uint128_host d_fixed126(dd v) {
+  uint128_host r = scaled_round_u(v.hi, 126);
+  if (v.lo > 0) r += scaled_round_u(v.lo, 126);
+  else if (v.lo < 0) r -= scaled_round_u(-v.lo, 126);
+  return r;
+}
+__global__ void __launch_bounds__(128) bsb_build_kernel(const BsbBuild A) {
+  __shared__ double s_p[64];
+  __shared__ dd s_q[64];
+  __shared__ uint128_host s_lane[32], s_thr[32], s_low[32];
+  const int r = blockIdx.x / A.K, k = blockIdx.x - r * A.K, tid = threadIdx.x, Kp = A.Kp;
+  const BGraphHost& b = A.graphs[r];
+  const int ell = b.ell, tb = b.tb, L = b.L, top = b.top, blk = b.low + b.mid;
+  if (tid < b.m) {
+    const double x = A.p[A.p_off[r] + (size_t)k * b.m + A.perm[64 * r + tid]];
+    s_p[tid] = x;
+    s_q[tid] = dd_one_minus(x);
+  }
+  __syncthreads();
+  // mass of pattern v of the n arcs from internal position a on, without the
+  // x-th of them (x < 0: all; v has a bit for each arc that is left)
+  auto mass = [&](int a, int n, int v, int x) {
+    dd w = dd{1.0, 0.0};
+    for (int i = 0; i < n; ++i) {
+      if (i == x) continue;
+      w = dd_mul(w, v & 1 ? dd{s_p[a + i], 0.0} : s_q[a + i]);
+      v >>= 1;
+    }
+    return w;
+  };
+  const size_t gk = (size_t)r * A.K + k;
+  const int j = tid & 31;
+  if (tid < 32) {
+    s_lane[j] = j < (1 << ell) ? d_fixed126(mass(0, ell, j, -1)) : 0;
+  } else if (tid < 64) {
+    const dd w = mass(ell, tb, j, -1);
+    const bool on = j < (1 << tb);
+    s_thr[j] = on ? d_fixed126(w) : 0;
+    A.thw[b.thw_off + (size_t)j * Kp + k] = on ? fixed_u64(w, 63) : 0ull;
+  } else if (tid < 96) {
+    u128 v = u128{0, 0};
+    if (j < (1 << b.low)) v = to_fixed127(mass(top, b.low, j, -1));
+    s_low[j] = ((uint128_host)v.hi << 64) | v.lo;
+  } else {
+    u128 v = u128{0, 0};
+    const dd w = mass(top + b.low, b.mid, j, -1);
+    const bool on = j < (1 << b.mid);
+    if (on) v = to_fixed127(w);
+    A.mid[2 * (32 * gk + j)] = v.lo;
+    A.mid[2 * (32 * gk + j) + 1] = v.hi;
+    if (A.grad) A.fold[kBsbFold * gk + 72 + j] = on ? fixed_u64(w, 63) : 0ull;
+  }
+  for (int g = tid; g < (1 << L); g += 128) {
+    const dd w = mass(ell + tb, L, g, -1);
+    if (A.grad) {
+      const u128 v = to_fixed127(w);
+      A.wm2[b.wm2_off + ((size_t)g * Kp + k) * 2] = v.lo;
+      A.wm2[b.wm2_off + ((size_t)g * Kp + k) * 2 + 1] = v.hi;
+    } else {
+      A.wm[b.wm_off + (size_t)g * Kp + k] = fixed_u64(w, 63);
+    }
+  }
+  for (int l = 0, sh = 0; l < b.nlev; sh += b.lev_bits[l], ++l)
+    for (int v = tid; v < (1 << b.lev_bits[l]); v += 128)
+      A.pt[b.pt_off + (size_t)k * b.pt_size + b.lev_off[l] + v] = to_mx(mass(top + blk + sh, b.lev_bits[l], v, -1));
+  __syncthreads();
+  const uint128_host half = (uint128_host)1 << 63;
+  for (int e = tid; e < 1024; e += 128) {
+    uint128_host sl = 0, st = 0;
+    for (int i = 0; i < 8; ++i)
+      if ((e >> i) & 1) {
+        sl += s_lane[8 * (e >> 8) + i];
+        st += s_thr[8 * (e >> 8) + i];
+      }
+    A.lt[b.lt_off + (size_t)e * Kp + k] = (unsigned long long)((sl + half) >> 64);
+    if (A.grad) A.tt[b.tt_off + (size_t)e * Kp + k] = (unsigned long long)((st + half) >> 64);
+  }
+  for (int e = tid; e < 128; e += 128) {
+    uint128_host s = 0;
+    for (int i = 0; i < 4; ++i)
+      if ((e >> i) & 1) s += s_low[4 * (e >> 4) + i];
+    A.nib[2 * (128 * gk + e)] = (unsigned long long)s;
+    A.nib[2 * (128 * gk + e) + 1] = (unsigned long long)(s >> 64);
+  }
+  if (!A.grad) return;
+  // lane and thread pattern masses without each of their arcs
+  for (int e = tid; e < 320; e += 128) {
+    const int part = e >= 160, x = (e % 160) >> 5, n = part ? tb : ell, a = part ? ell : 0;
+    if (x >= n || j >= (1 << n)) continue;
+    const int v = (j & ((1 << x) - 1)) | ((j >> (x + 1)) << x);
+    (part ? A.thwex + b.thwex_off : A.lwex + b.lwex_off)[((size_t)(x * 32 + j)) * Kp + k] = fixed_u64(mass(a, n, v, x), 63);
+  }
+  // the fold's arcs and masses (laid out as BsFoldParams)
+  unsigned long long* F = A.fold + kBsbFold * gk;
+  if (tid < 10) {
+    const int part = tid / 5, i = tid % 5, n = part ? b.mid : b.low;
+    F[tid] = i < n ? fixed_u64(dd{s_p[top + (part ? b.low : 0) + i], 0.0}, 63) : 0ull;
+  }
+  if (tid < 62) {
+    const int part = tid >= 31, e = tid % 31, n = part ? b.mid : b.low, a = top + (part ? b.low : 0);
+    const int i = e < 16 ? 0 : e < 24 ? 1 : e < 28 ? 2 : e < 30 ? 3 : 4;   // masses of the arcs above arc i
+    const int v = e - (i == 0 ? 0 : i == 1 ? 16 : i == 2 ? 24 : i == 3 ? 28 : 30), above = n - i - 1 > 0 ? n - i - 1 : 0;
+    F[10 + tid] = v < (1 << above) ? fixed_u64(mass(a + i + 1, above, v, -1), 63) : 0ull;
+  }
+}
+
+// Puts this call's tables on the device: built on the host and copied, or for
+// merged batches built there from the reliabilities alone.
+static int bsb_upload(BsBatch& E, const pbat_graph* graphs, const double* p, cudaStream_t st) {
+  char* d = (char*)E.scr->dmem;
+  char* h = (char*)E.scr->hmem;
+  auto copy = [&](size_t at, size_t bytes) { return cudaMemcpyAsync(d + at, h + at, bytes, cudaMemcpyHostToDevice, st); };
+  cudaError_t e;
+  if (!E.merged) {
+    bsb_tables(E, graphs, p);
+    e = copy(0, E.o_upload_end);
+    return e == cudaSuccess ? PBAT_OK : fail(PBAT_ECUDA, "upload failed: %s", cudaGetErrorString(e));
+  }
+  if (!E.static_ready) {
+    // what does not depend on the reliabilities, once: descriptors, packed
+    // counts, arc orders, and zeros where the tables have no entry
+    unsigned long long* nt = (unsigned long long*)(h + E.o_nt);
+    unsigned char* perm = (unsigned char*)(h + E.o_perm);
+    unsigned long long* off = (unsigned long long*)(h + E.o_poff);
+    std::vector<unsigned long long> first(E.G, 0);
+    for (int i = 1; i < E.G; ++i) first[i] = first[i - 1] + (unsigned long long)E.K * graphs[i - 1].n_arcs;
+    for (int r = 0; r < E.G; ++r) {
+      const BGraphHost& b = E.bg[r];
+      bsb_count_table(E.plans[b.gidx].ell, nt + b.nt_off);
+      for (int k = 0; k < b.m; ++k) perm[64 * r + k] = (unsigned char)E.plans[b.gidx].perm[k];
+      off[r] = first[b.gidx];
+    }
+    e = cudaMemsetAsync(d, 0, E.o_upload_end, st);
+    if (e == cudaSuccess) e = copy(E.o_graphs, sizeof(BGraphHost) * E.G);
+    if (e == cudaSuccess) e = copy(E.o_nt, 8 * E.n_nt);
+    if (e == cudaSuccess) e = copy(E.o_perm, E.o_p - E.o_perm);
+    if (e != cudaSuccess) return fail(PBAT_ECUDA, "upload failed: %s", cudaGetErrorString(e));
+    E.static_ready = true;
+  }
+  memcpy(h + E.o_p, p, 8 * E.n_p);
+  if ((e = copy(E.o_p, 8 * E.n_p)) != cudaSuccess)
+    return fail(PBAT_ECUDA, "upload failed: %s", cudaGetErrorString(e));
+  auto at = [&](size_t o) { return (unsigned long long*)(d + o); };
+  BsbBuild A{(const BGraphHost*)(d + E.o_graphs), (const unsigned char*)(d + E.o_perm), at(E.o_poff),
+             (const double*)(d + E.o_p), at(E.o_lt), at(E.o_wm), at(E.o_thw), at(E.o_wm2), at(E.o_tt), at(E.o_lwex),
+             at(E.o_thwex), at(E.o_nib), at(E.o_mid), at(E.o_fold), (MxHost*)(d + E.o_pt), E.K, E.Kp, E.grad ? 1 : 0};
+  bsb_build_kernel<<<E.G * E.K, 128, 0, st>>>(A);
+  if ((e = cudaGetLastError()) != cudaSuccess)
+    return fail(PBAT_ECUDA, "batched tables: %s", cudaGetErrorString(e));
+  return PBAT_OK;
 }
 
 static int bsb_enqueue(BsBatch& E, cudaStream_t st, unsigned long long budget_ns) {
@@ -1418,9 +1594,7 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
       clear_error();
       return;
     }
-    bsb_tables(T, graphs, p);
-    bool ok = cudaMemcpyAsync(T.scr->dmem, T.scr->hmem, T.o_upload_end, cudaMemcpyHostToDevice, st) ==
-              cudaSuccess;
+    bool ok = bsb_upload(T, graphs, p, st) == PBAT_OK;
     // (merged runs are short: the second of two counts)
     for (int rep = 0; ok && rep < (T.merged ? 2 : 1); ++rep)
       ok = cudaEventRecord(a, st) == cudaSuccess && bsb_enqueue(T, st, 0) == PBAT_OK &&
@@ -1520,11 +1694,9 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
     return code;
   };
   const unsigned long long budget = o.time_budget_s > 0 ? (unsigned long long)(o.time_budget_s * 1e9) : 0ull;
-  bsb_tables(*E, graphs, p);
   char* d = (char*)E->scr->dmem;
   char* h = (char*)E->scr->hmem;
-  if (cudaMemcpyAsync(d, h, E->o_upload_end, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return done(fail(PBAT_ECUDA, "upload failed: %s", cudaGetErrorString(cudaGetLastError())));
+  if (const int rc = bsb_upload(*E, graphs, p, st)) return done(rc);
   if (!E->exec) {
     cudaStream_t cs;
     if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess)
