@@ -81,17 +81,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "144a0eff24a2e04d": (51080047 / 2**40, 5656576, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "3326fae9e2a0d23b": (51111310 / 2**40, 7172352, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "d6bbbd149d626633": (18785233 / 2**40, 563968, "profiles/bs_kernel_undirected24x40.md"),
+    "8562a0ea3d516ec7": (18741463 / 2**40, 565248, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "a1a59d928cebfbe7": (1143022 / 2**34, 258560, "profiles/bs_kernel_grad_directed20x34.md"),
+    "da30d7dd42d47de3": (1352709 / 2**34, 247296, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "2070c50cd69727f3": (879618 / 2**34, 107520, "profiles/bs_kernel_directed20x34.md"),
+    "01218a14c42ae95a": (879618 / 2**34, 107520, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "2f12e7d3edd30eb2": (1648898 / 2**27, 475904, "profiles/bs_kernel_grad_grid3x6.md"),
+    "1a30d000589d9776": (1718510 / 2**27, 462848, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "e9d8951d579e3800": (1067596 / 2**27, 156672, "profiles/bs_kernel_grid3x6.md"),
+    "4e6b8981adebc73f": (1057835 / 2**27, 157184, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

@@ -246,7 +246,7 @@ static unsigned long long full_counts(int ell) {
 // or the per-word connectivity program is small (registers to spare); on
 // GB300: 3x6 grid (L = 5) 70.5 -> 66.7 us, 34-arc directed network (12
 // operations per word) 1.54 -> 1.43 ms, but the 40-arc network (260
-// operations per word) 144.7 -> 157.6 ms, so that one keeps global slots.
+// operations per word) 144.7 -> 157.6 ms, so that one keeps them in slots.
 static bool acc_in_registers(const BsPlan& bp) { return bp.L <= 6 || bp.ops_var <= 128; }
 
 // Walk arcs unrolled per step (2^in_bits words with compile-time walk words):
@@ -598,7 +598,8 @@ int bs_prepare(const GraphIn& g, const double* p, bool grad, const pbat_options&
       bl.Q.inv_q[k] = dd_recip_dd(dd_one_minus(pk));
     }
     bl.smem = (size_t)(4 * 256 * 2 + 2 * (1 << bp.L) + 4 * 256 + (bp.L + 1) * bl.nthr) * 8 +
-              (size_t)std::max(L_out, 1) * bl.nthr * 16 + (size_t)(m + 1) * 8 + rel_bytes;
+              (size_t)std::max(L_out, 1) * bl.nthr * 16 + (size_t)(m + 1) * 8 + rel_bytes +
+              (size_t)(bl.nthr / 32) * (1 + 2 * (bp.merge ? top : m)) * 24 + 8;   // per-warp sums
   }
   if (bl.smem > (size_t)dev.smem_optin)
     return fail(PBAT_ERANGE, "bit-sliced kernel needs %zu B of shared memory", bl.smem);

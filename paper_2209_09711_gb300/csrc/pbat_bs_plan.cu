@@ -563,15 +563,16 @@ static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPl
     bp.L = std::max(0, std::min(lmax, m - bp.ell - bp.tb - std::max(o.prefix_bits, r)));
   } else if (!one_by_one && o.prune && o.launches != 1) {
     // Items merged by signature cost little each, so there are many and short
-    // ones; their number is bounded by the table of item slots (2^24).  GB300,
-    // R / fused in us, source/sink-near prefixes: 27 arcs L = 3: 42 / 54 (5: 37
-    // / 61, 8: 60 / 100); 31 arcs L = 5: 68 / 109 (3: 97 / 134, 8: 107 / 176);
-    // 34 arcs directed L = 6: 60 / 82 (4: 56 / 78, 8: 78 / 118); 40 arcs,
-    // prune-aware, L = 6: 140 / 269 (8: 158 / 285, 10: 970 fused).  Below
-    // 24 arcs one launch that walks every item left is faster (23 arcs, L = 2:
-    // 29 / 36 against 29 / 54), with about 2^11 items.
-    bp.L = free_bits < 14 ? std::max(0, free_bits - 11)
-                          : std::min(lmax, std::max(free_bits - 24, std::min(6, (free_bits - 6) / 3)));
+    // ones, up to 2^24 of them; fewer states are walked in one launch, about
+    // 2^10 items.  GB300, source/sink-near prefixes, R / fused in us: 40 arcs
+    // (prune-aware) L = 6 115 / 264 (8: 124 / 274, 10: 970 fused); 34 arcs
+    // directed L = 6 36 / 62 (3: 38 / 71, 8: 40 / 77); 31 arcs L = 5 33 / 74
+    // (3: 62 / 102, 8: 54 / 137); 27 arcs merged L = 3 19 / 46, in one launch L =
+    // 5 19 / 37; 26 arcs merged L = 3 15 / 37, one launch L = 6 13 / 24 (4: 18 /
+    // 38); 23 arcs one launch L = 3 10 / 20 (1: 16 / 33, 6: 15 / 31).
+    const bool merge = free_bits >= (p_for_grad ? 18 : 17);
+    bp.L = merge ? std::min(lmax, std::max(free_bits - 24, std::min(6, (free_bits - 6) / 3)))
+                 : std::max(0, std::min(6, free_bits - 10));
   } else {
     // every item walked by itself: about 2^11 of them, measured best on GB300
     // for 27..40 arcs (larger items amortise the per-item epilogue, which is

@@ -37,9 +37,8 @@ bool bs_walk_ok(const double* p, int a);
 constexpr int kMaxSigBits = 63;
 // Items from which a run merges them by default (pbat_options.launches 0):
 // below, one launch is a few microseconds long and further ones cost more
-// than they save (GB300, R / fused: 2^11 items of 23 arcs 29 / 36 us in one
-// launch, 29 / 54 merged; 2^14 items of 27 arcs 58 / 90 against 42 / 54).
-constexpr unsigned long long kMergeItems = 1ull << 12;
+// than they save (see bs_plan_roles).
+constexpr unsigned long long kMergeItems = 1ull << 13;
 constexpr unsigned long long kMaxMergeItems = 1ull << 24;   // a slot number for each in the fused kernel
 constexpr unsigned long long kMaxMergeBlocks = 1ull << 14;
 

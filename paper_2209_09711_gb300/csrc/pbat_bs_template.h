@@ -180,7 +180,6 @@ struct facc;
 struct BsWork {
   u64* counter; u32* status; u64* stats;
   dd* part_acc; u64* part_n; dd* out_acc; u64* out_n;
-  facc* wacc;       // fused kernel: per warp, R and the two sums of every arc
   u64* out_limbs;   // [n_acc][8]: 256-bit fixed point at scale 2^250, 32 bits per limb
   // merged runs: the classes in the order they were met (their slots), how
   // many there are, and the walking launch's ticket
@@ -397,39 +396,50 @@ __device__ __forceinline__ u128 bs_fold2(u128 V0, u128 V1, u64 p, u64 w, u128& G
   u128_add(V0, x.lo, x.hi);
   return V0;
 }
-// A fold block's 32 items per lane: V over them by the five low arcs (see
-// bs_kernel_grad_p3).  V(j): item j's conditional reliability (scale 2^124);
-// p, w: the low arcs' p and the masses above each, as in BsFoldParams.
+// A fold block's 32 items per lane, folded over the five low arcs (see
+// bs_kernel_grad_p3): the items 8 q to 8 q + 7 over the lowest three, then
+// the four results over the other two.  item(j): item j's conditional
+// reliability (scale 2^124); p, w: the low arcs' p and the masses above each,
+// as in BsFoldParams; G: the sums per arc.
+template <class Item>
+__device__ __forceinline__ u128 bs_fold_group(const u64* p, const u64* w, int q, u128 (&G)[5], Item item) {
+  u128 V[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) V[i] = item(8 * q + i);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[0], w[4 * q + i], G[0]);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[1], w[16 + 2 * q + i], G[1]);
+  return bs_fold2(V[0], V[1], p[2], w[24 + q], G[2]);
+}
+__device__ __forceinline__ u128 bs_fold_groups(const u64* p, const u64* w, u128 (&V)[4], u128 (&G)[5]) {
+#pragma unroll
+  for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[3], w[28 + i], G[3]);
+  return bs_fold2(V[0], V[1], p[4], w[30], G[4]);
+}
 template <class Item>
 __device__ __forceinline__ u128 bs_fold_low(const u64* p, const u64* w, u128 (&G)[5], Item item) {
-  u128 top[4];   // folded over the lowest three arcs
+  u128 V[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    u128 V[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) V[i] = item(8 * q + i);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[0], w[4 * q + i], G[0]);
-#pragma unroll
-    for (int i = 0; i < 2; ++i) V[i] = bs_fold2(V[2 * i], V[2 * i + 1], p[1], w[16 + 2 * q + i], G[1]);
-    top[q] = bs_fold2(V[0], V[1], p[2], w[24 + q], G[2]);
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i) top[i] = bs_fold2(top[2 * i], top[2 * i + 1], p[3], w[28 + i], G[3]);
-  return bs_fold2(top[0], top[1], p[4], w[30], G[4]);
+  for (int q = 0; q < 4; ++q) V[q] = bs_fold_group(p, w, q, G, item);
+  return bs_fold_groups(p, w, V, G);
+}
+// Sum over the lanes of a low arc's G by the mid patterns' masses (2^124).
+__device__ __forceinline__ u128 bs_fold_sum(u128 G, u64 m_mid) {
+  const u128 g = warp_sum_u128(mul64x128_shr64(m_mid, G.lo, G.hi));   // 2^122
+  return u128{g.lo << 2, (g.hi << 2) | (g.lo >> 62)};
 }
 // The mid arcs over the lanes, and the block's sums per arc (scale 2^124):
-// lane l ends with low arc l's, lane `low` + l with mid arc l's, in X; every
-// lane with the block's V.
+// lane l ends with low arc l's (from FIRST on), lane `low` + l with mid arc
+// l's, in X; every lane with the block's V.
+template <int FIRST>
 __device__ __forceinline__ u128 bs_fold_mid(u128 V, const u128 (&G)[5], int low, int mid, const u64* p, const u64* w,
                                             u64 m_mid, int lane, u128& X) {
   X = u128{0ull, 0ull};
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
+  for (int i = FIRST; i < 5; ++i) {
     if (i >= low) break;
-    u128 g = mul64x128_shr64(m_mid, G[i].lo, G[i].hi);   // 2^122
-    g = warp_sum_u128(g);
-    g = u128{g.lo << 2, (g.hi << 2) | (g.lo >> 62)};
+    const u128 g = bs_fold_sum(G[i], m_mid);
     if (lane == i) X = g;
   }
 #pragma unroll
@@ -517,13 +527,16 @@ __device__ __forceinline__ void bs_item_counts(const u32* rel, u64* s_nbins, int
 // with integer atomics (every sum is non-negative, and integer addition is
 // exact, so the order of the blocks does not matter); then the block's N_k
 // counts.  The host converts the result once.
-__device__ __forceinline__ void bs_write_out(const BsWork& W, const facc* s_acc, int stride, int n_acc,
-                                             const u64* s_nbins, int nthr) {
+__device__ __forceinline__ void bs_add_out(u64* limbs, const facc* s_acc, int stride, int n_acc, int nthr) {
   for (int i = threadIdx.x; i < n_acc; i += nthr) {
     facc t = s_acc[i];
     for (int w = 1; w < nthr / 32; ++w) facc_add(t, s_acc[w * stride + i].v, s_acc[w * stride + i].E);
-    bs_limb_add(W.out_limbs + 8 * i, t.v, 127 - t.E);   // v * 2^(-123 - E) at scale 2^250
+    bs_limb_add(limbs + 8 * i, t.v, 127 - t.E);   // v * 2^(-123 - E) at scale 2^250
   }
+}
+__device__ __forceinline__ void bs_write_out(const BsWork& W, const facc* s_acc, int stride, int n_acc,
+                                             const u64* s_nbins, int nthr) {
+  bs_add_out(W.out_limbs, s_acc, stride, n_acc, nthr);
   for (int i = threadIdx.x; i <= BS_M; i += nthr)
     if (s_nbins[i]) atomicAdd(&W.out_n[i], s_nbins[i]);
 }
@@ -893,8 +906,10 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u64* s_bins = s_tt + 4 * 256;                             // [L + 1][NTHR]
   u128* s_A = (u128*)(s_bins + (BS_L + 1) * BS_NTHR);       // [BS_OUT][NTHR]
   u64* s_nbins = (u64*)(s_A + (BS_OUT > 0 ? BS_OUT : 1) * BS_NTHR);
-  // per warp, in global scratch: R, then A_k and B_k of every arc k
-  facc* g_acc = W.wacc + (size_t)blockIdx.x * (BS_NTHR / 32) * (1 + 2 * BS_M);
+  // per warp: R, then A_k and B_k of every arc k (of a class: of the arcs
+  // below the prefix)
+  constexpr int n_acc = PHASE == 2 ? 1 + 2 * BS_TOP : 1 + 2 * BS_M, m_acc = PHASE == 2 ? BS_TOP : BS_M;
+  facc* s_acc = (facc*)(((size_t)(s_nbins + BS_M + 1) + (BS_NTHR / 32) * (BS_TOP + 1) * 4 + 7) & ~(size_t)7);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < 4 * 256; i += BS_NTHR) s_lt[i] = ((const ulonglong2*)lane_tab)[i];
   for (int i = tid; i < 4 * 256; i += BS_NTHR) s_tt[i] = thr_tab[i];
@@ -908,9 +923,9 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     next = (u64)warp * gridDim.x + blockIdx.x;
     if (blockIdx.x >= n_list || *W.status) return;   // no class, or a run that the host discards
   }
-  for (int i = tid; i < (BS_NTHR / 32) * (1 + 2 * BS_M); i += BS_NTHR) g_acc[i] = facc{u128{0ull, 0ull}, 0, 0};
+  for (int i = tid; i < (BS_NTHR / 32) * n_acc; i += BS_NTHR) s_acc[i] = facc{u128{0ull, 0ull}, 0, 0};
   __syncthreads();
-  facc* acc = g_acc + warp * (1 + 2 * BS_M);
+  facc* acc = s_acc + warp * n_acc;
   u64* bins = s_bins + tid;
   u128* A = s_A + tid;
   const BsTr tr = bs_tr_init(lane);
@@ -920,9 +935,8 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   u64 n_walk = 0, n_full = 0, n_dead = 0;
 #if BS_ACC_REG
   // short items: this lane's accumulators -- R and the two sums of internal
-  // arcs `lane` and `lane + 32` -- in registers, so an item costs no global
-  // round trip.  Long items keep them all in the global slots: registers are
-  // worth more to the walk.
+  // arcs `lane` and `lane + 32` -- in registers.  Long items keep them all in
+  // the shared slots: registers are worth more to the walk.
   facc accR = facc{u128{0ull, 0ull}, 0, 0}, accA = accR, accB = accR;
 #if BS_M > 32
   facc accA2 = accR, accB2 = accR;
@@ -1096,7 +1110,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     BS_FACTORS();
     facc accR, accA, accB;
     if (lane == 0) accR = acc[0];
-    if (lane < BS_M) {
+    if (lane < m_acc) {
       accA = acc[1 + 2 * lane];
       accB = acc[2 + 2 * lane];
     }
@@ -1124,7 +1138,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     }
 #if !BS_ACC_REG
     if (lane == 0) acc[0] = accR;
-    if (lane < BS_M) {
+    if (lane < m_acc) {
       acc[1 + 2 * lane] = accA;
       acc[2 + 2 * lane] = accB;
     }
@@ -1154,12 +1168,12 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   }
 #if BS_ACC_REG
   if (lane == 0) acc[0] = accR;
-  if (lane < BS_M) {
+  if (lane < m_acc) {
     acc[1 + 2 * lane] = accA;
     acc[2 + 2 * lane] = accB;
   }
 #if BS_M > 32
-  if (lane + 32 < BS_M) {
+  if (PHASE == 0 && lane + 32 < BS_M) {
     acc[1 + 2 * (lane + 32)] = accA2;
     acc[2 + 2 * (lane + 32)] = accB2;
   }
@@ -1169,7 +1183,7 @@ __device__ __forceinline__ void bs_kernel_grad_body(
   // gradient (A - B for prefix arcs, A / p - B / (1 - p) for walk arcs, A
   // for lane and thread arcs)
   __syncthreads();
-  bs_write_out(W, g_acc, 1 + 2 * BS_M, 1 + 2 * BS_M, s_nbins, BS_NTHR);
+  bs_write_out(W, s_acc, n_acc, n_acc, s_nbins, BS_NTHR);
 }
 
 #define KERNEL_G_ARGS const __grid_constant__ BsParams P, const __grid_constant__ BsGradParams Q, \
@@ -1206,63 +1220,89 @@ struct BsFoldParams {
   u64 wmid[31];         // of the mid arcs above mid arc b
   u64 mid[32];          // mid pattern masses (2^63)
 };
-extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR) bs_kernel_grad_p3(
-    const __grid_constant__ BsParams P, const __grid_constant__ BsFoldParams Q, const mx* __restrict__ ptab,
-    const BsWork W) {
-  __shared__ u64 s_none[BS_M + 1];   // no counts here
+// Few blocks (TEAM): the four warps of a thread block share one, a group of
+// eight items per lane each, and the first folds their results -- a block is
+// otherwise 15 us of one warp's latency.
+template <bool TEAM>
+__device__ __forceinline__ void bs_fold_body(const BsParams& P, const BsFoldParams& Q, const mx* __restrict__ ptab,
+                                             const BsWork& W) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  facc* g_acc = W.wacc + (size_t)blockIdx.x * (BS_MERGE_NTHR / 32) * (1 + 2 * BS_M);
-  facc* acc = g_acc + warp * (1 + 2 * BS_M);
-  for (int i = tid; i <= BS_M; i += BS_MERGE_NTHR) s_none[i] = 0ull;
-  bs_wait_previous();
-  // (the walking launch uses the same slots, so not before it has ended)
-  for (int i = lane; i < 1 + 2 * BS_M; i += 32) acc[i] = facc{u128{0ull, 0ull}, 0, 0};
+  // A_k and B_k of every prefix arc, per warp
+  __shared__ facc s_acc[BS_MERGE_NTHR / 32][2 * BS_D];
+  __shared__ u128 s_V[TEAM ? 4 : 1][32], s_X[TEAM ? 4 : 1][4];   // a team's folded groups and sums
+  facc* acc = s_acc[warp];
+  for (int i = lane; i < 2 * BS_D; i += 32) acc[i] = facc{u128{0ull, 0ull}, 0, 0};
   __syncwarp();
+  bs_wait_previous();
   // an earlier launch ran out of time or slots: its masks and slots are not
   // all written, and the host discards the run
   if (*(volatile u32*)W.status) return;
   const u64 nblk = P.n_tasks >> BS_BLK, blk0 = P.task_lo >> BS_BLK;
-  const u64 nwarps = (u64)gridDim.x * (BS_MERGE_NTHR / 32);
+  const u64 step = TEAM ? (u64)gridDim.x : (u64)gridDim.x * (BS_MERGE_NTHR / 32);
   const u64 m_mid = Q.mid[lane];
   const u64 t_start = bs_timer();
   // lane l < BS_BLK: arc l of the block; lanes: arcs `lane` and `lane + 32` above it
   facc accP = facc{u128{0ull, 0ull}, 0, 0}, accA = accP, accB = accP, accA2 = accP, accB2 = accP;
-  for (u64 b = (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; b < nblk; b += nwarps) {
-    if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
+  for (u64 b = TEAM ? blockIdx.x : (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; b < nblk; b += step) {
+    if (!TEAM && P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
     const u64 hi = blk0 + b;
     const uint2 m = W.cmask[b * 32 + lane];
-    if (!__any_sync(0xffffffffu, m.x | m.y)) continue;
+    if (!__any_sync(0xffffffffu, m.x | m.y)) continue;   // (the same in every warp of a team)
     const u32* cls = W.cls + (b << BS_BLK) + lane;
-    u128 G[5];
+    u128 G[5], X, V;
 #pragma unroll
     for (int i = 0; i < 5; ++i) G[i] = u128{0ull, 0ull};
-    u128 V = bs_fold_low(Q.p, Q.wlow, G, [&](int j) {
+    auto item = [&](int j) {
       u128 v = u128{0ull, (m.x >> j) & 1u ? 1ull << 60 : 0ull};
       if ((m.y >> j) & 1u) {
         const ulonglong2 s = W.csum[cls[j << BS_MID]];
         v = u128{s.x, s.y};
       }
       return v;
-    });
-    u128 X;   // the block's sums, lane l: arc l's
-    V = bs_fold_mid(V, G, BS_LOW, BS_MID, Q.p + 5, Q.wmid, m_mid, lane, X);
+    };
+    if constexpr (TEAM) {
+      s_V[warp][lane] = bs_fold_group(Q.p, Q.wlow, warp, G, item);
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const u128 g = bs_fold_sum(G[i], m_mid);
+        if (lane == i) s_X[warp][i] = g;
+      }
+      __syncthreads();
+      if (warp == 0) {
+        u128 T[4] = {s_V[0][lane], s_V[1][lane], s_V[2][lane], s_V[3][lane]};
+        V = bs_fold_mid<3>(bs_fold_groups(Q.p, Q.wlow, T, G), G, BS_LOW, BS_MID, Q.p + 5, Q.wmid, m_mid, lane, X);
+        if (lane < 3 && lane < BS_LOW)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) u128_add(X, s_X[q][lane].lo, s_X[q][lane].hi);
+      }
+      __syncthreads();
+      if (warp != 0) continue;
+    } else {
+      V = bs_fold_mid<0>(bs_fold_low(Q.p, Q.wlow, G, item), G, BS_LOW, BS_MID, Q.p + 5, Q.wmid, m_mid, lane, X);
+    }
     const mx w = bs_level_mass(P.nlev_hi, P.hi_bits, P.hi_off, ptab, hi);
     if (lane < BS_BLK) facc_add(accP, mx_prod(w, X), w.e);
     const u128 Sv = mx_prod(w, V);
     if (lane < BS_HI) { if ((hi >> lane) & 1ull) facc_add(accA, Sv, w.e); else facc_add(accB, Sv, w.e); }
     if (lane + 32 < BS_HI) { if ((hi >> (lane + 32)) & 1ull) facc_add(accA2, Sv, w.e); else facc_add(accB2, Sv, w.e); }
   }
-  if (lane < BS_BLK) acc[1 + 2 * (BS_TOP + lane)] = accP;
+  if (lane < BS_BLK) acc[2 * lane] = accP;
   if (lane < BS_HI) {
-    acc[1 + 2 * (BS_TOP + BS_BLK + lane)] = accA;
-    acc[2 + 2 * (BS_TOP + BS_BLK + lane)] = accB;
+    acc[2 * (BS_BLK + lane)] = accA;
+    acc[2 * (BS_BLK + lane) + 1] = accB;
   }
   if (lane + 32 < BS_HI) {
-    acc[1 + 2 * (BS_TOP + BS_BLK + lane + 32)] = accA2;
-    acc[2 + 2 * (BS_TOP + BS_BLK + lane + 32)] = accB2;
+    acc[2 * (BS_BLK + lane + 32)] = accA2;
+    acc[2 * (BS_BLK + lane + 32) + 1] = accB2;
   }
   __syncthreads();
-  bs_write_out(W, g_acc, 1 + 2 * BS_M, 1 + 2 * BS_M, s_none, BS_MERGE_NTHR);
+  bs_add_out(W.out_limbs + 8 * (1 + 2 * BS_TOP), s_acc[0], 2 * BS_D, 2 * BS_D, BS_MERGE_NTHR);
+}
+extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR, 5) bs_kernel_grad_p3(
+    const __grid_constant__ BsParams P, const __grid_constant__ BsFoldParams Q, const mx* __restrict__ ptab,
+    const BsWork W) {
+  if (gridDim.x * (BS_MERGE_NTHR / 32) > P.n_tasks >> BS_BLK) bs_fold_body<true>(P, Q, ptab, W);
+  else bs_fold_body<false>(P, Q, ptab, W);
 }
 #endif
 #endif
@@ -1946,7 +1986,7 @@ extern "C" __global__ void __launch_bounds__(BSB_MNTHR) bs_batch_grad_p3(
       return v;
     });
     u128 X;
-    V = bs_fold_mid(V, Gs, low, mid, f + 5, f + 41, f[72 + lane], lane, X);
+    V = bs_fold_mid<0>(V, Gs, low, mid, f + 5, f + 41, f[72 + lane], lane, X);
     const mx w = bsb_hi_mass(B, pt, k, hi);
     u64* out = limbs + B->out_off + (size_t)k * (1 + 2 * B->m) * BSB_LIMBS;
     if (lane < blk) bsb_limb_add(out + (1 + 2 * (top + lane)) * BSB_LIMBS, mx_prod(w, X), w.e);

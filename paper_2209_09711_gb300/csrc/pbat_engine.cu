@@ -762,7 +762,9 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
     while (J->split_log2 < 5 && (mg.blocks << (J->split_log2 + 1)) <= 8ull * J->dev.sms) ++J->split_log2;
     J->grid1 = fit(1, mg.blocks << J->split_log2, 4);
     J->grid2 = fit(2, std::min(n_items, mg.slots), (int)warps_per_block);
-    J->grid3 = fit(3, mg.blocks, 4);
+    // (a thread block for each item block while they all fit at once, see bs_fold_body)
+    J->grid3 = fit(3, mg.blocks * 4, 4);
+    if ((unsigned long long)J->grid3 < mg.blocks) J->grid3 = fit(3, mg.blocks & ~3ull, 4);
   }
   const int m = g.m;
   // accumulators per block: the frontier kernel and the bit-sliced R kernel
@@ -794,10 +796,6 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   const size_t o_part_acc = off; off = up16(off + part_bytes);
   const size_t o_part_n = off; off = up16(off + (J->bs ? 0 : (size_t)grid * (m + 1) * 8));
   const size_t o_out_acc = off; off = up16(off + (size_t)n_acc * sizeof(dd));
-  // per-warp slots of every block of the largest of the launches' grids
-  const long long warps_max = std::max<long long>(std::max<long long>(grid, J->grid2) * warps_per_block, J->grid3 * 4LL);
-  const size_t wacc_bytes = (J->bs && bs_grad(*J->bs)) ? (size_t)warps_max * (1 + 2 * m) * 24 : 0;
-  const size_t o_wacc = off; off = up16(off + wacc_bytes);
   const size_t o_wmid = off; off = up16(off + wmid.size() * sizeof(u128));
   size_t o_lane = 0, o_thr = 0, o_wmid64 = 0, o_ptab = 0, o_ptabx = 0, o_mtab = 0, o_tab_end = 0;
   if (J->bs) {
@@ -841,7 +839,6 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   J->W.out_acc = (dd*)(d + o_out_acc);
   J->W.out_n = (unsigned long long*)(d + o_out_n);
   J->W.out_limbs = limbs_bytes ? (unsigned long long*)(d + o_out_limbs) : nullptr;
-  J->W.wacc = wacc_bytes ? (void*)(d + o_wacc) : nullptr;
   J->W.list = (unsigned int*)(d + o_list);
   J->W.key = (unsigned long long*)(d + o_key);
   J->W.cmass = (unsigned long long*)(d + o_cmass);

@@ -54,7 +54,6 @@ struct DevWork {
   unsigned long long* part_n;   // [grid][m + 1]
   dd* out_acc;                  // [n_acc]
   unsigned long long* out_n;    // [m + 1]
-  void* wacc;                   // fused bit-sliced kernel: per-warp accumulators (24 B each)
   unsigned long long* out_limbs;  // bit-sliced kernels: [n_acc][8] 256-bit fixed point, scale 2^250
   // merged runs of the bit-sliced kernels (BsWork in the kernel source): the
   // classes' slots, their count and ticket, the class table, and per item
