@@ -389,15 +389,42 @@ static void bs_generate_sig(const GraphIn& g, BsPlan& bp) {
     const int a = bp.perm[k];
     isb[g.tail[a]] = isb[g.head[a]] = true;
   }
-  Elim C(g.n, g.directed != 0, g.source, g.sink);
-  for (int k = top; k < m; ++k) {
-    const int a = bp.perm[k];
-    C.or_in(g.tail[a], g.head[a], "a[" + std::to_string(k) + "]");
-  }
   std::vector<int> bnd{g.source, g.sink}, rest;
   for (int v = 0; v < g.n; ++v) {
     if (!isb[v]) rest.push_back(v);
     else if (v != g.source && v != g.sink) bnd.push_back(v);
+  }
+  bp.nsig = -1;
+  // Which pairs the prefix arcs can join at all, and so the words needed:
+  // known before anything is generated, as the closure's program grows with
+  // the cube of the nodes (up to 64; within kMaxSigBits words it is short).
+  std::vector<uint64_t> reach(g.n);
+  for (int v = 0; v < g.n; ++v) reach[v] = 1ull << v;
+  for (bool grew = true; grew;) {
+    grew = false;
+    auto join = [&](int u, int v) {
+      if (g.directed && (v == g.source || u == g.sink)) return;
+      if (reach[v] & ~reach[u]) reach[u] |= reach[v], grew = true;
+    };
+    for (int k = top; k < m; ++k) {
+      const int u = g.tail[bp.perm[k]], v = g.head[bp.perm[k]];
+      join(u, v);
+      if (!g.directed) join(v, u);
+    }
+  }
+  int need = 0;
+  for (size_t i = 0; i < bnd.size(); ++i) {
+    int pairs = 0;
+    for (size_t j = 0; j < (g.directed ? bnd.size() : i); ++j)
+      pairs += i != j && (reach[bnd[i]] >> bnd[j] & 1) && !(g.directed && i == 0 && j == 1);
+    if (g.directed) need += pairs;
+    else for (; pairs; pairs >>= 1) ++need;
+  }
+  if (need > kMaxSigBits) return;
+  Elim C(g.n, g.directed != 0, g.source, g.sink);
+  for (int k = top; k < m; ++k) {
+    const int a = bp.perm[k];
+    C.or_in(g.tail[a], g.head[a], "a[" + std::to_string(k) + "]");
   }
   C.eliminate_all(rest);
   // transitive closure over the boundary (Warshall's algorithm)
@@ -447,7 +474,6 @@ static void bs_generate_sig(const GraphIn& g, BsPlan& bp) {
         emit(e);
       }
   }
-  bp.nsig = -1;
   if (nsig > kMaxSigBits) return;
   bp.nsig = nsig;
   // The two ends of the prune come from the same closure: an item is connected
