@@ -2,8 +2,9 @@
 """PBAT benchmark: states/s of exact two-terminal reliability on one GB300.
 
 A step is one pass of the whole enumeration (prefix split, exact monotone
-prune, Gray walk, connectivity of every state, exact accumulation of R,
-N_k and dR/dp into 256-bit fixed-point results) over the 2^m states of the
+prune, prefixes merged by the network they leave, Gray walk and connectivity
+of one prefix per class, exact accumulation of R, N_k and dR/dp into 256-bit
+fixed-point results) over the 2^m states of the
 workload, with the tables already resident on the device.  The headline
 workload is the largest single network, 24 nodes and 40 arcs (2^40
 states).  ``value`` is 2^m / device time of the fused R + N_k + dR/dp step
@@ -81,17 +82,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "3326fae9e2a0d23b": (51111310 / 2**40, 7172352, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "3243cd366da80781": (51114699 / 2**40, 7168000, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "8562a0ea3d516ec7": (18741463 / 2**40, 565248, "profiles/bs_kernel_undirected24x40.md"),
+    "53e373a42c63628a": (18744953 / 2**40, 591872, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "da30d7dd42d47de3": (1352709 / 2**34, 247296, "profiles/bs_kernel_grad_directed20x34.md"),
+    "bb6d95b1e164d3cc": (1352709 / 2**34, 246528, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "01218a14c42ae95a": (879618 / 2**34, 107520, "profiles/bs_kernel_directed20x34.md"),
+    "a2af33993624a428": (879618 / 2**34, 107776, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "1a30d000589d9776": (1718510 / 2**27, 462848, "profiles/bs_kernel_grad_grid3x6.md"),
+    "e8a2ba6380e98e4a": (1719499 / 2**27, 462336, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "4e6b8981adebc73f": (1057835 / 2**27, 157184, "profiles/bs_kernel_grid3x6.md"),
+    "c20797897baf0476": (1046350 / 2**27, 165376, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152
@@ -327,8 +328,7 @@ def _single_record(pb, name, steps, warmup, stream, flush, barrier, ws):
 
 def _batched_record(pb, steps, warmup, stream, ws):
     """The batched workload: 64 networks x 16 p-vectors through
-    pbat_reliability_batched (one persistent launch replayed from a CUDA
-    graph).  Device time from the library's events around the graph launch;
+    pbat_reliability_batched (merged launches replayed from a CUDA graph).  Device time from the library's events around the graph launch;
     the call time includes tables, upload and read-back."""
     import torch
     nets, pvecs = synth.workload_batched()
@@ -356,11 +356,11 @@ def _batched_record(pb, steps, warmup, stream, ws):
             "outputs": "R per (network, p-vector), N_k per network",
             "value": ws * states / (ms / 1e3), "pairs_per_s": ws * states * K / (ms / 1e3),
             "ms_per_step": ms, "call_ms": call, "launches": launches,
-            "kernel": "bs_batch (one persistent launch, CUDA graph replay)", "R00": float(R[0][0]),
+            "kernel": "bs_batch* (merged launches, CUDA graph replay)", "R00": float(R[0][0]),
             "fused": {"value": ws * states / (gms / 1e3), "pairs_per_s": ws * states * K / (gms / 1e3),
                       "ms_per_step": gms, "call_ms": gcall, "launches": glaunches,
                       "outputs": "R, N_k and dR/dp per (network, p-vector)",
-                      "kernel": "bs_batch_grad (one persistent launch, CUDA graph replay)"},
+                      "kernel": "bs_batch_grad* (merged launches, CUDA graph replay)"},
             "fused_over_r_only_time": gms / ms}
 
 

@@ -250,7 +250,8 @@ static unsigned long long full_counts(int ell) {
 static bool acc_in_registers(const BsPlan& bp) { return bp.L <= 6 || bp.ops_var <= 128; }
 
 // Walk arcs unrolled per step (2^in_bits words with compile-time walk words):
-// three give more independent words to the R kernel (GB300: 40-arc network
+// three give more independent words to the R kernel (GB300, one launch that
+// walks every item, here and in the figures below: 40-arc network
 // 106.5 -> 87.8 ms, 34-arc directed 541 -> 495 us) and to the fused kernel
 // when its accumulators are in registers (34-arc 1437 -> 1385 us), but the
 // fused kernel with a large program loses registers to them (40-arc 147.4 ->
@@ -1552,8 +1553,8 @@ int bsb_source_for(int G, const pbat_graph* graphs, int K, const pbat_options& o
 // module and runs the batch once; the fastest launch wins.  The gradient
 // module (elig given) is tuned the same way.  The register cap is not
 // tuned: on GB300 the 64-network workload ran fastest at the default launch
-// bounds of 4 blocks per SM (R module 5.42 ms; 3, 6 and 2 blocks: 5.61, 6.82
-// and 5.91 ms).  Returns false when no candidate ran (the planner's
+// bounds of 4 blocks per SM (R module, every item walked by itself: 5.42 ms; 3,
+// 6 and 2 blocks: 5.61, 6.82 and 5.91 ms).  Returns false when no candidate ran (the planner's
 // defaults are kept).
 static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, const pbat_options& o,
                      cudaStream_t st, const DeviceInfo& dev, const std::vector<std::string>* elig, bool per_item,

@@ -550,12 +550,12 @@ __device__ __forceinline__ void bs_write_out(const BsWork& W, const facc* s_acc,
 //             of its signature: its mass, its popcount;
 //   bs_walk   walks one item of every class for all of them;
 //   bs_fold   (fused kernel) the prefix arcs' gradient from the items' sums.
-// Against walking every item left (GB300; a 24-node, 40-arc network, 2^40
-// states): fused 49.1 -> 0.26 ms, R 20.2 -> 0.12 ms; a 20-node, 34-arc
-// directed network 0.36 -> 0.055 and 0.58 -> 0.050 ms; the 3x6 grid 0.100 ->
-// 0.048 and 0.055 -> 0.026 ms.  The large runs are bound by instruction
-// issue (bs_merge and bs_fold work per 32 items, bs_walk per class), the
-// small ones by the latency of their three launches.
+// Against walking every item left (GB300, whole passes through the API): a
+// 24-node, 40-arc network (2^40 states) fused 49.3 -> 0.30 ms, R 20.2 -> 0.17
+// ms; a 20-node, 34-arc directed network 0.38 -> 0.072 and 0.65 -> 0.086 ms;
+// 11 nodes, 31 arcs, fused 0.39 -> 0.13 ms.  The large runs are bound by
+// instruction issue (bs_merge and bs_fold work per 32 items, bs_walk per
+// class), the small ones by the latency of their two or three launches.
 // ---------------------------------------------------------------------------
 #if BS_MERGE
 #define BS_BLK (BS_LOW + BS_MID)   // prefix arcs inside a merge block
@@ -1228,7 +1228,7 @@ __device__ __forceinline__ void bs_fold_body(const BsParams& P, const BsFoldPara
                                              const BsWork& W) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // A_k and B_k of every prefix arc, per warp
-  __shared__ facc s_acc[BS_MERGE_NTHR / 32][2 * BS_D];
+  __shared__ facc s_acc[BS_MERGE_NTHR / 32][BS_D ? 2 * BS_D : 1];
   __shared__ u128 s_V[TEAM ? 4 : 1][32], s_X[TEAM ? 4 : 1][4];   // a team's folded groups and sums
   facc* acc = s_acc[warp];
   for (int i = lane; i < 2 * BS_D; i += 32) acc[i] = facc{u128{0ull, 0ull}, 0, 0};
@@ -1829,9 +1829,8 @@ __device__ __forceinline__ void bsb_finish_grad(
 //   bs_batch*_p2  adds each item's masses and popcount to its class
 //   bs_batch*     walks one item of every class (bsb_conn, bsb_finish)
 //   bs_batch*_p3  (gradient) folds the prefix arcs, per block and p-vector
-// GB300, against a walk for every item left: 64 networks x 16 p-vectors, R
-// 9.6 -> 0.62 ms; 20 x 7 with the gradient 0.91 -> 0.36 ms (prune 1), 0.16
-// (prune 2).  The walking launch is bound by instruction issue and the table
+// GB300, against a walk for every item left: 64 networks (2.9e10 states) x 16
+// p-vectors, R 5.42 -> 0.43 ms, with the gradient 24.1 -> 1.89 ms.  The walking launch is bound by instruction issue and the table
 // rows it reads through L1, the others by the latency of the table and the
 // class memory, hence the several warps per block of items.
 // ---------------------------------------------------------------------------
