@@ -432,6 +432,9 @@ struct Job {
   bool merged = false;
   int grid1 = 0, grid2 = 0, grid3 = 0, split_log2 = 0;
   size_t clear_bytes = 0;
+  // the job that this one took the place of (job_rerun), kept while a stream
+  // capture of its launches may be replayed into its buffers
+  Job* before = nullptr;
   // the inputs, kept to re-run the exact frontier kernel when R is too small
   // for the bit-sliced kernel's fixed-point error bound
   std::vector<int32_t> tail_copy, head_copy;
@@ -625,8 +628,8 @@ static int autotune(const GraphIn& g, const double* p, bool grad, pbat_options& 
   // than 128 and 224 threads the R kernel 7% faster than 256
   if (!large) nts.push_back(64), nts.push_back(96);
   for (int nt : {128, 160, 192, 224, 256}) nts.push_back(nt);
-  // a register cap of two blocks per SM: on GB300 the fused kernel of the
-  // 40-arc network in prune-aware mode went from 26.0 to 24.7 ms with it
+  // a register cap of two blocks per SM: on GB300 the one-launch fused kernel
+  // of the 40-arc network in prune-aware mode went from 26.0 to 24.7 ms with it
   if (o.occupancy >= 0) occs.push_back(o.occupancy);
   else occs = {0, 2};
   double best_ms = 1e300;
@@ -971,8 +974,12 @@ static int job_rerun(Job* J, pbat_options o, bool keep, cudaStream_t st, double*
   int rc = job_create(J->g, J->p_copy.data(), J->pl.grad, &o, &F);
   if (!rc && !(rc = job_upload(F, st)) && !(rc = job_launch(F, st)))
     rc = job_read(F, st, R_out, Nk_out, J->pl.grad ? dRdp_out : nullptr, opt);
-  if (keep && !rc) std::swap(*J, *F);
-  job_destroy(F);
+  if (keep && !rc) {
+    std::swap(*J, *F);
+    J->before = F;
+  } else {
+    job_destroy(F);
+  }
   return rc;
 }
 
@@ -1069,6 +1076,7 @@ int job_read(Job* J, cudaStream_t st, double* R_out, uint64_t* Nk_out, double* d
 
 void job_destroy(Job* J) {
   if (!J) return;
+  job_destroy(J->before);
   if (J->bs) bs_delete(J->bs);
   event_pairs_release(J->dev.device, J->evs);
   scratch_release(J->scr);

@@ -176,6 +176,33 @@ def test_more_classes_than_the_table_holds(pb):
 
 
 @pytest.mark.gpu
+def test_replay_after_the_class_table_overflowed(pb):
+    """A capture of a merged plan's launches stays valid when a read has found
+    too many classes and taken the plan to one launch: its replays write to
+    the captured job's own buffers, not to memory given back."""
+    import torch
+    tail, head, rng = synth.random_connected_undirected(20, 38, 902)
+    net = synth.Network(20, tail, head, synth.uniform_p(rng, 38, 0.7, 0.95), 0, 19)
+    # (another block size than the test above, whose plan is known not to merge)
+    plan = pb.Plan(net, opts=pb.options(autotune=0, launches=2, walk_bits=4, block_threads=64))
+    stream = torch.cuda.Stream()
+    plan.execute(stream.cuda_stream)   # loads the kernels
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        plan.execute(stream.cuda_stream)
+    graph.replay()
+    torch.cuda.synchronize()
+    first = plan.read(stream.cuda_stream)
+    other = pb.reliability_net(net, opts=pb.options(autotune=0, launches=1, walk_bits=4))
+    graph.replay()
+    torch.cuda.synchronize()
+    plan.execute(stream.cuda_stream)
+    again = plan.read(stream.cuda_stream)
+    assert first.Nk == again.Nk == other.Nk
+    assert first.R == again.R and _same(first.R, other.R, 1e-12 * other.R)
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("vectors", [1, 7, 17, 40])
 @pytest.mark.parametrize("grad", [False, True])
 def test_merged_batches(pb, vectors, grad):
