@@ -176,6 +176,23 @@ def test_more_classes_than_the_table_holds(pb):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("p, launches", [(0.5, 3), (0.7, 3), (0.75, 1), (0.95, 1)])
+def test_small_gradients_keep_their_split(pb, p, launches):
+    """The fused kernel of the complete graph of 8 nodes: six other arcs at
+    the source fail with (1 - p)^6, above 2^-11 merged, below in one launch
+    with that route's very results."""
+    arcs = [(u, v) for u in range(8) for v in range(u)]
+    net = synth.Network(8, [u for u, _ in arcs], [v for _, v in arcs], [p] * 28, 7, 0)
+    res = pb.reliability_net(net, grad=True, opts=pb.options(autotune=0))
+    one = pb.reliability_net(net, grad=True, opts=pb.options(autotune=0, launches=1))
+    assert res.stats[5] == launches
+    assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R)
+    for x, y in zip(res.grad, one.grad):
+        assert x == y if launches == 1 else _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56)
+    assert pb.reliability_net(net, opts=pb.options(autotune=0)).stats[5] == 2
+
+
+@pytest.mark.gpu
 def test_replay_after_the_class_table_overflowed(pb):
     """A capture of a merged plan's launches stays valid when a read has found
     too many classes and taken the plan to one launch: its replays write to
