@@ -95,7 +95,8 @@ typedef struct pbat_options {
                            items left into classes whose prefixes leave the same network, one
                            that walks each class once, and for the gradient one that adds the
                            prefix arcs' (at most 2^24 items and 2^18 classes, else one
-                           launch); 0 (default) = merged from 2^13 items on, else one launch,
+                           launch); 0 (default) = merged from 2^13 items on, else one launch
+                           (so too a gradient that is all below about 2^-11, under 38 arcs),
                            or the autotuner's choice when it runs.  Results do not depend on
                            it. */
   int range_bits;       /* 0 (default) = whole space.  Otherwise only the states whose
