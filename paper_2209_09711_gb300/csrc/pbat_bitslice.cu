@@ -324,12 +324,23 @@ struct BsCached {
 static std::mutex g_bsplan_mu;
 static std::map<std::string, BsCached> g_bsplan;
 
+// What a plan takes from the width of a range: whether the items are few enough
+// or many enough to be merged.  Their number is the width times a power of two
+// and so are the limits, so the width's logarithm rounded down and up decides.
+static long long width_class(const pbat_options& o) {
+  if (o.range_bits <= 0) return 0;
+  const uint64_t w = o.range_hi - o.range_lo;
+  if (!w) return -1;
+  return 2 * (64 - __builtin_clzll(w)) + ((w & (w - 1)) != 0);
+}
+
 static std::string bs_plan_key(const GraphIn& g, const double* p, bool grad, const pbat_options& o,
                                int nthr, int device) {
   std::string k;
   auto put = [&](long long v) { k.append((const char*)&v, sizeof v); };
   put(device); put(g.n); put(g.m); put(g.directed); put(g.source); put(g.sink); put(grad);
-  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(nthr); put(o.prune); put(o.launches);
+  put(o.walk_bits); put(o.prefix_bits); put(o.range_bits); put(width_class(o));
+  put(nthr); put(o.prune); put(o.launches);
   put(std::max(0, o.occupancy));
   k.append((const char*)g.tail, sizeof(int32_t) * g.m);
   k.append((const char*)g.head, sizeof(int32_t) * g.m);

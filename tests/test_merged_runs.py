@@ -160,6 +160,35 @@ def test_merged_runs_of_ranges_and_extreme_reliabilities(pb):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("wide_first", [False, True])
+@pytest.mark.parametrize("grad", [False, True])
+def test_ranges_of_other_widths_plan_for_themselves(pb, wide_first, grad):
+    """One network's ranges of the same number of bits, narrow and wide, in
+    either order: each takes the route of its own number of items, whatever
+    range was planned before."""
+    # (a network of its own for each order and kernel: plans are kept by network)
+    seed = 640 + 2 * wide_first + grad
+    # by default: 2^10 items a division, merged from 2^13 on
+    net = synth.random_small(seed, n=12, m=30, p_lo=0.3, p_hi=0.95)
+    widths = [(0, 1, 1), (5, 12, 1), (8, 16, 3 if grad else 2), (0, 64, 3 if grad else 2), (7, 7, 1)]
+    for lo, hi, launches in reversed(widths) if wide_first else widths:
+        opt = dict(range_bits=6, range_lo=lo, range_hi=hi, walk_bits=4, algo=pb.ALGO_BITSLICE)
+        res = pb.reliability_net(net, grad=grad, opts=pb.options(**opt))
+        assert res.stats[5] == launches, (lo, hi)
+        one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
+        assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+    # merged when asked for: 2^18 items a division, at most 2^24 merged
+    net = synth.random_small(seed + 10, n=9, m=36, p_lo=0.3, p_hi=0.95)
+    widths = [(3, 4, 3 if grad else 2), (64, 128, 3 if grad else 2), (64, 129, 1), (0, 256, 1)]
+    for lo, hi, launches in reversed(widths) if wide_first else widths:
+        opt = dict(range_bits=8, range_lo=lo, range_hi=hi, prune=2, walk_bits=0, algo=pb.ALGO_BITSLICE)
+        res = pb.reliability_net(net, grad=grad, opts=pb.options(launches=2, **opt))
+        assert res.stats[5] == launches, (lo, hi)
+        one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
+        assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+
+
+@pytest.mark.gpu
 def test_more_classes_than_the_table_holds(pb):
     """A network of 2^24 items in more than 2^18 classes: the merged run is
     given up and every item walked, with the same counts and reliability, for
