@@ -82,17 +82,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "3243cd366da80781": (51114699 / 2**40, 7168000, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "b354841fd795531d": (51297915 / 2**40, 7164672, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "53e373a42c63628a": (18744953 / 2**40, 591872, "profiles/bs_kernel_undirected24x40.md"),
+    "9ce88ff5e095ca61": (18774375 / 2**40, 562176, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "bb6d95b1e164d3cc": (1352709 / 2**34, 246528, "profiles/bs_kernel_grad_directed20x34.md"),
+    "3c05a51e1037662e": (1353625 / 2**34, 248576, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "a2af33993624a428": (879618 / 2**34, 107776, "profiles/bs_kernel_directed20x34.md"),
+    "33a6e68dbb1689fe": (882294 / 2**34, 109568, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "e8a2ba6380e98e4a": (1719499 / 2**27, 462336, "profiles/bs_kernel_grad_grid3x6.md"),
+    "09f23962e7f661d7": (1716533 / 2**27, 462336, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "c20797897baf0476": (1046350 / 2**27, 165376, "profiles/bs_kernel_grid3x6.md"),
+    "cb47608e39d098ec": (1055757 / 2**27, 163072, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

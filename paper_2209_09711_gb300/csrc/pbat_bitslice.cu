@@ -977,7 +977,7 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  for (;;) {\n"
       "    const u64 cls = next;\n"
       "    if (cls >= n_cls) break;\n"
-      "    if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); break; }\n"
+      "    if (bs_time_up(budget_ns, t0, status, lane)) break;\n"
       "    next = ~0ull;\n"
       "    if (n_cls > n_warps) {\n"
       "      if (lane == 0) next = n_warps + atomicAdd(A.ticket, 1ull);\n"
@@ -1032,7 +1032,7 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
             "  for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks << A.split_log2;\n"
             "       v += (u64)gridDim.x * (BSB_MNTHR / 32)) {\n"
             "    const u64 t = v >> A.split_log2;\n"
-            "    if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); break; }\n"
+            "    if (bs_time_up(budget_ns, t0, status, lane)) break;\n"
             "    const int net = bsb_block_net(graphs, G, t);\n"
             "    const u64 hi = t - graphs[net].blk_begin;\n"
             "    u32 full = 0u, left = 0u;\n"

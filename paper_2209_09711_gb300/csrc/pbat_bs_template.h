@@ -221,6 +221,20 @@ __device__ __forceinline__ void bs_let_next_start() { asm volatile("griddepcontr
 __device__ __forceinline__ u64 bs_timer() {
   u64 t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t;
 }
+// Whether a warp's time is up, the same answer in every lane: lane 0 reads the
+// clock.  The loops that ask go on with collectives of the whole warp, and the
+// lanes come here from code where they part, so each lane reading for itself
+// could leave some of them waiting for the others.
+__device__ __forceinline__ bool bs_time_up(u64 budget_ns, u64 t_start, u32* status, int lane) {
+  if (!budget_ns) return false;
+  __syncwarp();
+  int up = 0;
+  if (lane == 0 && bs_timer() - t_start > budget_ns) {
+    atomicOr(status, 1u);
+    up = 1;
+  }
+  return __shfl_sync(0xffffffffu, up, 0) != 0;
+}
 
 // Mass of the prefix arcs of `prefix`: product over table levels.
 __device__ __forceinline__ mx bs_level_mass(int nlev, const int* bits, const int* off,
@@ -583,7 +597,7 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
   for (u64 t = (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; t < nblk << split_log2; t += nwarps) {
     const u64 b = t >> split_log2;
     const u32 part = (u32)t & ((1u << split_log2) - 1u);
-    if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
+    if (bs_time_up(P.budget_ns, t_start, W.status, lane)) break;
     const u64 hi = blk0 + b;
     u32 a[BS_M], z[BS_NSIG > 0 ? BS_NSIG : 1], dn, up;
 #pragma unroll
@@ -1244,7 +1258,7 @@ __device__ __forceinline__ void bs_fold_body(const BsParams& P, const BsFoldPara
   // lane l < BS_BLK: arc l of the block; lanes: arcs `lane` and `lane + 32` above it
   facc accP = facc{u128{0ull, 0ull}, 0, 0}, accA = accP, accB = accP, accA2 = accP, accB2 = accP;
   for (u64 b = TEAM ? blockIdx.x : (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; b < nblk; b += step) {
-    if (!TEAM && P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); break; }
+    if (!TEAM && bs_time_up(P.budget_ns, t_start, W.status, lane)) break;
     const u64 hi = blk0 + b;
     const uint2 m = W.cmask[b * 32 + lane];
     if (!__any_sync(0xffffffffu, m.x | m.y)) continue;   // (the same in every warp of a team)

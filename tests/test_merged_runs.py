@@ -104,6 +104,44 @@ def test_signature_is_the_residual_network(pb, directed, prune):
                 assert (sig[i] == sig[j]) == (res[i] == res[j]), (seed, i, j)
 
 
+def _merged_sources(pb):
+    """The kernels of a merged run, of one network and of a batch, R and gradient."""
+    tail, head, rng = synth.random_connected_undirected(12, 30, 77)
+    net = synth.Network(12, tail, head, synth.uniform_p(rng, 30, 0.7, 0.95), 0, 11)
+    for grad in (False, True):
+        batch = (pb.batch_grad_kernel_source([net, net], [[net.p] * 3] * 2) if grad
+                 else pb.batch_kernel_source([net, net], 3))
+        for src in (pb.kernel_source(net, pb.options(launches=2), grad=grad), batch):
+            assert re.search(r"#define BSB?_MERGE 1", src)
+            yield src
+
+
+def _openers(src, at):
+    """The statement at a position, and the headers of the blocks around it."""
+    out, depth, i = [src[max(src.rfind(c, 0, at) for c in ";{}"):at]], 0, at
+    while i > 0:
+        i -= 1
+        if src[i] == "}":
+            depth += 1
+        elif src[i] == "{":
+            depth -= 1
+            if depth < 0:
+                depth = 0
+                out.append(src[max(src.rfind(c, 0, i) for c in ";{}"):i])
+    return out
+
+
+def test_a_warp_reads_the_clock_in_one_lane(pb):
+    """The time limit: what follows a check are collectives of the whole warp,
+    so one lane decides for all.  Every comparison with the clock is made by
+    lane 0 alone (the kernels are not run for this)."""
+    for src in _merged_sources(pb):
+        places = [m.start() for m in re.finditer(r"bs_timer\(\) -", src)]
+        assert places
+        for at in places:
+            assert any("lane == 0" in o for o in _openers(src, at)), src[at - 200:at + 60]
+
+
 def _same(a, b, tol):
     return abs(a - b) <= tol
 
