@@ -82,17 +82,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "b354841fd795531d": (51297915 / 2**40, 7164672, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "9339d9597661dd9d": (51309917 / 2**40, 7158272, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "9ce88ff5e095ca61": (18774375 / 2**40, 562176, "profiles/bs_kernel_undirected24x40.md"),
+    "55e2110d63735bc3": (18791803 / 2**40, 561152, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "3c05a51e1037662e": (1353625 / 2**34, 248576, "profiles/bs_kernel_grad_directed20x34.md"),
+    "6223a26866165e86": (1355673 / 2**34, 250368, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "33a6e68dbb1689fe": (882294 / 2**34, 109568, "profiles/bs_kernel_directed20x34.md"),
+    "c6da5851d80ee436": (882294 / 2**34, 109568, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "09f23962e7f661d7": (1716533 / 2**27, 462336, "profiles/bs_kernel_grad_grid3x6.md"),
+    "c917d3c65fa15ac2": (1723243 / 2**27, 463616, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "cb47608e39d098ec": (1055757 / 2**27, 163072, "profiles/bs_kernel_grid3x6.md"),
+    "0defd9c65cd97826": (1065593 / 2**27, 161792, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

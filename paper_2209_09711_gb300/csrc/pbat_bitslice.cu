@@ -970,7 +970,7 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  const u64 t0 = bs_timer();\n";
   kern += E.merged ?
       "  rel[lane] = 0u;\n"
-      "  if (*(volatile u32*)status) return;\n"
+      "  if (bs_warp_given_up(status, lane)) return;\n"
       "  const u64 n_cls = *A.n_classes, n_warps = (u64)gridDim.x * (BSB_NTHR / 32);\n"
       "  u64 next = (u64)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;\n"
       "  __syncwarp();\n"

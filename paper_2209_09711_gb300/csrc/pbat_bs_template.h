@@ -236,6 +236,17 @@ __device__ __forceinline__ bool bs_time_up(u64 budget_ns, u64 t_start, u32* stat
   return __shfl_sync(0xffffffffu, up, 0) != 0;
 }
 
+// Whether the run was given up, out of time or of class slots (the host then
+// discards it), the same answer in every thread of a block or of a warp: one
+// reads the word, which other blocks of the same launch may be setting.
+__device__ __forceinline__ bool bs_block_given_up(const u32* status) {
+  return __syncthreads_or(threadIdx.x == 0 && *(volatile const u32*)status != 0u) != 0;
+}
+__device__ __forceinline__ bool bs_warp_given_up(const u32* status, int lane) {
+  const u32 s = lane == 0 ? *(volatile const u32*)status : 0u;
+  return __shfl_sync(0xffffffffu, s, 0) != 0u;
+}
+
 // Mass of the prefix arcs of `prefix`: product over table levels.
 __device__ __forceinline__ mx bs_level_mass(int nlev, const int* bits, const int* off,
                                             const mx* __restrict__ ptab, u64 prefix) {
@@ -707,9 +718,10 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
     bs_wait_previous();
     n_list = *W.list_n;
     next = (u64)warp * gridDim.x + blockIdx.x;
-    if (blockIdx.x >= n_list || *W.status) return;   // no class, or a run that the host discards
+    if (blockIdx.x >= n_list) return;   // no class
   }
-  __syncthreads();
+  if (PHASE != 2) __syncthreads();
+  else if (bs_block_given_up(W.status)) return;
   u64* bins = s_bins + tid;
   const bool thr_on = lane < (1 << BS_TB);
   const u64 thw = thr_on ? P.thw[lane] : 0ull;
@@ -935,10 +947,11 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     bs_let_next_start();
     n_list = *W.list_n;
     next = (u64)warp * gridDim.x + blockIdx.x;
-    if (blockIdx.x >= n_list || *W.status) return;   // no class, or a run that the host discards
+    if (blockIdx.x >= n_list) return;   // no class
   }
   for (int i = tid; i < (BS_NTHR / 32) * n_acc; i += BS_NTHR) s_acc[i] = facc{u128{0ull, 0ull}, 0, 0};
-  __syncthreads();
+  if (PHASE != 2) __syncthreads();
+  else if (bs_block_given_up(W.status)) return;
   facc* acc = s_acc + warp * n_acc;
   u64* bins = s_bins + tid;
   u128* A = s_A + tid;
@@ -1246,11 +1259,9 @@ __device__ __forceinline__ void bs_fold_body(const BsParams& P, const BsFoldPara
   __shared__ u128 s_V[TEAM ? 4 : 1][32], s_X[TEAM ? 4 : 1][4];   // a team's folded groups and sums
   facc* acc = s_acc[warp];
   for (int i = lane; i < 2 * BS_D; i += 32) acc[i] = facc{u128{0ull, 0ull}, 0, 0};
-  __syncwarp();
   bs_wait_previous();
-  // an earlier launch ran out of time or slots: its masks and slots are not
-  // all written, and the host discards the run
-  if (*(volatile u32*)W.status) return;
+  // (the masks and slots of a run that was given up are not all written)
+  if (bs_block_given_up(W.status)) return;
   const u64 nblk = P.n_tasks >> BS_BLK, blk0 = P.task_lo >> BS_BLK;
   const u64 step = TEAM ? (u64)gridDim.x : (u64)gridDim.x * (BS_MERGE_NTHR / 32);
   const u64 m_mid = Q.mid[lane];
@@ -1940,8 +1951,8 @@ __device__ __forceinline__ void bsb_merge_block(const BGraph* __restrict__ B, in
 extern "C" __global__ void __launch_bounds__(BSB_MNTHR) BSB_SCATTER(
     const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u32* status) {
   __shared__ mx s_hi[BSB_MNTHR / 32][64];
-  if (*(volatile u32*)status) return;   // out of time or slots: the host discards the run
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (bs_warp_given_up(status, lane)) return;
   for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks * A.parts; v += (u64)gridDim.x * (BSB_MNTHR / 32)) {
     const u64 t = v / A.parts;
     const int part = (int)(v - t * A.parts);
@@ -1974,8 +1985,8 @@ extern "C" __global__ void __launch_bounds__(BSB_MNTHR) BSB_SCATTER(
 extern "C" __global__ void __launch_bounds__(BSB_MNTHR) bs_batch_grad_p3(
     const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u64* limbs,
     const u32* status) {
-  if (*(volatile const u32*)status) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (bs_warp_given_up(status, lane)) return;
   for (u64 t = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; t < A.n_blocks * K; t += (u64)gridDim.x * (BSB_MNTHR / 32)) {
     const u64 b = t / K;
     const int k = (int)(t - b * K);

@@ -142,6 +142,18 @@ def test_a_warp_reads_the_clock_in_one_lane(pb):
             assert any("lane == 0" in o for o in _openers(src, at)), src[at - 200:at + 60]
 
 
+def test_a_block_or_a_warp_reads_the_status_in_one_thread(pb):
+    """The word that says that a run was given up, which other blocks of the
+    same launch may be setting: only the two functions that read it for a whole
+    block or warp do, and a thread that does not return goes on to barriers or
+    collectives (the kernels are not run for this)."""
+    for src in _merged_sources(pb):
+        reads = list(re.finditer(r"(?<!u32)\*(?:\(volatile (?:const )?u32\*\))?(?:W\.)?status", src))
+        assert len(reads) == 2
+        for m in reads:
+            assert any("_given_up(" in o for o in _openers(src, m.start())), src[m.start() - 200:m.end()]
+
+
 def _same(a, b, tol):
     return abs(a - b) <= tol
 
