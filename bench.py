@@ -82,17 +82,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "9339d9597661dd9d": (51309917 / 2**40, 7158272, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "fb7df71bff6f2408": (51049950 / 2**40, 7045888, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "55e2110d63735bc3": (18791803 / 2**40, 561152, "profiles/bs_kernel_undirected24x40.md"),
+    "a88084a1ef4ad807": (18672325 / 2**40, 476416, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "6223a26866165e86": (1355673 / 2**34, 250368, "profiles/bs_kernel_grad_directed20x34.md"),
+    "f0baa0f8084c97fa": (1321683 / 2**34, 242688, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "c6da5851d80ee436": (882294 / 2**34, 109568, "profiles/bs_kernel_directed20x34.md"),
+    "58e1477a6b95c5b9": (873986 / 2**34, 110336, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "c917d3c65fa15ac2": (1723243 / 2**27, 463616, "profiles/bs_kernel_grad_grid3x6.md"),
+    "f9e02ae0c7da9494": (1719066 / 2**27, 465664, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "0defd9c65cd97826": (1065593 / 2**27, 161792, "profiles/bs_kernel_grid3x6.md"),
+    "90468b5ed8689557": (1034867 / 2**27, 162560, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

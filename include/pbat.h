@@ -107,7 +107,11 @@ typedef struct pbat_options {
   uint64_t range_lo;
   uint64_t range_hi;
   double time_budget_s; /* > 0: the device stops after this many seconds and the call
-                           returns PBAT_ETIMEOUT; 0 = no limit */
+                           returns PBAT_ETIMEOUT; 0 = no limit.  A kernel looks at the
+                           clock before each work item (or block of items), and the
+                           launches of one enumeration or batch all count from the first
+                           one's start.  An enumeration that is run again (AUTO's exact
+                           re-run, one launch after too many classes) has the limit anew */
   uint64_t stats[8];    /* out, filled by the last call that took these options:
                            [0] states enumerated by walking (of a class of merged items: one
                            item's), [1] the other states, resolved by the prune or with

@@ -789,7 +789,7 @@ struct BGraphHost {
 };
 // Host mirror of BMerge in the kernel source.
 struct BMergeHost {
-  void *key, *id_of, *net, *rep, *hist, *cmass, *csum, *cmask, *ent, *n_classes, *ticket;
+  void *key, *id_of, *net, *rep, *hist, *cmass, *csum, *cmask, *ent, *n_classes, *ticket, *start;
   unsigned long long n_blocks;
   int split_log2, parts;
   unsigned cap;
@@ -966,8 +966,7 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  u64* nkw = s_nk + (threadIdx.x >> 5) * 65;\n"
       "  u32* rel = (u32*)(s_nk + (BSB_NTHR / 32) * 65) + (threadIdx.x >> 5) * 33;   // merged: counts below the prefix\n"
       "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n"
-      "  int cur = -1;   // network whose counts nkw holds\n"
-      "  const u64 t0 = bs_timer();\n";
+      "  int cur = -1;   // network whose counts nkw holds\n";
   kern += E.merged ?
       "  rel[lane] = 0u;\n"
       "  if (bs_warp_given_up(status, lane)) return;\n"
@@ -977,7 +976,7 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  for (;;) {\n"
       "    const u64 cls = next;\n"
       "    if (cls >= n_cls) break;\n"
-      "    if (bs_time_up(budget_ns, t0, status, lane)) break;\n"
+      "    if (budget_ns && bs_time_up(budget_ns, A.start, status, lane)) break;\n"
       "    next = ~0ull;\n"
       "    if (n_cls > n_warps) {\n"
       "      if (lane == 0) next = n_warps + atomicAdd(A.ticket, 1ull);\n"
@@ -985,12 +984,13 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "    }\n"
       "    const int lo = (int)A.net[cls];\n"
       "    const u64 prefix = A.rep[cls];\n" :
+      "  const u64 t0 = bs_timer();\n"
       "  for (;;) {\n"
       "    u64 task = 0;\n"
       "    const u64 cls = 0;\n"
       "    if (lane == 0) {\n"
       "      task = atomicAdd(counter, 1ull);\n"
-      "      if (budget_ns && bs_timer() - t0 > budget_ns) { atomicOr(status, 1u); task = ~0ull; }\n"
+      "      if (budget_ns && bs_late(budget_ns, t0, status)) task = ~0ull;\n"
       "    }\n"
       "    task = __shfl_sync(0xffffffffu, task, 0);\n"
       "    if (task >= total) break;\n"
@@ -1028,11 +1028,10 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
             "  extern __shared__ u32 s_sig[];\n"
             "  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;\n"
             "  u32* zs = s_sig + warp * " + std::to_string(std::max(1, E.nsig_max) * 32) + ";\n"
-            "  const u64 t0 = bs_timer();\n"
             "  for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks << A.split_log2;\n"
             "       v += (u64)gridDim.x * (BSB_MNTHR / 32)) {\n"
             "    const u64 t = v >> A.split_log2;\n"
-            "    if (bs_time_up(budget_ns, t0, status, lane)) break;\n"
+            "    if (budget_ns && bs_time_up(budget_ns, A.start, status, lane)) break;\n"
             "    const int net = bsb_block_net(graphs, G, t);\n"
             "    const u64 hi = t - graphs[net].blk_begin;\n"
             "    u32 full = 0u, left = 0u;\n"
@@ -1157,7 +1156,7 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   E.o_upload_end = off;
   E.o_limbs = off; off = a256(off + 8 * E.n_out);
   E.o_nk = off; off = a256(off + 8 * (size_t)E.nk_total);
-  E.o_counter = off; off = a256(off + 3 * 8);   // and, merged, the number of classes and their ticket
+  E.o_counter = off; off = a256(off + 4 * 8);   // and, merged, the number of classes, their ticket and the start
   E.o_status = off; off = a256(off + 4);
   E.o_end = off;
   if ((rc = scratch_acquire(dev.device, E.o_end, E.o_end, &E.scr))) return rc;
@@ -1183,6 +1182,7 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
     M.key = d + key; M.id_of = d + id_of; M.net = d + net; M.rep = d + rep; M.hist = d + hist;
     M.cmass = d + cmass; M.csum = d + csum; M.cmask = d + cmask; M.ent = d + ent;
     M.n_classes = u + E.o_counter + 8; M.ticket = u + E.o_counter + 16;
+    M.start = u + E.o_counter + 24;
     M.nib = u + E.o_nib; M.mid = u + E.o_mid; M.fold = u + E.o_fold;
     E.smem1 = (size_t)(kMergeThreads / 32) * std::max(1, E.nsig_max) * 32 * 4;
     auto fit = [&](cudaKernel_t k, size_t smem, unsigned long long warps) {
@@ -1524,7 +1524,7 @@ static int bsb_enqueue(BsBatch& E, cudaStream_t st, unsigned long long budget_ns
                    &limbs, &nk, &counter, &status, &bud, (void*)&E.M};
   if (E.merged) {
     void* a1[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &limbs, &nk, &status, &bud};
-    void* a2[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &status};
+    void* a2[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &status, &bud};
     if ((e = cudaMemsetAsync(E.M.key, 0, E.key_bytes, st)) != cudaSuccess ||
         (e = cudaLaunchKernel((const void*)E.jit.kernel_p1, dim3(E.grid1), dim3(kMergeThreads), a1, E.smem1, st)) != cudaSuccess ||
         (e = cudaLaunchKernel((const void*)E.jit.kernel_p2, dim3(E.grid2), dim3(kMergeThreads), a2, 0, st)) != cudaSuccess)
@@ -1533,7 +1533,7 @@ static int bsb_enqueue(BsBatch& E, cudaStream_t st, unsigned long long budget_ns
   e = cudaLaunchKernel((const void*)E.jit.kernel, dim3(E.grid), dim3(kBsbThreads),
                        E.grad ? gargs : args, E.smem, st);
   if (e == cudaSuccess && E.merged && E.grad) {
-    void* a3[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &limbs, &status};
+    void* a3[] = {(void*)&graphs, &G, &K, (void*)&pt, (void*)&E.M, &limbs, &status, &bud};
     e = cudaLaunchKernel((const void*)E.jit.kernel_p3, dim3(E.grid3), dim3(kMergeThreads), a3, 0, st);
   }
   if (e != cudaSuccess) return fail(PBAT_ECUDA, "batched launch: %s", cudaGetErrorString(e));

@@ -186,6 +186,7 @@ struct BsWork {
   u32* list;
   u64* list_n;
   u64* counter2;
+  u64* start;   // and when it began (bs_run_late)
   // per slot: the signature (0: unused), the summed mass of the class's items
   // in two chunks, their number by popcount (BS_HIST each), one of them, and
   // the sum S of that one
@@ -221,21 +222,42 @@ __device__ __forceinline__ void bs_let_next_start() { asm volatile("griddepcontr
 __device__ __forceinline__ u64 bs_timer() {
   u64 t; asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t)); return t;
 }
-// Whether a warp's time is up, the same answer in every lane: lane 0 reads the
-// clock.  The loops that ask go on with collectives of the whole warp, and the
-// lanes come here from code where they part, so each lane reading for itself
-// could leave some of them waiting for the others.
-__device__ __forceinline__ bool bs_time_up(u64 budget_ns, u64 t_start, u32* status, int lane) {
-  if (!budget_ns) return false;
+__device__ __forceinline__ bool bs_late(u64 budget_ns, u64 t_start, u32* status) {
+  const u64 now = bs_timer();
+  if (now <= t_start || now - t_start <= budget_ns) return false;
+  atomicOr(status, 1u);
+  return true;
+}
+// The launches of a merged run all count its time limit from when the first
+// warp of the first one asked, kept beside the status.  (Another SM's clock may
+// have been read a little later than this one's.)
+__device__ __forceinline__ bool bs_run_late(u64 budget_ns, u64* start, u32* status) {
+  u64 first = *(volatile u64*)start;
+  if (!first) {
+    const u64 now = bs_timer();
+    first = atomicCAS(start, 0ull, now);
+    if (!first) first = now;
+  }
+  return bs_late(budget_ns, first, status);
+}
+// Whether the time is up, the same answer in every lane of a warp or every
+// thread of a block: one lane reads the clock.  The loops that ask go on with
+// collectives of the whole warp, and the lanes come here from code where they
+// part, so each lane reading for itself could leave some of them waiting for
+// the others.  Out of line, and called under a limit only: inlined, it made
+// the compiler join the parted lanes of bs_merge_body's loop over the classes
+// later (24 nodes, 40 arcs, L = 6: 44.5 -> 60.3 M warp instructions, 103 -> 129 us).
+__device__ __noinline__ bool bs_time_up(u64 budget_ns, u64* start, u32* status, int lane) {
   __syncwarp();
   int up = 0;
-  if (lane == 0 && bs_timer() - t_start > budget_ns) {
-    atomicOr(status, 1u);
-    up = 1;
-  }
+  if (lane == 0) up = bs_run_late(budget_ns, start, status);
   return __shfl_sync(0xffffffffu, up, 0) != 0;
 }
-
+__device__ __noinline__ bool bs_block_time_up(u64 budget_ns, u64* start, u32* status) {
+  int up = 0;
+  if (threadIdx.x == 0) up = bs_run_late(budget_ns, start, status);
+  return __syncthreads_or(up) != 0;
+}
 // Whether the run was given up, out of time or of class slots (the host then
 // discards it), the same answer in every thread of a block or of a warp: one
 // reads the word, which other blocks of the same launch may be setting.
@@ -599,7 +621,6 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
   __syncthreads();
   const u128 m_mid = u128{mtab[128 + lane].x, mtab[128 + lane].y};
   facc accR = facc{u128{0ull, 0ull}, 0, 0};
-  const u64 t_start = bs_timer();
   // a block's items left to walk are shared by 2^split_log2 warps (each takes
   // every so manyeth bit of the words), so that few blocks still fill the GPU
   const u64 nwarps = (u64)gridDim.x * (BS_MERGE_NTHR / 32);
@@ -608,7 +629,7 @@ __device__ __forceinline__ void bs_merge_body(const BsParams& P, const mx* __res
   for (u64 t = (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; t < nblk << split_log2; t += nwarps) {
     const u64 b = t >> split_log2;
     const u32 part = (u32)t & ((1u << split_log2) - 1u);
-    if (bs_time_up(P.budget_ns, t_start, W.status, lane)) break;
+    if (P.budget_ns && bs_time_up(P.budget_ns, W.start, W.status, lane)) break;
     const u64 hi = blk0 + b;
     u32 a[BS_M], z[BS_NSIG > 0 ? BS_NSIG : 1], dn, up;
 #pragma unroll
@@ -741,7 +762,8 @@ __device__ __forceinline__ void bs_kernel_body(const BsParams& P, const u64* __r
     }
     if (lane == 0) {
       if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
-      if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); task = ~0ull; }
+      if (P.budget_ns && (phase == 2 ? bs_run_late(P.budget_ns, W.start, W.status)
+                                     : bs_late(P.budget_ns, t_start, W.status))) task = ~0ull;
     }
     task = __shfl_sync(0xffffffffu, task, 0);
     u64 prefix;
@@ -982,7 +1004,8 @@ __device__ __forceinline__ void bs_kernel_grad_body(
     }
     if (lane == 0) {
       if constexpr (phase == 0) task = atomicAdd(W.counter, 1ull);
-      if (P.budget_ns && bs_timer() - t_start > P.budget_ns) { atomicOr(W.status, 1u); task = ~0ull; }
+      if (P.budget_ns && (phase == 2 ? bs_run_late(P.budget_ns, W.start, W.status)
+                                     : bs_late(P.budget_ns, t_start, W.status))) task = ~0ull;
     }
     task = __shfl_sync(0xffffffffu, task, 0);
     u64 prefix;
@@ -1265,11 +1288,11 @@ __device__ __forceinline__ void bs_fold_body(const BsParams& P, const BsFoldPara
   const u64 nblk = P.n_tasks >> BS_BLK, blk0 = P.task_lo >> BS_BLK;
   const u64 step = TEAM ? (u64)gridDim.x : (u64)gridDim.x * (BS_MERGE_NTHR / 32);
   const u64 m_mid = Q.mid[lane];
-  const u64 t_start = bs_timer();
   // lane l < BS_BLK: arc l of the block; lanes: arcs `lane` and `lane + 32` above it
   facc accP = facc{u128{0ull, 0ull}, 0, 0}, accA = accP, accB = accP, accA2 = accP, accB2 = accP;
   for (u64 b = TEAM ? blockIdx.x : (u64)blockIdx.x * (BS_MERGE_NTHR / 32) + warp; b < nblk; b += step) {
-    if (!TEAM && bs_time_up(P.budget_ns, t_start, W.status, lane)) break;
+    if (P.budget_ns && (TEAM ? bs_block_time_up(P.budget_ns, W.start, W.status)
+                             : bs_time_up(P.budget_ns, W.start, W.status, lane))) break;
     const u64 hi = blk0 + b;
     const uint2 m = W.cmask[b * 32 + lane];
     if (!__any_sync(0xffffffffu, m.x | m.y)) continue;   // (the same in every warp of a team)
@@ -1381,7 +1404,7 @@ struct BMerge {
   u64* key; u32* id_of;
   u32* net; u64* rep; u32* hist; u64* cmass; ulonglong2* csum;
   uint2* cmask; uint2* ent;
-  u64* n_classes; u64* ticket;
+  u64* n_classes; u64* ticket; u64* start;   // start: when the run began (bs_run_late)
   u64 n_blocks;
   // few blocks: 2^split_log2 warps share one in the first (its words and its
   // p-vectors), `parts` in the second launch (its p-vectors)
@@ -1949,11 +1972,13 @@ __device__ __forceinline__ void bsb_merge_block(const BGraph* __restrict__ B, in
   }
 }
 extern "C" __global__ void __launch_bounds__(BSB_MNTHR) BSB_SCATTER(
-    const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u32* status) {
+    const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u32* status,
+    u64 budget_ns) {
   __shared__ mx s_hi[BSB_MNTHR / 32][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (bs_warp_given_up(status, lane)) return;
   for (u64 v = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; v < A.n_blocks * A.parts; v += (u64)gridDim.x * (BSB_MNTHR / 32)) {
+    if (budget_ns && bs_time_up(budget_ns, A.start, status, lane)) break;
     const u64 t = v / A.parts;
     const int part = (int)(v - t * A.parts);
     u32 left = A.cmask[t * 32 + lane].y;
@@ -1984,10 +2009,11 @@ extern "C" __global__ void __launch_bounds__(BSB_MNTHR) BSB_SCATTER(
 #if BSB_GRAD
 extern "C" __global__ void __launch_bounds__(BSB_MNTHR) bs_batch_grad_p3(
     const BGraph* __restrict__ graphs, int G, int K, const mx* __restrict__ pt, const BMerge A, u64* limbs,
-    const u32* status) {
+    u32* status, u64 budget_ns) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (bs_warp_given_up(status, lane)) return;
   for (u64 t = (u64)blockIdx.x * (BSB_MNTHR / 32) + warp; t < A.n_blocks * K; t += (u64)gridDim.x * (BSB_MNTHR / 32)) {
+    if (budget_ns && bs_time_up(budget_ns, A.start, status, lane)) break;
     const u64 b = t / K;
     const int k = (int)(t - b * K);
     const uint2 m = A.cmask[b * 32 + lane];

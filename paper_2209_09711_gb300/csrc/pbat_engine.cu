@@ -817,6 +817,7 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   const size_t o_stats = off; off = up16(off + 3 * 8);
   const size_t o_list_n = off; off = up16(off + 8);     // number of classes and their ticket
   const size_t o_counter2 = off; off = up16(off + 8);
+  const size_t o_start = off; off = up16(off + 8);      // when a merged run began (time limit)
   const size_t o_out_n = off; off = up16(off + (size_t)(m + 1) * 8);
   const size_t limbs_bytes = J->bs ? (size_t)n_acc * 8 * 8 : 0;
   const size_t o_out_limbs = off; off = up16(off + limbs_bytes);
@@ -885,6 +886,7 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   J->W.cls = (unsigned int*)(d + o_cls);
   J->W.list_n = (unsigned long long*)(d + o_list_n);
   J->W.counter2 = (unsigned long long*)(d + o_counter2);
+  J->W.start = (unsigned long long*)(d + o_start);
   J->d_wmid = (u128*)(d + o_wmid);
   J->h_region = h + h_region;
   J->h_acc = (dd*)(h + h_acc);

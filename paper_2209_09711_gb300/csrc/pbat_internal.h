@@ -61,6 +61,7 @@ struct DevWork {
   unsigned int* list;
   unsigned long long* list_n;
   unsigned long long* counter2;
+  unsigned long long* start;
   unsigned long long* key;
   unsigned long long* cmass;
   unsigned int* hist;

@@ -134,12 +134,12 @@ def _openers(src, at):
 def test_a_warp_reads_the_clock_in_one_lane(pb):
     """The time limit: what follows a check are collectives of the whole warp,
     so one lane decides for all.  Every comparison with the clock is made by
-    lane 0 alone (the kernels are not run for this)."""
+    lane 0 or thread 0 alone (the kernels are not run for this)."""
     for src in _merged_sources(pb):
-        places = [m.start() for m in re.finditer(r"bs_timer\(\) -", src)]
+        places = [m.start() for m in re.finditer(r"bs_timer\(\) -|(?<!bool )(?<!return )bs_(?:run_)?late\(", src)]
         assert places
         for at in places:
-            assert any("lane == 0" in o for o in _openers(src, at)), src[at - 200:at + 60]
+            assert any("lane == 0" in o or "threadIdx.x == 0" in o for o in _openers(src, at)), src[at - 200:at + 60]
 
 
 def test_a_block_or_a_warp_reads_the_status_in_one_thread(pb):
@@ -252,6 +252,38 @@ def test_more_classes_than_the_table_holds(pb):
         res = plan.read()
         assert res.stats[5] == 1
         assert res.Nk == want.Nk and _same(res.R, want.R, 1e-12 * want.R)
+
+
+@pytest.mark.gpu
+def test_time_limit_of_merged_runs(pb):
+    """A limit far below the run's length ends merged runs, plain, with the
+    gradient and in batches, with the error that says so; the next call is
+    right.  So does one that no launch of the run reaches by itself: the
+    launches count from the first one's start."""
+    net = synth.workload_random_24_40()
+    for grad in (False, True):
+        opt = dict(autotune=0, launches=2, walk_bits=6, prune=2)
+        with pytest.raises(pb.PbatError, match="PBAT_ETIMEOUT"):
+            pb.reliability_net(net, grad=grad, opts=pb.options(time_budget_s=1e-9, **opt))
+        for _ in range(2):
+            res = pb.reliability_net(net, grad=grad, opts=pb.options(time_budget_s=10.0, **opt))
+        assert res.stats[5] == (3 if grad else 2) and sum(res.Nk) == sum(pb.reliability_net(net).Nk)
+        if grad:   # (about a fifth, half and 0.3 of the run)
+            with pytest.raises(pb.PbatError, match="PBAT_ETIMEOUT"):
+                pb.reliability_net(net, grad=True, opts=pb.options(time_budget_s=0.7e-9 * res.stats[4], **opt))
+    nets, pvecs = synth.workload_batched()
+    for grad in (False, True):
+        with pytest.raises(pb.PbatError, match="PBAT_ETIMEOUT"):
+            pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(autotune=0, time_budget_s=1e-9))
+        for _ in range(2):
+            o = pb.options(autotune=0, time_budget_s=10.0)
+            R, Nk, _ = pb.reliability_batched(nets, pvecs, grad=grad, opts=o)
+        if grad:   # (the walk takes 0.8 of the run, the fold after it 0.1)
+            with pytest.raises(pb.PbatError, match="PBAT_ETIMEOUT"):
+                pb.reliability_batched(nets, pvecs, grad=True,
+                                       opts=pb.options(autotune=0, time_budget_s=0.92e-9 * o.stats[4]))
+        one = pb.reliability_net(nets[0], p=pvecs[0][3], grad=False)
+        assert Nk[0] == one.Nk and _same(R[0][3], one.R, 1e-12 * one.R)
 
 
 @pytest.mark.gpu
