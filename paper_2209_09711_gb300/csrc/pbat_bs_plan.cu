@@ -559,6 +559,15 @@ static void bs_smaller_walk(const GraphIn& g, BsPlan& bp, const double* p_for_gr
   bp = std::move(best);
 }
 
+int bs_space(const pbat_options& o, int free_bits) {
+  const unsigned long long width = o.range_hi - o.range_lo;
+  return o.range_bits > 0 && width > 1 ? free_bits + 64 - __builtin_clzll(width - 1) : free_bits;
+}
+
+static unsigned long long plan_items(const BsPlan& bp, const pbat_options& o) {
+  return bp.r > 0 ? (o.range_hi - o.range_lo) << (bp.d - bp.r) : 1ull << bp.d;
+}
+
 static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
                          const double* p_for_grad, bool one_by_one);
 
@@ -566,9 +575,11 @@ int bs_make_plan(const GraphIn& g, const pbat_options& o, int nthr, BsPlan& bp,
                  const double* p_for_grad) {
   if (fault_at("plan")) return fail(PBAT_EINVAL, "injected fault: planning");
   const int rc = bs_plan_roles(g, o, nthr, bp, p_for_grad, false);
-  // items that cannot be merged keep the walk length of a one-launch run
+  // items that cannot be merged -- by their signatures, or as there are too many
+  // (wide ranges of many bits) -- keep the walk length of a one-launch run
   const bool lengths_free = o.walk_bits < 0 && o.prefix_bits < 0 && o.prune && o.launches != 1;
-  if (rc || bp.nsig >= 0 || !lengths_free) return rc;
+  const bool too_many = !rc && !bp.merge && plan_items(bp, o) >= kMergeItems;
+  if (rc || !lengths_free || (bp.nsig >= 0 && !too_many)) return rc;
   bp = BsPlan();
   return bs_plan_roles(g, o, nthr, bp, p_for_grad, true);
 }
@@ -596,9 +607,15 @@ static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPl
     // (3: 62 / 102, 8: 54 / 137); 27 arcs merged L = 3 19 / 46, in one launch L =
     // 5 19 / 37; 26 arcs merged L = 3 15 / 37, one launch L = 6 13 / 24 (4: 18 /
     // 38); 23 arcs one launch L = 3 10 / 20 (1: 16 / 33, 6: 15 / 31).
-    const bool merge = free_bits >= (p_for_grad ? 18 : 17);
-    bp.L = merge ? std::min(lmax, std::max(free_bits - 24, std::min(6, (free_bits - 6) / 3)))
-                 : std::max(0, std::min(6, free_bits - 10));
+    // Of a range, with the arcs that its width stands for (36 arcs, the 2^16
+    // divisions of 16 bits, as if it were one division: 43 / 73 ms, in one launch
+    // as below 1.6 / 3.8), but leaving ten prefix arcs outside it for whole merge
+    // blocks (32 arcs, the 2^12 divisions of 12 bits: L = 5 193 / 285 us, 0 74 / 125).
+    const int space = bs_space(o, free_bits);
+    const bool merge = space >= (p_for_grad ? 18 : 17);
+    const int rule = std::min(std::min(6, (space - 6) / 3), std::max(0, free_bits - 10));
+    bp.L = merge ? std::min(lmax, std::max(space - 24, rule))
+                 : std::max(0, std::min(6, space - 10));
   } else {
     // every item walked by itself: about 2^11 of them, measured best on GB300
     // for 27..40 arcs (larger items amortise the per-item epilogue, which is
@@ -694,7 +711,7 @@ static int bs_plan_roles(const GraphIn& g, const pbat_options& o, int nthr, BsPl
   bp.low = std::min(5, bp.d - r);
   bp.mid = std::min(5, bp.d - r - bp.low);
   if (o.prune && !(bp.pex >> (top + bp.low + bp.mid))) bs_generate_sig(g, bp);
-  const unsigned long long items = r > 0 ? (o.range_hi - o.range_lo) << (bp.d - r) : 1ull << bp.d;
+  const unsigned long long items = plan_items(bp, o);
   bp.merge = bp.nsig >= 0 && o.launches != 1 && bp.d - r <= 24 && items > 0 && items <= kMaxMergeItems &&
              items >> (bp.low + bp.mid) <= kMaxMergeBlocks && (o.launches == 2 || items >= kMergeItems);
   return PBAT_OK;

@@ -42,6 +42,10 @@ constexpr unsigned long long kMergeItems = 1ull << 13;
 constexpr unsigned long long kMaxMergeItems = 1ull << 24;   // a slot number for each in the fused kernel
 constexpr unsigned long long kMaxMergeBlocks = 1ull << 14;
 
+// log2 of the items that a walk of no arcs would leave, rounded up: the arcs
+// outside the range that are not lane or thread arcs, and the range's width.
+int bs_space(const pbat_options& o, int free_bits);
+
 // Plan one network for the bit-sliced kernels (Sec. 4.3 equal division:
 // lane, thread, walk and prefix arcs, range arcs on top) and generate its
 // connectivity program.  p_for_grad: the reliabilities when planning the

@@ -29,6 +29,7 @@
 #include <vector>
 
 #include "pbat.h"
+#include "pbat_bs_plan.h"
 #include "pbat_engine.h"
 #include "pbat_internal.h"
 #include "pbat_nvtx.h"
@@ -637,8 +638,8 @@ static int autotune(const GraphIn& g, const double* p, bool grad, pbat_options& 
   for (const bool merge : {true, false}) {
     if (merge ? (!mode || o.launches == 1) : best.L >= 0) continue;
     // merged: around the planner's choice (see bs_plan_roles)
-    const int mid = (free_bits - 6) / 3;
-    const int lo = merge ? std::max({0, free_bits - 24, mid - 3}) : std::max(0, lmax - (large ? 2 : 6));
+    const int space = bs_space(o, free_bits), mid = (space - 6) / 3;
+    const int lo = merge ? std::max({0, space - 24, mid - 3}) : std::max(0, lmax - (large ? 2 : 6));
     std::vector<pbat_options> cands;
     for (int L = lo; L <= (merge ? std::min(lmax, mid + 1) : lmax); ++L)
       for (int nt : nts)

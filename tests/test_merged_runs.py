@@ -104,6 +104,33 @@ def test_signature_is_the_residual_network(pb, directed, prune):
                 assert (sig[i] == sig[j]) == (res[i] == res[j]), (seed, i, j)
 
 
+@pytest.mark.parametrize("m, bits, lo, hi, items_log2, merged", [
+    # as many items as their walks are meant to leave, whatever the division:
+    # the whole space, one division of it, an eighth in several divisions
+    (36, 0, 0, 0, 20, True), (36, 3, 1, 2, 18, True), (39, 3, 0, 8, 23, True), (36, 6, 8, 16, 18, True),
+    # not fewer than ten prefix arcs outside the range, for whole merge blocks
+    (32, 12, 0, 1 << 12, 22, True), (34, 12, 0, 1 << 12, 22, True), (40, 10, 0, 1 << 10, 24, True),
+    # wide ranges of many bits: more than 2^14 blocks of items, or more than 2^24
+    # items -- one launch, and its long walks
+    (36, 16, 0, 1 << 16, 16, False), (36, 16, 1 << 15, 1 << 16, 15, False), (36, 20, 0, 1 << 18, 18, False),
+    (48, 10, 0, 1 << 10, 28, False),
+    # narrow ranges: about 2^10 items in one launch, fewer where there are no more
+    (36, 16, 7, 9, 10, False), (36, 24, 5, 6, 2, False), (30, 10, 0, 3, 10, False),
+])
+@pytest.mark.parametrize("grad", [False, True])
+def test_walk_length_of_ranges(pb, m, bits, lo, hi, items_log2, merged, grad):
+    """The planner's walk length follows the number of items of the range
+    asked for, not that of one division."""
+    tail, head, rng = synth.random_connected_undirected(12, m, 31)
+    net = synth.Network(12, tail, head, synth.uniform_p(rng, m, 0.7, 0.95), 0, 11)
+    src = pb.kernel_source(net, pb.options(range_bits=bits, range_lo=lo, range_hi=hi), grad=grad)
+    D = {k: int(v) for k, v in re.findall(r"#define (BS_\w+) (-?\d+)", src)}
+    width = (hi - lo) if bits else 1
+    items = width << (D["BS_D"] - bits)
+    assert (items - 1).bit_length() == items_log2, D
+    assert D["BS_MERGE"] == merged
+
+
 def _merged_sources(pb):
     """The kernels of a merged run, of one network and of a batch, R and gradient."""
     tail, head, rng = synth.random_connected_undirected(12, 30, 77)
