@@ -967,7 +967,10 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  u32* rel = (u32*)(s_nk + (BSB_NTHR / 32) * 65) + (threadIdx.x >> 5) * 33;   // merged: counts below the prefix\n"
       "  for (int i = lane; i < 65; i += 32) nkw[i] = 0ull;\n"
       "  int cur = -1;   // network whose counts nkw holds\n";
+  // (t0 is read here, limit or not: without a read of the clock at this place
+  // the compiler's schedule of the loop made it 49 -> 56 us, 2 networks x 17)
   kern += E.merged ?
+      "  const u64 t0 = budget_ns ? bs_run_start(A.start) : bs_timer();\n"
       "  rel[lane] = 0u;\n"
       "  if (bs_warp_given_up(status, lane)) return;\n"
       "  const u64 n_cls = *A.n_classes, n_warps = (u64)gridDim.x * (BSB_NTHR / 32);\n"
@@ -976,7 +979,12 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       "  for (;;) {\n"
       "    const u64 cls = next;\n"
       "    if (cls >= n_cls) break;\n"
-      "    if (budget_ns && bs_time_up(budget_ns, A.start, status, lane)) break;\n"
+      "    if (budget_ns) {\n"
+      "      int up = 0;\n"
+      "      __syncwarp();\n"
+      "      if (lane == 0) up = bs_late(budget_ns, t0, status);\n"
+      "      if (__shfl_sync(0xffffffffu, up, 0)) break;\n"
+      "    }\n"
       "    next = ~0ull;\n"
       "    if (n_cls > n_warps) {\n"
       "      if (lane == 0) next = n_warps + atomicAdd(A.ticket, 1ull);\n"

@@ -186,7 +186,7 @@ struct BsWork {
   u32* list;
   u64* list_n;
   u64* counter2;
-  u64* start;   // and when it began (bs_run_late)
+  u64* start;   // and when it began (bs_run_start)
   // per slot: the signature (0: unused), the summed mass of the class's items
   // in two chunks, their number by popcount (BS_HIST each), one of them, and
   // the sum S of that one
@@ -231,14 +231,17 @@ __device__ __forceinline__ bool bs_late(u64 budget_ns, u64 t_start, u32* status)
 // The launches of a merged run all count its time limit from when the first
 // warp of the first one asked, kept beside the status.  (Another SM's clock may
 // have been read a little later than this one's.)
-__device__ __forceinline__ bool bs_run_late(u64 budget_ns, u64* start, u32* status) {
+__device__ __forceinline__ u64 bs_run_start(u64* start) {
   u64 first = *(volatile u64*)start;
   if (!first) {
     const u64 now = bs_timer();
     first = atomicCAS(start, 0ull, now);
     if (!first) first = now;
   }
-  return bs_late(budget_ns, first, status);
+  return first;
+}
+__device__ __forceinline__ bool bs_run_late(u64 budget_ns, u64* start, u32* status) {
+  return bs_late(budget_ns, bs_run_start(start), status);
 }
 // Whether the time is up, the same answer in every lane of a warp or every
 // thread of a block: one lane reads the clock.  The loops that ask go on with
@@ -1404,7 +1407,7 @@ struct BMerge {
   u64* key; u32* id_of;
   u32* net; u64* rep; u32* hist; u64* cmass; ulonglong2* csum;
   uint2* cmask; uint2* ent;
-  u64* n_classes; u64* ticket; u64* start;   // start: when the run began (bs_run_late)
+  u64* n_classes; u64* ticket; u64* start;   // start: when the run began (bs_run_start)
   u64 n_blocks;
   // few blocks: 2^split_log2 warps share one in the first (its words and its
   // p-vectors), `parts` in the second launch (its p-vectors)
