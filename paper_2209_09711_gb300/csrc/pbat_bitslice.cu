@@ -800,6 +800,7 @@ struct BMergeHost {
 constexpr int kBsbThreads = 128;
 constexpr int kBsbMinBlocks = 4;  // default launch bounds: 4 blocks of 128 threads, <= 128 registers
 constexpr int kBsbMaxWalk = 5;  // 2^L connectivity words per thread staged in shared memory
+constexpr int kBsbMergedWalk = 4;
 constexpr int kBsbLimbs = 8;    // 32-bit chunks of a 256-bit value at scale 2^250, in 64-bit atomics
 constexpr int kBsbMaxGraphs = 256;
 constexpr unsigned long long kBsbMaxItems = 1ull << 24;   // merged: of all networks together
@@ -880,12 +881,12 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
   E.K = K;
   E.plans.resize(G);
   items.assign(G, 0ull);
-  for (int i = 0; i < G; ++i) {
+  auto plan = [&](int i, int walk_bits) {
     GraphIn g{graphs[i].n_nodes, graphs[i].n_arcs, graphs[i].tail, graphs[i].head,
               graphs[i].directed, graphs[i].source, graphs[i].sink};
     pbat_options oo;
     pbat_options_init(&oo);
-    oo.walk_bits = std::min(o.walk_bits >= 0 ? o.walk_bits : kBsbMaxWalk, kBsbMaxWalk);
+    oo.walk_bits = walk_bits;
     oo.prune = o.prune;   // prune == 2: prune-aware prefix arcs
     // the gradient module divides walk-arc sums by p and 1 - p: only arcs
     // eligible under every p-vector may be walk arcs
@@ -894,12 +895,26 @@ static int bsb_source(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       pe.resize(g.m);
       for (int a = 0; a < g.m; ++a) pe[a] = E.elig[i][a] == '1' ? 0.5 : 0.0;
     }
-    int rc = bs_make_plan(g, oo, kBsbThreads, E.plans[i], E.grad ? pe.data() : nullptr);
-    if (rc) return rc;
+    E.plans[i] = BsPlan();
+    return bs_make_plan(g, oo, kBsbThreads, E.plans[i], E.grad ? pe.data() : nullptr);
+  };
+  auto plan_all = [&](int walk_bits) {
+    int rc = PBAT_OK;
+    for (int i = 0; i < G && !rc; ++i) rc = plan(i, walk_bits);
+    E.merged = !rc && !E.per_item && bsb_mergeable(E.plans, o);
+    return rc;
+  };
+  // untuned and merged: shorter walks than one by one (GB300, 20 networks x 7
+  // p-vectors, L = 5 / 4 / 3: gradient 551 / 358 / 414 us, R 157 / 135 / 151; 64 x
+  // 16, R 3.0 / 2.7 / 3.4 ms), where they leave no more items than can be merged
+  const bool merge = o.walk_bits < 0 && !o.autotune && o.prune && !E.per_item;
+  int rc = plan_all(merge ? kBsbMergedWalk : std::min(o.walk_bits >= 0 ? o.walk_bits : kBsbMaxWalk, kBsbMaxWalk));
+  if (!rc && merge && !E.merged) rc = plan_all(kBsbMaxWalk);
+  if (rc) return rc;
+  for (int i = 0; i < G; ++i) {
     items[i] = 1ull << E.plans[i].d;
     E.lmax = std::max(E.lmax, E.plans[i].L);
   }
-  E.merged = !E.per_item && bsb_mergeable(E.plans, o);
   for (const BsPlan& bp : E.plans) E.nsig_max = std::max(E.nsig_max, bp.nsig);
   E.order.resize(G);
   for (int i = 0; i < G; ++i) E.order[i] = i;
@@ -1685,11 +1700,6 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
         ob.prune = mode;
         ob.occupancy = occ;
       }
-    } else if (o.walk_bits < 0 && o.prune && !per_item) {
-      // untuned and merged: shorter walks than one by one (GB300, 20 networks
-      // x 7 p-vectors, L = 5 / 4 / 3: gradient 551 / 358 / 414 us, R 157 / 135 /
-      // 151; 64 x 16, R 3.0 / 2.7 / 3.4 ms)
-      ob.walk_bits = 4;
     }
     std::unique_ptr<BsBatch> ne(new BsBatch());
     ne->key = key;

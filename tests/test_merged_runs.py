@@ -131,6 +131,25 @@ def test_walk_length_of_ranges(pb, m, bits, lo, hi, items_log2, merged, grad):
     assert D["BS_MERGE"] == merged
 
 
+@pytest.mark.parametrize("m, n, walk, merged", [(26, 9, 4, 1), (39, 9, 5, 1), (40, 9, 5, 0), (34, 12, 5, 0)])
+@pytest.mark.parametrize("grad", [False, True])
+def test_walk_length_of_batches(pb, m, n, walk, merged, grad):
+    """Untuned batches walk four arcs where they are merged, five where that
+    makes the items few enough to be (39 arcs), and five as ever where they are
+    not: too many items (40 arcs), too long a signature (directed, 12 nodes)."""
+    net = synth.random_small(8600 + m, n=n, m=m, directed=n == 12, p_lo=0.2, p_hi=0.9)
+    small = synth.random_small(8700, n=6, m=12, p_lo=0.2, p_hi=0.9)
+    # (the sum of the items is limited: 39 arcs reach the limit alone)
+    nets = [net] if m == 39 else [net, small]
+    o = pb.options(autotune=0)
+    src = (pb.batch_grad_kernel_source(nets, [[g.p] * 3 for g in nets], o) if grad
+           else pb.batch_kernel_source(nets, 3, o))
+    assert f"#define BSB_LMAX {walk}\n" in src and f"#define BSB_MERGE {merged}\n" in src
+    # without the prune nothing is merged
+    src = pb.batch_kernel_source(nets, 3, pb.options(autotune=0, prune=0))
+    assert "#define BSB_LMAX 5\n" in src and "#define BSB_MERGE 0\n" in src
+
+
 def _merged_sources(pb):
     """The kernels of a merged run, of one network and of a batch, R and gradient."""
     tail, head, rng = synth.random_connected_undirected(12, 30, 77)
