@@ -9,6 +9,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -837,7 +838,12 @@ struct BsBatch {
   bool static_ready = false;
   size_t o_perm = 0, o_poff = 0, o_p = 0, n_p = 0;
   size_t smem1 = 0, o_nib = 0, o_mid = 0, o_fold = 0, key_bytes = 0;
-  Scratch* mscr = nullptr;
+  // the class memory that M points into, allocated apart: it is given back
+  // when other batches need it (bsb_trim)
+  void* mmem = nullptr;
+  size_t mbytes = 0;
+  std::function<void(char*)> place;   // M's pointers, given the class memory
+  unsigned long long used = 0;        // by the last call that used this batch
   BMergeHost M{};
 };
 
@@ -851,11 +857,66 @@ static bool bsb_mergeable(const std::vector<BsPlan>& plans, const pbat_options& 
   return items <= kBsbMaxItems;
 }
 
+// Class memory that the kept batches may hold together: up to about 2 GB each
+// (2^24 items), so that a sweep over many sets of networks does not fill the
+// GPU; those used longest ago give theirs back first.
+constexpr size_t kBsbKeepBytes = (size_t)4 << 30;
+
 static std::mutex g_bsb_mu;
 static std::vector<BsBatch*> g_bsb;
+static unsigned long long g_bsb_calls = 0;
 static std::set<std::string> g_bsb_unmergeable;   // batches whose classes did not fit
 
 static size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
+
+// (the captured graph holds the memory's address, so it goes with it)
+static void bsb_drop_class_memory(BsBatch& E) {
+  if (E.exec) cudaGraphExecDestroy(E.exec);
+  E.exec = nullptr;
+  if (E.mmem) cudaFree(E.mmem);
+  E.mmem = nullptr;
+}
+static void bsb_release(BsBatch& E) {
+  bsb_drop_class_memory(E);
+  scratch_release(E.scr);
+  E.scr = nullptr;
+}
+// Takes class memory from batches that no call is using, longest unused first,
+// until the kept ones hold at most `keep` bytes together.
+static void bsb_trim(int device, size_t keep) {
+  for (;;) {
+    BsBatch* old = nullptr;
+    {
+      std::lock_guard<std::mutex> lk(g_bsb_mu);
+      size_t held = 0;
+      for (auto* e : g_bsb) {
+        if (e->device != device || !e->mmem) continue;
+        held += e->mbytes;
+        if (!e->busy && (!old || e->used < old->used)) old = e;
+      }
+      if (!old || held <= keep) return;
+      old->busy = true;
+    }
+    bsb_drop_class_memory(*old);
+    std::lock_guard<std::mutex> lk(g_bsb_mu);
+    old->busy = false;
+  }
+}
+static int bsb_class_memory(BsBatch& E) {
+  if (!E.merged || E.mmem) return PBAT_OK;
+  bsb_trim(E.device, kBsbKeepBytes - std::min(kBsbKeepBytes, E.mbytes));
+  if (cudaMalloc(&E.mmem, E.mbytes) != cudaSuccess) {
+    cudaGetLastError();
+    bsb_trim(E.device, 0);
+    if (cudaMalloc(&E.mmem, E.mbytes) != cudaSuccess) {
+      cudaGetLastError();
+      E.mmem = nullptr;
+      return fail(PBAT_ENOMEM, "cudaMalloc of %zu B failed", E.mbytes);
+    }
+  }
+  E.place((char*)E.mmem);
+  return PBAT_OK;
+}
 
 static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const pbat_options& o,
                       const DeviceInfo& dev, const std::vector<unsigned long long>& items);
@@ -1199,11 +1260,12 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
     const size_t rep = take(8ull * M.cap), hist = take(4ull * M.cap * M.hist_stride);
     const size_t cmass = take(16ull * M.cap * K), csum = take(E.grad ? 16ull * M.cap * K : 0);
     const size_t cmask = take(8ull * 32 * blocks), ent = take(8ull * E.total);
-    if ((rc = scratch_acquire(dev.device, mo, 0, &E.mscr))) return rc;
-    char* d = (char*)E.mscr->dmem;
+    E.mbytes = mo;
+    E.place = [=, &M](char* d) {
+      M.key = d + key; M.id_of = d + id_of; M.net = d + net; M.rep = d + rep; M.hist = d + hist;
+      M.cmass = d + cmass; M.csum = d + csum; M.cmask = d + cmask; M.ent = d + ent;
+    };
     char* u = (char*)E.scr->dmem;
-    M.key = d + key; M.id_of = d + id_of; M.net = d + net; M.rep = d + rep; M.hist = d + hist;
-    M.cmass = d + cmass; M.csum = d + csum; M.cmask = d + cmask; M.ent = d + ent;
     M.n_classes = u + E.o_counter + 8; M.ticket = u + E.o_counter + 16;
     M.start = u + E.o_counter + 24;
     M.nib = u + E.o_nib; M.mid = u + E.o_mid; M.fold = u + E.o_fold;
@@ -1624,9 +1686,8 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
   auto run = [&](const pbat_options& t) {
     BsBatch T;
     new_batch(T);
-    if (bsb_build(T, G, graphs, K, t, dev) != PBAT_OK) {
-      scratch_release(T.scr);
-      scratch_release(T.mscr);
+    if (bsb_build(T, G, graphs, K, t, dev) != PBAT_OK || bsb_class_memory(T) != PBAT_OK) {
+      bsb_release(T);
       clear_error();
       return;
     }
@@ -1650,8 +1711,7 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
       cudaGetLastError();
       clear_error();
     }
-    scratch_release(T.scr);
-    scratch_release(T.mscr);
+    bsb_release(T);
   };
   std::vector<pbat_options> cands;
   for (int mode : (o.prune == 1 ? std::vector<int>{1, 2} : std::vector<int>{o.prune}))
@@ -1711,8 +1771,7 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
     }
     int rc = bsb_build(*ne, G, graphs, K, ob, dev);
     if (rc) {
-      scratch_release(ne->scr);
-      scratch_release(ne->mscr);
+      bsb_release(*ne);
       return rc;
     }
     E = ne.release();
@@ -1722,8 +1781,10 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
   auto done = [&](int code) {
     std::lock_guard<std::mutex> lk(g_bsb_mu);
     E->busy = false;
+    E->used = ++g_bsb_calls;
     return code;
   };
+  if (const int rc = bsb_class_memory(*E)) return done(rc);
   const unsigned long long budget = o.time_budget_s > 0 ? (unsigned long long)(o.time_budget_s * 1e9) : 0ull;
   char* d = (char*)E->scr->dmem;
   char* h = (char*)E->scr->hmem;
@@ -1778,8 +1839,10 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
     {
       std::lock_guard<std::mutex> lk(g_bsb_mu);
       g_bsb_unmergeable.insert(key);
-      E->busy = false;
+      g_bsb.erase(std::find(g_bsb.begin(), g_bsb.end(), E));
     }
+    bsb_release(*E);
+    delete E;
     return run_batched_bs(G, graphs, K, p, o, st, R_out, Nk_out, key, dev, kernel_ns, elig, dRdp_out, coarse);
   }
   if (*(unsigned int*)(h + E->o_status) & 1u) return done(fail(PBAT_ETIMEOUT, "time budget ran out on the device"));

@@ -401,3 +401,33 @@ def test_merged_batches(pb, vectors, grad):
                 if grad:
                     for x, y in zip(g[i][k], g0[i][k]):
                         assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (net.name, k)
+
+
+@pytest.mark.gpu
+def test_batches_give_their_class_memory_back(pb):
+    """Sets of networks one after another, of about 1 GB of class memory each
+    (38 arcs, 2^24 items): what the library keeps stays bounded, and the first
+    set is answered again, its memory taken and its graph captured anew.  A
+    batch with more classes than fit keeps none of it."""
+    import torch
+    free0 = torch.cuda.mem_get_info()[0]
+    nets = [synth.random_small(8900 + i, n=9, m=38, p_lo=0.3, p_hi=0.95) for i in range(7)]
+    opt = dict(autotune=0, algo=pb.ALGO_BITSLICE)
+    first = []
+    for net in nets + nets[:2]:
+        R, Nk, _ = pb.reliability_batched([net], [[net.p] * 2], opts=pb.options(**opt))
+        first.append((R[0][0], Nk[0]))
+        assert R[0][0] == R[0][1]
+    assert first[:2] == first[7:]
+    one = pb.reliability_net(nets[0], opts=pb.options(autotune=0))
+    assert first[0][1] == one.Nk and _same(first[0][0], one.R, 1e-12 * one.R)
+    held = free0 - torch.cuda.mem_get_info()[0]
+    assert held < (5 << 30), held
+    tail, head, rng = synth.random_connected_undirected(20, 38, 902)
+    net = synth.Network(20, tail, head, synth.uniform_p(rng, 38, 0.7, 0.95), 0, 19)
+    free1 = torch.cuda.mem_get_info()[0]
+    for _ in range(2):
+        R, Nk, _ = pb.reliability_batched([net], [[net.p] * 64], opts=pb.options(**opt))
+        one = pb.reliability_net(net, opts=pb.options(autotune=0, launches=1))
+        assert Nk[0] == one.Nk and _same(R[0][63], one.R, 1e-12 * one.R)
+    assert free1 - torch.cuda.mem_get_info()[0] < (256 << 20)
