@@ -35,8 +35,10 @@
  *   - Environment: PBAT_AUTOTUNE_CACHE names a file that keeps the
  *     autotuner's choices across processes.  PBAT_FAULT, for failure-
  *     detection tests, lists host-side sites to fail ("plan", "compile",
- *     "alloc", "launch", comma-separated): each fails as its real call can,
- *     with the same error code, before any GPU work of that step.
+ *     "alloc", "classes", "launch", comma-separated): each fails as its real
+ *     call can, with the same error code, before any GPU work of that step.
+ *     Without memory for the classes of a merged run ("classes") a call walks
+ *     every work item by itself instead of failing.
  *   - `cuda_stream` is a cudaStream_t (NULL = the legacy default stream).
  *     The calls are synchronous: they return after the results are on the
  *     host.  Calls are re-entrant; concurrent calls from several host

@@ -904,6 +904,7 @@ static void bsb_trim(int device, size_t keep) {
 }
 static int bsb_class_memory(BsBatch& E) {
   if (!E.merged || E.mmem) return PBAT_OK;
+  if (fault_at("classes")) return fail(PBAT_ENOMEM, "injected fault: class memory allocation");
   bsb_trim(E.device, kBsbKeepBytes - std::min(kBsbKeepBytes, E.mbytes));
   if (cudaMalloc(&E.mmem, E.mbytes) != cudaSuccess) {
     cudaGetLastError();
@@ -1730,24 +1731,19 @@ static bool bsb_tune(int G, const pbat_graph* graphs, int K, const double* p, co
   return found;
 }
 
-// R (and N_k) of a batch with the bit-sliced batched kernel; with `elig`
-// (one string of '0'/'1' walk-arc eligibility per network) the gradient
-// module also returns dR/dp in dRdp_out (the layout of p), and lists in
-// *coarse the (network, p-vector) pairs whose R or gradient the
-// fixed-point error bounds cannot certify to 1e-12 (the caller re-runs them
-// exactly).  Returns PBAT_ENOTSUP when the batch is outside the module's
-// limits (the caller then uses the frontier kernel).
 int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, const pbat_options& o,
                    cudaStream_t st, double* R_out, uint64_t* Nk_out, const std::string& key,
                    const DeviceInfo& dev, uint64_t* kernel_ns, const std::vector<std::string>* elig,
-                   double* dRdp_out, std::vector<std::pair<int, int>>* coarse) {
-  NvtxRange nv("pbat batched");
-  if (G > kBsbMaxGraphs) return PBAT_ENOTSUP;
+                   double* dRdp_out, std::vector<std::pair<int, int>>* coarse);
+
+// One batch by one route: merged where it can be, or every item by itself.
+static int run_batched_route(int G, const pbat_graph* graphs, int K, const double* p, const pbat_options& o,
+                             cudaStream_t st, double* R_out, uint64_t* Nk_out, const std::string& key,
+                             const DeviceInfo& dev, uint64_t* kernel_ns, const std::vector<std::string>* elig,
+                             double* dRdp_out, std::vector<std::pair<int, int>>* coarse, bool per_item) {
   BsBatch* E = nullptr;
-  bool per_item = false;
   {
     std::lock_guard<std::mutex> lk(g_bsb_mu);
-    per_item = g_bsb_unmergeable.count(key) != 0;
     for (auto* e : g_bsb)
       if (!e->busy && e->key == key && e->per_item == per_item) { e->busy = true; E = e; break; }
   }
@@ -1907,6 +1903,33 @@ int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, cons
   }
   if (Nk_out) memcpy(Nk_out, nk, sizeof(uint64_t) * E->nk_total);
   return done(PBAT_OK);
+}
+
+// R (and N_k) of a batch with the bit-sliced batched kernel; with `elig`
+// (one string of '0'/'1' walk-arc eligibility per network) the gradient
+// module also returns dR/dp in dRdp_out (the layout of p), and lists in
+// *coarse the (network, p-vector) pairs whose R or gradient the
+// fixed-point error bounds cannot certify to 1e-12 (the caller re-runs them
+// exactly).  Returns PBAT_ENOTSUP when the batch is outside the module's
+// limits (the caller then uses the frontier kernel).
+int run_batched_bs(int G, const pbat_graph* graphs, int K, const double* p, const pbat_options& o,
+                   cudaStream_t st, double* R_out, uint64_t* Nk_out, const std::string& key,
+                   const DeviceInfo& dev, uint64_t* kernel_ns, const std::vector<std::string>* elig,
+                   double* dRdp_out, std::vector<std::pair<int, int>>* coarse) {
+  NvtxRange nv("pbat batched");
+  if (G > kBsbMaxGraphs) return PBAT_ENOTSUP;
+  bool per_item;
+  {
+    std::lock_guard<std::mutex> lk(g_bsb_mu);
+    per_item = g_bsb_unmergeable.count(key) != 0;
+  }
+  int rc = run_batched_route(G, graphs, K, p, o, st, R_out, Nk_out, key, dev, kernel_ns, elig, dRdp_out, coarse, per_item);
+  if (rc == PBAT_ENOMEM && !per_item) {
+    // no room for the classes: every item by itself, which needs the tables only
+    clear_error();
+    rc = run_batched_route(G, graphs, K, p, o, st, R_out, Nk_out, key, dev, kernel_ns, elig, dRdp_out, coarse, true);
+  }
+  return rc;
 }
 
 }  // namespace pbat

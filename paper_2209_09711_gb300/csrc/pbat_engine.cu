@@ -91,9 +91,10 @@ int fail(int code, const char* fmt, ...) {
 void clear_error() { t_last_error.clear(); }
 
 // Host-side fault injection, for failure-detection tests: PBAT_FAULT holds a
-// comma-separated list of sites -- "plan", "compile", "alloc", "launch" --
-// and a listed site fails the way its real call can, with the same error
-// code, before any GPU work of that step.  Nothing on the device is faulted.
+// comma-separated list of sites -- "plan", "compile", "alloc", "launch",
+// "classes" (the class memory of merged runs) -- and a listed site fails the
+// way its real call can, with the same error code, before any GPU work of
+// that step.  Nothing on the device is faulted.
 bool fault_at(const char* site) {
   const char* f = getenv("PBAT_FAULT");
   if (!f || !*f) return false;
@@ -350,6 +351,27 @@ int device_info(DeviceInfo& out) {
 
 static std::vector<Scratch*> g_pool;
 
+// Frees the buffers that no call or plan holds.
+static void scratch_give_back(int device) {
+  std::vector<Scratch*> idle;
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (size_t i = 0; i < g_pool.size();) {
+      if (g_pool[i]->busy || g_pool[i]->device != device) {
+        ++i;
+        continue;
+      }
+      idle.push_back(g_pool[i]);
+      g_pool.erase(g_pool.begin() + i);
+    }
+  }
+  for (Scratch* s : idle) {
+    cudaFree(s->dmem);
+    cudaFreeHost(s->hmem);
+    delete s;
+  }
+}
+
 int scratch_acquire(int device, size_t dbytes, size_t hbytes, Scratch** out) {
   if (fault_at("alloc")) return fail(PBAT_ENOMEM, "injected fault: device scratch allocation");
   {
@@ -368,8 +390,12 @@ int scratch_acquire(int device, size_t dbytes, size_t hbytes, Scratch** out) {
   s->hbytes = std::max<size_t>(hbytes, 1 << 16);
   if (cudaMalloc(&s->dmem, s->dbytes) != cudaSuccess) {
     cudaGetLastError();
-    delete s;
-    return fail(PBAT_ENOMEM, "cudaMalloc of %zu B failed", dbytes);
+    scratch_give_back(device);
+    if (cudaMalloc(&s->dmem, s->dbytes) != cudaSuccess) {
+      cudaGetLastError();
+      delete s;
+      return fail(PBAT_ENOMEM, "cudaMalloc of %zu B failed", dbytes);
+    }
   }
   if (cudaMallocHost(&s->hmem, s->hbytes) != cudaSuccess) {
     cudaGetLastError();
@@ -866,7 +892,20 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
     hoff = up16(hoff + (o_tab_end - o_lane));  // same layout as the device tables
   }
   const size_t hbytes = hoff;
-  if ((rc = scratch_acquire(J->dev.device, dbytes, hbytes, &J->scr))) return rc;
+  if (J->merged && fault_at("classes")) rc = fail(PBAT_ENOMEM, "injected fault: class memory allocation");
+  else rc = scratch_acquire(J->dev.device, dbytes, hbytes, &J->scr);
+  if (rc == PBAT_ENOMEM && J->merged) {
+    // no room for the classes (up to about 200 MB): one launch, which needs little
+    pbat_options one;
+    pbat_options_init(&one);
+    if (opt) one = *opt;
+    one.launches = 1;
+    one.autotune = 0;
+    J.reset();
+    clear_error();
+    return job_create(g, p, grad, &one, out);
+  }
+  if (rc) return rc;
   char* d = (char*)J->scr->dmem;
   char* h = (char*)J->scr->hmem;
   J->W.counter = (unsigned long long*)(d + o_counter);

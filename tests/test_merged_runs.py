@@ -431,3 +431,34 @@ def test_batches_give_their_class_memory_back(pb):
         one = pb.reliability_net(net, opts=pb.options(autotune=0, launches=1))
         assert Nk[0] == one.Nk and _same(R[0][63], one.R, 1e-12 * one.R)
     assert free1 - torch.cuda.mem_get_info()[0] < (256 << 20)
+
+
+@pytest.mark.gpu
+def test_no_room_for_the_classes(pb, monkeypatch):
+    """Where the class memory of a merged run cannot be had, every item is
+    walked by itself, with the same results; a kept plan too."""
+    net = synth.random_small(8950, n=9, m=28, p_lo=0.3, p_hi=0.95)
+    small = synth.random_small(8951, n=6, m=14, p_lo=0.3, p_hi=0.95)
+    nets, pvecs = [net, small], [[net.p] * 3, [small.p] * 3]
+    o = dict(autotune=0)
+    want = [pb.reliability_net(net, grad=g, opts=pb.options(**o)) for g in (False, True)]
+    assert [w.stats[5] for w in want] == [2, 3]
+    monkeypatch.setenv("PBAT_FAULT", "classes")
+    for grad in (False, True):
+        one = pb.reliability_net(net, grad=grad, opts=pb.options(**o))
+        plan = pb.Plan(net, grad=grad, opts=pb.options(launches=2, **o))
+        plan.execute()
+        kept = plan.read()
+        R, Nk, gr = pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(**o))
+        for res in (one, kept):
+            assert res.stats[5] == 1 and res.Nk == want[grad].Nk == Nk[0]
+            assert _same(res.R, want[grad].R, 2 * 2.0**-53 * res.R) and _same(R[0][2], res.R, 2.0**-52)
+            if grad:
+                for x, y, z in zip(res.grad, want[1].grad, gr[0][2]):
+                    assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56) and _same(z, y, 2 * 2.0**-53 * abs(y) + 2.0**-56)
+    monkeypatch.delenv("PBAT_FAULT")
+    for grad in (False, True):
+        res = pb.reliability_net(net, grad=grad, opts=pb.options(**o))
+        assert res.stats[5] == want[grad].stats[5] and res.R == want[grad].R
+        R2, Nk2, _ = pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(**o))
+        assert Nk2 == Nk and _same(R2[0][2], R[0][2], 2.0**-52)
