@@ -419,7 +419,7 @@ static void merge_tables(const double* p, const pbat_options& o, int m, BsLaunch
     sh += bits;
   }
   // the enumerated mass is at most 2^-mass_exp
-  const double mass = range_mass(m, p, o);
+  const double mass = range_mass(p, o);
   P.mass_exp = mass > 0.0 && mass < 1.0 ? std::max(0, -(ilogb(mass) + 1)) : 0;
   bl.mtab.assign(2 * (128 + 32), 0ull);
   block_tables(p, low, bp.low, bp.mid, bl.mtab.data(), bl.mtab.data() + 256);

@@ -471,26 +471,6 @@ struct Job {
 
 static size_t up16(size_t x) { return (x + 15) & ~(size_t)15; }
 
-// Probability mass of the states an enumeration covers: 1 for the whole
-// space, else the mass of the prefixes [range_lo, range_hi) of the first
-// range_bits input arcs (a digit-by-digit sum, O(range_bits)).
-double range_mass(int m, const double* p, const pbat_options& o) {
-  (void)m;
-  if (o.range_bits <= 0) return 1.0;
-  const int r = o.range_bits;
-  auto below = [&](unsigned long long x) {  // mass of prefixes < x (x <= 2^r)
-    if (x >= (1ull << r)) return 1.0L;
-    long double acc = 0.0L, run = 1.0L;
-    for (int i = 0; i < r; ++i) {  // input arc i is bit r-1-i of the prefix
-      const int bit = (int)((x >> (r - 1 - i)) & 1ull);
-      if (bit) acc += run * (1.0L - (long double)p[i]);
-      run *= bit ? (long double)p[i] : 1.0L - (long double)p[i];
-    }
-    return acc;
-  };
-  return (double)(below(o.range_hi) - below(o.range_lo));
-}
-
 int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, Job** out);
 int job_upload(Job* J, cudaStream_t st);
 int job_launch(Job* J, cudaStream_t st);
@@ -756,7 +736,7 @@ int job_create(const GraphIn& g, const double* p, bool grad, pbat_options* opt, 
   J->g.head = J->head_copy.data();
   J->p_copy.assign(p, p + g.m);
   J->opt_copy = o;
-  J->mass = range_mass(g.m, p, o);
+  J->mass = range_mass(p, o);
   if ((rc = device_info(J->dev))) return rc;
   std::vector<u128> wmid;
   int per_sm = 0, nthr = 128;

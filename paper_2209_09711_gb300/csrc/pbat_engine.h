@@ -67,7 +67,6 @@ struct BsMerge {
   int hist = 0;
 };
 
-double range_mass(int m, const double* p, const pbat_options& o);
 int run_single(const GraphIn& g, const double* p, bool grad, pbat_options* opt, void* stream,
                double* R_out, uint64_t* Nk_out, double* dRdp_out);
 
@@ -200,6 +199,28 @@ inline dd limbs256_to_dd(const unsigned long long* limbs) {
   const int e = 64 * (h - 1) - lz - 250;   // the value is t * 2^e
   const double a = (double)(uint64_t)(t >> 75), b = (double)(uint64_t)((t >> 22) & ((1ull << 53) - 1));
   return fast_two_sum(ldexp(a, e + 75), ldexp(b, e + 22));
+}
+
+// Probability mass of the states an enumeration covers: 1 for the whole space,
+// else the mass of the prefixes [range_lo, range_hi) of the first range_bits
+// input arcs.  A sum of blocks of 2^k prefixes, all of them positive, so it is
+// good to a few roundings however small: the difference of the masses below
+// the two ends loses a division of 1e-40 entirely.
+inline double range_mass(const double* p, const pbat_options& o) {
+  if (o.range_bits <= 0) return 1.0;
+  auto block = [&](uint64_t v, int bits) {   // its first `bits` arcs are fixed
+    long double w = 1.0L;
+    for (int i = 0; i < bits; ++i)
+      w *= ((v >> (bits - 1 - i)) & 1) ? (long double)p[i] : 1.0L - (long double)p[i];
+    return w;
+  };
+  long double sum = 0.0L;
+  uint64_t lo = o.range_lo, hi = o.range_hi;
+  for (int bits = o.range_bits; lo < hi; --bits, lo >>= 1, hi >>= 1) {
+    if (lo & 1) sum += block(lo++, bits);
+    if (hi & 1) sum += block(--hi, bits);
+  }
+  return (double)sum;
 }
 
 inline dd dd_recip(double x) {

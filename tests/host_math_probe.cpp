@@ -11,6 +11,7 @@
 //   R <x bits>              dd_recip(x)                  -> <hi bits> <lo bits>
 //   P <n> <p bits> x n      product_table over arcs 0..n-1 -> 2^n lines <hi bits> <lo bits>
 //   T <n> <hi lo bits> x n  byte_table_sums(w, n, out, 1)  -> 1024 lines <value>
+//   G <r> <lo> <hi> <p bits> x r  range_mass of divisions lo..hi-1 -> <bits>
 //   X <hi bits> <lo bits> <scale>  fixed_u64({hi, lo}, scale) -> <value>
 #include <cstdio>
 #include <cstring>
@@ -56,6 +57,18 @@ int main() {
         if (scanf("%llx", &limbs[i]) != 1) return 1;
       const dd r = limbs256_to_dd(limbs);
       printf("%llx %llx\n", bits(r.hi), bits(r.lo));
+    } else if (op == 'G') {
+      pbat_options o{};
+      unsigned long long lo, hi, v;
+      double p[64];
+      if (scanf("%d %llx %llx", &o.range_bits, &lo, &hi) != 3) return 1;
+      o.range_lo = lo;
+      o.range_hi = hi;
+      for (int i = 0; i < o.range_bits; ++i) {
+        if (scanf("%llx", &v) != 1) return 1;
+        p[i] = dbl(v);
+      }
+      printf("%llx\n", bits(range_mass(p, o)));
     } else if (op == 'B') {
       int n, k;
       if (scanf("%d %d", &n, &k) != 2) return 1;

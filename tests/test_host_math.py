@@ -200,3 +200,37 @@ def test_fixed_point_rounding_of_double_doubles(probe):
     for (h, l, sc), (v,) in zip(cases, out):
         exact = (Fraction(h) + Fraction(l)) * 2 ** sc
         assert abs(int(v, 16) - exact) <= 1, (h, l, sc)
+
+
+def test_mass_of_a_range(probe):
+    """The mass of the divisions lo..hi-1, a scale and an error bound of the
+    kernels: good to a few roundings of a double, also where it is far below
+    the mass of the divisions before it."""
+    rng = random.Random(40)
+    cases = []
+    for r in list(range(1, 9)) + [12, 20, 33, 62]:
+        for _ in range(30):
+            near = rng.choice([0.5, 1e-2, 1e-4])
+            p = [rng.choice([near, 1 - near]) * rng.uniform(0.9, 1.0) for _ in range(r)]
+            lo = rng.choice([0, 1, (1 << r) // 2, (1 << r) - 1, rng.randrange(1 << r)])
+            hi = rng.choice([lo, lo + 1, 1 << r, rng.randint(lo, 1 << r)])
+            cases.append((r, lo, max(lo, min(hi, 1 << r)), p))
+    cases.append((12, 1 << 11, (1 << 11) + 1, [0.9999] * 12))
+    out = probe([f"G {r} {lo:x} {hi:x} " + " ".join(f"{_bits(x):x}" for x in p) for r, lo, hi, p in cases])
+    for (r, lo, hi, p), o in zip(cases, out):
+        def below(x):   # exact mass of the divisions before x
+            if x >> r:
+                return Fraction(1)
+            acc, run = Fraction(0), Fraction(1)
+            for i in range(r):
+                f = Fraction(p[i])
+                if (x >> (r - 1 - i)) & 1:
+                    acc += run * (1 - f)
+                    run *= f
+                else:
+                    run *= 1 - f
+            return acc
+        want = below(hi) - below(lo)
+        got = Fraction(_dbl(int(o[0], 16)))
+        # 62 products of up to 62 factors in at least 64 bits, once rounded to 53
+        assert abs(got - want) <= want * (Fraction(1, 1 << 53) + Fraction(128, 1 << 64)), (r, lo, hi)

@@ -462,3 +462,22 @@ def test_no_room_for_the_classes(pb, monkeypatch):
         assert res.stats[5] == want[grad].stats[5] and res.R == want[grad].R
         R2, Nk2, _ = pb.reliability_batched(nets, pvecs, grad=grad, opts=pb.options(**o))
         assert Nk2 == Nk and _same(R2[0][2], R[0][2], 2.0**-52)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("grad", [False, True])
+def test_divisions_of_tiny_mass(pb, grad):
+    """A division of mass 1e-44 that comes after one of 1e-4: the scale of the
+    classes' masses is its own."""
+    tail, head, _ = synth.random_connected_undirected(14, 40, 12)
+    p = [0.9999] * 12 + [0.95] * 28
+    net = synth.Network(14, tail, head, p, 0, 13)
+    for lo in (0, 1, 1 << 11, (1 << 11) + (1 << 10)):
+        opt = dict(range_bits=12, range_lo=lo, range_hi=lo + 1, autotune=0, algo=pb.ALGO_BITSLICE)
+        res = pb.reliability_net(net, grad=grad, opts=pb.options(launches=2, **opt))
+        one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
+        assert res.stats[5] == (3 if grad else 2) and res.Nk == one.Nk
+        assert one.R > 0 and abs(res.R - one.R) <= 1e-15 * one.R, (lo, res.R, one.R)
+        if grad:   # (of the range's mass: the gradient of a fixed arc is R / p or - R / (1 - p))
+            for x, y in zip(res.grad, one.grad):
+                assert abs(x - y) <= 1e-15 * max(abs(y), one.R)
