@@ -206,7 +206,8 @@ void pbat_plan_destroy(pbat_plan plan);
 /* Describe a plan (no device work): out8 = {algo (PBAT_ALGO_FRONTIER or
  * PBAT_ALGO_BITSLICE), lane arcs, thread arcs (0 for the frontier kernel),
  * walk arcs, prefix arcs, threads per block, blocks, 1 if the gradient is
- * computed}. */
+ * computed}.  Threads and blocks are those of the one launch, or of a merged
+ * run's launch that walks the classes. */
 int pbat_plan_describe(pbat_plan plan, int* out8);
 /* Copy the plan's statistics (the pbat_options.stats[8] layout, as filled by
  * the last pbat_plan_read) into stats_out[8]. */

@@ -1337,7 +1337,7 @@ int pbat_plan_describe(pbat_plan plan, int* out8) {
     out8[4] = J->pl.d;
   }
   out8[5] = J->grid_nthr;
-  out8[6] = J->grid;
+  out8[6] = J->merged ? J->grid2 : J->grid;
   out8[7] = J->pl.grad ? 1 : 0;
   return PBAT_OK;
 }

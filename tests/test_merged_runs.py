@@ -481,3 +481,18 @@ def test_divisions_of_tiny_mass(pb, grad):
         if grad:   # (of the range's mass: the gradient of a fixed arc is R / p or - R / (1 - p))
             for x, y in zip(res.grad, one.grad):
                 assert abs(x - y) <= 1e-15 * max(abs(y), one.R)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("grad", [False, True])
+def test_description_of_a_merged_plan(pb, grad):
+    """Blocks of the launch that walks the classes: three nodes leave at most
+    eight signatures, two blocks of four warps, for 2^10 items."""
+    arcs = [(k % 3, (k + 1) % 3) for k in range(20)]
+    net = synth.Network(3, [u for u, _ in arcs], [v for _, v in arcs], [0.5] * 20, 0, 2)
+    for launches, blocks in ((2, 2), (1, 256)):
+        plan = pb.Plan(net, grad=grad, opts=pb.options(launches=launches, walk_bits=0, block_threads=128))
+        plan.execute()
+        assert plan.read().stats[5] == ((3 if grad else 2) if launches == 2 else 1)
+        d = plan.describe()
+        assert d["blocks"] == blocks and d["prefix_bits"] == 10, d
