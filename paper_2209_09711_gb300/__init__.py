@@ -223,7 +223,10 @@ def _graphs(nets):
     lists = [x if isinstance(x, (list, tuple)) else np.asarray(x, dtype=np.int32)
              for net in nets for x in (net.tail, net.head)]
     sizes = [len(x) for x in lists]
-    ends = np.fromiter(chain.from_iterable(lists), np.int32, sum(sizes))
+    try:
+        ends = np.fromiter(chain.from_iterable(lists), np.int32, sum(sizes))
+    except (TypeError, ValueError):   # nodes that are arrays of one element themselves
+        ends = np.concatenate([np.asarray(x, dtype=np.int32).ravel()[:len(x)] for x in lists])
     table = np.zeros(len(nets), dtype=_GRAPH_DTYPE)
     at = ends.ctypes.data + 4 * np.cumsum([0] + sizes[:-1])
     table["tail"], table["head"] = at[0::2], at[1::2]
@@ -241,7 +244,10 @@ def _rows(pv, K):
     if (isinstance(pv, (list, tuple)) and len(pv) == K and all(isinstance(row, (list, tuple)) for row in pv)
             and len({len(row) for row in pv}) == 1):
         # lists of floats: half the time of np.asarray
-        return np.fromiter(chain.from_iterable(pv), np.float64, K * len(pv[0]))
+        try:
+            return np.fromiter(chain.from_iterable(pv), np.float64, K * len(pv[0]))
+        except (TypeError, ValueError):   # deeper lists, elements that are arrays
+            pass
     return np.asarray(pv, dtype=np.float64).reshape(K, -1).ravel()
 
 
