@@ -1211,7 +1211,7 @@ static int bsb_layout(BsBatch& E, int G, const pbat_graph* graphs, int K, const 
       b.tt_off = (int)tt; tt += (size_t)1024 * Kp;
       b.lwex_off = (int)lwex; lwex += (size_t)5 * 32 * Kp;
       b.thwex_off = (int)thwex; thwex += (size_t)5 * 32 * Kp;
-      b.ptex_off = (int)ptex; ptex += (size_t)K * bp.d * 128;
+      b.ptex_off = (int)ptex; ptex += E.merged ? 0 : (size_t)K * bp.d * 128;
       b.out_off = (int)outl; outl += (size_t)K * (1 + 2 * b.m) * kBsbLimbs;
     }
   }

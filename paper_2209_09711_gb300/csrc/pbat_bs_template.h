@@ -1830,7 +1830,6 @@ __device__ __forceinline__ void bsb_finish_grad(
     }
     // ---- prefix factors of p-vector k and the additions to its results
     const mx* tk = pt + Bp->pt_off + (size_t)k * pt_size;
-    const mx* exk = ptex + Bp->ptex_off + ((size_t)k * d << 7);
     const mx wpre = BSB_MERGE ? bs_class_mass(A.cmass + 2 * (cls * K + k), 0)
                               : bsb_prefix_mass(tk, nlev, lev_bits, lev_off, prefix);
     u64* out = gl + (size_t)k * stride * BSB_LIMBS;
@@ -1842,8 +1841,8 @@ __device__ __forceinline__ void bsb_finish_grad(
       bsb_limb_add(out + (1 + 2 * lane) * BSB_LIMBS, mx_prod(wpre, myX), wpre.e);
       bsb_limb_add(out + (2 + 2 * lane) * BSB_LIMBS, mx_prod(wpre, myY), wpre.e);
     }
-    continue;
-#endif
+#else
+    const mx* exk = ptex + Bp->ptex_off + ((size_t)k * d << 7);
     if (lane < m) {
       u128 X = u128{0ull, 0ull}, Y = u128{0ull, 0ull};
       mx f = wpre;
@@ -1869,6 +1868,7 @@ __device__ __forceinline__ void bsb_finish_grad(
       const bool on = (prefix >> j) & 1ull;
       bsb_limb_add(out + ((on ? 1 : 2) + 2 * (lane + 32)) * BSB_LIMBS, mx_prod(f, S), f.e);
     }
+#endif
   }
 }
 #if BSB_MERGE
