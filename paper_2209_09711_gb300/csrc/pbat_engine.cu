@@ -36,7 +36,7 @@
 
 namespace pbat {
 
-size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide);
+size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide, bool lane_tab);
 const void* frontier_kernel_ptr(bool grad, bool wide);
 cudaError_t launch_frontier(bool grad, bool wide, int grid, int nthr, size_t smem,
                             cudaStream_t st, const FrontierParams& P, const u128* wmid,
@@ -246,7 +246,12 @@ int make_plan(const GraphIn& g, const double* p, bool grad, const pbat_options& 
   pl.n_tasks = hi - lo;
   pl.wide = g.n > 32;
   pl.nthr = o.block_threads > 0 ? o.block_threads : 128;
-  pl.smem = frontier_smem_bytes(g.n, m, pl.L, pl.nthr, grad, pl.wide);
+  pl.lane_tab = true;
+  pl.smem = frontier_smem_bytes(g.n, m, pl.L, pl.nthr, grad, pl.wide, true);
+  if (pl.smem > (size_t)dev.smem_optin) {
+    pl.lane_tab = false;
+    pl.smem = frontier_smem_bytes(g.n, m, pl.L, pl.nthr, grad, pl.wide, false);
+  }
   if (pl.smem > (size_t)dev.smem_optin)
     return fail(PBAT_ERANGE, "shared memory %zu B exceeds %d B (lower walk_bits)", pl.smem,
                 dev.smem_optin);
@@ -271,6 +276,7 @@ void build_params(const GraphIn& g, const double* p, const Plan& pl, const pbat_
   P.walk_bits = pl.L;
   P.prefix_bits = pl.d;
   P.prune = pl.prune;
+  P.lane_tab = pl.lane_tab;
   P.task_lo = pl.task_lo;
   P.n_tasks = pl.n_tasks;
   P.budget_ns = o.time_budget_s > 0 ? (unsigned long long)(o.time_budget_s * 1e9) : 0ull;

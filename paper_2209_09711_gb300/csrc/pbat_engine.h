@@ -39,6 +39,7 @@ struct Plan {
   int prune = 1;
   int nthr = 128;
   size_t smem = 0;
+  bool lane_tab = false;   // the gradient's lane masses in shared memory too
   unsigned long long task_lo = 0, n_tasks = 0;
   std::vector<int> perm;  // internal arc position -> input arc index
 };

@@ -215,9 +215,10 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
   off = align16(off + (size_t)nwarps * (1 + m) * sizeof(dd));
   unsigned long long* s_nbins = reinterpret_cast<unsigned long long*>(smem + off);
   if (GRAD) off = align16(off + (size_t)(m + 1) * sizeof(unsigned long long));
-  LaneMass* s_lwx = reinterpret_cast<LaneMass*>(smem + off);   // lane masses without each lane arc
+  // lane masses without each lane arc (from the parameters where they have no room here)
+  LaneMass* s_lwx = reinterpret_cast<LaneMass*>(smem + off);
 
-  if (GRAD)
+  if (GRAD && P.lane_tab)
     for (int i = tid; i < ell * 32; i += nthr) s_lwx[i] = P.lane_w_ex[i >> 5][i & 31];
   for (int i = tid; i < nW; i += nthr) s_wmid[i] = wmid_g[i];
   for (int i = tid; i < nwarps * (1 + m); i += nthr) s_wacc[i] = dd{0.0, 0.0};
@@ -366,7 +367,7 @@ __global__ void __launch_bounds__(256) frontier_kernel(const __grid_constant__ F
         const u128 o = u128{__shfl_xor_sync(0xffffffffu, T.lo, 1 << i), __shfl_xor_sync(0xffffffffu, T.hi, 1 << i)};
         const u128 df = (lane >> i) & 1 ? u128_sub(T, o) : u128_zero();
         int eg;
-        const u128 sg = warp_sum_scaled(df, s_lwx[i * 32 + lane], &eg);
+        const u128 sg = warp_sum_scaled(df, P.lane_tab ? s_lwx[i * 32 + lane] : P.lane_w_ex[i][lane], &eg);
         if (lane == i) {
           X = sg;
           eX = eg;
@@ -432,7 +433,7 @@ __global__ void __launch_bounds__(kReduceThreads) reduce_kernel(DevWork W, int n
   }
 }
 
-size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide) {
+size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide, bool lane_tab) {
   size_t off = 0;
   off = align16(off + ((size_t)1 << L) * sizeof(u128));
   off = align16(off + (size_t)n * nthr * (wide ? 8 : 4));
@@ -440,7 +441,7 @@ size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide) 
   if (grad) off = align16(off + (size_t)2 * L * nthr * sizeof(u128));
   off = align16(off + (size_t)(nthr / 32) * (1 + m) * sizeof(dd));
   off = align16(off + (size_t)(m + 1) * sizeof(unsigned long long));
-  if (grad) off += (size_t)kMaxLaneBits * 32 * sizeof(LaneMass);
+  if (grad && lane_tab) off += (size_t)kMaxLaneBits * 32 * sizeof(LaneMass);
   return off;
 }
 

@@ -29,7 +29,7 @@ struct FrontierParams {
   int n, m, directed, source, sink;
   int lane_bits, walk_bits, prefix_bits;
   int prune;
-  int pad0;
+  int lane_tab;                 // gradient: lane_w_ex is copied to shared memory
   unsigned long long task_lo;   // first prefix value
   unsigned long long n_tasks;   // number of prefix values (work items)
   unsigned long long budget_ns; // 0 = no deadline

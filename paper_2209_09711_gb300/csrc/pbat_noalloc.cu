@@ -38,7 +38,7 @@
 
 namespace pbat {
 
-size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide);
+size_t frontier_smem_bytes(int n, int m, int L, int nthr, bool grad, bool wide, bool lane_tab);
 const void* frontier_kernel_ptr(bool grad, bool wide);
 cudaError_t launch_frontier(bool grad, bool wide, int grid, int nthr, size_t smem,
                             cudaStream_t st, const FrontierParams& P, const u128* wmid,
@@ -211,7 +211,7 @@ static int run_noalloc(const GraphIn& g, const double* p, const pbat_options* op
   // launch shape: persistent grid, clamped to the partials that fit
   const bool wide = g.n > 32;
   const int nthr = o.block_threads > 0 ? o.block_threads : 128;
-  const size_t smem = frontier_smem_bytes(g.n, m, L, nthr, false, wide);
+  const size_t smem = frontier_smem_bytes(g.n, m, L, nthr, false, wide, false);
   const void* kfn = frontier_kernel_ptr(false, wide);
   cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return fail(PBAT_ECUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));

@@ -49,3 +49,24 @@ def test_frontier_prefix_past_a_warp(pb):
     net = synth.random_small(7300, n=9, m=48, p_lo=0.3, p_hi=0.9)
     for lo in (0, 0x123456789, 2**36 - 1):
         _check(pb, net, range_bits=36, range_lo=lo, range_hi=lo + 1)
+
+
+def test_frontier_at_the_shared_memory_limit(pb):
+    """64 nodes, walks of nine arcs, blocks of 256 threads and the gradient:
+    231,936 bytes of shared memory without the lane masses' table, with it
+    above the limit of 232,448.  The table then stays in the parameters."""
+    net = synth.random_small(7400, n=64, m=63, p_lo=0.3, p_hi=0.9)
+    # a path from source to sink, so that the division reaches it
+    tail = list(range(63))
+    net = synth.Network(64, tail, [k + 1 for k in tail], net.p, 0, 63)
+    for nthr in (256, 128):
+        res = pb.reliability_net(net, grad=True, opts=pb.options(algo=pb.ALGO_FRONTIER, walk_bits=9, block_threads=nthr,
+                                                                 range_bits=44, range_lo=2**44 - 1, range_hi=2**44))
+        want = 1.0
+        for p in net.p:
+            want *= p
+        # one state of the division's 2^19 reaches the sink
+        assert sum(res.Nk) == res.Nk[63] == 1
+        assert abs(res.R - want) <= 1e-14 * want
+        for g, p in zip(res.grad, net.p):
+            assert abs(g - want / p) <= 1e-14 * want / p
