@@ -82,17 +82,17 @@ SHAPES = {
 # fraction is reported as null.
 COUNTS = {
     # random-undirected-n24-m40: fused (L 8, 128 threads, prune 2, occupancy 2, launches 2)
-    "2462730491fd071e": (51074130 / 2**40, 7038720, "profiles/bs_kernel_grad_undirected24x40.md"),
+    "2462730491fd071e": (51051149 / 2**40, 7042560, "profiles/bs_kernel_grad_undirected24x40.md"),
     # random-undirected-n24-m40: r-only (L 8, 160 threads, prune 2, occupancy 2, launches 2)
-    "8a655a848b7ba44c": (18650719 / 2**40, 476416, "profiles/bs_kernel_undirected24x40.md"),
+    "8a655a848b7ba44c": (18666894 / 2**40, 475392, "profiles/bs_kernel_undirected24x40.md"),
     # random-directed-n20-m34: fused (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "b759304bc6095fa7": (1321683 / 2**34, 243712, "profiles/bs_kernel_grad_directed20x34.md"),
+    "b759304bc6095fa7": (1321683 / 2**34, 241920, "profiles/bs_kernel_grad_directed20x34.md"),
     # random-directed-n20-m34: r-only (L 7, 256 threads, prune 2, occupancy 0, launches 2)
-    "9701a4295c31e3d5": (873986 / 2**34, 110080, "profiles/bs_kernel_directed20x34.md"),
+    "9701a4295c31e3d5": (873986 / 2**34, 109824, "profiles/bs_kernel_directed20x34.md"),
     # grid-3x6: fused (L 1, 128 threads, prune 2, occupancy 2, launches 2)
-    "6dd45b0f9bf9cbde": (1735532 / 2**27, 467200, "profiles/bs_kernel_grad_grid3x6.md"),
+    "6dd45b0f9bf9cbde": (1739430 / 2**27, 467456, "profiles/bs_kernel_grad_grid3x6.md"),
     # grid-3x6: r-only (L 1, 192 threads, prune 2, occupancy 2, launches 2)
-    "1dcca192089d5124": (1042493 / 2**27, 178688, "profiles/bs_kernel_grid3x6.md"),
+    "1dcca192089d5124": (1048538 / 2**27, 162048, "profiles/bs_kernel_grid3x6.md"),
 }
 
 SM_COUNT = 152

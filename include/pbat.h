@@ -96,11 +96,13 @@ typedef struct pbat_options {
                            2 = merged: a launch that resolves what the prune can and puts the
                            items left into classes whose prefixes leave the same network, one
                            that walks each class once, and for the gradient one that adds the
-                           prefix arcs' (at most 2^24 items and 2^18 classes, else one
-                           launch); 0 (default) = merged from 2^13 items on, else one launch
-                           (so too a gradient that is all below about 2^-11, under 38 arcs),
-                           or the autotuner's choice when it runs.  Results do not depend on
-                           it. */
+                           prefix arcs' (at most 2^24 items in 2^14 blocks of up to
+                           2^10, and 2^18 classes, else one launch; so too without the up
+                           to 200 MB that they take); 0 (default) = merged from 2^13 items
+                           on, else one launch (so too a gradient that is all below about
+                           2^-11, under 38 arcs), or the autotuner's choice when it runs.
+                           N_k does not depend on it, R and dR/dp only by roundings within
+                           the stated bounds. */
   int range_bits;       /* 0 (default) = whole space.  Otherwise only the states whose
                            first range_bits coordinates, read as an integer, lie in
                            [range_lo, range_hi) -- the divisions range_lo..range_hi-1 of
@@ -167,7 +169,11 @@ typedef struct pbat_graph {
 /*
  * Many networks, each with n_pvec arc-reliability vectors, in one launch of
  * a CUDA graph (captured once and replayed).  Each state's connectivity is
- * computed once and weighted by every p-vector.
+ * computed once and weighted by every p-vector; with the prune on, items whose
+ * prefixes leave the same network are walked once, as in single merged runs
+ * (up to 2^24 items in all; the class memory, up to about 2 GB, is kept with
+ * the batch, 4 GB over all of them, and without room for it every item is
+ * walked by itself).
  * With dRdp_out, the gradient module gives R, N_k and dR/dp for every
  * (network, p-vector); pairs whose R or gradient the bit-sliced fixed-point
  * bounds cannot certify to 1e-12 (small R) are re-run exactly with the
@@ -261,15 +267,15 @@ int pbat_kernel_source(int n_nodes, int n_arcs, const int32_t* tail, const int32
                        const pbat_options* opt, char* buf, size_t cap);
 
 /* Diagnostic, no GPU needed: the CUDA C++ source of the batched bit-sliced
- * module (every network's connectivity program and the persistent kernel)
+ * module (every network's connectivity program and the batch's kernels)
  * for these networks and n_pvec p-vectors.  Same buffer convention as
  * pbat_kernel_source. */
 int pbat_batch_kernel_source(int n_graphs, const pbat_graph* graphs, int n_pvec,
                              const pbat_options* opt, char* buf, size_t cap);
 
 /* Diagnostic, no GPU needed: the CUDA C++ source of the batched gradient
- * module (every network's connectivity program and the persistent kernel
- * that also forms dR/dp for every p-vector).  p: as for
+ * module (every network's connectivity program and the kernels that also
+ * form dR/dp for every p-vector).  p: as for
  * pbat_reliability_batched, or NULL; it decides which arcs may be walk
  * arcs (p in [2^-20, 1 - 2^-20] under every p-vector).  Same buffer
  * convention as pbat_kernel_source. */

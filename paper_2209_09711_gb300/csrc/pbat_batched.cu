@@ -575,7 +575,7 @@ int run_batched(int G, const pbat_graph* graphs, int K, const double* p, pbat_op
   if (o.algo != PBAT_ALGO_FRONTIER) {
     // bit-sliced batched module: R and N_k, or with the gradient the
     // gradient module (every p-vector's exact per-arc sums from one
-    // connectivity pass per state); both one persistent launch
+    // connectivity pass per state); both one launch of a graph
     std::vector<double> Rb((size_t)G * K);
     std::vector<uint64_t> Nb;
     std::vector<double> Gb;
@@ -629,8 +629,8 @@ int run_batched(int G, const pbat_graph* graphs, int K, const double* p, pbat_op
       if (Nk_out) memcpy(Nk_out, Nb.data(), sizeof(uint64_t) * Nb.size());
       if (dRdp_out) memcpy(dRdp_out, Gb.data(), sizeof(double) * Gb.size());
       if (opt) {
-        opt->stats[4] = kns;   // device time of the batched launch
-        opt->stats[5] = 1;     // one persistent kernel for every p-vector
+        opt->stats[4] = kns;   // device time of the batch's graph
+        opt->stats[5] = 1;     // one graph for every network and p-vector
         opt->stats[7] = 1;
       }
       return PBAT_OK;

@@ -767,7 +767,7 @@ void bs_describe(const BsLaunch& bl, int* out6) {
 }  // namespace pbat
 
 // ---------------------------------------------------------------------------
-// Batched bit-sliced enumeration: one module, one persistent kernel.
+// Batched bit-sliced enumeration: one module, its launches replayed as a graph.
 // ---------------------------------------------------------------------------
 namespace pbat {
 

@@ -1361,11 +1361,12 @@ extern "C" __global__ void __launch_bounds__(BS_MERGE_NTHR, 5) bs_kernel_grad_p3
 
 
 // Batched: every network's connectivity program is a struct of static
-// functions (inv, var) with its sizes as constants; one persistent kernel
-// takes (network, prefix) items from one ticket -- networks with the most
-// items first -- and switches to that network's connectivity function
-// (bsb_conn), which only stages the item's 2^L connectivity words in shared
-// memory.  The accumulate (bsb_finish) is written once in the kernel body,
+// functions (inv, var, and sig where items are merged) with its sizes as
+// constants.  The walking kernel takes one item of every class -- or, where
+// items are not merged, (network, prefix) items from one ticket, networks
+// with the most items first -- and switches to that network's connectivity
+// function (bsb_conn), which only stages the item's 2^L connectivity words in
+// shared memory.  The accumulate (bsb_finish) is written once in the kernel body,
 // so the module's compile time barely grows with the number of networks: it
 // weights each word by every p-vector, 16 at a time in registers (byte
 // tables interleaved by p-vector, read through L1), and adds each item's

@@ -324,7 +324,7 @@ def test_time_limit_of_merged_runs(pb):
         for _ in range(2):
             o = pb.options(autotune=0, time_budget_s=10.0)
             R, Nk, _ = pb.reliability_batched(nets, pvecs, grad=grad, opts=o)
-        if grad:   # (the walk takes 0.8 of the run, the fold after it 0.1)
+        if grad:   # (the fold, last, takes a tenth to a quarter of the run)
             with pytest.raises(pb.PbatError, match="PBAT_ETIMEOUT"):
                 pb.reliability_batched(nets, pvecs, grad=True,
                                        opts=pb.options(autotune=0, time_budget_s=0.92e-9 * o.stats[4]))
