@@ -266,22 +266,27 @@ def test_ranges_of_other_widths_plan_for_themselves(pb, wide_first, grad):
     seed = 640 + 2 * wide_first + grad
     # by default: 2^10 items a division, merged from 2^13 on
     net = synth.random_small(seed, n=12, m=30, p_lo=0.3, p_hi=0.95)
-    widths = [(0, 1, 1), (5, 12, 1), (8, 16, 3 if grad else 2), (0, 64, 3 if grad else 2), (7, 7, 1)]
+    merged = 3 if grad else 2
+    widths = [(0, 1, 1), (5, 12, 1), (8, 16, merged), (0, 64, merged), (7, 7, 1), (9, 42, merged)]
     for lo, hi, launches in reversed(widths) if wide_first else widths:
         opt = dict(range_bits=6, range_lo=lo, range_hi=hi, walk_bits=4, algo=pb.ALGO_BITSLICE)
         res = pb.reliability_net(net, grad=grad, opts=pb.options(**opt))
         assert res.stats[5] == launches, (lo, hi)
         one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
         assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+        for x, y in zip(res.grad if grad else (), one.grad if grad else ()):
+            assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (lo, hi, x, y)
     # merged when asked for: 2^18 items a division, at most 2^24 merged
     net = synth.random_small(seed + 10, n=9, m=36, p_lo=0.3, p_hi=0.95)
-    widths = [(3, 4, 3 if grad else 2), (64, 128, 3 if grad else 2), (64, 129, 1), (0, 256, 1)]
+    widths = [(3, 4, merged), (64, 128, merged), (64, 129, 1), (0, 256, 1), (5, 30, merged)]
     for lo, hi, launches in reversed(widths) if wide_first else widths:
         opt = dict(range_bits=8, range_lo=lo, range_hi=hi, prune=2, walk_bits=0, algo=pb.ALGO_BITSLICE)
         res = pb.reliability_net(net, grad=grad, opts=pb.options(launches=2, **opt))
         assert res.stats[5] == launches, (lo, hi)
         one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
         assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+        for x, y in zip(res.grad if grad else (), one.grad if grad else ()):
+            assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (lo, hi, x, y)
 
 
 @pytest.mark.gpu
@@ -496,3 +501,21 @@ def test_description_of_a_merged_plan(pb, grad):
         assert plan.read().stats[5] == ((3 if grad else 2) if launches == 2 else 1)
         d = plan.describe()
         assert d["blocks"] == blocks and d["prefix_bits"] == 10, d
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("bits, lo, hi, merged", [(10, 0, 1 << 10, True), (12, 700, 3100, True), (3, 2, 7, True),
+                                                  (16, 5, 50001, False), (20, 3, 1 << 18, False)])
+def test_default_plans_of_wide_ranges(pb, bits, lo, hi, merged):
+    """Ranges by the planner's own lengths, whole, ragged and of more blocks
+    than are merged, against one launch."""
+    tail, head, rng = synth.random_connected_undirected(14, 34, 77)
+    net = synth.Network(14, tail, head, synth.uniform_p(rng, 34, 0.6, 0.95), 0, 13)
+    for grad in (False, True):
+        opt = dict(range_bits=bits, range_lo=lo, range_hi=hi, autotune=0, algo=pb.ALGO_BITSLICE)
+        res = pb.reliability_net(net, grad=grad, opts=pb.options(**opt))
+        one = pb.reliability_net(net, grad=grad, opts=pb.options(launches=1, **opt))
+        assert res.stats[5] == ((3 if grad else 2) if merged else 1)
+        assert res.Nk == one.Nk and _same(res.R, one.R, 2 * 2.0**-53 * one.R + 2.0**-53)
+        for x, y in zip(res.grad if grad else (), one.grad if grad else ()):
+            assert _same(x, y, 2 * 2.0**-53 * abs(y) + 2.0**-56), (x, y)
